@@ -23,9 +23,12 @@
 // shuffle dot products, no block barriers).  All reductions have a fixed
 // order, so the factors are identical from run to run.  Converged factors are
 // copied from per-worker scratch to a bump-allocated arena; blocks that do not
-// fit are reported and re-run after the arena grows.  The factor columns are
-// kept as float pairs and the residuals formed in double-float arithmetic; the
-// FP64 pipe (64 cycles per warp instruction) is left to the stopping test.
+// fit are reported and re-run after the arena grows.  The CTA workers keep the
+// factor columns as float pairs and form the residuals in double-float
+// arithmetic; the warp workers keep them in FP64 and form the residuals with
+// FP64 FMAs (measured: the float-pair residuals are 24% faster on the large
+// blocks of a level-8 sphere with 80-panel leaves, 5-8% slower on the small
+// blocks, where the FP32 units are already the busier pipe).
 #include <algorithm>
 #include <cmath>
 #include <map>
@@ -39,6 +42,7 @@ namespace hm {
 
 // CTA sizes of the persistent kernel (the autotuner picks one; 128 by default)
 constexpr int ACA_THREADS = 128;
+constexpr int ACA_MAX_WARPS = 8;
 constexpr int SMALL_MAX_DIM = 256;  // warp-mode blocks: m, n <= this
 constexpr int HUGE_SUM = 2560;      // CTA-mode blocks with m + n above this use the large scratch
 // per-warp shared doubles in warp mode: fixed record, U/W row values, bitmaps, norm terms
@@ -77,37 +81,38 @@ struct AcaArgs {
 };
 
 struct Best {
-    float h, l;  // the signed value, a normalised pair
-    int idx;     // index (INT_MAX = none)
+    double a;  // |value|
+    int idx;   // index (INT_MAX = none)
+    double v;  // signed value
 };
 
-// larger |h + l| (of normalised pairs: by h, then by l with h's sign), the
-// lower index on ties; a Best without an index loses to any other but a NaN
 __device__ __forceinline__ bool better(const Best &x, const Best &y) {
-    if (x.idx == 0x7fffffff) return false;
-    if (y.idx == 0x7fffffff) return x.h == x.h;
-    const float xa = fabsf(x.h), ya = fabsf(y.h);
-    if (xa != ya) return xa > ya;
-    const float xl = x.h < 0.0f ? -x.l : x.l, yl = y.h < 0.0f ? -y.l : y.l;
-    return xl > yl || (xl == yl && x.idx < y.idx);
+    return x.a > y.a || (x.a == y.a && x.idx < y.idx);
 }
 
 __device__ __forceinline__ Best warp_argmax(Best b) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         Best c;
-        c.h = __shfl_xor_sync(0xffffffffu, b.h, o);
-        c.l = __shfl_xor_sync(0xffffffffu, b.l, o);
+        c.a = __shfl_xor_sync(0xffffffffu, b.a, o);
         c.idx = __shfl_xor_sync(0xffffffffu, b.idx, o);
+        c.v = __shfl_xor_sync(0xffffffffu, b.v, o);
         if (better(c, b)) b = c;
     }
     return b;
+}
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
 // shared scratch of one ACA worker (CTA or warp)
 struct AcaShared {
     float *fix;     // [64]  fixed panel record (float panel table row)
     double *vec;    // [kmax] U(i_r, :) or W(j_r, :)
+    double *red;    // [warps] sum partials (CTA mode)
     Best *bred;     // [warps] argmax partials (CTA mode)
     uint32_t *urow, *ucol;
     long long *ibc; // broadcast slot (CTA mode)
@@ -119,55 +124,99 @@ constexpr int NORM_STRIDE = 2 + 2 * MAX_KMAX;
 
 // Terms of the Frobenius norm of the approximant after step r, accumulated in
 // FP32 from the high parts of the factor columns (the estimate only
-// decides when to stop): res[l] = u_r . u_l, res[NORM_W + l] = w_r . w_l for
-// l <= r.  Eight columns per pass over the vectors; the lanes' sums of the
-// eight are reduced together (each exchange halves the columns a lane still
-// carries), then one shared-memory round over the warps.
-constexpr int NORM_W = MAX_KMAX + 1;
+// decides when to stop): res[0] = |u_r|^2, res[1] = |w_r|^2,
+// res[2 + l] = u_r . u_l, res[2 + r + l] = w_l . w_r (l < r).  One pass over
+// the columns, per-warp shuffle reductions, one shared-memory round.
 template <bool CTA, int NT>
-__device__ __noinline__ void norm_terms(const FF *U, const FF *W, int m, int n, int r, const AcaShared &sh) {
+__device__ void norm_terms(const float *Uf, const float *Wf, int m, int n, int r, const AcaShared &sh) {
     const int gs = CTA ? NT : 32, t = CTA ? (int)threadIdx.x : (int)(threadIdx.x & 31);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nvals = 2 + 2 * r;
+    const float *ur = Uf + (int64_t)r * m, *wr = Wf + (int64_t)r * n;
     float *st = CTA ? sh.stage + warp * NORM_STRIDE : sh.stage;
-#pragma unroll 1
-    for (int side = 0; side < 2; ++side, st += NORM_W) {
-        const FF *X = side ? W : U;
-        const int cnt = side ? n : m;
-        const FF *xr = X + (int64_t)r * cnt;
-#pragma unroll 1
-        for (int c0 = 0; c0 <= r; c0 += 8) {
-            float acc[8];
+    for (int c0 = 0; c0 < nvals; c0 += 8) {
+        float acc[8];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) acc[c] = 0.0f;
-            const FF *xc = X + (int64_t)c0 * cnt;
-#pragma unroll 1
-            for (int k = t; k < cnt; k += gs) {
-                const float u = xr[k].h;
-                const FF *p = xc + k;
+        for (int c = 0; c < 8; ++c) acc[c] = 0.0f;
+        for (int k = t; k < m; k += gs) {
+            const float u = ur[k];
 #pragma unroll
-                for (int c = 0; c < 8; ++c, p += cnt)
-                    if (c0 + c <= r) acc[c] = fmaf(u, p->h, acc[c]);
+            for (int c = 0; c < 8; ++c) {
+                const int v = c0 + c;
+                if (v == 0) acc[c] = fmaf(u, u, acc[c]);
+                else if (v >= 2 && v < 2 + r) acc[c] = fmaf(u, Uf[(int64_t)(v - 2) * m + k], acc[c]);
             }
+        }
+        for (int j = t; j < n; j += gs) {
+            const float w = wr[j];
 #pragma unroll
-            for (int h = 4, o = 16; h > 0; h >>= 1, o >>= 1) {
-                const bool up = lane & o;
-#pragma unroll
-                for (int c = 0; c < h; ++c) {
-                    const float mine = up ? acc[c + h] : acc[c], other = up ? acc[c] : acc[c + h];
-                    acc[c] = mine + __shfl_xor_sync(0xffffffffu, other, o);
-                }
+            for (int c = 0; c < 8; ++c) {
+                const int v = c0 + c;
+                if (v == 1) acc[c] = fmaf(w, w, acc[c]);
+                else if (v >= 2 + r && v < nvals) acc[c] = fmaf(w, Wf[(int64_t)(v - 2 - r) * n + j], acc[c]);
             }
-            float a = acc[0];
-            a += __shfl_xor_sync(0xffffffffu, a, 2);
-            a += __shfl_xor_sync(0xffffffffu, a, 1);
-            if ((lane & 3) == 0 && c0 + (lane >> 2) <= r) st[c0 + (lane >> 2)] = a;
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            float a = acc[c];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (lane == 0 && c0 + c < nvals) st[c0 + c] = a;
         }
     }
     if (CTA) {
         __syncthreads();
-#pragma unroll 1
-        for (int v = t; v < NORM_STRIDE; v += gs) {
-            if ((v < NORM_W ? v : v - NORM_W) > r) continue;
+        for (int v = t; v < nvals; v += gs) {
+            float a = 0.0f;
+            for (int w = 0; w < NT / 32; ++w) a += sh.stage[w * NORM_STRIDE + v];
+            sh.res[v] = a;
+        }
+        __syncthreads();
+    } else {
+        __syncwarp();
+    }
+}
+
+template <bool CTA, int NT>
+__device__ void norm_terms(const FF *Uf, const FF *Wf, int m, int n, int r, const AcaShared &sh) {
+    const int gs = CTA ? NT : 32, t = CTA ? (int)threadIdx.x : (int)(threadIdx.x & 31);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nvals = 2 + 2 * r;
+    const FF *ur = Uf + (int64_t)r * m, *wr = Wf + (int64_t)r * n;
+    float *st = CTA ? sh.stage + warp * NORM_STRIDE : sh.stage;
+    for (int c0 = 0; c0 < nvals; c0 += 8) {
+        float acc[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[c] = 0.0f;
+        for (int k = t; k < m; k += gs) {
+            const float u = ur[k].h;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const int v = c0 + c;
+                if (v == 0) acc[c] = fmaf(u, u, acc[c]);
+                else if (v >= 2 && v < 2 + r) acc[c] = fmaf(u, Uf[(int64_t)(v - 2) * m + k].h, acc[c]);
+            }
+        }
+        for (int j = t; j < n; j += gs) {
+            const float w = wr[j].h;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const int v = c0 + c;
+                if (v == 1) acc[c] = fmaf(w, w, acc[c]);
+                else if (v >= 2 + r && v < nvals) acc[c] = fmaf(w, Wf[(int64_t)(v - 2 - r) * n + j].h, acc[c]);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            float a = acc[c];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (lane == 0 && c0 + c < nvals) st[c0 + c] = a;
+        }
+    }
+    if (CTA) {
+        __syncthreads();
+        for (int v = t; v < nvals; v += gs) {
             float a = 0.0f;
             for (int w = 0; w < NT / 32; ++w) a += sh.stage[w * NORM_STRIDE + v];
             sh.res[v] = a;
@@ -185,6 +234,17 @@ struct Grp {
     __device__ __forceinline__ static void sync() {
         if (CTA) __syncthreads();
         else __syncwarp();
+    }
+    __device__ __forceinline__ static double sum(double v, const AcaShared &sh) {
+        v = warp_sum(v);
+        if (!CTA) return v;
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        if (lane == 0) sh.red[w] = v;
+        __syncthreads();
+        double t = 0.0;
+        for (int k = 0; k < NT / 32; ++k) t += sh.red[k];
+        __syncthreads();
+        return t;
     }
     __device__ __forceinline__ static Best argmax(Best b, const AcaShared &sh) {
         b = warp_argmax(b);
@@ -211,42 +271,46 @@ struct Grp {
 
 __device__ __forceinline__ bool bit(const uint32_t *bm, int k) { return (bm[k >> 5] >> (k & 31)) & 1u; }
 
-// Entry of the Galerkin matrix for the pair of the panel whose shared-memory
-// record is `fix` (at Morton position gf, fixed during a pass) and the panel at
-// position gv, read from the float panel table.  Far-field pairs in
-// double-float; touching pairs (which admissible blocks do not contain in
-// practice) by the FP64 regularised rule, with the row's panel first.
-// The regular rule runs over the points of the row-role panel in a rolled
-// loop that reads that panel's record as it goes, and loads the column-role
-// record into registers up front.  G(x, y) = G(y, x), so the pair is evaluated
-// with the fixed record in the row role in both passes: the varying record,
-// read from L2, is then loaded once per entry.  The value is the same entry up
-// to rounding (~1e-15 relative, the order of the double-float sums).
-// One out-of-line copy serves every call: with the passes' and the norm's
-// code unrolled and repeated (160 KB, now 110 KB with the rare paths) a quarter
-// of the warps' time was spent waiting for instructions.  655,220 panels,
-// leaves of 80 rows, eps 1e-6: 263 -> 220 ms (stalls per issue, 81,920 panels:
-// no instruction 2.5 -> 0.7, long scoreboard 2.0, wait 1.4; issue slots 65 %
-// busy, FP32 pipe 50 %).
-__device__ __noinline__ static FF aca_entry(const float *fix, bool fixed_is_row, int gf, int gv, const AcaArgs &A) {
-    const float *rec = A.pf + gv;
-    const int st = (int)A.npad;
+// One out-of-line copy of the far-field evaluation shared by every call site
+// (row and column passes, CTA and warp workers).
+__device__ __noinline__ static FF far_entry(const float *r, int rs, const float *c, int cs, const QuadParams &qp) {
     FF e;
-    const int32_t vf[3] = {__float_as_int(fix[PF_VID]), __float_as_int(fix[PF_VID + 1]),
-                           __float_as_int(fix[PF_VID + 2])};
-    const int32_t vv[3] = {__float_as_int(rec[(int64_t)PF_VID * st]), __float_as_int(rec[(int64_t)(PF_VID + 1) * st]),
-                           __float_as_int(rec[(int64_t)(PF_VID + 2) * st])};
-    const int kind = shared_vertices(vf, vv);
-    if (kind) {
-        const double *area = A.pt + (int64_t)PT_AREA * A.npad;
-        return ff_from(fixed_is_row ? singular_entry_serial(A.V, vf, vv, kind, area[gf], area[gv], A.qp)
-                                    : singular_entry_serial(A.V, vv, vf, kind, area[gv], area[gf], A.qp));
-    }
-    if (!regular_entry_ff2(fix, 1, rec, st, A.qp, e.h, e.l)) e = regular_entry_near(fix, 1, rec, st, A.qp);
+    if (!regular_entry_ff2(r, rs, c, cs, qp, e.h, e.l)) e = regular_entry_near(r, rs, c, cs, qp);
     return e;
 }
 
-// ACA of one block; U (m x kmax) and W (n x kmax) column-major
+// Entry of the Galerkin matrix for the row panel at Morton position gi and the
+// column panel at gj; `fix` is the shared-memory record of the panel that is
+// fixed during the pass (the row panel when fixed_is_row, else the column
+// panel), the other record is read from the float panel table.  Far-field
+// pairs in float-float; touching pairs (which admissible blocks do not contain
+// in practice) by the FP64 regularised rule.
+__device__ __forceinline__ FF aca_entry(const float *fix, bool fixed_is_row, int64_t gi, int64_t gj,
+                                        const AcaArgs &A) {
+    const int64_t var = fixed_is_row ? gj : gi;
+    const float *rec = A.pf + var;
+    const int64_t st = A.npad;
+    const int32_t vf[3] = {__float_as_int(fix[PF_VID]), __float_as_int(fix[PF_VID + 1]),
+                           __float_as_int(fix[PF_VID + 2])};
+    const int32_t vv[3] = {__float_as_int(rec[PF_VID * st]), __float_as_int(rec[(PF_VID + 1) * st]),
+                           __float_as_int(rec[(PF_VID + 2) * st])};
+    const int kind = shared_vertices(vf, vv);
+    if (kind) {
+        const double ai = A.pt[(int64_t)PT_AREA * A.npad + gi], aj = A.pt[(int64_t)PT_AREA * A.npad + gj];
+        return ff_from(fixed_is_row ? singular_entry_serial(A.V, vf, vv, kind, ai, aj, A.qp)
+                                    : singular_entry_serial(A.V, vv, vf, kind, ai, aj, A.qp));
+    }
+    // The regular rule sums over the points of the row-role panel in a rolled
+    // loop that reads that panel's record as it goes, and loads the
+    // column-role record into registers up front.  G(x, y) = G(y, x), so the
+    // pair is evaluated with the fixed (shared-memory) record in the row role
+    // in both passes: the varying record, read from L2, is then loaded once
+    // per entry instead of once per outer step.  The value is the same entry
+    // up to rounding (~1e-14 relative, the order of the double-float sums).
+    return far_entry(fix, 1, rec, (int)st, A.qp);
+}
+
+// ACA of one block (CTA workers); U (m x kmax) and W (n x kmax) column-major
 // in scratch, as float pairs: the residual rows and columns (entry minus the
 // rank-one terms so far) are formed in double-float arithmetic on the FP32
 // units, to ~2^-48 of the largest term, like the entries themselves.
@@ -256,96 +320,85 @@ __device__ int aca_block(const AcaArgs &A, int rb, int m, int cb, int n, FF *U, 
     using G = Grp<CTA, NT>;
     const int gs = G::size(), t = G::rank();
     const int wr = (m + 31) >> 5, wc = (n + 31) >> 5;
-#pragma unroll 1
     for (int k = t; k < wr; k += gs) sh.urow[k] = 0u;
-#pragma unroll 1
     for (int k = t; k < wc; k += gs) sh.ucol[k] = 0u;
     G::sync();
     const int rmax = min(A.kmax, min(m, n));
-    const float tiny = 8.881784197001252e-16f;  // 2^-50
+    const double tiny = 8.881784197001252e-16;  // 2^-50
     FF *vec = reinterpret_cast<FF *>(sh.vec);
     int r = 0, i = 0;
-    const double eps2 = A.eps * A.eps;
-    double s2 = 0.0;
-    float delta1 = 0.0f;
+    double s2 = 0.0, delta1 = 0.0;
     bool converged = false;
     while (r < rmax) {
-        // pass 0: residual of row i, and its largest entry in an unused column
-        // (jp); pass 1: residual of column jp and its largest in an unused row.
-        // One copy of the code for both (see aca_entry).
-        int jp = 0;
-        bool retry = false;
-        Best best;
-#pragma unroll 1
-        for (int pass = 0; pass < 2; ++pass) {
-            const int fp = pass ? cb + jp : rb + i, v0 = pass ? rb : cb, nvar = pass ? m : n;
-            const FF *src = pass ? W + jp : U + i;  // row jp of W or row i of U
-            const int src_ld = pass ? n : m;
-            FF *M = pass ? U : W, *dst = M + (int64_t)r * nvar;
-            const uint32_t *used = pass ? sh.urow : sh.ucol;
-#pragma unroll 1
-            for (int q = t; q < PF_ROWS; q += gs) sh.fix[q] = A.pf[(int64_t)q * A.npad + fp];
-#pragma unroll 1
-            for (int l = t; l < r; l += gs) vec[l] = src[(int64_t)l * src_ld];
-            G::sync();
-            best = Best{0.0f, 0.0f, 0x7fffffff};
-#pragma unroll 1
-            for (int k = t; k < nvar; k += gs) {
-                const FF e = aca_entry(sh.fix, pass == 0, fp, v0 + k, A);
-                float hs = e.h, lo = e.l;
-                const FF *p = M + k;
-#pragma unroll 4
-                for (int l = 0; l < r; ++l, p += nvar) ff_sub_prod(hs, lo, vec[l], *p);
-                FF v;
-                fast_two_sum(hs, lo, v.h, v.l);
-                dst[k] = v;
-                if (!bit(used, k)) {
-                    const Best c{v.h, v.l, k};
-                    if (better(c, best)) best = c;
-                }
-            }
-            best = G::argmax(best, sh);
-            if (pass == 0) {
-                if (t == 0) sh.urow[i >> 5] |= 1u << (i & 31);
-                G::sync();
-                const FF delta{best.h, best.l};
-                const bool zero_row = (r == 0) ? (delta.h == 0.0f) : (fabsf(delta.h) <= tiny * delta1);
-                if (zero_row || best.idx == 0x7fffffff) {
-                    retry = true;
-                    break;
-                }
-                if (r == 0) delta1 = fabsf(delta.h);
-                jp = best.idx;
-                const FF inv_delta = ff_recip(delta);
-#pragma unroll 2
-                for (int j = t; j < n; j += gs) dst[j] = ff_mul(dst[j], inv_delta);
+        // ---- residual of row i ----
+        for (int q = t; q < PF_ROWS; q += gs) sh.fix[q] = A.pf[(int64_t)q * A.npad + rb + i];
+        for (int l = t; l < r; l += gs) vec[l] = U[(int64_t)l * m + i];
+        G::sync();
+        Best best{-1.0, 0x7fffffff, 0.0};
+        for (int j = t; j < n; j += gs) {
+            const FF e = aca_entry(sh.fix, true, rb + i, cb + j, A);
+            float hs = e.h, lo = e.l;
+            for (int l = 0; l < r; ++l) ff_sub_prod(hs, lo, vec[l], W[(int64_t)l * n + j]);
+            FF v;
+            fast_two_sum(hs, lo, v.h, v.l);
+            W[(int64_t)r * n + j] = v;
+            if (!bit(sh.ucol, j)) {
+                const double vd = ff_to(v);
+                const Best c{fabs(vd), j, vd};
+                if (better(c, best)) best = c;
             }
         }
-        if (retry) {
+        best = G::argmax(best, sh);
+        if (t == 0) sh.urow[i >> 5] |= 1u << (i & 31);
+        G::sync();
+        const double delta = best.v;
+        const bool zero_row = (r == 0) ? (delta == 0.0) : (fabs(delta) <= tiny * delta1);
+        if (zero_row || best.idx == 0x7fffffff) {
             // lowest unused row
             int cand = 0x7fffffff;
-#pragma unroll 1
             for (int k = t; k < m; k += gs)
                 if (!bit(sh.urow, k)) { cand = k; break; }
-            Best c{0.0f, 0.0f, cand};
+            Best c{0.0, cand, 0.0};
             c = G::argmax(c, sh);
             if (c.idx == 0x7fffffff) break;
             i = c.idx;
             continue;
         }
+        if (r == 0) delta1 = fabs(delta);
+        const int jp = best.idx;
+        const FF inv_delta = ff_from(1.0 / delta);
+        for (int j = t; j < n; j += gs) W[(int64_t)r * n + j] = ff_mul(W[(int64_t)r * n + j], inv_delta);
+        // ---- residual of column jp ----
+        for (int q = t; q < PF_ROWS; q += gs) sh.fix[q] = A.pf[(int64_t)q * A.npad + cb + jp];
+        for (int l = t; l < r; l += gs) vec[l] = W[(int64_t)l * n + jp];
+        G::sync();
+        Best nb{-1.0, 0x7fffffff, 0.0};
+        for (int k = t; k < m; k += gs) {
+            const FF e = aca_entry(sh.fix, false, rb + k, cb + jp, A);
+            float hs = e.h, lo = e.l;
+            for (int l = 0; l < r; ++l) ff_sub_prod(hs, lo, vec[l], U[(int64_t)l * m + k]);
+            FF u;
+            fast_two_sum(hs, lo, u.h, u.l);
+            U[(int64_t)r * m + k] = u;
+            if (!bit(sh.urow, k)) {
+                const double ud = ff_to(u);
+                const Best c{fabs(ud), k, ud};
+                if (better(c, nb)) nb = c;
+            }
+        }
         if (t == 0) sh.ucol[jp >> 5] |= 1u << (jp & 31);
         // ---- Frobenius norm of the approximant ----
         norm_terms<CTA, NT>(U, W, m, n, r, sh);
         const float *res = CTA ? sh.res : sh.stage;
-        float cross = 0.0f;
-#pragma unroll 1
-        for (int l = 0; l < r; ++l) cross = fmaf(res[l], res[NORM_W + l], cross);
-        const double step2 = (double)res[r] * (double)res[NORM_W + r];
-        s2 += 2.0 * (double)cross + step2;
+        const double nu2 = res[0], nw2 = res[1];
+        double cross = 0.0;
+        for (int l = 0; l < r; ++l) cross += (double)res[2 + l] * (double)res[2 + r + l];
+        s2 = s2 + 2.0 * cross + nu2 * nw2;
         ++r;
-        if (step2 <= eps2 * s2) { converged = true; break; }
-        if (best.idx == 0x7fffffff) { converged = true; break; }
-        i = best.idx;
+        nb = G::argmax(nb, sh);
+        if (sqrt(nu2) * sqrt(nw2) <= A.eps * sqrt(s2)) { converged = true; break; }
+        if (nb.idx == 0x7fffffff) { converged = true; break; }
+        i = nb.idx;
         G::sync();
     }
     *hit_kmax = !converged && r == A.kmax && r < min(m, n);
@@ -373,21 +426,128 @@ __device__ void aca_store(const AcaArgs &A, int64_t b, int m, int n, int k, cons
     // reads contiguously
     double *dst = A.arena + off;
     const int64_t mk = (int64_t)m * k, nk = (int64_t)n * k;
-#pragma unroll 2
     for (int64_t e = t; e < mk; e += gs) dst[e] = ff_to(U[e]);
-    dst += mk;
-    const int kd = max(k, 1);
-    int j = t / kd, l = t - j * kd;
-    const int dj = gs / kd, dl = gs - dj * kd;
-#pragma unroll 1
     for (int64_t e = t; e < nk; e += gs) {
-        dst[e] = ff_to(W[(int64_t)l * n + j]);
-        l += dl;
-        j += dj;
-        if (l >= k) {
-            l -= k;
-            ++j;
+        const int64_t j = e / k, l = e - j * k;
+        dst[mk + e] = ff_to(W[l * n + j]);
+    }
+}
+
+// The same ACA with the factor columns in FP64 (U, W) plus FP32 shadows (Uf,
+// Wf) for the norm terms, the rank-one updates of the residuals in FP64.
+// Used by the warp workers (small blocks), where the FP32 units are the
+// busier pipe; the CTA workers (large blocks) use the float-pair form.
+template <bool CTA, int NT>
+__device__ int aca_block_d(const AcaArgs &A, int rb, int m, int cb, int n, double *U, double *W, float *Uf, float *Wf,
+                         const AcaShared &sh, bool *hit_kmax) {
+    using G = Grp<CTA, NT>;
+    const int gs = G::size(), t = G::rank();
+    const int wr = (m + 31) >> 5, wc = (n + 31) >> 5;
+    for (int k = t; k < wr; k += gs) sh.urow[k] = 0u;
+    for (int k = t; k < wc; k += gs) sh.ucol[k] = 0u;
+    G::sync();
+    const int rmax = min(A.kmax, min(m, n));
+    const double tiny = 8.881784197001252e-16;  // 2^-50
+    int r = 0, i = 0;
+    double s2 = 0.0, delta1 = 0.0;
+    bool converged = false;
+    while (r < rmax) {
+        // ---- residual of row i ----
+        for (int q = t; q < PF_ROWS; q += gs) sh.fix[q] = A.pf[(int64_t)q * A.npad + rb + i];
+        for (int l = t; l < r; l += gs) sh.vec[l] = U[(int64_t)l * m + i];
+        G::sync();
+        Best best{-1.0, 0x7fffffff, 0.0};
+        for (int j = t; j < n; j += gs) {
+            double v = ff_to(aca_entry(sh.fix, true, rb + i, cb + j, A));
+            for (int l = 0; l < r; ++l) v -= sh.vec[l] * W[(int64_t)l * n + j];
+            W[(int64_t)r * n + j] = v;
+            if (!bit(sh.ucol, j)) {
+                const Best c{fabs(v), j, v};
+                if (better(c, best)) best = c;
+            }
         }
+        best = G::argmax(best, sh);
+        if (t == 0) sh.urow[i >> 5] |= 1u << (i & 31);
+        G::sync();
+        const double delta = best.v;
+        const bool zero_row = (r == 0) ? (delta == 0.0) : (fabs(delta) <= tiny * delta1);
+        if (zero_row || best.idx == 0x7fffffff) {
+            // lowest unused row
+            int cand = 0x7fffffff;
+            for (int k = t; k < m; k += gs)
+                if (!bit(sh.urow, k)) { cand = k; break; }
+            Best c{0.0, cand, 0.0};
+            c = G::argmax(c, sh);
+            if (c.idx == 0x7fffffff) break;
+            i = c.idx;
+            continue;
+        }
+        if (r == 0) delta1 = fabs(delta);
+        const int jp = best.idx;
+        const double inv_delta = 1.0 / delta;
+        for (int j = t; j < n; j += gs) {
+            const double w = W[(int64_t)r * n + j] * inv_delta;
+            W[(int64_t)r * n + j] = w;
+            Wf[(int64_t)r * n + j] = (float)w;
+        }
+        // ---- residual of column jp ----
+        for (int q = t; q < PF_ROWS; q += gs) sh.fix[q] = A.pf[(int64_t)q * A.npad + cb + jp];
+        for (int l = t; l < r; l += gs) sh.vec[l] = W[(int64_t)l * n + jp];
+        G::sync();
+        Best nb{-1.0, 0x7fffffff, 0.0};
+        for (int k = t; k < m; k += gs) {
+            double u = ff_to(aca_entry(sh.fix, false, rb + k, cb + jp, A));
+            for (int l = 0; l < r; ++l) u -= sh.vec[l] * U[(int64_t)l * m + k];
+            U[(int64_t)r * m + k] = u;
+            Uf[(int64_t)r * m + k] = (float)u;
+            if (!bit(sh.urow, k)) {
+                const Best c{fabs(u), k, u};
+                if (better(c, nb)) nb = c;
+            }
+        }
+        if (t == 0) sh.ucol[jp >> 5] |= 1u << (jp & 31);
+        // ---- Frobenius norm of the approximant ----
+        norm_terms<CTA, NT>(Uf, Wf, m, n, r, sh);
+        const float *res = CTA ? sh.res : sh.stage;
+        const double nu2 = res[0], nw2 = res[1];
+        double cross = 0.0;
+        for (int l = 0; l < r; ++l) cross += (double)res[2 + l] * (double)res[2 + r + l];
+        s2 = s2 + 2.0 * cross + nu2 * nw2;
+        ++r;
+        nb = G::argmax(nb, sh);
+        if (sqrt(nu2) * sqrt(nw2) <= A.eps * sqrt(s2)) { converged = true; break; }
+        if (nb.idx == 0x7fffffff) { converged = true; break; }
+        i = nb.idx;
+        G::sync();
+    }
+    *hit_kmax = !converged && r == A.kmax && r < min(m, n);
+    return r;
+}
+
+template <bool CTA, int NT>
+__device__ void aca_store(const AcaArgs &A, int64_t b, int m, int n, int k, const double *U, const double *W,
+                          const AcaShared &sh) {
+    using G = Grp<CTA, NT>;
+    const int gs = G::size(), t = G::rank();
+    const int64_t need = (int64_t)k * (m + n);
+    long long off = 0;
+    if (t == 0) off = (long long)atomicAdd(A.arena_top, (unsigned long long)need);
+    off = G::bcast(off, sh);
+    if (t == 0) A.rank[b] = k;
+    if ((int64_t)off + need > A.arena_cap) {
+        if (t == 0) A.uw_off[b] = -1;
+        return;
+    }
+    if (t == 0) A.uw_off[b] = (int64_t)off;
+    // U_b column-major (m x k); W_b row-major (n x k): row j of W_b holds the
+    // k coefficients of column j of the block, which the projection W_b^T x
+    // reads contiguously
+    double *dst = A.arena + off;
+    const int64_t mk = (int64_t)m * k, nk = (int64_t)n * k;
+    for (int64_t e = t; e < mk; e += gs) dst[e] = U[e];
+    for (int64_t e = t; e < nk; e += gs) {
+        const int64_t j = e / k, l = e - j * k;
+        dst[mk + e] = W[l * n + j];
     }
 }
 
@@ -397,6 +557,7 @@ template <int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) aca_kernel(AcaArgs A) {
     constexpr int WARPS = NT / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double s_red[WARPS];
     __shared__ Best s_bred[WARPS];
     __shared__ long long s_ibc;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -404,7 +565,6 @@ __global__ void __launch_bounds__(NT, MINB) aca_kernel(AcaArgs A) {
     // ---------------- phase 1: large blocks, whole CTA ----------------
     // 1a: the huge blocks (and an overflow re-run) on the first big_ctas CTAs,
     // whose scratch fits any block; 1b: the other large blocks on every CTA
-#pragma unroll 1
     for (int tier = 0; tier < 2; ++tier) {
         if (tier == 0 && (int)blockIdx.x >= A.big_ctas) continue;
         if (tier == 1 && A.todo) break;
@@ -412,6 +572,7 @@ __global__ void __launch_bounds__(NT, MINB) aca_kernel(AcaArgs A) {
         double *d = reinterpret_cast<double *>(smem_raw);
         sh.fix = reinterpret_cast<float *>(d);
         sh.vec = d + 32;
+        sh.red = s_red;
         sh.bred = s_bred;
         sh.ibc = &s_ibc;
         sh.urow = reinterpret_cast<uint32_t *>(d + 32 + MAX_KMAX);
@@ -449,13 +610,14 @@ __global__ void __launch_bounds__(NT, MINB) aca_kernel(AcaArgs A) {
         double *d = reinterpret_cast<double *>(smem_raw) + (int64_t)warp * WARP_SMEM_DOUBLES;
         sh.fix = reinterpret_cast<float *>(d);
         sh.vec = d + 32;
+        sh.red = nullptr;
         sh.bred = nullptr;
         sh.ibc = nullptr;
         sh.urow = reinterpret_cast<uint32_t *>(d + 32 + MAX_KMAX);
         sh.ucol = sh.urow + words;
         sh.stage = reinterpret_cast<float *>(d + 32 + MAX_KMAX + words);
         sh.res = sh.stage;
-        FF *U = reinterpret_cast<FF *>(A.scr_small + ((int64_t)blockIdx.x * WARPS + warp) * A.small_stride);
+        double *U = A.scr_small + ((int64_t)blockIdx.x * WARPS + warp) * A.small_stride;
         for (;;) {
             int q = 0;
             if (lane == 0) q = (int)atomicAdd(A.q_small, 1ull);
@@ -464,9 +626,11 @@ __global__ void __launch_bounds__(NT, MINB) aca_kernel(AcaArgs A) {
             const int64_t b = A.work[A.n_big + q];
             const int32_t rb = A.adm[4 * b], re = A.adm[4 * b + 1], cb = A.adm[4 * b + 2], ce = A.adm[4 * b + 3];
             const int m = re - rb, n = ce - cb;
-            FF *W = U + (int64_t)m * A.kmax;
+            double *W = U + (int64_t)m * A.kmax;
+            float *Uf = reinterpret_cast<float *>(W + (int64_t)n * A.kmax);
+            float *Wf = Uf + (int64_t)m * A.kmax;
             bool hit = false;
-            const int k = aca_block<false, NT>(A, rb, m, cb, n, U, W, sh, &hit);
+            const int k = aca_block_d<false, NT>(A, rb, m, cb, n, U, W, Uf, Wf, sh, &hit);
             if (hit && lane == 0) atomicAdd(A.kmax_hit, 1);
             __syncwarp();
             aca_store<false, NT>(A, b, m, n, k, U, W, sh);
@@ -690,7 +854,7 @@ void assemble_aca(const hm_tree *tr, hm_matrix *A, const QuadParams &qp, cudaStr
         a.work = d_work.as<int32_t>();
         a.n_big = n_big;
         a.n_work = (int64_t)work.size();
-        a.small_stride = (int64_t)max_sum_small * kmax;  // U, W as float pairs
+        a.small_stride = ((int64_t)max_sum_small * kmax * 3 + 1) / 2;  // U, W in FP64 + FP32 shadows
         scr_small.alloc(sizeof(double) * a.small_stride * grid * (tc.nt / 32));
         a.scr_small = scr_small.as<double>();
         a.arena_top = ctr4;
