@@ -275,7 +275,7 @@ __device__ __forceinline__ bool bit(const uint32_t *bm, int k) { return (bm[k >>
 // (row and column passes, CTA and warp workers).
 __device__ __noinline__ static FF far_entry(const float *r, int rs, const float *c, int cs, const QuadParams &qp) {
     FF e;
-    if (!regular_entry_ff2(r, rs, c, cs, qp, e.h, e.l)) e = regular_entry_near(r, rs, c, cs, qp);
+    regular_entry_ff2(r, rs, c, cs, qp, e.h, e.l);
     return e;
 }
 

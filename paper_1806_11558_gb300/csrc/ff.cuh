@@ -74,31 +74,7 @@ __device__ __forceinline__ FF ff_from(double x) {
     split_double(x, r.h, r.l);
     return r;
 }
-// h + l of a normalised pair as a double, rounded to nearest.  The FP64 pipe
-// takes 64 cycles per warp instruction and conversions go through it too, so the
-// bits are put together by integer operations: h's bits give a double, l
-// rounded to that double's last place is added to them.  Where h is a power of
-// two (the last place below it is half as large), small, or not finite: by FP64.
-__device__ __forceinline__ double ff_to(FF a) {
-    const uint32_t hb = __float_as_uint(a.h), e = (hb >> 23) & 0xffu;
-    if (e < 52u || e == 255u || (hb & 0x7fffffu) == 0u) return (double)a.h + (double)a.l;
-    // l 2^(52 - (e - 127)), |l| <= 2^(e - 127 - 24)
-    int li = __float2int_rn(__fmul_rn(a.l, __uint_as_float((306u - e) << 23)));
-    li = (int)hb < 0 ? -li : li;
-    const unsigned long long m = ((unsigned long long)(hb & 0x7fffffffu) << 29) + (896ull << 52) + (long long)li;
-    return __longlong_as_double((long long)(m | ((unsigned long long)(hb & 0x80000000u) << 32)));
-}
-
-// 1 / a of a normalised pair, to ~2^-47: the reciprocal y of the high part and
-// its correction y (r + r^2), r = 1 - a y
-__device__ __forceinline__ FF ff_recip(FF a) {
-    const float y = __frcp_rn(a.h);
-    float r = __fmaf_rn(-a.h, y, 1.0f);
-    r = __fmaf_rn(-a.l, y, r);
-    FF o;
-    fast_two_sum(y, __fmul_rn(y, __fmaf_rn(r, r, r)), o.h, o.l);
-    return o;
-}
+__device__ __forceinline__ double ff_to(FF a) { return (double)a.h + (double)a.l; }
 
 // a * b, normalised, to ~2^-47 relative
 __device__ __forceinline__ FF ff_mul(FF a, FF b) {
@@ -303,8 +279,7 @@ __device__ __noinline__ static FF regular_entry_near(const float *__restrict__ R
 
 // Regular entry a_ij = |Ti||Tj|/(4 pi) sum_p sum_q w_p w_q / |x_p - y_q| for
 // panel records R (row, test) and C (column, trial); element k of a record at
-// R[k * rs], as the float pair (eh, el), not normalised.  Returns false, with
-// no value, for a pair that regular_entry_near has to evaluate.
+// R[k * rs].  Returns the float pair (eh, el), not normalised.
 //
 // The squared distances come from the orbits of the rule: with the centroid
 // difference D and the scaled vertex offsets u_k (row) and w_l (column),
@@ -320,7 +295,7 @@ __device__ __noinline__ static FF regular_entry_near(const float *__restrict__ R
 // rounding each, so r^2 carries ~2^-48 |D|^2.  The arithmetic pipe is the bound:
 // about 1,850 operations per entry against 4,200 with the 49 differences.
 // Measured on a sphere of 655,220 panels (leaves of 80 rows, eps 1e-6): near
-// field 153 -> 95 ms, ACA 381 -> 265 ms by this alone.  Against the sum in 80-bit arithmetic
+// field 153 -> 95 ms, ACA 381 -> 265 ms.  Against the sum in 80-bit arithmetic
 // (separations of 3 to 300 radii): 3e-15 rms, where the differences with a
 // first-order root gave 7e-15.
 //
@@ -329,14 +304,19 @@ __device__ __noinline__ static FF regular_entry_near(const float *__restrict__ R
 // of the smallest r^2, |Q| < P, and two inverse distances outweigh a third.
 // Other pairs (a few per row of the near field) take regular_entry_near, as
 // do distances whose squares leave the range where the low parts are normal.
-__device__ __forceinline__ bool regular_entry_ff2(const float *__restrict__ R, int rs, const float *__restrict__ C,
+__device__ __forceinline__ void regular_entry_ff2(const float *__restrict__ R, int rs, const float *__restrict__ C,
                                                   int cs, const QuadParams &qp, float &eh_out, float &el_out) {
     float Dh[3], Dl[3];
     centroid_diff(R, rs, C, cs, Dh, Dl);
     float R0h, R0l;
     ff_dot3(Dh, Dl, Dh, Dl, R0h, R0l);
     const float rad = __fadd_rn(R[PF_RAD * rs], C[PF_RAD * cs]);
-    if (!(R0h >= 9.0f * rad * rad && R0h > 1e-18f && R0h < 1e30f)) return false;
+    if (!(R0h >= 9.0f * rad * rad && R0h > 1e-18f && R0h < 1e30f)) {
+        const FF e = regular_entry_near(R, rs, C, cs, qp);
+        eh_out = e.h;
+        el_out = e.l;
+        return;
+    }
     // w' = -2 w; Q_l for both orbits
     float wh[2][3], wl[2][3], Qh[6], Ql[6];
 #pragma unroll
@@ -451,7 +431,13 @@ __device__ __forceinline__ bool regular_entry_ff2(const float *__restrict__ R, i
     float ah, al;
     fast_two_sum(acc_h, acc_l, ah, al);
     entry_scale(ah, al, R, rs, C, cs, eh_out, el_out);
-    return true;
+}
+
+__device__ __forceinline__ double regular_entry_ff(const float *__restrict__ R, int rs, const float *__restrict__ C,
+                                                   int cs, const QuadParams &qp) {
+    float eh, el;
+    regular_entry_ff2(R, rs, C, cs, qp, eh, el);
+    return (double)eh + (double)el;
 }
 
 }  // namespace hm

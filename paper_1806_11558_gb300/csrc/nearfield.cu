@@ -83,21 +83,15 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t phase,
     }
 }
 
-// Pairs of a dense block that regular_entry_ff2 leaves to regular_entry_near
-// wait in a list of the CTA and are evaluated together at the end: a few
-// lanes of many warps would otherwise each make their warp run that longer
-// path (655,220 panels, leaves of 80 rows: 95 -> 81 ms; issue slots 80 % busy).
-constexpr int NF_LIST = 2048;
-
 // Shared-memory layout of nearfield_kernel: two 128-byte aligned panel tiles
 // (FP64: [PT_ROWS][box_cols] doubles; float pairs: [PF_ROWS][box_cols]
-// floats), then the mbarrier and (float pairs) the list of near pairs.
+// floats), then the mbarrier.
 __host__ __device__ constexpr int nf_rec_bytes(bool ff) { return ff ? PF_ROWS * 4 : PT_ROWS * 8; }
 __host__ __device__ constexpr int nf_tile_bytes(bool ff, int box_cols) {
     return ((nf_rec_bytes(ff) * box_cols) + 127) / 128 * 128;
 }
 __host__ __device__ constexpr int nf_smem_bytes(bool ff, int box_cols) {
-    return 128 + 2 * nf_tile_bytes(ff, box_cols) + 16 + (ff ? 2 * NF_LIST : 0);
+    return 128 + 2 * nf_tile_bytes(ff, box_cols) + 16;
 }
 
 // ---------------------------------------------------------------------------
@@ -106,7 +100,7 @@ __host__ __device__ constexpr int nf_smem_bytes(bool ff, int box_cols) {
 constexpr int NF_THREADS = 128;
 
 // FF: the regular entries from the float-pair table in double-float
-// arithmetic (regular_entry_ff2, ~1e-14 relative) on the FP32 pipes; else from
+// arithmetic (regular_entry_ff, ~1e-14 relative) on the FP32 pipes; else from
 // the FP64 table in FP64.
 template <bool FF>
 __global__ void __launch_bounds__(NF_THREADS) nearfield_kernel(const __grid_constant__ CUtensorMap pt_map,
@@ -135,10 +129,7 @@ __global__ void __launch_bounds__(NF_THREADS) nearfield_kernel(const __grid_cons
     Rec *tR = reinterpret_cast<Rec *>(sm);
     Rec *tC = reinterpret_cast<Rec *>(sm + tile_bytes);
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + 2 * tile_bytes);
-    uint16_t *list = reinterpret_cast<uint16_t *>(bar + 2);
-    __shared__ int n_list;
     if (threadIdx.x == 0) {
-        n_list = 0;
         mbar_init(bar, 1);
         fence_barrier_init();
     }
@@ -220,33 +211,10 @@ __global__ void __launch_bounds__(NF_THREADS) nearfield_kernel(const __grid_cons
         }
         if (valid && !touch) {
             double a;
-            if constexpr (FF) {
-                hm::FF v;
-                if (!regular_entry_ff2(R, box_cols, C, box_cols, qp, v.h, v.l)) {
-                    const int k = mn <= 65536 ? atomicAdd(&n_list, 1) : NF_LIST;
-                    if (k < NF_LIST) {
-                        list[k] = (uint16_t)e;
-                        continue;
-                    }
-                    v = regular_entry_near(R, box_cols, C, box_cols, qp);
-                }
-                fast_two_sum(v.h, v.l, v.h, v.l);
-                a = ff_to(v);
-            } else {
+            if constexpr (FF)
+                a = regular_entry_ff(R, box_cols, C, box_cols, qp);
+            else
                 a = regular_entry(R, box_cols, C, box_cols, qp);
-            }
-            arena[blk_base + (int64_t)i * blk_ld + j] = a;
-            if (mirror) arena[par_base + (int64_t)j * par_ld + i] = a;
-        }
-    }
-    if constexpr (FF) {
-        __syncthreads();
-        const int nl = min(n_list, NF_LIST);
-        for (int k = threadIdx.x; k < nl; k += NF_THREADS) {
-            const int e = list[k], i = e / n, j = e - i * n;
-            hm::FF v = regular_entry_near(tR + i + ro, box_cols, tC + j + co, box_cols, qp);
-            fast_two_sum(v.h, v.l, v.h, v.l);
-            const double a = ff_to(v);
             arena[blk_base + (int64_t)i * blk_ld + j] = a;
             if (mirror) arena[par_base + (int64_t)j * par_ld + i] = a;
         }
