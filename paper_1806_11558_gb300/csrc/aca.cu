@@ -273,9 +273,10 @@ __device__ __forceinline__ bool bit(const uint32_t *bm, int k) { return (bm[k >>
 
 // One out-of-line copy of the far-field evaluation shared by every call site
 // (row and column passes, CTA and warp workers).
-__device__ __noinline__ static FF far_entry(const float *r, int rs, const float *c, int cs, const QuadParams &qp) {
+__device__ __noinline__ static FF far_entry(const float *r, int rs, const float *c, int cs, const float *wh,
+                                            const float *wl) {
     FF e;
-    regular_entry_ff2(r, rs, c, cs, qp, e.h, e.l);
+    regular_entry_ff2(r, rs, c, cs, wh, wl, e.h, e.l);
     return e;
 }
 
@@ -307,7 +308,7 @@ __device__ __forceinline__ FF aca_entry(const float *fix, bool fixed_is_row, int
     // in both passes: the varying record, read from L2, is then loaded once
     // per entry instead of once per outer step.  The value is the same entry
     // up to rounding (~1e-14 relative, the order of the double-float sums).
-    return far_entry(fix, 1, rec, (int)st, A.qp);
+    return far_entry(fix, 1, rec, (int)st, A.qp.w_h, A.qp.w_l);
 }
 
 // ACA of one block (CTA workers); U (m x kmax) and W (n x kmax) column-major

@@ -233,9 +233,6 @@ struct QuadParams {
     double gw[MAX_SS];
     float w_h[NQ];       // the 7 weights as float pairs (w = w_h + w_l)
     float w_l[NQ];
-    double orbit;        // u_k = orbit (V_k - c): offsets of points 1..3 from the centroid
-    float rho[4];        // offsets of points 4..6 over those of 1..3, and its square, as float pairs
-    float cw[12];        // weights of the six classes of point pairs (centroid, orbit 1, orbit 2), float pairs
 };
 
 // 7-point rule from its closed form; Gauss-Legendre nodes by Newton's method

@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(NF_THREADS) nearfield_kernel(const __grid_cons
         if (valid && !touch) {
             double a;
             if constexpr (FF)
-                a = regular_entry_ff(R, box_cols, C, box_cols, qp);
+                a = regular_entry_ff(R, box_cols, C, box_cols, qp.w_h, qp.w_l);
             else
                 a = regular_entry(R, box_cols, C, box_cols, qp);
             arena[blk_base + (int64_t)i * blk_ld + j] = a;

@@ -315,17 +315,6 @@ QuadParams make_quad(int ss_order) {
         q.w_h[k] = (float)q.w[k];
         q.w_l[k] = (float)(q.w[k] - (double)q.w_h[k]);
     }
-    // a point (a, a, 1 - 2a) lies at (1 - 3a) (V - centroid) from the centroid
-    q.orbit = 1.0 - 3.0 * a[0];
-    const double rho = (1.0 - 3.0 * a[1]) / (1.0 - 3.0 * a[0]), wo[3] = {q.w[0], wa[0], wa[1]};
-    auto pair = [](double v, float *o) {
-        o[0] = (float)v;
-        o[1] = (float)(v - (double)o[0]);
-    };
-    pair(rho, q.rho);
-    pair(rho * rho, q.rho + 2);
-    for (int i = 0, c = 0; i < 3; ++i)
-        for (int j = i; j < 3; ++j, ++c) pair(wo[i] * wo[j], q.cw + 2 * c);
     // Gauss-Legendre on [-1, 1]: roots of P_n by Newton's method started from
     // cos(pi (k + 3/4) / (n + 1/2)); weights 2 / ((1 - x^2) P_n'(x)^2); then
     // mapped to [0, 1].

@@ -135,51 +135,27 @@ __global__ void panel_table_kernel(const double *V, const int32_t *T, const int3
         const int32_t i = perm[k];
         const int32_t t0 = T[3 * (int64_t)i], t1 = T[3 * (int64_t)i + 1], t2 = T[3 * (int64_t)i + 2];
         const double *a = V + 3 * (int64_t)t0, *b = V + 3 * (int64_t)t1, *c = V + 3 * (int64_t)t2;
-        // float record: the centroid as three floats (the third from the
-        // vertices' differences to the first two, so a point's representation
-        // error is relative to the panel size) and the scaled vertex offsets
-        double cr[3], u[3][3];
+        // float-pair record: the centroid as (h, l) and every quadrature point
+        // as an offset from that represented centroid h + l (exact in FP64),
+        // so a point's representation error is relative to the panel size
+        double cr[3];
         for (int d = 0; d < 3; ++d) {
             float h, l;
             split_double(cent[3 * (int64_t)i + d], h, l);
             pf[(int64_t)(PF_CH + d) * npad + k] = h;
             pf[(int64_t)(PF_CL + d) * npad + k] = l;
             cr[d] = __dadd_rn((double)h, (double)l);
-            const double e0 = __dsub_rn(a[d], cr[d]), e1 = __dsub_rn(b[d], cr[d]), e2 = __dsub_rn(c[d], cr[d]);
-            const double r = __dadd_rn(__dadd_rn(e0, e1), e2) / 3.0;
-            pf[(int64_t)(PF_CM + d) * npad + k] = (float)r;
-            u[0][d] = __dmul_rn(qp.orbit, __dsub_rn(e0, r));
-            u[1][d] = __dmul_rn(qp.orbit, __dsub_rn(e1, r));
-            for (int v = 0; v < 2; ++v) {
-                split_double(u[v][d], h, l);
-                pf[(int64_t)(PF_U + 6 * v + d) * npad + k] = h;
-                pf[(int64_t)(PF_U + 6 * v + 3 + d) * npad + k] = l;
-                u[v][d] = __dadd_rn((double)h, (double)l);
-            }
-            u[2][d] = -__dadd_rn(u[0][d], u[1][d]);
-            split_double(u[2][d], h, l);
-            pf[(int64_t)(PF_U + 12 + d) * npad + k] = h;
-            pf[(int64_t)(PF_U + 15 + d) * npad + k] = l;
         }
-        const double rho = (double)qp.rho[0] + (double)qp.rho[1];
-        double nmax = 0.0;
-        for (int v = 0; v < 3; ++v) {
-            float h, l;
-            const double nv2 = u[v][0] * u[v][0] + u[v][1] * u[v][1] + u[v][2] * u[v][2];
-            nmax = nv2 > nmax ? nv2 : nmax;
-            split_double(nv2, h, l);
-            pf[(int64_t)(PF_N + 2 * v) * npad + k] = h;
-            pf[(int64_t)(PF_N + 2 * v + 1) * npad + k] = l;
-            split_double(rho * rho * nv2, h, l);
-            pf[(int64_t)(PF_N2 + 2 * v) * npad + k] = h;
-            pf[(int64_t)(PF_N2 + 2 * v + 1) * npad + k] = l;
-        }
-        pf[(int64_t)PF_RAD * npad + k] = __double2float_ru(sqrt(nmax));
         for (int q = 0; q < NQ; ++q)
-            for (int d = 0; d < 3; ++d)
-                pt[(int64_t)(7 * d + q) * npad + k] =
-                    __dadd_rn(__dadd_rn(__dmul_rn(qp.bary[q][0], a[d]), __dmul_rn(qp.bary[q][1], b[d])),
-                              __dmul_rn(qp.bary[q][2], c[d]));
+            for (int d = 0; d < 3; ++d) {
+                const double xq = __dadd_rn(__dadd_rn(__dmul_rn(qp.bary[q][0], a[d]), __dmul_rn(qp.bary[q][1], b[d])),
+                                            __dmul_rn(qp.bary[q][2], c[d]));
+                pt[(int64_t)(7 * d + q) * npad + k] = xq;
+                float h, l;
+                split_double(__dsub_rn(xq, cr[d]), h, l);
+                pf[(int64_t)(PF_AH + 7 * d + q) * npad + k] = h;
+                pf[(int64_t)(PF_AL + 7 * d + q) * npad + k] = l;
+            }
         pf[(int64_t)(PF_VID + 0) * npad + k] = __int_as_float(t0);
         pf[(int64_t)(PF_VID + 1) * npad + k] = __int_as_float(t1);
         pf[(int64_t)(PF_VID + 2) * npad + k] = __int_as_float(t2);
