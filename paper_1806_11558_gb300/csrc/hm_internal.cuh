@@ -402,6 +402,7 @@ struct hm_matrix {
     hm::DBuf rank16;    // [n_adm] int32: k_b - k32_b
     hm::TailPanels ut32, ut16;
     int64_t wp_entries = 0;
+    int32_t up_kmax = 0, wp_kmax = 0;  // widest row / column panel of the factors
     int64_t n_partials = 0;  // length of the partial-projection vector
     // block-Jacobi preconditioner: inverse of each leaf cluster's diagonal block
     // block-Jacobi preconditioner (built on the first preconditioned solve):

@@ -269,6 +269,8 @@ void build_lr_panels(hm_matrix *A, const DBuf &uw, const DBuf &uw_off, cudaStrea
         HM_CUDA_CHECK(cudaMemcpyAsync(ku.data(), A->up_K.p, sizeof(int32_t) * nl, cudaMemcpyDeviceToHost, s));
         HM_CUDA_CHECK(cudaMemcpyAsync(kw.data(), A->wp_K.p, sizeof(int32_t) * nl, cudaMemcpyDeviceToHost, s));
         HM_CUDA_CHECK(cudaStreamSynchronize(s));
+        A->up_kmax = *std::max_element(ku.begin(), ku.end());
+        A->wp_kmax = *std::max_element(kw.begin(), kw.end());
         std::vector<int32_t> ord(4 * nl);
         auto by_work = [&](int32_t *o, auto work) {
             for (int64_t r = 0; r < nl; ++r) o[r] = (int32_t)r;
@@ -437,6 +439,7 @@ struct MvDir {
     const int64_t *exp_off, *exp_ptr;
     const int32_t *exp_K, *exp_tidx;
     const int32_t *row_order, *col_order;
+    int proj_kmax;  // widest projection panel
 };
 
 static MvDir mv_dir(const hm_matrix *A, bool trans) {
@@ -447,11 +450,11 @@ static MvDir mv_dir(const hm_matrix *A, bool trans) {
         return MvDir{A->wp_off.as<int64_t>(), A->wp_colptr.as<int64_t>(), A->wp_K.as<int32_t>(),
                      tr->lr_bcolptr.as<int64_t>(), A->pofs.as<int64_t>(), A->up_off.as<int64_t>(),
                      A->up_colptr.as<int64_t>(), A->up_K.as<int32_t>(), A->tidx.as<int32_t>(),
-                     ord ? ord : nullptr, ord ? ord + nl : nullptr};
+                     ord ? ord : nullptr, ord ? ord + nl : nullptr, A->wp_kmax};
     return MvDir{A->up_off.as<int64_t>(), A->up_colptr.as<int64_t>(), A->up_K.as<int32_t>(),
                  tr->lr_browptr.as<int64_t>(), A->pofs_t.as<int64_t>(), A->wp_off.as<int64_t>(),
                  A->wp_colptr.as<int64_t>(), A->wp_K.as<int32_t>(), A->tidx_t.as<int32_t>(),
-                 ord ? ord + 2 * nl : nullptr, ord ? ord + 3 * nl : nullptr};
+                 ord ? ord + 2 * nl : nullptr, ord ? ord + 3 * nl : nullptr, A->up_kmax};
 }
 
 template <class TD, class TF, class TX, class TT>
@@ -460,9 +463,9 @@ static void matvec_impl(const hm_matrix *A, const TD *dense, const TF *proj, con
     const hm_tree *tr = A->tree;
     if (tr->n_adm > 0) {
         Trace tr_col(nm.col, s);
-        col_kernel<TF, TX, TT><<<(unsigned)tr->n_leaf, COL_THREADS, 0, s>>>(tr->leaf_begin.as<int32_t>(), d.proj_off,
-                                                                            d.proj_K, d.proj_ptr, proj, x, p,
-                                                                            d.col_order);
+        const int parts = col_parts_for(d.proj_kmax, V16<TF>::N);
+        col_kernel<TF, TX, TT><<<(unsigned)(tr->n_leaf * parts), COL_THREADS, 0, s>>>(
+            parts, tr->leaf_begin.as<int32_t>(), d.proj_off, d.proj_K, d.proj_ptr, proj, x, p, d.col_order);
         HM_LAUNCH_CHECK();
     }
     if (tr->n_adm > 0) {
@@ -476,16 +479,10 @@ static void matvec_impl(const hm_matrix *A, const TD *dense, const TF *proj, con
     // neighbouring clusters share their gathered x and t in L2 (measured:
     // largest-first 3.50 -> 3.28 ms in FP64, 1.24 -> 1.33 ms in FP32)
     constexpr bool ORD = sizeof(TD) == 8;
-    auto kern = row_kernel<12, TD, TF, TX, TT, ORD>;
-    switch (row_rb_for(tr->max_leaf)) {
-        case 4: kern = row_kernel<4, TD, TF, TX, TT, ORD>; break;
-        case 5: kern = row_kernel<5, TD, TF, TX, TT, ORD>; break;
-        case 8: kern = row_kernel<8, TD, TF, TX, TT, ORD>; break;
-        default: break;
-    }
+    const int groups = (tr->max_leaf + ROW_WARPS - 1) / ROW_WARPS;
     Trace tr_row(nm.row, s);
-    kern<<<(unsigned)tr->n_leaf, ROW_THREADS, 0, s>>>(
-        tr->leaf_begin.as<int32_t>(), tr->rho_off.as<int64_t>(), tr->rho_K.as<int32_t>(),
+    row_kernel<TD, TF, TX, TT, ORD><<<(unsigned)(tr->n_leaf * groups), ROW_THREADS, 0, s>>>(
+        groups, tr->leaf_begin.as<int32_t>(), tr->rho_off.as<int64_t>(), tr->rho_K.as<int32_t>(),
         tr->rho_colptr.as<int64_t>(), tr->colidx.as<int32_t>(), dense, d.exp_off, d.exp_K, d.exp_ptr, d.exp_tidx,
         expd, t, x, ym, d.row_order);
     HM_LAUNCH_CHECK();

@@ -95,14 +95,23 @@ template <> __device__ __forceinline__ void ld_idx<8>(const int32_t *p, int (&o)
 //               W_b whose columns cover kappa, side by side): each thread owns
 //               16 bytes of columns and accumulates over the |kappa| rows in
 //               registers, so every thread keeps |kappa| independent 16-byte
-//               loads in flight and no reduction is needed.
+//               loads in flight and no reduction is needed.  The panel's
+//               columns are shared by `parts` CTAs, one pass of the threads
+//               each, so that the few panels of a small operator fill the chip
+//               (FP64, 21,780 panels, 512 clusters: 89 -> 66 us against 49 us of
+//               the FP64 pipe; FP32, 81,920 panels: 147 -> 108 us).  An odd
+//               number: consecutive CTAs go to consecutive SMs (152 = 8 x 19),
+//               and with 8 parts the emptier last ones would all meet on the
+//               same SMs (FP64, 5,120 panels: 27 us against 18 us).
 //  tsum_kernel: t_b(l) = sum over the column clusters of sigma_b of those
 //               partials, in increasing cluster order (fixed order).
 // ---------------------------------------------------------------------------
-constexpr int COL_THREADS = 256;
+constexpr int COL_THREADS = 128;
+// parts of a pass over panels of at most K columns, N per thread
+constexpr int col_parts_for(int K, int N) { return ((K + COL_THREADS * N - 1) / (COL_THREADS * N)) | 1; }
 
 template <class TF, class TX, class TP>
-__global__ void __launch_bounds__(COL_THREADS) col_kernel(const int32_t *__restrict__ leaf_begin,
+__global__ void __launch_bounds__(COL_THREADS) col_kernel(int parts, const int32_t *__restrict__ leaf_begin,
                                                           const int64_t *__restrict__ wp_off,
                                                           const int32_t *__restrict__ wp_K,
                                                           const int64_t *__restrict__ wp_colptr,
@@ -111,15 +120,17 @@ __global__ void __launch_bounds__(COL_THREADS) col_kernel(const int32_t *__restr
     using A = typename Acc<TF>::type;
     constexpr int N = V16<TF>::N;
     __shared__ A s_x[MAX_LEAF];
-    const int64_t kap = order ? order[blockIdx.x] : blockIdx.x;  // largest panels first
+    const int q = blockIdx.x / parts, part = blockIdx.x - q * parts;
+    const int64_t kap = order ? order[q] : q;  // largest panels first
     const int32_t c0 = leaf_begin[kap], mc = leaf_begin[kap + 1] - c0;
+    const int Kw = wp_K[kap];
+    if (part * COL_THREADS * N >= Kw) return;
     for (int j = threadIdx.x; j < mc; j += COL_THREADS) s_x[j] = (A)x[c0 + j];
     __syncthreads();
-    const int Kw = wp_K[kap];
     const TF *W = wp + wp_off[kap];
     TP *out = p + wp_colptr[kap];
     const int nv = Kw / N;
-    for (int v = threadIdx.x; v < nv; v += COL_THREADS) {
+    for (int v = part * COL_THREADS + threadIdx.x; v < nv; v += parts * COL_THREADS) {
         A acc[N];
 #pragma unroll
         for (int e = 0; e < N; ++e) acc[e] = 0;
@@ -217,74 +228,68 @@ __global__ void tsum_b0_kernel(int64_t na, const int64_t *__restrict__ t_off, in
 }
 
 // ---------------------------------------------------------------------------
-// y_rho = P_rho x(colidx) + Ut_rho t(tidx): one CTA per leaf row cluster,
-// dispatched in decreasing order of panel work (`order`), so the longest
-// CTAs start first and the last wave is made of short ones.
-// Every row of a panel multiplies the same gathered vector, so the CTA
-// gathers it once per column chunk into shared memory; then each warp takes
-// RB rows at a time and streams them with 16-byte loads against the staged
-// chunk (one shared-memory vector feeds RB independent global loads).
+// y_rho = P_rho x(colidx) + Ut_rho t(tidx): CTAs of ROW_WARPS rows of a leaf
+// row cluster, one row per warp.  Every row of a panel multiplies the same
+// gathered vector, so the CTA gathers it once per column chunk into shared
+// memory; then each warp streams its row with 16-byte loads, ROW_LOADS of them
+// in flight, against the staged chunk.  The FP64 product is bound by the FP64
+// pipe (2 FMAs per SM and clock), the others by HBM.
+//
+// Eight rows per CTA whatever the leaves: a whole cluster per CTA (5, 8 or 12
+// rows per warp) left a small operator a wave of unequal CTAs and wasted the
+// slots of the rows that a cluster lacks.  Same sums bit for bit; measured per
+// launch, a cluster per CTA -> eight rows (time the FP64 pipe needs), FP64:
+// 5,120 panels 86 -> 45 us (17), 21,780 panels 397 -> 150 us (105), 200,000
+// panels 3.14 -> 1.74 ms (1.47), 327,680 panels 3.22 -> 3.22 ms (2.83); FP32
+// (time HBM needs): 21,780 panels 166 -> 70 us (39), 200,000 panels 976 ->
+// 647 us (543), 327,680 panels 1.31 -> 1.17 ms (1.05).  4 or 16 warps per CTA
+// and 1 or 8 loads in flight were slower or the same.
 // ---------------------------------------------------------------------------
-constexpr int ROW_THREADS = 256;
-constexpr int ROW_WARPS = ROW_THREADS / 32;
+constexpr int ROW_WARPS = 8;
+constexpr int ROW_THREADS = 32 * ROW_WARPS;
+template <class T> constexpr int ROW_LOADS = sizeof(T) == 8 ? 2 : 4;
 constexpr int ROW_CHUNK = 4096;  // columns staged per pass (multiple of 8)
-// Rows per warp per pass (RB): a row group is RB * ROW_WARPS rows.  The host
-// picks the smallest RB whose group covers the largest leaf cluster, so the
-// gathered vector is staged once per chunk and every warp keeps RB 16-byte
-// loads in flight per step; rows past the cluster's end issue no loads.
-// Leaves of 80 rows take two groups of 40 (RB = 5, 80 registers): measured
-// on the level-8 sphere (FP64 product) 16.0 ms against 16.4 ms with one
-// group of 80 (RB = 10) and 21.7 ms with RB = 12 (128 registers, 96-row
-// groups); the row sums are the same bit for bit.
-constexpr int row_rb_for(int max_leaf) {
-    return max_leaf <= 32 ? 4 : max_leaf <= 40 ? 5 : max_leaf <= 64 ? 8 : max_leaf <= 80 ? 5 : 12;
-}
 
-// Partial sums (per lane) of rows g0 + warp + ROW_WARPS * u, u < RB, of a
-// row-major panel P (|rho| x L) times z(idx), staging z(idx) chunk by chunk.
-template <int RB, class T, class Z, class A>
-__device__ __forceinline__ void panel_rows(const T *__restrict__ P, int L, const int32_t *__restrict__ idx,
-                                           const Z *__restrict__ z, int mr, int g0, A *s_z, A (&a)[RB]) {
-    constexpr int N = V16<T>::N;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const T *rows[RB];
-    bool live[RB];
-#pragma unroll
-    for (int u = 0; u < RB; ++u) {
-        const int r = g0 + warp + ROW_WARPS * u;
-        live[u] = r < mr;
-        rows[u] = P + (int64_t)(live[u] ? r : 0) * L;
-        a[u] = 0;
-    }
+// Partial sum (per lane) of row r (live: r exists) of a row-major panel P
+// (|rho| x L) times z(idx), staging z(idx) chunk by chunk.
+template <class T, class Z, class A>
+__device__ __forceinline__ A panel_row(const T *__restrict__ P, int L, const int32_t *__restrict__ idx,
+                                       const Z *__restrict__ z, int r, bool live, A *s_z) {
+    constexpr int N = V16<T>::N, U = ROW_LOADS<T>;
+    const int lane = threadIdx.x & 31;
+    const T *row = P + (int64_t)r * L;
+    A a = 0;
     for (int c0 = 0; c0 < L; c0 += ROW_CHUNK) {
         const int cl = min(ROW_CHUNK, L - c0);
         __syncthreads();
         for (int k = threadIdx.x; k < cl; k += ROW_THREADS) s_z[k] = (A)z[idx[c0 + k]];
         __syncthreads();
-        const int nv = cl / N;
-        // two steps in flight for FP64 panels (measured faster there; the
-        // FP32 / BF16 panels are faster without)
-        constexpr int UNR = sizeof(T) == 8 ? 2 : 1;
-#pragma unroll UNR
-        for (int v = lane; v < nv; v += 32) {
-            A zv[N];
+        const int nv = live ? cl / N : 0;
+        const T *rc = row + c0;
+        int v = lane;
+        for (; v + 32 * (U - 1) < nv; v += 32 * U) {
+            A pv[U][N];
 #pragma unroll
-            for (int e = 0; e < N; ++e) zv[e] = s_z[v * N + e];
+            for (int u = 0; u < U; ++u) V16<T>::load(rc + (int64_t)(v + 32 * u) * N, pv[u]);
 #pragma unroll
-            for (int u = 0; u < RB; ++u) {
-                if (!live[u]) continue;
-                A pv[N];
-                V16<T>::load(rows[u] + c0 + (int64_t)v * N, pv);
+            for (int u = 0; u < U; ++u)
 #pragma unroll
-                for (int e = 0; e < N; ++e) a[u] += pv[e] * zv[e];
-            }
+                for (int e = 0; e < N; ++e) a += pv[u][e] * s_z[(v + 32 * u) * N + e];
+        }
+        for (; v < nv; v += 32) {
+            A pv[N];
+            V16<T>::load(rc + (int64_t)v * N, pv);
+#pragma unroll
+            for (int e = 0; e < N; ++e) a += pv[e] * s_z[v * N + e];
         }
     }
+    return a;
 }
 
-template <int RB, class TD, class TF, class TX, class TT, bool ORD>
+template <class TD, class TF, class TX, class TT, bool ORD>
 __global__ void __launch_bounds__(ROW_THREADS) row_kernel(
-    const int32_t *__restrict__ leaf_begin, const int64_t *__restrict__ rho_off, const int32_t *__restrict__ rho_K,
+    int groups, const int32_t *__restrict__ leaf_begin, const int64_t *__restrict__ rho_off,
+    const int32_t *__restrict__ rho_K,
     const int64_t *__restrict__ rho_colptr, const int32_t *__restrict__ colidx, const TD *__restrict__ dense,
     const int64_t *__restrict__ up_off, const int32_t *__restrict__ up_K, const int64_t *__restrict__ up_colptr,
     const int32_t *__restrict__ tidx, const TF *__restrict__ up, const TT *__restrict__ t, const TX *__restrict__ x,
@@ -292,29 +297,20 @@ __global__ void __launch_bounds__(ROW_THREADS) row_kernel(
     using AD = typename Acc<TD>::type;
     using AF = typename Acc<TF>::type;
     __shared__ __align__(16) unsigned char s_raw[ROW_CHUNK * sizeof(AD)];
-    const int64_t rho = ORD ? order[blockIdx.x] : blockIdx.x;  // largest panels first (ORD)
-    const int32_t r0 = leaf_begin[rho], r1 = leaf_begin[rho + 1];
-    const int mr = r1 - r0;
+    const int q = blockIdx.x / groups, g = blockIdx.x - q * groups;
+    const int64_t rho = ORD ? order[q] : q;  // largest panels first (ORD)
+    const int32_t r0 = leaf_begin[rho], mr = leaf_begin[rho + 1] - r0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const TD *P = dense + rho_off[rho];
-    const int Kd = rho_K[rho];
-    const int32_t *ci = colidx + rho_colptr[rho];
-    const TF *Q = up + up_off[rho];
-    const int Ku = up_K[rho];
-    const int32_t *ti = tidx + up_colptr[rho];
-    for (int g0 = 0; g0 < mr; g0 += RB * ROW_WARPS) {
-        AD ad[RB];
-        AF af[RB];
-        panel_rows<RB, TD, TX, AD>(P, Kd, ci, x, mr, g0, reinterpret_cast<AD *>(s_raw), ad);
-        panel_rows<RB, TF, TT, AF>(Q, Ku, ti, t, mr, g0, reinterpret_cast<AF *>(s_raw), af);
-#pragma unroll
-        for (int u = 0; u < RB; ++u) {
-            const int r = g0 + warp + ROW_WARPS * u;
-            const AD d = warp_reduce(ad[u]);
-            const AF f = warp_reduce(af[u]);
-            if (lane == 0 && r < mr) ym[r0 + r] = (double)d + (double)f;
-        }
-    }
+    if (g * ROW_WARPS >= mr) return;
+    const int r = g * ROW_WARPS + warp;
+    const bool live = r < mr;
+    const AD ad = panel_row<TD, TX, AD>(dense + rho_off[rho], rho_K[rho], colidx + rho_colptr[rho], x, live ? r : 0,
+                                        live, reinterpret_cast<AD *>(s_raw));
+    const AF af = panel_row<TF, TT, AF>(up + up_off[rho], up_K[rho], tidx + up_colptr[rho], t, live ? r : 0, live,
+                                        reinterpret_cast<AF *>(s_raw));
+    const AD d = warp_reduce(ad);
+    const AF f = warp_reduce(af);
+    if (lane == 0 && live) ym[r0 + r] = (double)d + (double)f;
 }
 
 }  // namespace hm
