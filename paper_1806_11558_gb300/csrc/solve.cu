@@ -43,10 +43,17 @@ static void apply(const hm_matrix *A, hm_dtype prec, const double *x, double *y,
 constexpr int DOT_THREADS = 512;
 constexpr int DOT_CHUNK = 8;  // vectors per register pass
 
-// out[l] = V_l . w for l < nv (+ out[l] when accumulate), one launch: every
-// block writes its partial sums part[blk][l]; the block that finishes last
-// (a ticket counter, reset by it for the next call) adds the partials of
-// each l in a fixed order (lanes over blocks, then a fixed shuffle tree).
+// out[l] = V_l . w for l < nv (+ out[l] when accumulate), one launch.  Block
+// (b, c) takes the elements of part b of the vectors of chunk c (DOT_CHUNK of
+// them) and writes its partial sums part[b][l]; of the blocks of a chunk the
+// one that finishes last (a ticket per chunk, reset by it for the next call)
+// adds the chunk's partials in a fixed order (lanes over blocks, then a fixed
+// shuffle tree).  An FP64 addition occupies its pipe for 64 cycles per warp,
+// so the warp sums of the chunk's 8 vectors are formed together: each exchange
+// halves the vectors a lane still carries (9 additions instead of 40, in the
+// order of the plain tree).  Mean over the passes of a solve, one block per
+// part with the chunks in turn -> this: 21,780 elements, up to 66 vectors 39.5
+// -> 13.1 us; 5,120 elements, up to 30 vectors 24.9 -> 11.2 us (the same sums).
 __global__ void __launch_bounds__(DOT_THREADS) dots_kernel(const double *__restrict__ V, int64_t ld, int nv,
                                                             const double *__restrict__ w, int64_t n,
                                                             double *__restrict__ part, double *__restrict__ out,
@@ -56,45 +63,52 @@ __global__ void __launch_bounds__(DOT_THREADS) dots_kernel(const double *__restr
     __shared__ double s[DOT_THREADS / 32][DOT_CHUNK];
     __shared__ bool s_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c0 = blockIdx.y * DOT_CHUNK;
+    if (c0 >= nv) return;  // graph form: the grid covers the longest basis
     const int64_t per = (n + gridDim.x - 1) / gridDim.x;
     const int64_t i0 = (int64_t)blockIdx.x * per, i1 = min(n, i0 + per);
-    for (int c0 = 0; c0 < nv; c0 += DOT_CHUNK) {
-        double acc[DOT_CHUNK];
+    double acc[DOT_CHUNK];
 #pragma unroll
-        for (int c = 0; c < DOT_CHUNK; ++c) acc[c] = 0.0;
-        for (int64_t i = i0 + threadIdx.x; i < i1; i += DOT_THREADS) {
-            const double wi = w[i];
+    for (int c = 0; c < DOT_CHUNK; ++c) acc[c] = 0.0;
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += DOT_THREADS) {
+        const double wi = w[i];
 #pragma unroll
-            for (int c = 0; c < DOT_CHUNK; ++c)
-                if (c0 + c < nv) acc[c] = fma(V[(int64_t)(c0 + c) * ld + i], wi, acc[c]);
-        }
+        for (int c = 0; c < DOT_CHUNK; ++c)
+            if (c0 + c < nv) acc[c] = fma(V[(int64_t)(c0 + c) * ld + i], wi, acc[c]);
+    }
+    // lanes with bits 4, 3, 2 = c end with vector c's sum
+    static_assert(DOT_CHUNK == 8, "three halving exchanges");
 #pragma unroll
-        for (int c = 0; c < DOT_CHUNK; ++c) {
-            double v = acc[c];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) s[warp][c] = v;
+    for (int h = DOT_CHUNK / 2, o = 16; h > 0; h >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int c = 0; c < h; ++c) {
+            const double mine = up ? acc[c + h] : acc[c], other = up ? acc[c] : acc[c + h];
+            acc[c] = mine + __shfl_xor_sync(0xffffffffu, other, o);
         }
-        __syncthreads();
-        if (threadIdx.x < DOT_CHUNK && c0 + (int)threadIdx.x < nv) {
-            double t = 0.0;
-            for (int k = 0; k < DOT_THREADS / 32; ++k) t += s[k][threadIdx.x];
-            part[(int64_t)blockIdx.x * nv + c0 + threadIdx.x] = t;
-        }
-        __syncthreads();
+    }
+    for (int o = 2; o > 0; o >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+    if ((lane & 3) == 0) s[warp][lane >> 2] = acc[0];
+    __syncthreads();
+    if (threadIdx.x < DOT_CHUNK && c0 + (int)threadIdx.x < nv) {
+        double t = 0.0;
+        for (int k = 0; k < DOT_THREADS / 32; ++k) t += s[k][threadIdx.x];
+        part[(int64_t)blockIdx.x * nv + c0 + threadIdx.x] = t;
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    if (threadIdx.x == 0) s_last = atomicAdd(ticket + blockIdx.y, 1u) == gridDim.x - 1;
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    for (int l = warp; l < nv; l += DOT_THREADS / 32) {
+    const int l = c0 + warp;
+    if (warp < DOT_CHUNK && l < nv) {
         double t = 0.0;
         for (int b = lane; b < (int)gridDim.x; b += 32) t += __ldcg(part + (int64_t)b * nv + l);
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
         if (lane == 0) out[l] = accumulate ? out[l] + t : t;
     }
-    if (threadIdx.x == 0) *ticket = 0u;
+    if (threadIdx.x == 0) ticket[blockIdx.y] = 0u;
 }
 
 // w -= sum_l V_l h_l
@@ -403,30 +417,32 @@ __global__ void __launch_bounds__(BJ_INV_THREADS) bj_invert_smem_kernel(const in
 
 // z_b = D_b^{-1} v_b: one thread per row over the column-major inverse
 // (consecutive threads read consecutive rows of one column), v_b staged in
-// shared memory; each row sums its columns in order.  trans: z = D^{-T} v,
+// shared memory; each row sums its columns in order.  Blocks of 64 rows, so
+// that the ~100 blocks of a small operator fill the chip, with eight loads in
+// flight: the loads' latency is the bound there (21,780 rows in 200-row blocks,
+// FP64: 55 -> 34 us against 128 threads per block).  trans: z = D^{-T} v,
 // the preconditioner of the transposed system (row-major reading).
 // TD = double: the FP64 preconditioner; TD = float: its FP32 rounding with
 // FP32 accumulation, for the inner solves on the low-precision copies.
-// grid.y = column of [cols][n] vectors.
-constexpr int BJ_THREADS = 128;
+// grid.y = group of 64 rows.
+constexpr int BJ_THREADS = 64;
 template <class TD>
 __global__ void __launch_bounds__(BJ_THREADS) bj_apply_kernel(const int32_t *begin, const int64_t *bj_off,
-                                                              const TD *bj, const double *v, double *z, int trans,
-                                                              int64_t n) {
+                                                              const TD *bj, const double *v, double *z, int trans) {
     __shared__ TD s_v[BJ_MAXM];
     const int64_t r = blockIdx.x;
     const int32_t r0 = begin[r], m = begin[r + 1] - r0;
     const TD *D = bj + bj_off[r];
-    const double *vc = v + (int64_t)blockIdx.y * n;
-    double *zc = z + (int64_t)blockIdx.y * n;
-    for (int j = threadIdx.x; j < m; j += BJ_THREADS) s_v[j] = (TD)vc[r0 + j];
+    const int i = blockIdx.y * BJ_THREADS + threadIdx.x;
+    if ((int)blockIdx.y * BJ_THREADS >= m) return;
+    for (int j = threadIdx.x; j < m; j += BJ_THREADS) s_v[j] = (TD)v[r0 + j];
     __syncthreads();
-    for (int i = threadIdx.x; i < m; i += BJ_THREADS) {
-        TD acc = 0;
-        const int64_t si = trans ? m : 1, sj = trans ? 1 : m;
-        for (int j = 0; j < m; ++j) acc = fma(D[j * sj + i * si], s_v[j], acc);
-        zc[r0 + i] = (double)acc;
-    }
+    if (i >= m) return;
+    TD acc = 0;
+    const int64_t si = trans ? m : 1, sj = trans ? 1 : m;
+#pragma unroll 8
+    for (int j = 0; j < m; ++j) acc = fma(D[j * sj + i * si], s_v[j], acc);
+    z[r0 + i] = (double)acc;
 }
 
 // The same for up to BJ_NC columns per CTA (grid.y = column groups): the
@@ -569,13 +585,13 @@ void bj_apply_cols(const hm_matrix *A, const double *v, double *z, int cols, boo
         HM_LAUNCH_CHECK();
         return;
     }
-    const dim3 grid((unsigned)A->n_bj, (unsigned)cols);
+    const dim3 grid((unsigned)A->n_bj, (unsigned)((A->bj_mmax + BJ_THREADS - 1) / BJ_THREADS));
     if (low)
         bj_apply_kernel<float><<<grid, BJ_THREADS, 0, s>>>(A->bj_begin.as<int32_t>(), A->bj_off.as<int64_t>(),
-                                                           A->bj32.as<float>(), v, z, trans ? 1 : 0, A->tree->n);
+                                                           A->bj32.as<float>(), v, z, trans ? 1 : 0);
     else
         bj_apply_kernel<double><<<grid, BJ_THREADS, 0, s>>>(A->bj_begin.as<int32_t>(), A->bj_off.as<int64_t>(),
-                                                            A->bj.as<double>(), v, z, trans ? 1 : 0, A->tree->n);
+                                                            A->bj.as<double>(), v, z, trans ? 1 : 0);
     HM_LAUNCH_CHECK();
 }
 
@@ -619,15 +635,18 @@ struct Gmres {
         z.alloc(sizeof(double) * n);
         d.alloc(sizeof(double) * n);
         nrm.alloc(sizeof(double) * 2);
-        ticket.alloc(sizeof(unsigned int));
-        HM_CUDA_CHECK(cudaMemsetAsync(ticket.p, 0, sizeof(unsigned int), s));
+        const int chunks = (m + 1 + DOT_CHUNK - 1) / DOT_CHUNK;
+        ticket.alloc(sizeof(unsigned int) * chunks);
+        HM_CUDA_CHECK(cudaMemsetAsync(ticket.p, 0, sizeof(unsigned int) * chunks, s));
         ctl.alloc(sizeof(LoopCtl));
     }
     // out[0..nv) = V_l . w (accumulate adds to out)
     void dots(const double *Vb, int nv, const double *wv, double *out, int accumulate, cudaStream_t s,
               const LoopCtl *c = nullptr) {
         Trace trace("gmres_dots", s);
-        dots_kernel<<<nblk, DOT_THREADS, 0, s>>>(Vb, n, nv, wv, n, part.as<double>(), out, accumulate,
+        // the graph form (c) takes the basis size from the device: its grid covers all m vectors
+        const dim3 grid((unsigned)nblk, (unsigned)(((c ? m : nv) + DOT_CHUNK - 1) / DOT_CHUNK));
+        dots_kernel<<<grid, DOT_THREADS, 0, s>>>(Vb, n, nv, wv, n, part.as<double>(), out, accumulate,
                                                  ticket.as<unsigned int>(), c);
         HM_LAUNCH_CHECK();
     }
