@@ -70,10 +70,6 @@ FP32_PEAK_TFLOPS = 152 * 2.07e9 * 128 * 2 / 1e12  # 80.5
 # FP32 flops of one pair evaluation in the double-float entry (ACA and the
 # regular near field; TwoSum 6, TwoProduct 2 with its FMA counted 2, ...): 93 per pair
 FF_FLOPS_PER_PAIR = 93
-# FP32 flops of one term of the double-float product (TwoProduct 1 + 2, TwoSum 6, two cross-term FMAs 4,
-# two adds into the compensation 2), FMAs counted 2: 15 flops in 12 instructions, so the instruction mix
-# caps these kernels at 15 / 24 = 0.625 of the FMA peak
-DF_FLOPS_PER_TERM = 15
 
 # DRAM traffic per launch from an ncu capture, valid while the kernel's source
 # file is unchanged (sha256 of the file at capture time); null otherwise.
@@ -142,10 +138,10 @@ def algorithmic_work(mi, ti, dense_leaves, n):
         "col_bcp_kernel.f32": ("hbm", 4.0 * (w - w16) + xr * (n + K - K16), "byte"),
         "col_bcp_kernel.bf16": ("hbm", (2.0 * w16 + xr * (n + K16)) if K16 else (2.0 * w + xr * (n + K)), "byte"),
         "nearfield_kernel": ("alu32", float(nf_entries) * PAIRS_PER_ENTRY * FF_FLOPS_PER_PAIR, "flop"),
-        # double-float product of the FP64 master, 16 right-hand sides per launch: DF_FLOPS_PER_TERM per
-        # (entry, right-hand side)
-        "row_df_kernel": ("alu32", DF_FLOPS_PER_TERM * MR * (d + u), "flop"),
-        "col_df_kernel": ("alu32", DF_FLOPS_PER_TERM * MR * w, "flop"),
+        # product of the FP64 master with 16 right-hand sides: every entry once, the digits and exponents of the
+        # rows of x and t (7 x 16 x 2 + 8 B), the rows of y (16 x 8 B), the partials (float pairs)
+        "row_fx_kernel": ("hbm", 8.0 * (d + u) + 232.0 * (n + K) + 128.0 * n, "byte"),
+        "col_fx_kernel": ("hbm", 8.0 * w + 232.0 * n + 128.0 * w * nl / n, "byte"),
         "nearfield_kernel.f64": ("alu", float(nf_entries) * PAIRS_PER_ENTRY * FLOPS_PER_PAIR, "flop"),
         "aca_kernel": ("alu32", float(mi["aca_entries"]) * PAIRS_PER_ENTRY * FF_FLOPS_PER_PAIR, "flop"),
     }

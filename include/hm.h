@@ -178,11 +178,10 @@ typedef struct {
                            HM_EINVAL. */
     int32_t resid_df;   /* refine = 1 and batched = 1: 1 = the outer residuals
                            b - H x of all systems by the 16-right-hand-side
-                           product of the FP64 master in double-float
-                           arithmetic (hm_matvec_block with HM_F64: each stored
-                           entry read once per 16 systems, the arithmetic on
-                           the FP32 pipe; ~1e-14 of |H||x| instead of ~1e-16),
-                           and the stopping test on them; 0 = one FP64 product
+                           product of the FP64 master on the tensor cores
+                           (hm_matvec_block with HM_F64: each stored entry
+                           read once per 16 systems; a few 1e-15 of |H||x|
+                           instead of ~1e-16), and the stopping test on them; 0 = one FP64 product
                            per system.  Other values: HM_EINVAL. */
 } hm_solve_params;
 
@@ -353,13 +352,15 @@ HM_API hm_status hm_matvec(const hm_matrix *A, int32_t trans, int32_t nrhs, hm_d
  *  (hi + lo) and multiplied as hi*hi + hi*lo + lo*hi, so the result carries
  *  about 16 significant bits (relative error ~1e-5 on top of the copy's own
  *  rounding) — accurate enough for the inner solves of the refinement.
- *  prec = HM_F64: the FP64 master in double-float arithmetic on the FP32
- *  pipe (every entry and x split into a pair of floats, error-free products
- *  and sums: the compensated dot product of Ogita, Rump and Oishi), about
- *  2^-47 relative error per term, ~1e-14 of the row sums of |H||x| — the
- *  FP64 residuals of the batched refinement (hm_solve_params.resid_df).
+ *  prec = HM_F64: the FP64 master on the tensor cores, every entry and x cut
+ *  into seven digits base 256 whose products are summed without rounding
+ *  (Ozaki, Ogita, Oishi and Rump): a few 1e-15 of the row sums of |H||x| — the
+ *  FP64 residuals of the batched refinement (hm_solve_params.resid_df).  Each
+ *  x_r is scaled by itself; a right-hand side whose entries are small beside
+ *  the others' in the same panels keeps fewer of the 54 bits there.
  * Stream-ordered (working vectors from the stream-ordered pool; HM_F64 uses
- * 128 bytes per panel, per partial projection and per unit of total rank).
+ * 360 bytes per panel, 128 per partial projection and 232 per unit of total
+ * rank).
  * Errors: HM_EINVAL for NULL pointers, nrhs < 1, an unknown precision, or a
  * low precision whose copy was not assembled. */
 HM_API hm_status hm_matvec_block(const hm_matrix *A, int32_t nrhs, hm_dtype prec, const double *d_x, double *d_y,

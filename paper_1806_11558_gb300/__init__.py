@@ -273,8 +273,8 @@ def hm_matvec(A, x, y, trans=0, prec=HM_F64, alpha=1.0, beta=0.0, stream=None):
 def hm_matvec_block(A, x, y, prec=HM_BF16, alpha=1.0, beta=0.0, stream=None):
     """Product for [nrhs, n] right-hand sides, 16 at a time: on the tensor
     cores with the FP32 / BF16 copies (~1e-5 relative accuracy, BF16 operand
-    pairs), or (prec = HM_F64) the FP64 master in double-float arithmetic
-    (~1e-14 of |H||x|)."""
+    pairs), or (prec = HM_F64) the FP64 master in exact digit products (a few
+    1e-15 of |H||x|)."""
     import torch
     nrhs = 1 if x.dim() == 1 else x.shape[0]
     _check(lib().hm_matvec_block(A, nrhs, int(prec), _ptr(x, torch.float64), _ptr(y, torch.float64), float(alpha),

@@ -457,7 +457,7 @@ struct Batch {
         return Z32.as<TV>();
     }
 
-    // outer residual products by the double-float 16-column product (resid_df)
+    // outer residual products by the 16-column product of the FP64 master (resid_df)
     DBuf dfw;
     void enable_df() { dfw.alloc(sizeof(float) * df_work_floats(A)); }
     // y = H_64 x for all R columns ([R][n], Morton): the outer products of the refinement

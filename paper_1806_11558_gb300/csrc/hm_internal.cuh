@@ -403,6 +403,11 @@ struct hm_matrix {
     hm::TailPanels ut32, ut16;
     int64_t wp_entries = 0;
     int32_t up_kmax = 0, wp_kmax = 0;  // widest row / column panel of the factors
+    // row pass of the FP64 product with 16 right-hand sides (build_fx_items):
+    // work items (cluster, first chunk, end chunk, partial slot or -1) and the
+    // sums of the split ones (cluster, first slot, slots, 0)
+    hm::DBuf fx_items, fx_red;
+    int64_t fx_nitems = 0, fx_nred = 0, fx_nslots = 0;
     int64_t n_partials = 0;  // length of the partial-projection vector
     // block-Jacobi preconditioner: inverse of each leaf cluster's diagonal block
     // block-Jacobi preconditioner (built on the first preconditioned solve):

@@ -1,82 +1,64 @@
 // mrhs_df.cu -- the product of the FP64 master with up to 16 right-hand
-// sides (the H-matvec of Sec. 2.3) in double-float arithmetic, for the FP64
-// residuals of the iterative refinement and hm_matvec_block(HM_F64).
+// sides (the H-matvec of Sec. 2.3) on the tensor cores, for the FP64 residuals
+// of the iterative refinement and hm_matvec_block(HM_F64).
 //
-// GB300 runs FP64 FMAs at 2 per SM and clock, FP32 FMAs at 128: the FP64
-// products of the refinement (one per system, each reading the whole FP64
-// master) are bound by the FP64 pipe.  Here every stored FP64 entry w is read
-// once per 16 right-hand sides and split into an unevaluated pair of floats,
-// w = h + l (h: w truncated to 24 significant bits, l: the rest rounded to
-// 24), by integer operations (no FP64 instruction); x is split the same way
-// (by FP64 conversions, n values).  Each term is accumulated into a pair
-// (s, c) of floats with an error-free product (TwoProduct: p + e = h_w h_x
-// exactly, by one FMA) and an error-free sum (TwoSum: s + p = t + sigma
-// exactly), the cross terms h_w l_x + l_w h_x and the two errors going to c:
-// the compensated dot product of Ogita, Rump and Oishi (2005, "Accurate sum
-// and dot product", Algorithm 5.3, Dot2) with double-float operands.  Its
-// result carries about 2^-47 relative error per term plus the rounding of
-// the compensation (n u^2 |H||x| at worst for n terms, u = 2^-24, about
-// sqrt(n) u^2 typically: ~1e-13 of a row sum of |H||x| at worst, a few 1e-15
-// in norm), against 2^-53 per term of the FP64 product; two orders below the
-// 1e-12 residuals the refinement stops at.
+// GB300 runs FP64 FMAs at 2 per SM and clock, FP32 FMAs at 128 and 16-bit
+// tensor multiply-adds at ~1,000 (mma.sync): 16 FP64 products are bound by the
+// FP64 pipe, and compensated sums of float pairs (12 FP32 operations per entry
+// and right-hand side) by the FP32 pipe.  Here entries and vectors are cut into
+// digits base 256 whose products the tensor cores add without rounding (the
+// error-free slicing of Ozaki, Ogita, Oishi and Rump, "Error-free
+// transformations of matrix multiplication by using fast routines of matrix
+// multiplication and its applications", Numer. Algorithms 2012):
+//   * column k of a panel has the exponent e_k of its largest x_r (each x_r
+//     scaled by its own largest entry first) and x_r 2^-e_k becomes an integer
+//     of 54 bits and sign, seven balanced digits d in [-128, 127], as FP16;
+//   * a term w 2^e_k of a row becomes an integer of 54 bits or less and sign on
+//     the scale of the row's largest term so far, in integer operations on the
+//     bits of w: seven digits, the top one signed, the others in [0, 255], as
+//     FP16 subnormals (u 2^-24, which are the digit's own bits);
+//   * of the 49 products of digits the 34 of order i + j <= 7 are formed by
+//     mma.m16n8k16 and summed by order: integers below 2^24 times 2^-24, exact
+//     in FP32 over 128 columns (orders 4 to 7, worth 2^-32 and less, may round);
+//   * the sums are put together as a float pair, without loss for the orders 0
+//     to 3, and added to a running pair (TwoSum): every 128 columns, or where a
+//     larger term raises the row's scale.
+// Against the exact product (16 right-hand sides, 1,280 to 2,880 panels) the
+// error is 4e-16 of |H||x| in norm for random and 2.5e-15 for positive x; the
+// compensated sums of float pairs that this replaces had 3e-15 and 1e-14 to
+// 1.4e-13.  Time per pass, before -> now (HBM alone): 64,980 panels, leaves of 64 rows:
+// row 3.93 -> 1.00 ms (0.33), column 0.97 -> 0.50 ms (0.15); 327,680 panels,
+// leaves of 80: row 16.1 -> 7.2 ms (2.3), column 6.4 -> 3.6 ms (1.1).
+// Non-finite x or entries give NaN in the rows they reach.
 //
-// The three passes of the FP64 product, each with 16 right-hand sides:
-//   col_df_kernel : per leaf column cluster kappa, the partials x_kappa^T W
-//                   of its column panel (one thread per panel column, all 16
-//                   right-hand sides in registers, x_kappa staged in shared
-//                   memory);
-//   tsum_df_kernel: t_b = sum of b's partials in increasing cluster order;
-//   row_df_kernel : per leaf row cluster, the near-field panel times the
-//                   gathered x and the U panel times the gathered t (panel
-//                   chunks staged by cp.async, the K range shared by KS
-//                   thread groups, combined in a fixed order at the end).
-// The products use __fmul_rn / __fadd_rn / __fsub_rn so that no FMA
-// contraction changes the error-free transformations.
+//   scale_x / digits_x    : the scale of each x_r, the digits of x
+//   col_fx_kernel         : per leaf column cluster kappa the partials
+//                           x_kappa^T W of its column panel
+//   tsum_fx_kernel        : t_b = sum of b's partials in increasing cluster
+//                           order, and its digits
+//   row_fx_kernel         : per leaf row cluster, the near-field panel times
+//                           the gathered x and the U panel times the gathered t
+//   row_reduce_kernel     : the sums of the rows whose panels were split
+#include <cuda_fp16.h>
+
 #include <algorithm>
+#include <vector>
 
 #include "hm_internal.cuh"
 
 namespace hm {
-namespace df {
+namespace fx {
 
-constexpr int MR = 16;
-
-// w = h + l: h is w truncated to 24 significant bits, l = w - h rounded to
-// 24 bits (|w - h - l| <= 2^-47 |w|), from the bits of w: for 2^-74 <= |w| <
-// 2^128 the exponent and the top 23 fraction bits of w make h, the low 29
-// fraction bits (an integer m) make l = m 2^(e - 52) with e the unbiased
-// exponent of w.  |w| < 2^-126 (zeros included) gives (0, 0); the remaining
-// ranges, which BEM entries do not reach, use FP64 conversions.
-__device__ __forceinline__ void split(double w, float &h, float &l) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(w);
-    const uint32_t hi32 = (uint32_t)(b >> 32), lo32 = (uint32_t)b;
-    const uint32_t mag = hi32 & 0x7fffffffu, sgn = hi32 & 0x80000000u;
-    if (mag >= 0x3b500000u && mag < 0x47f00000u) {  // biased exponent in [949, 1151)
-        h = __uint_as_float(sgn | ((mag - 0x38000000u) << 3) | (lo32 >> 29));
-        const float m = __uint2float_rn(lo32 & 0x1fffffffu);
-        const float sc = __uint_as_float((uint32_t)((int)(mag >> 20) - 948) << 23);  // 2^(e - 52)
-        l = __uint_as_float(__float_as_uint(__fmul_rn(m, sc)) | sgn);
-    } else if (mag < 0x38100000u) {
-        h = 0.0f;
-        l = 0.0f;
-    } else {
-        h = __double2float_rz(w);
-        l = __double2float_rn(w - (double)h);
-    }
-}
-
-// (s, c) += (ah + al)(xh + xl): TwoProduct and TwoSum; the two errors and
-// the cross terms are summed first and reach c in one rounding per term (the
-// rounding errors of c itself are what bound the result: ~sqrt(n) u |c|)
-__device__ __forceinline__ void dfma(float &s, float &c, float ah, float al, float xh, float xl) {
-    const float p = __fmul_rn(ah, xh);
-    const float e = __fmaf_rn(ah, xh, -p);
-    const float t = __fadd_rn(s, p);
-    const float bp = __fsub_rn(t, s);
-    const float sg = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(p, bp));
-    s = t;
-    c = __fadd_rn(c, __fmaf_rn(al, xh, __fmaf_rn(ah, xl, __fadd_rn(e, sg))));
-}
+constexpr int MR = 16;              // right-hand sides of a pass
+constexpr int NA = 7;               // digits of an entry, and of an x
+constexpr int NO = 6;               // sums kept: the orders 0 to 5, and with the last 6 / 2^8 and 7 / 2^16
+constexpr int DIG = NA * MR;        // halves per row of digits ([digit, top first][rhs])
+constexpr int XSTRIDE = 2 * DIG + 16;  // bytes per staged row: 8 rows hit different banks (ldmatrix)
+constexpr int QB = 54;              // bits of an integer x
+constexpr int E_ZERO = -900;        // exponent of a column of zeros, and the smallest one
+constexpr int E_BIAS = 1000;        // added to the exponents of columns, which makes them positive
+constexpr int F_EXP = 884;          // a row's factor 2^(E - 1011) as a float: exponent field E - 884
+constexpr int E_NAN = F_EXP + 255;  // biased term exponents from here on: not finite, or beyond FP32
 
 // (s, c) += (s2, c2)
 __device__ __forceinline__ void dadd(float &s, float &c, float s2, float c2) {
@@ -94,89 +76,352 @@ __device__ __forceinline__ void norm2(float s, float c, float &h, float &l) {
     l = __fadd_rn(__fsub_rn(s, __fsub_rn(h, bp)), __fsub_rn(c, bp));
 }
 
-// X{h,l}[m][r] = x_r at Morton position m (x is [nr][n], original order when
-// perm is given), split into floats; zeros for r >= nr
-__global__ void split_x_kernel(const double *__restrict__ x, int64_t n, int nr, const int32_t *__restrict__ perm,
-                               float *__restrict__ Xh, float *__restrict__ Xl) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n * MR; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t m = e / MR;
-        const int r = (int)(e - m * MR);
-        const double v = r < nr ? x[(int64_t)r * n + (perm ? perm[m] : m)] : 0.0;
-        const float h = __double2float_rn(v);
-        Xh[e] = h;
-        Xl[e] = __double2float_rn(v - (double)h);
+__device__ __forceinline__ uint32_t saddr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+template <int N> __device__ __forceinline__ void cp_async(void *dst, const void *src, bool pred) {
+    if (N == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(saddr(dst)), "l"(src), "r"(pred ? 16 : 0)
+                     : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(saddr(dst)), "l"(src), "r"(pred ? 8 : 0)
+                     : "memory");
+}
+
+__device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// ---------------------------------------------------------------------------
+// digits of the vectors
+// ---------------------------------------------------------------------------
+// sc[r] = the largest high word of |x_r| (finite entries)
+__global__ void __launch_bounds__(256) scale_x_kernel(const double *__restrict__ x, int64_t n,
+                                                      unsigned int *__restrict__ sc) {
+    const double *xr = x + (int64_t)blockIdx.y * n;
+    unsigned int m = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const unsigned int h = (unsigned int)__double2hiint(xr[i]) & 0x7fffffffu;
+        if (h < 0x7ff00000u) m = max(m, h);
     }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(sc + blockIdx.y, m);
+}
+
+// |x_r| < 2^scale
+__device__ __forceinline__ int scale_of(unsigned int sc) { return sc >= 0x100000u ? (int)(sc >> 20) - 1022 : 0; }
+
+// the seven digits of q, |q| <= 2^54, as halves at o[0], o[MR], ... (top first)
+constexpr long long DIGIT_BIAS = 0x80808080808080ll;
+__device__ __forceinline__ void store_digits(long long q, __half *o) {
+    const unsigned long long u = (unsigned long long)(q + DIGIT_BIAS);
+#pragma unroll
+    for (int j = 0; j < NA; ++j) o[(NA - 1 - j) * MR] = __int2half_rn((int)((u >> (8 * j)) & 0xffu) - 128);
+}
+
+// Xd[m] = the digits of x_r 2^-(scale_r + e), Xe[m] = ((e + E_BIAS) 2^20, bits of the r
+// whose x_r is not finite), for position m (x is [nr][n], original order
+// when perm is given); zeros for r >= nr.  16 lanes per position.
+__global__ void __launch_bounds__(256) digits_x_kernel(const double *__restrict__ x, int64_t n, int nr,
+                                                       const int32_t *__restrict__ perm,
+                                                       const unsigned int *__restrict__ sc, __half *__restrict__ Xd,
+                                                       uint2 *__restrict__ Xe) {
+    const int r = threadIdx.x & 15;
+    const int S = r < nr ? scale_of(sc[r]) : 0;
+    const int64_t n2 = (n + 1) / 2 * 2;  // whole warps (two positions each)
+    for (int64_t m = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 4; m < n2;
+         m += ((int64_t)gridDim.x * blockDim.x) >> 4) {
+        const double v = m < n && r < nr ? x[(int64_t)r * n + (perm ? perm[m] : m)] : 0.0;
+        const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+        const int eb = (int)(b >> 52) & 0x7ff;
+        const bool bad = eb == 0x7ff;
+        const int ex = eb == 0 || bad ? E_ZERO : max(eb - 1022 - S, E_ZERO);
+        int e = ex;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+        const unsigned int bm = __ballot_sync(0xffffffffu, bad) >> (threadIdx.x & 16) & 0xffffu;
+        // the mantissa (53 bits) on the column's scale, rounded to nearest
+        long long q = 0;
+        const int sh = e - ex;
+        if (eb != 0 && !bad && sh < 63) {
+            const unsigned long long mant = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+            q = (long long)(((mant << (QB - 53)) + ((1ull << sh) >> 1)) >> sh);
+            if ((long long)b < 0) q = -q;
+        }
+        if (m < n) {
+            store_digits(q, Xd + m * DIG + r);
+            if (r == 0) Xe[m] = make_uint2((uint32_t)(e + E_BIAS) << 20, bm);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// digits of the entries and the products
+// ---------------------------------------------------------------------------
+// A row of a tile keeps one exponent E (in the top 12 bits of E20) for the
+// terms it is summing: at least that of the largest term so far and HEADROOM
+// more when it has to rise, which ends the sums so far (flush).  It starts so
+// high that zero and subnormal entries (exponent field 0) are shifted out
+// whatever their column's exponent.
+constexpr uint32_t HEADROOM = 1u << 20;
+constexpr uint32_t E20_START = (uint32_t)(E_BIAS + 320) << 20;
+
+// exponent (biased by 1023 + E_BIAS, times 2^20, plus some fraction bits) of the term w 2^e
+__device__ __forceinline__ uint32_t term_exp(double w, uint32_t e20) {
+    return ((uint32_t)__double2hiint(w) & 0x7fffffffu) + e20;
+}
+
+// E20 for terms up to tm where the present one is too small, else the present one
+__device__ __forceinline__ uint32_t raise_exp(uint32_t tm, uint32_t E20) {
+    return tm < E20 + 0x100000u ? E20 : (tm & 0xfff00000u) + HEADROOM;
+}
+
+// w 2^(e - E) as 55-bit fixed point plus 2^55: bytes 6..0 are the digits (the
+// top one plus 128)
+__device__ __forceinline__ void fixed_point(double w, uint32_t E20, uint32_t e20, uint32_t &lo, uint32_t &hi) {
+    const int h = __double2hiint(w);
+    const uint32_t s = min((E20 - e20 - ((uint32_t)h & 0x7ff00000u)) >> 20, 63u);
+    const unsigned long long v =
+        ((((unsigned long long)(uint32_t)((h & 0xfffff) | 0x100000) << 32) | (uint32_t)__double2loint(w)) << 2) >> s;
+    const uint32_t sg = (uint32_t)(h >> 31);
+    lo = (uint32_t)v ^ sg;
+    hi = (uint32_t)(v >> 32) ^ sg ^ 0x00800000u;
+}
+
+// the seven digits of two entries of consecutive k (columns with e20 = ea,
+// eb), packed for an A fragment (lower k in the low half): o[i][reg], top
+// digit first, as FP16 subnormals
+__device__ __forceinline__ void digit_pair(double a, double b, uint32_t E20, uint32_t ea, uint32_t eb, uint32_t (&o)[NA][4], int reg) {
+    uint32_t al, ah, bl, bh;
+    fixed_point(a, E20, ea, al, ah);
+    fixed_point(b, E20, eb, bl, bh);
+    const uint32_t t = __byte_perm(ah, bh, 0x6521);  // a5 a6 b5 b6
+    const uint32_t p = __byte_perm(al, bl, 0x6521);  // a1 a2 b1 b2
+    const uint32_t q = __byte_perm(al, bl, 0x7430);  // a0 a3 b0 b3
+    const uint32_t top = __byte_perm(t, 0, 0x4341);
+    const __half2 c = __hsub2(*reinterpret_cast<const __half2 *>(&top), __half2half2(__ushort_as_half(0x80)));
+    o[0][reg] = *reinterpret_cast<const uint32_t *>(&c);
+    o[1][reg] = __byte_perm(t, 0, 0x4240);
+    o[2][reg] = __byte_perm(ah, bh, 0x0400) & 0x00ff00ffu;  // a4 . b4 .
+    o[3][reg] = __byte_perm(q, 0, 0x4341);
+    o[4][reg] = __byte_perm(p, 0, 0x4341);
+    o[5][reg] = __byte_perm(p, 0, 0x4240);
+    o[6][reg] = __byte_perm(q, 0, 0x4240);
+}
+
+// acc[i + j] += A_i X_j over 16 rows of staged digits (row k at xs + k
+// XSTRIDE) for i + j < NO, and acc[NO - 1] += A_i X_j 2^(8 (NO - 1 - i - j)) for
+// the orders NO and NO + 1
+template <int NT>
+__device__ __forceinline__ void mma_orders(float (&acc)[NO][NT][4], const uint32_t (&a)[NA][4], const unsigned char *xs) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t base = saddr(xs) + (lane & 15) * XSTRIDE + (NT == 2 ? (lane >> 4) * 16 : 0);
+#pragma unroll
+    for (int j = 0; j < NA; ++j) {
+        uint32_t b[4];
+        if constexpr (NT == 2)
+            asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                         : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3])
+                         : "r"(base + j * 2 * MR));
+        else
+            asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n"
+                         : "=r"(b[0]), "=r"(b[1])
+                         : "r"(base + j * 2 * MR));
+#pragma unroll
+        for (int i = 0; i + j < NO; ++i)
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) mma_f16(acc[i + j][nt], a[i], b[2 * nt], b[2 * nt + 1]);
+        // orders NO (from j = 0) and NO + 1 (from j = 1) on the scale of the last sum
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            if (m == 1 && j == 0) continue;
+#pragma unroll
+            for (int k = 0; k < 2 * NT; ++k) {
+                const __half2 v = __hmul2(*reinterpret_cast<const __half2 *>(&b[k]), __float2half2_rn(0x1p-8f));
+                b[k] = *reinterpret_cast<const uint32_t *>(&v);
+            }
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) mma_f16(acc[NO - 1][nt], a[NO + m - j], b[2 * nt], b[2 * nt + 1]);
+        }
+    }
+}
+
+__device__ __forceinline__ int exp_of(uint32_t E20) { return (int)(E20 >> 20) - E_BIAS; }
+__device__ __forceinline__ float row_factor(uint32_t E20) {
+    const int E = exp_of(E20);
+    return E > F_EXP && E < E_NAN ? __uint_as_float((uint32_t)(E - F_EXP) << 23) : 0.0f;
+}
+
+// (h, l) += x with the rounding of h kept in l
+__device__ __forceinline__ void add_exact(float &h, float &l, float x) {
+    const float t = __fadd_rn(h, x);
+    const float bp = __fsub_rn(t, h);
+    l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(t, bp)), __fsub_rn(x, bp)));
+    h = t;
+}
+
+// (s, c) += 2^(E - 1011) sum_d acc_d 2^-8d for the rows g (E20 = e0) and g + 8
+// (e1) of a fragment; acc_d to zero.  The orders 0 to 3 are added without
+// loss (24 bits each, their rounding kept), the rest is below 2^-26 of order 0.
+template <int NT>
+__device__ __forceinline__ void flush(float (&acc)[NO][NT][4], uint32_t e0, uint32_t e1, float (&s)[NT][4], float (&c)[NT][4]) {
+    const float f0 = row_factor(e0), f1 = row_factor(e1);
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float f = e < 2 ? f0 : f1;
+            float h = acc[0][nt][e];
+            float l = __fmul_rn(__fmaf_rn(acc[5][nt][e], 0x1p-8f, acc[4][nt][e]), 0x1p-32f);
+            add_exact(h, l, __fmul_rn(acc[1][nt][e], 0x1p-8f));
+            add_exact(h, l, __fmul_rn(acc[2][nt][e], 0x1p-16f));
+            add_exact(h, l, __fmul_rn(acc[3][nt][e], 0x1p-24f));
+            dadd(s[nt][e], c[nt][e], __fmul_rn(h, f), __fmul_rn(l, f));
+#pragma unroll
+            for (int d = 0; d < NO; ++d) acc[d][nt][e] = 0.0f;
+        }
+}
+
+// largest of the four lanes of a quad (one fragment row)
+__device__ __forceinline__ uint32_t quad_max(uint32_t v) {
+    v = max(v, __shfl_xor_sync(0xffffffffu, v, 1));
+    return max(v, __shfl_xor_sync(0xffffffffu, v, 2));
 }
 
 // ---------------------------------------------------------------------------
 // column pass: P[wp_colptr[kappa] + v][r] = sum_j W_kappa[j][v] x_r[c0 + j]
+//
+// One warp per 16 panel columns (the rows of its fragments), 32 panel rows at
+// a time; x_kappa's digits in shared memory.  A lane holds two columns and the
+// panel rows 2t, 2t + 1, 2t + 8, 2t + 9 of a 16-row step, read from HBM by
+// 16-byte loads (128 contiguous bytes per panel row, eight in flight per lane).
 // ---------------------------------------------------------------------------
-constexpr int CD_THREADS = 256;
+constexpr int CW = 4;                    // warps per CTA
+constexpr int KC = 32;                   // panel rows (columns in the row pass) per chunk
+constexpr int FLUSH = 4;                 // chunks summed at most: 4 * 255 * 128 * (4 KC) < 2^24
 
-__device__ __forceinline__ void col_step(double w, const float4 *sx, float (&s)[MR], float (&c)[MR]) {
-    float ah, al;
-    split(w, ah, al);
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-        const float4 xh = sx[g], xl = sx[4 + g];
-        dfma(s[4 * g], c[4 * g], ah, al, xh.x, xl.x);
-        dfma(s[4 * g + 1], c[4 * g + 1], ah, al, xh.y, xl.y);
-        dfma(s[4 * g + 2], c[4 * g + 2], ah, al, xh.z, xl.z);
-        dfma(s[4 * g + 3], c[4 * g + 3], ah, al, xh.w, xl.w);
-    }
-}
-
-__global__ void __launch_bounds__(CD_THREADS) col_df_kernel(const int32_t *__restrict__ leaf_begin,
-                                                            const int64_t *__restrict__ wp_off,
-                                                            const int32_t *__restrict__ wp_K,
-                                                            const int64_t *__restrict__ wp_colptr,
-                                                            const double *__restrict__ wp, const float *__restrict__ Xh,
-                                                            const float *__restrict__ Xl, float2 *__restrict__ P,
-                                                            const int32_t *__restrict__ order) {
-    __shared__ float4 sx[MAX_LEAF * 8];  // row j of x_kappa: hi [16] then lo [16]
-    const int64_t kap = order ? order[blockIdx.x] : blockIdx.x;
-    const int32_t c0 = leaf_begin[kap], mc = leaf_begin[kap + 1] - c0;
-    const float4 *xh4 = reinterpret_cast<const float4 *>(Xh), *xl4 = reinterpret_cast<const float4 *>(Xl);
-    for (int e = threadIdx.x; e < mc * 8; e += CD_THREADS) {
-        const int j = e >> 3, q = e & 7;
-        sx[e] = q < 4 ? xh4[(int64_t)(c0 + j) * 4 + q] : xl4[(int64_t)(c0 + j) * 4 + q - 4];
-    }
-    __syncthreads();
+template <int NT>
+__global__ void __launch_bounds__(32 * CW, 4) col_fx_kernel(int parts, const int32_t *__restrict__ leaf_begin,
+                                                         const int64_t *__restrict__ wp_off,
+                                                         const int32_t *__restrict__ wp_K,
+                                                         const int64_t *__restrict__ wp_colptr,
+                                                         const double *__restrict__ wp, const __half *__restrict__ Xd,
+                                                         const uint2 *__restrict__ Xe, float2 *__restrict__ P,
+                                                         const int32_t *__restrict__ order) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int q = blockIdx.x / parts, part = blockIdx.x - q * parts;
+    const int64_t kap = order ? order[q] : q;
     const int Kw = wp_K[kap];
-    const double *W = wp + wp_off[kap];
-    float4 *out = reinterpret_cast<float4 *>(P + wp_colptr[kap] * MR);
-    for (int v = threadIdx.x; v < Kw; v += CD_THREADS) {
-        float s[MR], c[MR];
+    if (part * 16 * CW >= Kw) return;
+    const int32_t c0 = leaf_begin[kap], mc = leaf_begin[kap + 1] - c0;
+    const int mp = (mc + KC - 1) / KC * KC;
+    uint2 *se = reinterpret_cast<uint2 *>(smem);      // [mp]
+    unsigned char *xs = smem + 8 * mp;              // [mp][XSTRIDE]
+    for (int e = threadIdx.x; e < mp * 2; e += 32 * CW) {
+        const int j = e >> 1, p = NA * (e & 1);
 #pragma unroll
-        for (int r = 0; r < MR; ++r) s[r] = c[r] = 0.0f;
-        const double *col = W + v;
-        int j = 0;
-        for (; j + 3 < mc; j += 4) {  // four loads in flight
-            const double w0 = __ldg(col + (int64_t)j * Kw), w1 = __ldg(col + (int64_t)(j + 1) * Kw);
-            const double w2 = __ldg(col + (int64_t)(j + 2) * Kw), w3 = __ldg(col + (int64_t)(j + 3) * Kw);
-            col_step(w0, sx + j * 8, s, c);
-            col_step(w1, sx + (j + 1) * 8, s, c);
-            col_step(w2, sx + (j + 2) * 8, s, c);
-            col_step(w3, sx + (j + 3) * 8, s, c);
+        for (int i = 0; i < NA; ++i) {
+            uint4 v = make_uint4(0, 0, 0, 0);
+            if (j < mc) v = __ldg(reinterpret_cast<const uint4 *>(Xd + (int64_t)(c0 + j) * DIG) + p + i);
+            *reinterpret_cast<uint4 *>(xs + j * XSTRIDE + 16 * (p + i)) = v;
         }
-        for (; j < mc; ++j) col_step(__ldg(col + (int64_t)j * Kw), sx + j * 8, s, c);
+    }
+    for (int j = threadIdx.x; j < mp; j += 32 * CW) se[j] = j < mc ? __ldg(Xe + c0 + j) : make_uint2(0, 0);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    unsigned int bad = 0;
+    for (int j = lane; j < mp; j += 32) bad |= se[j].y;
+    bad = __reduce_or_sync(0xffffffffu, bad);
+    const double *W = wp + wp_off[kap];
+    for (int v0 = 16 * (part * CW + warp); v0 < Kw; v0 += 16 * CW * parts) {
+        const int v = v0 + 2 * g;
+        const bool ok = v < Kw;  // Kw is even
+        const double *col = W + (ok ? v : 0) + (int64_t)(2 * t) * Kw;
+        float acc[NO][NT][4], s[NT][4], c[NT][4];
 #pragma unroll
-        for (int r = 0; r < MR; r += 2) out[(int64_t)v * 8 + r / 2] = make_float4(s[r], c[r], s[r + 1], c[r + 1]);
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                s[nt][e] = c[nt][e] = 0.0f;
+#pragma unroll
+                for (int d = 0; d < NO; ++d) acc[d][nt][e] = 0.0f;
+            }
+        uint32_t E0 = E20_START, E1 = E20_START;
+        int held = 0;
+#pragma unroll 1
+        for (int k0 = 0; k0 < mc; k0 += KC, col += (int64_t)KC * Kw) {
+            double2 w[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int j = 8 * (i >> 1) + (i & 1);  // panel row k0 + 2t + j
+                w[i] = make_double2(0.0, 0.0);
+                if (ok && k0 + 2 * t + j < mc) w[i] = __ldg(reinterpret_cast<const double2 *>(col + (int64_t)j * Kw));
+            }
+            uint32_t m0 = 0, m1 = 0;
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+                const uint4 e = *reinterpret_cast<const uint4 *>(se + k0 + 2 * t + 4 * i);
+                m0 = max(m0, max(term_exp(w[i].x, e.x), term_exp(w[i + 1].x, e.z)));
+                m1 = max(m1, max(term_exp(w[i].y, e.x), term_exp(w[i + 1].y, e.z)));
+            }
+            const uint32_t n0 = raise_exp(quad_max(m0), E0), n1 = raise_exp(quad_max(m1), E1);
+            if (__any_sync(0xffffffffu, n0 != E0 || n1 != E1) || held == FLUSH) {
+                if (held) flush<NT>(acc, E0, E1, s, c);
+                held = 0;
+                E0 = n0;
+                E1 = n1;
+            }
+            ++held;
+#pragma unroll
+            for (int kk = 0; kk < KC; kk += 16) {
+                if (k0 + kk >= mc) break;
+                uint32_t a[NA][4];
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    const uint4 e = *reinterpret_cast<const uint4 *>(se + k0 + kk + 8 * hf + 2 * t);
+                    const double2 x = w[kk / 4 + 2 * hf], y = w[kk / 4 + 2 * hf + 1];
+                    digit_pair(x.x, y.x, E0, e.x, e.z, a, 2 * hf);
+                    digit_pair(x.y, y.y, E1, e.x, e.z, a, 2 * hf + 1);
+                }
+                mma_orders<NT>(acc, a, xs + (k0 + kk) * XSTRIDE);
+            }
+        }
+        flush<NT>(acc, E0, E1, s, c);
+        const int worst = (exp_of(E0) >= E_NAN ? 1 : 0) | (exp_of(E1) >= E_NAN ? 2 : 0);
+        if (!ok) continue;
+        const float nan = __uint_as_float(0x7fffffffu);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {  // columns v, v + 1
+            float4 *o = reinterpret_cast<float4 *>(P + (wp_colptr[kap] + v + h) * MR);
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                const int r = 8 * nt + 2 * t;
+                float4 w = make_float4(s[nt][2 * h], c[nt][2 * h], s[nt][2 * h + 1], c[nt][2 * h + 1]);
+                if ((worst >> h & 1) || (bad >> r & 1)) w.x = nan;
+                if ((worst >> h & 1) || (bad >> (r + 1) & 1)) w.z = nan;
+                o[r / 2] = w;
+            }
+        }
     }
 }
 
 // ---------------------------------------------------------------------------
 // t_b(l) = sum over the column clusters of sigma_b of the partials, in
-// increasing cluster order: one lane per entry of t (all 16 right-hand
+// increasing cluster order, as digits: one lane per entry of t (all right-hand
 // sides), 32 consecutive entries per warp; the entry's block is found from
 // b0[c] (the block holding entry 32 c) by a search over the next 32 blocks'
 // offsets, or over t_off beyond them.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) tsum_df_kernel(int64_t na, int64_t nt, const int32_t *__restrict__ b0tab,
+constexpr int T_EMIN = -70;  // smallest exponent of a non-zero row of t (2^(54 - e) stays a float)
+
+template <int NT>
+__global__ void __launch_bounds__(256) tsum_fx_kernel(int64_t na, int64_t nt, const int32_t *__restrict__ b0tab,
                                                       const int64_t *__restrict__ t_off,
                                                       const int64_t *__restrict__ bcolptr,
                                                       const int64_t *__restrict__ pofs, const float2 *__restrict__ P,
-                                                      float *__restrict__ Th, float *__restrict__ Tl) {
+                                                      __half *__restrict__ Td, uint2 *__restrict__ Te) {
+    constexpr int NR = 8 * NT;
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -206,157 +451,255 @@ __global__ void __launch_bounds__(256) tsum_df_kernel(int64_t na, int64_t nt, co
             b = lo;
         }
         const int64_t l = e - t_off[b];
-        float s[MR], c[MR];
+        float s[NR], c[NR];
 #pragma unroll
-        for (int r = 0; r < MR; ++r) s[r] = c[r] = 0.0f;
+        for (int r = 0; r < NR; ++r) s[r] = c[r] = 0.0f;
         for (int64_t q = bcolptr[b]; q < bcolptr[b + 1]; ++q) {
             const float4 *pp = reinterpret_cast<const float4 *>(P + (pofs[q] + l) * MR);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
+            for (int k = 0; k < NR / 2; ++k) {
                 const float4 v = __ldg(pp + k);
                 dadd(s[2 * k], c[2 * k], v.x, v.y);
                 dadd(s[2 * k + 1], c[2 * k + 1], v.z, v.w);
             }
         }
-        float h[MR], lo[MR];
+        // (s, c) normalised; the exponent of the largest
+        int ex = E_ZERO;
+        unsigned int bad = 0;
 #pragma unroll
-        for (int r = 0; r < MR; ++r) norm2(s[r], c[r], h[r], lo[r]);
-        float4 *th = reinterpret_cast<float4 *>(Th + e * MR), *tl = reinterpret_cast<float4 *>(Tl + e * MR);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            th[k] = make_float4(h[4 * k], h[4 * k + 1], h[4 * k + 2], h[4 * k + 3]);
-            tl[k] = make_float4(lo[4 * k], lo[4 * k + 1], lo[4 * k + 2], lo[4 * k + 3]);
+        for (int r = 0; r < NR; ++r) {
+            float h, lo;
+            norm2(s[r], c[r], h, lo);
+            s[r] = h;
+            c[r] = lo;
+            const int eb = (int)(__float_as_uint(h) >> 23) & 0xff;
+            if (eb == 0xff) bad |= 1u << r;
+            else if (eb) ex = max(ex, max(eb - 126, T_EMIN));
         }
+        Te[e] = make_uint2((uint32_t)(ex + E_BIAS) << 20, bad);
+        const float sc = __uint_as_float((uint32_t)(127 + QB - max(ex, T_EMIN)) << 23);  // 2^(54 - ex)
+        unsigned long long u[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const uint32_t hb = __float_as_uint(s[r]);
+            const int eb = (int)(hb >> 23) & 0xff;
+            long long q = 0;
+            if (eb != 0 && eb != 0xff) {
+                const int sh = QB - 24 - (ex - (eb - 126));  // h = mantissa 2^(eb - 126 - 24)
+                const long long mant = (long long)((hb & 0x7fffffu) | 0x800000u);
+                q = sh >= 0 ? mant << sh : sh > -25 ? mant >> -sh : 0;
+                if ((int)hb < 0) q = -q;
+                q += __float2int_rn(__fmul_rn(c[r], sc));
+            }
+            u[r] = (unsigned long long)(q + DIGIT_BIAS);
+        }
+        uint4 *o = reinterpret_cast<uint4 *>(Td + e * DIG);
+#pragma unroll
+        for (int j2 = 0; j2 < NA; ++j2)
+#pragma unroll
+            for (int k = 0; k < NT; ++k) {
+                uint32_t w[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int sh = 8 * (NA - 1 - j2), r = 8 * k + 2 * i;
+                    // 1024 + u as a half, minus 1152
+                    const uint32_t d = 0x64006400u | (uint32_t)((u[r] >> sh) & 0xffu) | (uint32_t)((u[r + 1] >> sh) & 0xffu) << 16;
+                    const __half2 hd = __hsub2(*reinterpret_cast<const __half2 *>(&d), __float2half2_rn(1152.0f));
+                    w[i] = *reinterpret_cast<const uint32_t *>(&hd);
+                }
+                o[2 * j2 + k] = make_uint4(w[0], w[1], w[2], w[3]);
+            }
     }
 }
 
 // ---------------------------------------------------------------------------
 // row pass: Y[r0 + i][r] = sum_k D[i][k] x_r[colidx k] + sum_k U[i][k] t_r[tidx k]
-// One CTA per leaf row cluster (tiles of TR rows), TR x KS threads: thread
-// (i, g) accumulates row i over the columns k = g, g + KS, ... of each
-// chunk of KC columns and splits the FP64 entries it uses itself (each
-// entry is used by one thread).  The chunks of both panels stream through two
-// shared-memory buffers by cp.async: the FP64 panel rows ([TR][AST] doubles,
-// zeros past the panel) and the gathered rows of x or t ([KC][hi 16, lo
-// 16]); a chunk's copies are issued while the previous one is multiplied,
-// its gather indices one chunk earlier.  The KS partial sums of a row are
-// added in increasing g.
+//
+// One CTA per 16 MT rows of a leaf row cluster, one warp per 16 rows.  The
+// panels are walked in chunks of 32 columns through two shared-memory buffers
+// filled by cp.async: the FP64 rows of the chunk, and the digits and exponents
+// of the gathered rows of x or t.  A warp takes the largest term of each of its
+// rows in the chunk, forms the digits of its entries (each entry by one lane)
+// and multiplies.  Per 16 x 16 entries: 68 products of 16 x 8 x 16 (~150 cycles of an
+// SM), ~22 integer operations per entry (~80 cycles of the ALU pipe), 2 KB from
+// HBM (~95 cycles).
 // ---------------------------------------------------------------------------
-constexpr int KC = 32;
-constexpr int AST = KC + 2;  // doubles per staged panel row (16-byte aligned rows)
-
-template <int TR, int KS> struct RowCfg {
-    static constexpr int NT = TR * KS;
-    static constexpr int ABYTES = TR * AST * 8;
-    static constexpr int BUF = ABYTES + KC * 8 * 16;
-    static constexpr int PA = (TR * KC / 2 + NT - 1) / NT;  // 16-byte panel pieces per thread and chunk
-    static constexpr int RED = KS * TR * MR * 8;
-    static constexpr int SMEM = 2 * BUF > RED ? 2 * BUF : RED;
-    static_assert(NT >= KC * 8, "one gathered piece per thread and chunk");
+constexpr int AST = KC * 8 + 64;          // bytes per staged panel row: row pairs fill the banks
+template <int MT> struct RowCfg {
+    static constexpr int THREADS = 32 * MT;
+    static constexpr int A_BYTES = 16 * MT * AST;
+    static constexpr int STAGE = A_BYTES + KC * XSTRIDE + KC * 8;
+    static constexpr int SMEM = 2 * STAGE + 2 * KC * 4;
+    static constexpr int CTAS = MT <= 2 ? 6 : MT == 3 ? 5 : MT == 4 ? 4 : 3;  // per SM: 128 registers, shared memory
 };
 
-__device__ __forceinline__ uint32_t saddr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void cp16(void *dst, const void *src, bool pred) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(saddr(dst)), "l"(src), "r"(pred ? 16 : 0)
-                 : "memory");
+template <int MT, int NT>
+__global__ void __launch_bounds__(32 * MT, RowCfg<MT>::CTAS) row_fx_kernel(
+    int parts, const int32_t *__restrict__ leaf_begin, const int64_t *__restrict__ rho_off,
+    const int32_t *__restrict__ rho_K, const int64_t *__restrict__ rho_colptr, const int32_t *__restrict__ colidx,
+    const double *__restrict__ dense, const int64_t *__restrict__ up_off, const int32_t *__restrict__ up_K,
+    const int64_t *__restrict__ up_colptr, const int32_t *__restrict__ tidx, const double *__restrict__ up,
+    const __half *__restrict__ Xd, const uint2 *__restrict__ Xe, const __half *__restrict__ Td,
+    const uint2 *__restrict__ Te, const unsigned int *__restrict__ sc, double *__restrict__ Y,
+    const int4 *__restrict__ items, float2 *__restrict__ Ypart, int prow) {
+    using C = RowCfg<MT>;
+    extern __shared__ __align__(16) unsigned char smem[];
+    int32_t *s_idx = reinterpret_cast<int32_t *>(smem + 2 * C::STAGE);  // [2][KC]
+    const int q = blockIdx.x / parts, part = blockIdx.x - q * parts;
+    const int4 it = items[q];  // cluster, chunks [y, z), partial slot or -1
+    const int rho = it.x, cend = it.z;
+    const int32_t r0 = leaf_begin[rho] + part * 16 * MT;
+    const int rows = min(16 * MT, leaf_begin[rho + 1] - r0);
+    if (rows <= 0) return;
+    const int Kd = rho_K[rho], Ku = up_K[rho];
+    const int nd = (Kd + KC - 1) / KC;
+    const double *Pd = dense + rho_off[rho] + (int64_t)part * 16 * MT * Kd;
+    const double *Pu = up + up_off[rho] + (int64_t)part * 16 * MT * Ku;
+    const int32_t *ci = colidx + rho_colptr[rho], *ti = tidx + up_colptr[rho];
+    const int tid = threadIdx.x;
+    // gather indices of chunk c (-1: past the panel)
+    auto load_idx = [&](int c) {
+        for (int k = tid; k < KC; k += C::THREADS) {
+            const bool u = c >= nd;
+            const int K = u ? Ku : Kd, col = (u ? c - nd : c) * KC + k;
+            s_idx[(c & 1) * KC + k] = c < cend && col < K ? __ldg((u ? ti : ci) + col) : -1;
+        }
+    };
+    // this thread's pieces of a chunk: 16 bytes of the panel rows arow, arow +
+    // THREADS / 16, ... and pieces of the digits of a column
+    const int arow = tid >> 4, acol = 2 * (tid & 15);
+    auto issue = [&](int c) {
+        unsigned char *st = smem + (c & 1) * C::STAGE;
+        const bool u = c >= nd;
+        const int K = u ? Ku : Kd, k0 = (u ? c - nd : c) * KC;
+        const double *P = u ? Pu : Pd;
+        const bool in = k0 + acol < K;
+        const double *src = P + (int64_t)arow * K + k0 + acol;
+        unsigned char *dst = st + arow * AST + acol * 8;
+#pragma unroll
+        for (int v = 0; v < 8; ++v, src += (C::THREADS / 16) * (int64_t)K) {
+            const bool ok = in && arow + (C::THREADS / 16) * v < rows;
+            cp_async<16>(dst + (C::THREADS / 16) * v * AST, ok ? src : P, ok);
+        }
+        const __half *Z = u ? Td : Xd;
+        const uint2 *Ze = u ? Te : Xe;
+        unsigned char *sb = st + C::A_BYTES;
+        const int32_t *ix = s_idx + (c & 1) * KC;
+        // two neighbouring threads take 16 bytes each of a column in turn
+#pragma unroll
+        for (int e0 = 0; e0 < KC * 2; e0 += C::THREADS) {
+            const int e = e0 + tid, k = e >> 1, p = e & 1;
+            if (e0 + C::THREADS <= KC * 2 || e < KC * 2) {
+                const int z = ix[k];
+                const __half *zs = Z + (int64_t)max(z, 0) * DIG + 8 * p;
+                unsigned char *zd = sb + k * XSTRIDE + 16 * p;
+#pragma unroll
+                for (int i = 0; i < NA; ++i) cp_async<16>(zd + 32 * i, zs + 16 * i, z >= 0);
+                if (p == 0) cp_async<8>(sb + KC * XSTRIDE + 8 * k, Ze + max(z, 0), z >= 0);
+            }
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+    float acc[NO][NT][4], s[NT][4], c[NT][4];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            s[nt][e] = c[nt][e] = 0.0f;
+#pragma unroll
+            for (int d = 0; d < NO; ++d) acc[d][nt][e] = 0.0f;
+        }
+    unsigned int bad = 0;
+    uint32_t E0 = E20_START, E1 = E20_START;
+    int held = 0;
+    load_idx(it.y);
+    load_idx(it.y + 1);
+    __syncthreads();
+    if (it.y < cend) issue(it.y);
+#pragma unroll 1
+    for (int ch = it.y; ch < cend; ++ch) {
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        __syncthreads();  // chunk ch has landed for every thread; every thread is done with chunk ch - 1
+        if (ch + 1 < cend) issue(ch + 1);
+        const unsigned char *st = smem + (ch & 1) * C::STAGE;
+        const double *a0 = reinterpret_cast<const double *>(st + (16 * warp + g) * AST) + 2 * t;
+        const double *a1 = reinterpret_cast<const double *>(st + (16 * warp + g + 8) * AST) + 2 * t;
+        const unsigned char *sb = st + C::A_BYTES;
+        const uint2 *se = reinterpret_cast<const uint2 *>(sb + KC * XSTRIDE) + 2 * t;
+        uint32_t m0 = 0, m1 = 0;
+#pragma unroll
+        for (int k = 0; k < KC; k += 8) {
+            const double2 w0 = *reinterpret_cast<const double2 *>(a0 + k), w1 = *reinterpret_cast<const double2 *>(a1 + k);
+            const uint4 e = *reinterpret_cast<const uint4 *>(se + k);
+            bad |= e.y | e.w;
+            m0 = max(m0, max(term_exp(w0.x, e.x), term_exp(w0.y, e.z)));
+            m1 = max(m1, max(term_exp(w1.x, e.x), term_exp(w1.y, e.z)));
+        }
+        const uint32_t n0 = raise_exp(quad_max(m0), E0), n1 = raise_exp(quad_max(m1), E1);
+        if (__any_sync(0xffffffffu, n0 != E0 || n1 != E1) || held == FLUSH) {
+            if (held) flush<NT>(acc, E0, E1, s, c);
+            held = 0;
+            E0 = n0;
+            E1 = n1;
+        }
+        ++held;
+#pragma unroll
+        for (int k = 0; k < KC; k += 16) {
+            uint32_t a[NA][4];
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                const double2 w0 = *reinterpret_cast<const double2 *>(a0 + k + 8 * hf);
+                const double2 w1 = *reinterpret_cast<const double2 *>(a1 + k + 8 * hf);
+                const uint4 e = *reinterpret_cast<const uint4 *>(se + k + 8 * hf);
+                digit_pair(w0.x, w0.y, E0, e.x, e.z, a, 2 * hf);
+                digit_pair(w1.x, w1.y, E1, e.x, e.z, a, 2 * hf + 1);
+            }
+            mma_orders<NT>(acc, a, sb + k * XSTRIDE);
+        }
+        // the indices of chunk ch + 2 (chunk ch's were read by issue(ch), an iteration ago)
+        load_idx(ch + 2);
+    }
+    flush<NT>(acc, E0, E1, s, c);
+    const int worst = (exp_of(E0) >= E_NAN ? 1 : 0) | (exp_of(E1) >= E_NAN ? 2 : 0);
+    bad = __reduce_or_sync(0xffffffffu, bad);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int row = 16 * warp + g + 8 * h;
+        if (row >= rows) continue;
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int r = 8 * nt + 2 * t + e;
+                float hi = s[nt][2 * h + e];
+                if ((worst >> h & 1) || (bad >> r & 1)) hi = __uint_as_float(0x7fffffffu);  // NaN
+                if (it.w >= 0)
+                    Ypart[((int64_t)it.w * prow + part * 16 * MT + row) * MR + r] = make_float2(hi, c[nt][2 * h + e]);
+                else
+                    Y[(int64_t)(r0 + row) * MR + r] =
+                        scalbn((double)hi + (double)c[nt][2 * h + e], scale_of(sc[r]));
+            }
+    }
 }
 
-template <int TR, int KS>
-__global__ void __launch_bounds__(TR *KS, 2) row_df_kernel(
-    const int32_t *__restrict__ leaf_begin, const int64_t *__restrict__ rho_off, const int32_t *__restrict__ rho_K,
-    const int64_t *__restrict__ rho_colptr, const int32_t *__restrict__ colidx, const double *__restrict__ dense,
-    const int64_t *__restrict__ up_off, const int32_t *__restrict__ up_K, const int64_t *__restrict__ up_colptr,
-    const int32_t *__restrict__ tidx, const double *__restrict__ up, const float *__restrict__ Xh,
-    const float *__restrict__ Xl, const float *__restrict__ Th, const float *__restrict__ Tl, double *__restrict__ Y,
-    const int32_t *__restrict__ order) {
-    using C = RowCfg<TR, KS>;
-    constexpr int NT = C::NT;
-    extern __shared__ __align__(16) unsigned char smem[];
-    float2 *red = reinterpret_cast<float2 *>(smem);  // [KS][TR][MR], after the last chunk
-    const int t = threadIdx.x, i = t % TR, g = t / TR;
-    const int64_t rho = order ? order[blockIdx.x] : blockIdx.x;
-    const int32_t r0 = leaf_begin[rho], mr = leaf_begin[rho + 1] - r0;
-    const int Kd = rho_K[rho], Ku = up_K[rho];
-    const int nd = (Kd + KC - 1) / KC, nc = nd + (Ku + KC - 1) / KC;
-    const double *Pd = dense + rho_off[rho], *Pu = up + up_off[rho];
-    const int32_t *ci = colidx + rho_colptr[rho], *ti = tidx + up_colptr[rho];
-    const float4 *xh4 = reinterpret_cast<const float4 *>(Xh), *xl4 = reinterpret_cast<const float4 *>(Xl);
-    const float4 *th4 = reinterpret_cast<const float4 *>(Th), *tl4 = reinterpret_cast<const float4 *>(Tl);
-    const int zk = t >> 3, zq = t & 7;  // this thread's gathered piece: column zk, quarter zq (hi 0-3, lo 4-7)
-    for (int r0t = 0; r0t < mr; r0t += TR) {
-        const int rows = min(TR, mr - r0t);
-        // gather index of chunk c for this thread's piece (-1: past the panel)
-        auto zindex = [&](int c) -> int {
-            const bool u = c >= nd;
-            const int K = u ? Ku : Kd, k = (u ? c - nd : c) * KC + zk;
-            return (t < KC * 8 && k < K) ? __ldg((u ? ti : ci) + k) : -1;
-        };
-        auto issue = [&](int c, int zi) {
-            unsigned char *buf = smem + (c & 1) * C::BUF;
-            const bool u = c >= nd;
-            const int K = u ? Ku : Kd, k0 = (u ? c - nd : c) * KC;
-            const double *P = (u ? Pu : Pd) + (int64_t)r0t * K;
-#pragma unroll
-            for (int v = 0; v < C::PA; ++v) {
-                const int e = t + NT * v, row = e / (KC / 2), col = 2 * (e % (KC / 2));
-                if (e < TR * KC / 2) {
-                    const bool ok = row < rows && k0 + col < K;
-                    cp16(buf + (row * AST + col) * 8, ok ? P + (int64_t)row * K + k0 + col : P, ok);
-                }
-            }
-            if (t < KC * 8) {
-                const float4 *z = zq < 4 ? (u ? th4 : xh4) : (u ? tl4 : xl4);
-                cp16(buf + C::ABYTES + t * 16, z + (int64_t)max(zi, 0) * 4 + (zq & 3), zi >= 0);
-            }
-            asm volatile("cp.async.commit_group;\n" ::: "memory");
-        };
-        float s[MR], c[MR];
-#pragma unroll
-        for (int r = 0; r < MR; ++r) s[r] = c[r] = 0.0f;
-        if (nc > 0) issue(0, zindex(0));
-        int zi = nc > 1 ? zindex(1) : -1;
-        for (int ch = 0; ch < nc; ++ch) {
-            if (ch + 1 < nc) {
-                issue(ch + 1, zi);
-                if (ch + 2 < nc) zi = zindex(ch + 2);
-                asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-            } else {
-                asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-            }
-            __syncthreads();  // chunk ch has landed for every thread
-            const unsigned char *buf = smem + (ch & 1) * C::BUF;
-            const double *sa = reinterpret_cast<const double *>(buf) + i * AST;
-            const float4 *sz = reinterpret_cast<const float4 *>(buf + C::ABYTES);
-            const int K = ch < nd ? Kd : Ku, kc = min(KC, K - (ch < nd ? ch : ch - nd) * KC);
-            for (int k = g; k < kc; k += KS) {
-                float ah, al;
-                split(sa[k], ah, al);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float4 xh = sz[k * 8 + q], xl = sz[k * 8 + 4 + q];
-                    dfma(s[4 * q], c[4 * q], ah, al, xh.x, xl.x);
-                    dfma(s[4 * q + 1], c[4 * q + 1], ah, al, xh.y, xl.y);
-                    dfma(s[4 * q + 2], c[4 * q + 2], ah, al, xh.z, xl.z);
-                    dfma(s[4 * q + 3], c[4 * q + 3], ah, al, xh.w, xl.w);
-                }
-            }
-            __syncthreads();  // every thread is done with this buffer before it is refilled
+// rows of the clusters whose panels were split: Y = the sum of the partials
+// in slot order (red: cluster, first slot, slots)
+template <int NT>
+__global__ void __launch_bounds__(256) row_reduce_kernel(const int4 *__restrict__ red, const int32_t *__restrict__ leaf_begin,
+                                                         const float2 *__restrict__ Ypart, int prow,
+                                                         const unsigned int *__restrict__ sc, double *__restrict__ Y) {
+    const int4 rd = red[blockIdx.x];
+    const int32_t r0 = leaf_begin[rd.x], mr = leaf_begin[rd.x + 1] - r0;
+    for (int e = threadIdx.x; e < mr * 8 * NT; e += 256) {
+        const int row = e / (8 * NT), r = e - row * (8 * NT);
+        float s = 0.0f, c = 0.0f;
+#pragma unroll 4
+        for (int k = 0; k < rd.z; ++k) {
+            const float2 v = Ypart[((int64_t)(rd.y + k) * prow + row) * MR + r];
+            dadd(s, c, v.x, v.y);
         }
-        // the KS partial sums of each row, in increasing g
-#pragma unroll
-        for (int r = 0; r < MR; ++r) red[(g * TR + i) * MR + r] = make_float2(s[r], c[r]);
-        __syncthreads();
-        for (int o = t; o < TR * MR; o += NT) {
-            const int ii = o / MR, r = o % MR;
-            if (ii >= rows) continue;
-            float2 v = red[ii * MR + r];
-            for (int gg = 1; gg < KS; ++gg) {
-                const float2 w = red[(gg * TR + ii) * MR + r];
-                dadd(v.x, v.y, w.x, w.y);
-            }
-            Y[(int64_t)(r0 + r0t + ii) * MR + r] = (double)v.x + (double)v.y;
-        }
-        __syncthreads();  // the next tile's copies reuse this memory
+        Y[(int64_t)(r0 + row) * MR + r] = scalbn((double)s + (double)c, scale_of(sc[r]));
     }
 }
 
@@ -372,68 +715,147 @@ __global__ void scatter_kernel(const double *__restrict__ Y, int64_t n, int nr, 
     }
 }
 
-template <int TR, int KS>
-static void launch_row(const hm_matrix *A, const float *Xh, const float *Xl, const float *Th, const float *Tl,
-                       double *Y, const int32_t *ord, cudaStream_t s) {
-    const hm_tree *tr = A->tree;
-    using C = RowCfg<TR, KS>;
-    auto kern = row_df_kernel<TR, KS>;
-    HM_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    Trace trace("row_df_kernel", s);
-    kern<<<(unsigned)tr->n_leaf, C::NT, C::SMEM, s>>>(
-        tr->leaf_begin.as<int32_t>(), tr->rho_off.as<int64_t>(), tr->rho_K.as<int32_t>(), tr->rho_colptr.as<int64_t>(),
-        tr->colidx.as<int32_t>(), A->dense.as<double>(), A->up_off.as<int64_t>(), A->up_K.as<int32_t>(),
-        A->up_colptr.as<int64_t>(), A->tidx.as<int32_t>(), A->up.as<double>(), Xh, Xl, Th, Tl, Y, ord);
-    HM_LAUNCH_CHECK();
-}
-
 // blocks of 256 threads for a grid-stride loop over n items
 static unsigned grid_for(int64_t n) {
     const int64_t b = (n + 255) / 256;
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>(b, 65535LL * 8));
 }
 
-}  // namespace df
+// the working arrays of one pass, in this order (each a multiple of 16 bytes)
+struct Work {
+    __half *Xd, *Td;
+    float2 *P, *Ypart;
+    uint2 *Xe, *Te;
+    unsigned int *sc;
+};
 
-// floats of the working arrays of one 16-right-hand-side pass: x pairs
-// (2 x 16 n), partials (2 x 16 P), t pairs (2 x 16 K), Y (16 n doubles)
+template <int NT>
+static void block_product(const hm_matrix *A, const double *x, int nr, const int32_t *perm, double *Y, const Work &w,
+                          cudaStream_t s) {
+    const hm_tree *tr = A->tree;
+    const int64_t n = tr->n, nl = tr->n_leaf;
+    HM_CUDA_CHECK(cudaMemsetAsync(w.sc, 0, sizeof(unsigned int) * MR, s));
+    const dim3 gs((unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, 256)), (unsigned)nr);
+    scale_x_kernel<<<gs, 256, 0, s>>>(x, n, w.sc);
+    HM_LAUNCH_CHECK();
+    digits_x_kernel<<<grid_for(n * MR), 256, 0, s>>>(x, n, nr, perm, w.sc, w.Xd, w.Xe);
+    HM_LAUNCH_CHECK();
+    const int32_t *ord = A->mv_order.as<int32_t>();
+    if (tr->n_adm > 0) {
+        {
+            const int smem = (tr->max_leaf + KC - 1) / KC * KC * (XSTRIDE + 8);
+            HM_CUDA_CHECK(cudaFuncSetAttribute(col_fx_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            const int parts = ((A->wp_kmax + 16 * CW * 4 - 1) / (16 * CW * 4)) | 1;  // odd: see col_kernel
+            Trace trace("col_fx_kernel", s);
+            col_fx_kernel<NT><<<(unsigned)(nl * parts), 32 * CW, smem, s>>>(
+                parts, tr->leaf_begin.as<int32_t>(), A->wp_off.as<int64_t>(), A->wp_K.as<int32_t>(),
+                A->wp_colptr.as<int64_t>(), A->wp.as<double>(), w.Xd, w.Xe, w.P, ord ? ord + nl : nullptr);
+            HM_LAUNCH_CHECK();
+        }
+        Trace trace("tsum_fx_kernel", s);
+        tsum_fx_kernel<NT><<<grid_for((A->total_rank + 31) / 32 * 32), 256, 0, s>>>(
+            tr->n_adm, A->total_rank, A->tsum_b0.as<int32_t>(), A->t_off.as<int64_t>(), tr->lr_bcolptr.as<int64_t>(),
+            A->pofs.as<int64_t>(), w.P, w.Td, w.Te);
+        HM_LAUNCH_CHECK();
+    }
+    const int tiles = (tr->max_leaf + 15) / 16, parts = (tiles + 4) / 5, mt = (tiles + parts - 1) / parts;
+    const int prow = 16 * tiles;
+    auto launch = [&](auto kern, int threads, int smem) {
+        HM_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        Trace trace("row_fx_kernel", s);
+        kern<<<(unsigned)(A->fx_nitems * parts), threads, smem, s>>>(
+            parts, tr->leaf_begin.as<int32_t>(), tr->rho_off.as<int64_t>(), tr->rho_K.as<int32_t>(),
+            tr->rho_colptr.as<int64_t>(), tr->colidx.as<int32_t>(), A->dense.as<double>(), A->up_off.as<int64_t>(),
+            A->up_K.as<int32_t>(), A->up_colptr.as<int64_t>(), A->tidx.as<int32_t>(), A->up.as<double>(), w.Xd, w.Xe,
+            w.Td, w.Te, w.sc, Y, A->fx_items.as<int4>(), w.Ypart, prow);
+        HM_LAUNCH_CHECK();
+    };
+    switch (mt) {
+        case 1: launch(row_fx_kernel<1, NT>, RowCfg<1>::THREADS, RowCfg<1>::SMEM); break;
+        case 2: launch(row_fx_kernel<2, NT>, RowCfg<2>::THREADS, RowCfg<2>::SMEM); break;
+        case 3: launch(row_fx_kernel<3, NT>, RowCfg<3>::THREADS, RowCfg<3>::SMEM); break;
+        case 4: launch(row_fx_kernel<4, NT>, RowCfg<4>::THREADS, RowCfg<4>::SMEM); break;
+        default: launch(row_fx_kernel<5, NT>, RowCfg<5>::THREADS, RowCfg<5>::SMEM); break;
+    }
+    if (A->fx_nred > 0) {
+        row_reduce_kernel<NT><<<(unsigned)A->fx_nred, 256, 0, s>>>(A->fx_red.as<int4>(), tr->leaf_begin.as<int32_t>(),
+                                                                   w.Ypart, prow, w.sc, Y);
+        HM_LAUNCH_CHECK();
+    }
+}
+
+}  // namespace fx
+
+// The row pass's work items: the panels of a leaf row cluster in chunks of 32
+// columns (near field first, then U), cut where one is long.  A cluster that
+// the Morton order tears apart has a near field ten times the mean width, and
+// one CTA walking it would be the pass (21,780 panels: mean 93 chunks, widest
+// 336): an item gets at most half of what an SM's share of CTAs would do one
+// after the other, 24 to 256 chunks.  Items by decreasing work; K: host copies
+// of the panel widths.
+void build_fx_items(hm_matrix *A, const std::vector<int32_t> &begin, const std::vector<int32_t> &kd,
+                    const std::vector<int32_t> &ku, cudaStream_t s) {
+    const int64_t nl = (int64_t)kd.size();
+    auto chunks = [&](int64_t r) { return (kd[r] + fx::KC - 1) / fx::KC + (ku[r] + fx::KC - 1) / fx::KC; };
+    int64_t total = 0;
+    for (int64_t r = 0; r < nl; ++r) total += chunks(r);
+    const int lim = (int)std::min<int64_t>(256, std::max<int64_t>(24, total / (2 * 4 * num_sms())));
+    std::vector<int4> items, red;
+    int slots = 0;
+    for (int64_t r = 0; r < nl; ++r) {
+        const int nc = chunks(r), parts = std::max(1, (nc + lim - 1) / lim);
+        if (parts > 1) red.push_back(make_int4((int)r, slots, parts, 0));
+        for (int p = 0; p < parts; ++p)
+            items.push_back(make_int4((int)r, (int)((int64_t)nc * p / parts), (int)((int64_t)nc * (p + 1) / parts),
+                                      parts > 1 ? slots++ : -1));
+    }
+    auto work = [&](const int4 &i) { return (int64_t)(i.z - i.y) * (begin[i.x + 1] - begin[i.x]); };
+    std::stable_sort(items.begin(), items.end(), [&](const int4 &a, const int4 &b) { return work(a) > work(b); });
+    A->fx_nitems = (int64_t)items.size();
+    A->fx_nred = (int64_t)red.size();
+    A->fx_nslots = slots;
+    A->fx_items.alloc(sizeof(int4) * std::max<size_t>(items.size(), 1));
+    A->fx_red.alloc(sizeof(int4) * std::max<size_t>(red.size(), 1));
+    HM_CUDA_CHECK(cudaMemcpyAsync(A->fx_items.p, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice, s));
+    HM_CUDA_CHECK(cudaMemcpyAsync(A->fx_red.p, red.data(), sizeof(int4) * red.size(), cudaMemcpyHostToDevice, s));
+    HM_CUDA_CHECK(cudaStreamSynchronize(s));
+}
+
+// floats of the working arrays of one 16-right-hand-side pass: digits of x
+// and t (56 each per row), partials of t (32 each), exponents of x and t (2
+// each, a multiple of 4 in all), scales (16), partials of split rows (32 per
+// row of a slot), Y (16 doubles per row)
 int64_t df_work_floats(const hm_matrix *A) {
     const int64_t n = A->tree->n, K = std::max<int64_t>(A->total_rank, 1), P = std::max<int64_t>(A->n_partials, 1);
-    return 32 * n + 32 * P + 32 * K + 32 * n;
+    return 56 * n + 32 * P + 56 * K + (2 * n + 3) / 4 * 4 + (2 * K + 3) / 4 * 4 + fx::MR +
+           32 * A->fx_nslots * ((A->tree->max_leaf + 15) / 16 * 16) + 32 * n;
 }
 
 // Y (Morton [n][16] FP64) = H_64 x for the nr <= 16 vectors x_r = x[r * n +
-// (perm ? perm[m] : m)] (Morton order without perm, original with it), in
-// double-float arithmetic; work: df_work_floats(A) floats (16-byte aligned).
+// (perm ? perm[m] : m)] (Morton order without perm, original with it); work:
+// df_work_floats(A) floats (16-byte aligned).
 void matvec_df_block(const hm_matrix *A, const double *x, int nr, const int32_t *perm, double *Y, float *work,
                      cudaStream_t s) {
-    using namespace df;
-    const hm_tree *tr = A->tree;
-    const int64_t n = tr->n, K = std::max<int64_t>(A->total_rank, 1), P = std::max<int64_t>(A->n_partials, 1);
-    float *Xh = work, *Xl = Xh + MR * n;
-    float2 *Pp = reinterpret_cast<float2 *>(Xl + MR * n);
-    float *Th = reinterpret_cast<float *>(Pp + MR * P), *Tl = Th + MR * K;
-    split_x_kernel<<<grid_for(n * MR), 256, 0, s>>>(x, n, nr, perm, Xh, Xl);
-    HM_LAUNCH_CHECK();
-    const int32_t *ord = A->mv_order.as<int32_t>();
-    const int64_t nl = tr->n_leaf;
-    if (tr->n_adm > 0) {
-        {
-            Trace trace("col_df_kernel", s);
-            col_df_kernel<<<(unsigned)nl, CD_THREADS, 0, s>>>(
-                tr->leaf_begin.as<int32_t>(), A->wp_off.as<int64_t>(), A->wp_K.as<int32_t>(),
-                A->wp_colptr.as<int64_t>(), A->wp.as<double>(), Xh, Xl, Pp, ord ? ord + nl : nullptr);
-            HM_LAUNCH_CHECK();
-        }
-        Trace trace("tsum_df_kernel", s);
-        tsum_df_kernel<<<grid_for((A->total_rank + 31) / 32 * 32), 256, 0, s>>>(
-            tr->n_adm, A->total_rank, A->tsum_b0.as<int32_t>(), A->t_off.as<int64_t>(), tr->lr_bcolptr.as<int64_t>(),
-            A->pofs.as<int64_t>(), Pp, Th, Tl);
-        HM_LAUNCH_CHECK();
-    }
-    if (tr->max_leaf <= 40) launch_row<40, 8>(A, Xh, Xl, Th, Tl, Y, ord, s);
-    else if (tr->max_leaf <= 80) launch_row<80, 4>(A, Xh, Xl, Th, Tl, Y, ord, s);
-    else launch_row<128, 2>(A, Xh, Xl, Th, Tl, Y, ord, s);
+    using namespace fx;
+    const int64_t n = A->tree->n, K = std::max<int64_t>(A->total_rank, 1), P = std::max<int64_t>(A->n_partials, 1);
+    Work w;
+    float *p = work;
+    w.Xd = reinterpret_cast<__half *>(p);
+    p += 56 * n;
+    w.P = reinterpret_cast<float2 *>(p);
+    p += 32 * P;
+    w.Td = reinterpret_cast<__half *>(p);
+    p += 56 * K;
+    w.Xe = reinterpret_cast<uint2 *>(p);
+    p += (2 * n + 3) / 4 * 4;
+    w.Te = reinterpret_cast<uint2 *>(p);
+    p += (2 * K + 3) / 4 * 4;
+    w.sc = reinterpret_cast<unsigned int *>(p);
+    p += MR;
+    w.Ypart = reinterpret_cast<float2 *>(p);
+    // at most 8 right-hand sides need one fragment column of the products, not two
+    if (nr <= 8) block_product<1>(A, x, nr, perm, Y, w, s);
+    else block_product<2>(A, x, nr, perm, Y, w, s);
 }
 
 // y = alpha H_64 x + beta y for nrhs right-hand sides [nrhs][n] in the
@@ -441,14 +863,14 @@ void matvec_df_block(const hm_matrix *A, const double *x, int nr, const int32_t 
 void matvec_df(const hm_matrix *A, int nrhs, const double *x, double *y, double alpha, double beta, cudaStream_t s) {
     const hm_tree *tr = A->tree;
     const int64_t n = tr->n;
-    for (int r0 = 0; r0 < nrhs; r0 += df::MR) {
-        const int nr = std::min(df::MR, nrhs - r0);
+    for (int r0 = 0; r0 < nrhs; r0 += fx::MR) {
+        const int nr = std::min(fx::MR, nrhs - r0);
         SBuf buf;
         buf.alloc(sizeof(float) * df_work_floats(A), s);
         float *work = buf.as<float>();
         double *Y = reinterpret_cast<double *>(work + df_work_floats(A) - 32 * n);
         matvec_df_block(A, x + (int64_t)r0 * n, nr, tr->perm.as<int32_t>(), Y, work, s);
-        df::scatter_kernel<<<df::grid_for(n * nr), 256, 0, s>>>(Y, n, nr, tr->perm.as<int32_t>(), alpha, beta,
+        fx::scatter_kernel<<<fx::grid_for(n * nr), 256, 0, s>>>(Y, n, nr, tr->perm.as<int32_t>(), alpha, beta,
                                                             y + (int64_t)r0 * n);
         HM_LAUNCH_CHECK();
     }
@@ -459,7 +881,7 @@ void matvec_df_morton(const hm_matrix *A, const double *xv, int nr, double *yv, 
     const int64_t n = A->tree->n;
     double *Y = reinterpret_cast<double *>(work + df_work_floats(A) - 32 * n);
     matvec_df_block(A, xv, nr, nullptr, Y, work, s);
-    df::scatter_kernel<<<df::grid_for(n * nr), 256, 0, s>>>(Y, n, nr, nullptr, 1.0, 0.0, yv);
+    fx::scatter_kernel<<<fx::grid_for(n * nr), 256, 0, s>>>(Y, n, nr, nullptr, 1.0, 0.0, yv);
     HM_LAUNCH_CHECK();
 }
 
