@@ -408,6 +408,10 @@ struct hm_matrix {
     // sums of the split ones (cluster, first slot, slots, 0)
     hm::DBuf fx_items, fx_red;
     int64_t fx_nitems = 0, fx_nred = 0, fx_nslots = 0;
+    // row pass of the FP32 / BF16 product with 16 right-hand sides
+    // (build_rm_items): work items (cluster, first row, end row, one row tile)
+    hm::DBuf rm_items;
+    int64_t rm_nitems = 0;
     int64_t n_partials = 0;  // length of the partial-projection vector
     // block-Jacobi preconditioner: inverse of each leaf cluster's diagonal block
     // block-Jacobi preconditioner (built on the first preconditioned solve):

@@ -191,6 +191,8 @@ void permute_from_morton(const hm_tree *tr, const double *ym, double alpha, doub
 
 void build_fx_items(hm_matrix *A, const std::vector<int32_t> &begin, const std::vector<int32_t> &kd,
                     const std::vector<int32_t> &ku, cudaStream_t s);
+void build_rm_items(hm_matrix *A, const std::vector<int32_t> &begin, const std::vector<int32_t> &kd,
+                    const std::vector<int32_t> &ku, cudaStream_t s);
 
 // Regroups the ACA output (uw: U_b column-major then W_b row-major at
 // uw_off[b]) into the low-rank row panels (U) and column panels (W).
@@ -285,6 +287,7 @@ void build_lr_panels(hm_matrix *A, const DBuf &uw, const DBuf &uw_off, cudaStrea
         by_work(ord.data() + 2 * nl, [&](int32_t r) { return rows(r) * ((int64_t)kd[r] + kw[r]); });
         by_work(ord.data() + 3 * nl, [&](int32_t r) { return rows(r) * (int64_t)ku[r]; });
         build_fx_items(A, lb, kd, ku, s);
+        build_rm_items(A, lb, kd, ku, s);
         A->mv_order.alloc(sizeof(int32_t) * 4 * nl);
         HM_CUDA_CHECK(cudaMemcpyAsync(A->mv_order.p, ord.data(), sizeof(int32_t) * 4 * nl, cudaMemcpyHostToDevice, s));
         HM_CUDA_CHECK(cudaStreamSynchronize(s));

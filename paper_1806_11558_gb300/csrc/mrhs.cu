@@ -124,7 +124,7 @@ __device__ __forceinline__ void rp_idx(const int32_t *__restrict__ idx, int K, i
     }
 }
 
-template <int MT, class TP, class C>
+template <int MT, class TP, class C, bool ONE>
 __device__ __forceinline__ void rp_load(unsigned char *stage, const TP *__restrict__ Pn, int K, int rows_valid, int c0,
                                         const int (&ir)[C::NJ], const __nv_bfloat16 *__restrict__ Zh,
                                         const __nv_bfloat16 *__restrict__ Zl) {
@@ -133,7 +133,8 @@ __device__ __forceinline__ void rp_load(unsigned char *stage, const TP *__restri
     __nv_bfloat16 *sBl = sBh + C::KS * RP_BSTRIDE;
     constexpr int PER = 16 / (int)sizeof(TP);  // elements per 16-byte copy
     constexpr int VPR = C::KS / PER;           // copies per row
-    for (int e = threadIdx.x; e < 16 * MT * VPR; e += C::THREADS) {
+    // the whole tile, or the one row tile of an item of a wide panel (ONE)
+    for (int e = threadIdx.x; e < (ONE ? 16 : 16 * MT) * VPR; e += C::THREADS) {
         const int r = e / VPR, v = e - (e / VPR) * VPR;
         const int col = c0 + PER * v;
         const bool ok = r < rows_valid && col < K;
@@ -152,7 +153,7 @@ __device__ __forceinline__ void rp_load(unsigned char *stage, const TP *__restri
     }
 }
 
-template <int MT, class TP, class C>
+template <int MT, class TP, class C, bool ONE>
 __device__ __forceinline__ void rp_compute(const unsigned char *stage, float (&acc)[C::template mth<MT>()][2][4]) {
     constexpr int MTH = C::template mth<MT>();
     const TP *sA = reinterpret_cast<const TP *>(stage);
@@ -169,7 +170,7 @@ __device__ __forceinline__ void rp_compute(const unsigned char *stage, float (&a
 #pragma unroll
     for (int ml = 0; ml < MTH; ++ml) {
         const int mt = mt0 + ml;
-        if (MTH != MT && mt >= MT) break;
+        if (ONE ? mt > 0 : MTH != MT && mt >= MT) break;
         if constexpr (sizeof(TP) == 4) {
             const float *r0 = reinterpret_cast<const float *>(sA) + (16 * mt + g) * (C::KS + RP_APAD) + kb + 2 * t;
             const float *r1 = r0 + 8 * (C::KS + RP_APAD);
@@ -210,7 +211,7 @@ __device__ __forceinline__ void rp_compute(const unsigned char *stage, float (&a
     }
 }
 
-template <int MT, class TP, class C>
+template <int MT, class TP, class C, bool ONE>
 __device__ __forceinline__ void rp_panel(unsigned char *sm, const TP *__restrict__ Pn, int K, int rows_valid,
                                          const int32_t *__restrict__ idx, const __nv_bfloat16 *__restrict__ Zh,
                                          const __nv_bfloat16 *__restrict__ Zl,
@@ -222,7 +223,7 @@ __device__ __forceinline__ void rp_panel(unsigned char *sm, const TP *__restrict
     for (int st = 0; st < ST - 1; ++st) {
         if (st < ns) {
             rp_idx<C>(idx, K, st * KS, ir);
-            rp_load<MT, TP, C>(sm + st * SB, Pn, K, rows_valid, st * KS, ir, Zh, Zl);
+            rp_load<MT, TP, C, ONE>(sm + st * SB, Pn, K, rows_valid, st * KS, ir, Zh, Zl);
         }
         cp_async_commit();
     }
@@ -231,10 +232,10 @@ __device__ __forceinline__ void rp_panel(unsigned char *sm, const TP *__restrict
         cp_async_wait<ST - 2>();
         __syncthreads();
         const int nx = sl + ST - 1;
-        if (nx < ns) rp_load<MT, TP, C>(sm + (nx % ST) * SB, Pn, K, rows_valid, nx * KS, ir, Zh, Zl);
+        if (nx < ns) rp_load<MT, TP, C, ONE>(sm + (nx % ST) * SB, Pn, K, rows_valid, nx * KS, ir, Zh, Zl);
         cp_async_commit();
         rp_idx<C>(idx, K, (nx + 1) * KS, ir);  // consumed one iteration later
-        rp_compute<MT, TP, C>(sm + (sl % ST) * SB, acc);
+        rp_compute<MT, TP, C, ONE>(sm + (sl % ST) * SB, acc);
     }
     cp_async_wait<0>();
     __syncthreads();
@@ -261,16 +262,17 @@ __global__ void __launch_bounds__(C::THREADS) row_mrhs_kernel(
     const int32_t *__restrict__ u16_K, const int64_t *__restrict__ u16_colptr, const int32_t *__restrict__ u16_tidx,
     const __nv_bfloat16 *__restrict__ u16, const __nv_bfloat16 *__restrict__ Th,
     const __nv_bfloat16 *__restrict__ Tl, const __nv_bfloat16 *__restrict__ Xh, const __nv_bfloat16 *__restrict__ Xl,
-    double *__restrict__ Y, YOut yo) {
+    double *__restrict__ Y, YOut yo, const int4 *__restrict__ items) {
     extern __shared__ __align__(16) unsigned char sm[];
-    const int64_t rho = blockIdx.x;
-    const int32_t r0 = leaf_begin[rho], mr = leaf_begin[rho + 1] - r0;
+    const int4 item = items[blockIdx.x];  // cluster, rows [y, z), 1 = one row tile of a wide panel
+    const int64_t rho = item.x;
+    const int32_t r0 = leaf_begin[rho];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const int Kd = rho_K[rho], Ku = up_K[rho];
     constexpr int MTH = C::template mth<MT>();
     const int kg = warp % C::KG, mt0 = MTH * (warp / C::KG);
-    for (int r0t = 0; r0t < mr; r0t += 16 * MT) {
-        const int rows = min(16 * MT, mr - r0t);
+    for (int r0t = item.y; r0t < item.z; r0t += 16 * MT) {
+        const int rows = min(16 * MT, item.z - r0t);
         float acc[MTH][2][4];
 #pragma unroll
         for (int ml = 0; ml < MTH; ++ml)
@@ -278,14 +280,20 @@ __global__ void __launch_bounds__(C::THREADS) row_mrhs_kernel(
             for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) acc[ml][nt][e] = 0.0f;
-        rp_panel<MT, float, C>(sm, dense + rho_off[rho] + (int64_t)r0t * Kd, Kd, rows, colidx + rho_colptr[rho], Xh,
-                               Xl, acc);
-        rp_panel<MT, TF, C>(sm, up + up_off[rho] + (int64_t)r0t * Ku, Ku, rows, tidx + up_colptr[rho], Th, Tl, acc);
-        if constexpr (TAIL) {
-            const int K16 = u16_K[rho];
-            rp_panel<MT, __nv_bfloat16, C>(sm, u16 + u16_off[rho] + (int64_t)r0t * K16, K16, rows,
-                                           u16_tidx + u16_colptr[rho], Th, Tl, acc);
-        }
+        auto panels = [&](auto one) {
+            constexpr bool ONE = decltype(one)::value;
+            rp_panel<MT, float, C, ONE>(sm, dense + rho_off[rho] + (int64_t)r0t * Kd, Kd, rows,
+                                        colidx + rho_colptr[rho], Xh, Xl, acc);
+            rp_panel<MT, TF, C, ONE>(sm, up + up_off[rho] + (int64_t)r0t * Ku, Ku, rows, tidx + up_colptr[rho], Th, Tl,
+                                     acc);
+            if constexpr (TAIL) {
+                const int K16 = u16_K[rho];
+                rp_panel<MT, __nv_bfloat16, C, ONE>(sm, u16 + u16_off[rho] + (int64_t)r0t * K16, K16, rows,
+                                                    u16_tidx + u16_colptr[rho], Th, Tl, acc);
+            }
+        };
+        if (item.w) panels(std::true_type{});
+        else panels(std::false_type{});
         // per-column-group sums -> shared memory -> fixed-order sum over the KG groups
         float *red = reinterpret_cast<float *>(sm);
 #pragma unroll
@@ -965,13 +973,52 @@ template <int MT, class C> static int row_smem() {
     return st > red ? st : red;
 }
 
+// The row pass's work items.  A cluster that the Morton order tears apart has
+// a near field up to ten times the mean width; taken in turn, the CTA that
+// walks it can end long after the others.  Clusters of more than twice the
+// mean width go first, widest first, one CTA per tile of 16 rows (the panel's
+// gathered rows are read once per tile); the others follow whole in Morton
+// order, whose neighbours share their gathered x and t in L2.  Leaves of more
+// than 80 rows are taken 64 rows at a time.  A row's sum is the same whichever
+// CTA forms it.  Measured, one CTA per cluster in Morton order -> this (time HBM
+// needs), us, FP32: 40,500 panels 272 -> 197 (80), 64,980 panels 374 -> 286 (166),
+// 81,920 panels, leaves of 80, 413 -> 351 (241), 327,680 panels, leaves of 80,
+// 1,525 -> 1,445 (1,151).
+constexpr int RM_ROWS = 64;  // rows of an item where the leaves have more than 80
+void build_rm_items(hm_matrix *A, const std::vector<int32_t> &begin, const std::vector<int32_t> &kd,
+                    const std::vector<int32_t> &ku, cudaStream_t s) {
+    const int64_t nl = (int64_t)kd.size();
+    auto width = [&](int64_t r) { return (int64_t)kd[r] + ku[r]; };
+    int64_t total = 0;
+    for (int64_t r = 0; r < nl; ++r) total += width(r);
+    std::vector<int32_t> wide;
+    std::vector<int4> items;
+    for (int64_t r = 0; r < nl; ++r)
+        if (width(r) * nl > 2 * total) wide.push_back((int32_t)r);
+    std::stable_sort(wide.begin(), wide.end(), [&](int32_t a, int32_t b) { return width(a) > width(b); });
+    for (int32_t r : wide)
+        for (int m = begin[r + 1] - begin[r], i = 0; i < m; i += 16)
+            items.push_back(make_int4(r, i, std::min(i + 16, m), 1));
+    const int step = A->tree->max_leaf > 80 ? RM_ROWS : 80;
+    for (int64_t r = 0; r < nl; ++r)
+        if (width(r) * nl <= 2 * total)
+            for (int m = begin[r + 1] - begin[r], i = 0; i < m; i += step)
+                items.push_back(make_int4((int)r, i, std::min(i + step, m), 0));
+    A->rm_nitems = (int64_t)items.size();
+    A->rm_items.alloc(sizeof(int4) * std::max<size_t>(items.size(), 1));
+    HM_CUDA_CHECK(cudaMemcpyAsync(A->rm_items.p, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice, s));
+    HM_CUDA_CHECK(cudaStreamSynchronize(s));
+}
+
 // Shapes of the row pass (warps x 16-column groups per slice x stages).  For
 // 80-row leaves (MT = 5) measured on the level-8 sphere, FP32 factors, ms per
 // product: 4x4x3 7.25, 4x4x2 7.64, 4x4x4 9.98, 8x4x3 7.32, 4x2x5 12.06,
 // 4x2x4 9.20, 8x2x4 8.64, 8x2x6 9.91, 8x8x3 9.00, 16x8x2 6.85, 16x8x3 8.32,
 // 16x16x2 6.65, 8x8x2 6.42-6.57: wide slices over 8 warps, two stages (111
-// KB of shared memory, two CTAs per SM).  The other tile counts keep 4x4x3
-// (8x8x2 would hold one CTA per SM for 128-row tiles).
+// KB of shared memory, two CTAs per SM).  Leaves of at most 48 rows (MT = 3)
+// and of more than 80 (items of 64 rows, MT = 4) keep 4x4x3; 128 rows in one
+// item left one CTA per SM: 200,000 panels, leaves of 98 rows, FP32, 1,598 us
+// in items of 128 rows, 1,230 in items of 64 (HBM needs 745).
 using RpShape5 = RpCfg<8, 8, 2>;
 using RpDefault = RpCfg<4, 4, 3>;
 
@@ -1031,14 +1078,14 @@ static void matvec_mrhs_impl(const hm_matrix *A, const TF *up, const float *X, d
         Trace tr_(f32 ? "row_mrhs_kernel.f32" : "row_mrhs_kernel.bf16", s);
         const TailPanels &U = tails ? A->ut32 : A->ut16;  // ut16: unused (TAIL = false) unless tails
         const TF *u = tails ? reinterpret_cast<const TF *>(A->ut32.data.p) : up;
-        kern<<<(unsigned)tr->n_leaf, threads, smem, s>>>(
+        kern<<<(unsigned)A->rm_nitems, threads, smem, s>>>(
             tr->leaf_begin.as<int32_t>(), tr->rho_off.as<int64_t>(), tr->rho_K.as<int32_t>(),
             tr->rho_colptr.as<int64_t>(), tr->colidx.as<int32_t>(), A->dense32.as<float>(),
             tails ? U.off.as<int64_t>() : A->up_off.as<int64_t>(), tails ? U.K.as<int32_t>() : A->up_K.as<int32_t>(),
             tails ? U.colptr.as<int64_t>() : A->up_colptr.as<int64_t>(),
             tails ? U.tidx.as<int32_t>() : A->tidx.as<int32_t>(), u, A->ut16.off.as<int64_t>(),
             A->ut16.K.as<int32_t>(), A->ut16.colptr.as<int64_t>(), A->ut16.tidx.as<int32_t>(),
-            A->ut16.data.as<__nv_bfloat16>(), Th, Tl, Xh, Xl, Y, yo);
+            A->ut16.data.as<__nv_bfloat16>(), Th, Tl, Xh, Xl, Y, yo, A->rm_items.as<int4>());
         HM_LAUNCH_CHECK();
     };
     if (A->params.mrhs_tcgen05 && A->mrhs_err.p) {  // the measured tcgen05 / TMEM row pass (mrhs_tc.cu)
@@ -1056,13 +1103,13 @@ static void matvec_mrhs_impl(const hm_matrix *A, const TF *up, const float *X, d
         if constexpr (sizeof(TF) == 4) {
             if (tiles <= 3) launch(row_mrhs_kernel<3, float, C, true>, row_smem<3, C>(), C::THREADS);
             else if (tiles <= 5) launch(row_mrhs_kernel<5, float, C5, true>, row_smem<5, C5>(), C5::THREADS);
-            else launch(row_mrhs_kernel<8, float, C, true>, row_smem<8, C>(), C::THREADS);
+            else launch(row_mrhs_kernel<4, float, C, true>, row_smem<4, C>(), C::THREADS);
         }
         return;
     }
     if (tiles <= 3) launch(row_mrhs_kernel<3, TF, C, false>, row_smem<3, C>(), C::THREADS);
     else if (tiles <= 5) launch(row_mrhs_kernel<5, TF, C5, false>, row_smem<5, C5>(), C5::THREADS);
-    else launch(row_mrhs_kernel<8, TF, C, false>, row_smem<8, C>(), C::THREADS);
+    else launch(row_mrhs_kernel<4, TF, C, false>, row_smem<4, C>(), C::THREADS);
 }
 
 // Y (Morton [n][16] FP64) = H X (Morton [n][16] FP32) with the FP32 near field
