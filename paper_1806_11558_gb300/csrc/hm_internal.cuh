@@ -231,8 +231,6 @@ struct QuadParams {
     int ss_n;            // Gauss-Legendre order on [0, 1] for touching pairs
     double gx[MAX_SS];
     double gw[MAX_SS];
-    float w_h[NQ];       // the 7 weights as float pairs (w = w_h + w_l)
-    float w_l[NQ];
 };
 
 // 7-point rule from its closed form; Gauss-Legendre nodes by Newton's method

@@ -102,8 +102,11 @@ constexpr int NF_THREADS = 128;
 // FF: the regular entries from the float-pair table in double-float
 // arithmetic (regular_entry_ff, ~1e-14 relative) on the FP32 pipes; else from
 // the FP64 table in FP64.
+// Bound by FP32 issue; four CTAs per SM: with 128 registers the column panel's
+// offsets stay in registers (655,220 panels 167 ms at 96 registers, 149 at 128;
+// 153 before the shorter entry).
 template <bool FF>
-__global__ void __launch_bounds__(NF_THREADS) nearfield_kernel(const __grid_constant__ CUtensorMap pt_map,
+__global__ void __launch_bounds__(NF_THREADS, 4) nearfield_kernel(const __grid_constant__ CUtensorMap pt_map,
                                                                 const int32_t *__restrict__ dense,
                                                                 const int64_t *__restrict__ base,
                                                                 const int32_t *__restrict__ ld,
@@ -212,7 +215,7 @@ __global__ void __launch_bounds__(NF_THREADS) nearfield_kernel(const __grid_cons
         if (valid && !touch) {
             double a;
             if constexpr (FF)
-                a = regular_entry_ff(R, box_cols, C, box_cols, qp.w_h, qp.w_l);
+                a = regular_entry_ff(R, box_cols, C, box_cols);
             else
                 a = regular_entry(R, box_cols, C, box_cols, qp);
             arena[blk_base + (int64_t)i * blk_ld + j] = a;

@@ -154,7 +154,7 @@ __global__ void panel_table_kernel(const double *V, const int32_t *T, const int3
                 float h, l;
                 split_double(__dsub_rn(xq, cr[d]), h, l);
                 pf[(int64_t)(PF_AH + 7 * d + q) * npad + k] = h;
-                pf[(int64_t)(PF_AL + 7 * d + q) * npad + k] = l;
+                pf[(int64_t)(PF_AL2 + 7 * d + q) * npad + k] = 2.0f * l;
             }
         pf[(int64_t)(PF_VID + 0) * npad + k] = __int_as_float(t0);
         pf[(int64_t)(PF_VID + 1) * npad + k] = __int_as_float(t1);
