@@ -297,18 +297,21 @@ __global__ void ss_edge_table_kernel(const QuadParams qp, SSPointFF *tab) {
 // (s, e) += (a, b) for non-negative float pairs
 __device__ __forceinline__ void ff_acc(float &s, float &e, float a, float b) {
     float t, u;
-    two_sum(s, a, t, u);
+    two_sum_pos(s, a, t, u);
     s = t;
     e = __fadd_rn(e, __fadd_rn(u, b));
 }
 
 // Sum over this lane's points of w / |D|, D = c0 E0 + c1 E1 - c2 E2 - c3 E3,
-// for the edge vectors E (common vertex: (a1, a2, b1, b2); common edge:
-// (a1, a2, b2, b1) with c3 = 0) as float pairs; returned as a float pair.
+// for the edge vectors E as float pairs (common vertex, NK = 4: (a1, a2, b1,
+// b2); common edge, NK = 3: (a1, a2, b2), c3 = 0); returned as a float pair.
+// WIDE: see regular_entry_ff2.
+template <int NK, bool WIDE>
 __device__ __forceinline__ void ss_sum_ff(const float Eh[4][3], const float El[4][3], const SSPointFF *__restrict__ tab,
-                                             int npts, int lane, float &acc_h, float &acc_l) {
+                                          int npts, int lane, float &acc_h, float &acc_l) {
     acc_h = 0.0f;
     acc_l = 0.0f;
+#pragma unroll 1
     for (int t = lane; t < npts; t += 32) {
         const SSPointFF p = tab[t];
         float dd_h = 0.0f, dd_l = 0.0f;
@@ -317,16 +320,21 @@ __device__ __forceinline__ void ss_sum_ff(const float Eh[4][3], const float El[4
             // D_d = c0 a1 + c1 a2 - c2 b1 - c3 b2
             float hs = 0.0f, lo = 0.0f;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
+            for (int k = 0; k < NK; ++k) {
                 const float sg = k < 2 ? 1.0f : -1.0f;
                 float ph, pe;
                 two_prod(p.ch[k], Eh[k][d], ph, pe);
                 pe = __fmaf_rn(p.ch[k], El[k][d], pe);
                 pe = __fmaf_rn(p.cl[k], Eh[k][d], pe);
-                float t1, e1;
-                two_sum(hs, sg * ph, t1, e1);
-                hs = t1;
-                lo = __fadd_rn(lo, __fmaf_rn(sg, pe, e1));
+                if (k == 0) {
+                    hs = ph;
+                    lo = pe;
+                } else {
+                    float t1, e1;
+                    two_sum(hs, sg * ph, t1, e1);
+                    hs = t1;
+                    lo = __fadd_rn(lo, __fmaf_rn(sg, pe, e1));
+                }
             }
             float Dh, Dl;
             fast_two_sum(hs, lo, Dh, Dl);
@@ -334,12 +342,19 @@ __device__ __forceinline__ void ss_sum_ff(const float Eh[4][3], const float El[4
             float qh, ql;
             two_prod(Dh, Dh, qh, ql);
             ql = __fmaf_rn(__fmul_rn(2.0f, Dh), Dl, ql);
-            ff_acc(dd_h, dd_l, qh, ql);
+            if (d == 0) {
+                dd_h = qh;
+                dd_l = ql;
+            } else {
+                ff_acc(dd_h, dd_l, qh, ql);
+            }
         }
         float r2h, r2l;
         fast_two_sum(dd_h, dd_l, r2h, r2l);
         // 1 / sqrt(r2): estimate + one Newton step with an exact residual
-        const float y0 = rsqrtf(r2h);
+        float y0;
+        if constexpr (WIDE) y0 = rsqrtf(r2h);
+        else asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(r2h));
         float yh, yl;
         two_prod(y0, y0, yh, yl);
         float mh, ml;
@@ -357,85 +372,122 @@ __device__ __forceinline__ void ss_sum_ff(const float Eh[4][3], const float El[4
     }
 }
 
-__global__ void singular_kernel(const SingularItem *__restrict__ items, int64_t count, const int32_t *__restrict__ trim,
-                                const double *__restrict__ V, const double *__restrict__ pt, int64_t npad,
-                                const QuadParams qp, double *__restrict__ arena,
-                                const SSPointFF *__restrict__ vtab, const SSPointFF *__restrict__ etab) {
-    const int lane = threadIdx.x & 31;
-    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (w >= count) return;
-    const SingularItem it = items[w];
-    const int32_t *ta = trim + 3 * (int64_t)it.i, *tb = trim + 3 * (int64_t)it.j;
-    const int32_t a[3] = {ta[0], ta[1], ta[2]}, bb[3] = {tb[0], tb[1], tb[2]};
-    const int kind = shared_vertices(a, bb);
-    int32_t P[3], Q[3];
-    touch_orient(a, bb, kind, P, Q);
-    const PairGeom g = pair_geom(V, P, Q);
-    const int n = qp.ss_n, n2 = n * n, n3 = n2 * n;
-    double s = 0.0;
-    bool ff_done = false;
-    if (kind == 3) {
-        // 1-D: three classes of regions, each counted twice with the eta1 / eta2 sums 1/2 and 1
-        for (int t = lane; t < 3 * n; t += 32) {
-            const int c = t / n, k = t - c * n;
-            const double e = qp.gx[k];
-            double s0, s1;
-            if (c == 0) { s0 = e; s1 = 1.0; }
-            else if (c == 1) { s0 = 1.0; s1 = e; }
-            else { s0 = -e; s1 = 1.0 - e; }
-            s += qp.gw[k] * inv_norm3(s0 * g.a1[0] + s1 * g.a2[0], s0 * g.a1[1] + s1 * g.a2[1],
-                                      s0 * g.a1[2] + s1 * g.a2[2]);
-        }
-    } else if (kind != 3 && (kind == 1 ? vtab : etab)) {
-        // double-float points; the lanes' partial sums as float pairs
-        float Eh[4][3], El[4][3];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            split_double(g.a1[d], Eh[0][d], El[0][d]);
-            split_double(g.a2[d], Eh[1][d], El[1][d]);
-            split_double(kind == 1 ? g.b1[d] : g.b2[d], Eh[2][d], El[2][d]);
-            split_double(kind == 1 ? g.b2[d] : g.b1[d], Eh[3][d], El[3][d]);
-        }
-        float ah, al;
-        ss_sum_ff(Eh, El, kind == 1 ? vtab : etab, kind == 1 ? 2 * n3 : 5 * n2, lane, ah, al);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float bh = __shfl_xor_sync(0xffffffffu, ah, o), bl = __shfl_xor_sync(0xffffffffu, al, o);
-            ff_acc(ah, al, bh, bl);
-        }
-        s = (double)ah + (double)al;  // the same value on every lane
-        ff_done = true;
-    } else if (kind == 2) {
-        // 2-D: D' = d0 a1 + u1 a2 - v1 b2 over the five regions, eta1 sum = 1/2
-        for (int t = lane; t < 5 * n2; t += 32) {
-            const int r = t / n2, rem = t - r * n2, k2 = rem / n, k3 = rem - k2 * n;
-            const double e2 = qp.gx[k2], e3 = qp.gx[k3], e23 = e2 * e3;
-            double d0, u1, v1, jp;
-            switch (r) {
-                case 0: d0 = e2; u1 = e3; v1 = 1.0 - e2; jp = 1.0; break;
-                case 1: d0 = e23; u1 = 1.0; v1 = e2 - e23; jp = e2; break;
-                case 2: d0 = -e2; u1 = 1.0 - e2; v1 = e23; jp = e2; break;
-                case 3: d0 = -e23; u1 = e2 - e23; v1 = 1.0; jp = e2; break;
-                default: d0 = -e23; u1 = 1.0 - e23; v1 = e2; jp = e2; break;
+// Bound by FP32 issue for common-vertex pairs (2 n^3 points); what FP64 there is
+// (64 cycles of a scheduler per warp instruction) is therefore shared out: lane
+// l < 12 forms and splits one component of one edge vector and the others take
+// it by shuffle, and the factor 4 |Ti| |Tj| / 3 is applied to the CTA's eight
+// sums by one warp.
+// Before (every lane all of it) -> now, ms: 5,120 panels 0.292 -> 0.212, 21,780
+// panels 1.147 -> 0.834, 655,220 panels 33.7 -> 24.5.
+constexpr int SING_WARPS = 8;
+__global__ void __launch_bounds__(32 * SING_WARPS) singular_kernel(
+    const SingularItem *__restrict__ items, int64_t count, const int32_t *__restrict__ trim,
+    const double *__restrict__ V, const double *__restrict__ pt, int64_t npad, const QuadParams qp,
+    double *__restrict__ arena, const SSPointFF *__restrict__ vtab, const SSPointFF *__restrict__ etab) {
+    __shared__ double s_sum[SING_WARPS];  // the sums, or their float pairs
+    __shared__ bool s_pair[SING_WARPS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t w0 = blockIdx.x * (int64_t)SING_WARPS;
+    if (w0 + warp < count) {
+        const SingularItem it = items[w0 + warp];
+        const int32_t *ta = trim + 3 * (int64_t)it.i, *tb = trim + 3 * (int64_t)it.j;
+        const int32_t a[3] = {ta[0], ta[1], ta[2]}, bb[3] = {tb[0], tb[1], tb[2]};
+        const int kind = shared_vertices(a, bb);
+        int32_t P[3], Q[3];
+        touch_orient(a, bb, kind, P, Q);
+        const int n = qp.ss_n, n2 = n * n, n3 = n2 * n;
+        double s = 0.0;
+        bool pair = false;
+        if (kind == 3) {
+            const PairGeom g = pair_geom(V, P, Q);
+            // 1-D: three classes of regions, each counted twice with the eta1 / eta2 sums 1/2 and 1
+            for (int t = lane; t < 3 * n; t += 32) {
+                const int c = t / n, k = t - c * n;
+                const double e = qp.gx[k];
+                double s0, s1;
+                if (c == 0) { s0 = e; s1 = 1.0; }
+                else if (c == 1) { s0 = 1.0; s1 = e; }
+                else { s0 = -e; s1 = 1.0 - e; }
+                s += qp.gw[k] * inv_norm3(s0 * g.a1[0] + s1 * g.a2[0], s0 * g.a1[1] + s1 * g.a2[1],
+                                          s0 * g.a1[2] + s1 * g.a2[2]);
             }
-            const double dx = d0 * g.a1[0] + u1 * g.a2[0] - v1 * g.b2[0];
-            const double dy = d0 * g.a1[1] + u1 * g.a2[1] - v1 * g.b2[1];
-            const double dz = d0 * g.a1[2] + u1 * g.a2[2] - v1 * g.b2[2];
-            s += qp.gw[k2] * qp.gw[k3] * jp * inv_norm3(dx, dy, dz);
-        }
-        s *= 0.5;
-    } else {
-        for (int t = lane; t < 2 * n3; t += 32) {
-            const int r = t / n3, rem = t - r * n3;
-            const int k1 = rem / n2, k2 = (rem / n) % n, k3 = rem % n;
-            s += ss_point(g, kind, r, k1, k2, k3, qp);
-        }
-    }
-    if (!ff_done) {
+        } else if (kind == 1 ? vtab : etab) {
+            // double-float points; the lanes' partial sums as float pairs
+            const int e = min(lane / 3, 3), d0 = lane % 3;  // edge vector and component of this lane
+            const int qe = kind == 1 ? e - 2 : 3 - e;       // of b1, b2 (kind 1) or b2, b1 (kind 2)
+            const int32_t to = e == 0 ? P[1] : e == 1 ? P[2] : qe == 0 ? Q[1] : Q[2];
+            const int32_t from = e == 0 ? P[0] : e == 1 ? P[1] : qe == 0 ? Q[0] : Q[1];
+            float eh, el;
+            split_double(V[3 * (int64_t)to + d0] - V[3 * (int64_t)from + d0], eh, el);
+            float Eh[4][3], El[4][3];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    Eh[k][d] = __shfl_sync(0xffffffffu, eh, 3 * k + d);
+                    El[k][d] = __shfl_sync(0xffffffffu, el, 3 * k + d);
+                }
+            auto lane_sum = [&](float x, float y) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const float xo = __shfl_xor_sync(0xffffffffu, x, o), yo = __shfl_xor_sync(0xffffffffu, y, o);
+                    ff_acc(x, y, xo, yo);
+                }
+                return FF{x, y};  // the same value on every lane
+            };
+            float ah, al;
+            if (kind == 1) ss_sum_ff<4, false>(Eh, El, vtab, 2 * n3, lane, ah, al);
+            else ss_sum_ff<3, false>(Eh, El, etab, 5 * n2, lane, ah, al);
+            FF a = lane_sum(ah, al);
+            if (!isfinite(a.h)) {
+                ss_sum_ff<4, true>(Eh, El, kind == 1 ? vtab : etab, kind == 1 ? 2 * n3 : 5 * n2, lane, ah, al);
+                a = lane_sum(ah, al);
+            }
+            s = __hiloint2double(__float_as_int(a.h), __float_as_int(a.l));
+            pair = true;
+        } else if (kind == 2) {
+            const PairGeom g = pair_geom(V, P, Q);
+            // 2-D: D' = d0 a1 + u1 a2 - v1 b2 over the five regions, eta1 sum = 1/2
+            for (int t = lane; t < 5 * n2; t += 32) {
+                const int r = t / n2, rem = t - r * n2, k2 = rem / n, k3 = rem - k2 * n;
+                const double e2 = qp.gx[k2], e3 = qp.gx[k3], e23 = e2 * e3;
+                double d0, u1, v1, jp;
+                switch (r) {
+                    case 0: d0 = e2; u1 = e3; v1 = 1.0 - e2; jp = 1.0; break;
+                    case 1: d0 = e23; u1 = 1.0; v1 = e2 - e23; jp = e2; break;
+                    case 2: d0 = -e2; u1 = 1.0 - e2; v1 = e23; jp = e2; break;
+                    case 3: d0 = -e23; u1 = e2 - e23; v1 = 1.0; jp = e2; break;
+                    default: d0 = -e23; u1 = 1.0 - e23; v1 = e2; jp = e2; break;
+                }
+                const double dx = d0 * g.a1[0] + u1 * g.a2[0] - v1 * g.b2[0];
+                const double dy = d0 * g.a1[1] + u1 * g.a2[1] - v1 * g.b2[1];
+                const double dz = d0 * g.a1[2] + u1 * g.a2[2] - v1 * g.b2[2];
+                s += qp.gw[k2] * qp.gw[k3] * jp * inv_norm3(dx, dy, dz);
+            }
+            s *= 0.5;
+        } else {
+            const PairGeom g = pair_geom(V, P, Q);
+            for (int t = lane; t < 2 * n3; t += 32) {
+                const int r = t / n3, rem = t - r * n3;
+                const int k1 = rem / n2, k2 = (rem / n) % n, k3 = rem % n;
+                s += ss_point(g, kind, r, k1, k2, k3, qp);
+            }
+        }
+        if (!pair) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        }
+        if (lane == 0) {
+            s_sum[warp] = s;
+            s_pair[warp] = pair;
+        }
     }
-    if (lane == 0) {
+    __syncthreads();
+    if (threadIdx.x < SING_WARPS && w0 + threadIdx.x < count) {
+        const SingularItem it = items[w0 + threadIdx.x];
+        double s = s_sum[threadIdx.x];
+        if (s_pair[threadIdx.x])
+            s = (double)__int_as_float(__double2hiint(s)) + (double)__int_as_float(__double2loint(s));
         const double ai = pt[(int64_t)PT_AREA * npad + it.i], aj = pt[(int64_t)PT_AREA * npad + it.j];
         const double a = 4.0 * ai * aj * (s / 3.0) * INV_4PI;
         arena[it.off] = a;
@@ -489,9 +541,8 @@ void assemble_nearfield(const hm_tree *tr, hm_matrix *A, const QuadParams &qp, c
             ss_edge_table_kernel<<<(ne + 255) / 256, 256, 0, s>>>(qp, vtab.as<SSPointFF>() + nv);
             HM_LAUNCH_CHECK();
         }
-        const int64_t threads = nsing * 32;
         Trace trace("singular_kernel", s);
-        singular_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(
+        singular_kernel<<<(unsigned)((nsing + SING_WARPS - 1) / SING_WARPS), 32 * SING_WARPS, 0, s>>>(
             items.as<SingularItem>(), nsing, tr->trim.as<int32_t>(), tr->V.as<double>(), tr->pt.as<double>(),
             tr->npad, qp, A->dense.as<double>(), vtab.as<SSPointFF>(),
             vtab.p ? vtab.as<SSPointFF>() + 2 * qp.ss_n * qp.ss_n * qp.ss_n : nullptr);
