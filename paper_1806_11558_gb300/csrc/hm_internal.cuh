@@ -242,10 +242,21 @@ QuadParams make_quad(int ss_order);
 // ----------------------------------------------------------------------------
 // exclusive scan of n int64 values (in may equal out); returns the total
 int64_t exclusive_scan_i64(const int64_t *d_in, int64_t *d_out, int64_t n, cudaStream_t s);
-// stable ascending sort of 64-bit keys with 32-bit payloads (LSD radix);
+// the same for `batch` arrays of n values, `stride` values apart; the totals to totals[]
+void exclusive_scans_i64(const int64_t *d_in, int64_t *d_out, int64_t stride, int64_t n, int batch, int64_t *totals,
+                         cudaStream_t s);
+// stable ascending sort of 64-bit keys with 32-bit payloads (LSD radix) by the
+// digits (bytes) of the keys that key_bits, a mask of the bits that a key may
+// have set, has bits in;
 // keys/vals are sorted in place, d_tmp_* are scratch of the same sizes
 void radix_sort_u64(uint64_t *d_keys, int32_t *d_vals, uint64_t *d_tmp_keys, int32_t *d_tmp_vals, int64_t n,
-                    int key_bits, cudaStream_t s);
+                    uint64_t key_bits, cudaStream_t s);
+// all bits of the numbers 0 .. n
+inline uint64_t bits_upto(uint64_t n) {
+    uint64_t m = 0;
+    while (m < n) m = 2 * m + 1;
+    return m;
+}
 void gather_i32(const int32_t *d_src, const int32_t *d_idx, int32_t *d_dst, int64_t n, cudaStream_t s);
 
 // ----------------------------------------------------------------------------

@@ -834,7 +834,7 @@ static void build_bcp(hm_matrix *A, BcpSet &S, hm_dtype prec, const int32_t *rk_
         bcp_keys_kernel<<<grid1d_m(na), 256, 0, s>>>(tr->adm.as<int32_t>(), rk_set, na, nb, key.as<uint64_t>(),
                                                       id.as<int32_t>());
         HM_LAUNCH_CHECK();
-        radix_sort_u64(key.as<uint64_t>(), id.as<int32_t>(), tkey.as<uint64_t>(), tid.as<int32_t>(), na, 2 * nb, s);
+        radix_sort_u64(key.as<uint64_t>(), id.as<int32_t>(), tkey.as<uint64_t>(), tid.as<int32_t>(), na, none, s);
         gather_i32(rk_set, id.as<int32_t>(), rk.as<int32_t>(), na, s);
         bcp_head_kernel<<<grid1d_m(na + 1), 256, 0, s>>>(key.as<uint64_t>(), rk.as<int32_t>(), na, none,
                                                           head.as<int64_t>(), rk64.as<int64_t>());
@@ -857,8 +857,7 @@ static void build_bcp(hm_matrix *A, BcpSet &S, hm_dtype prec, const int32_t *rk_
                                                            ng, nb, S.K.as<int32_t>(), S.rows.as<int32_t>(),
                                                            cnt.as<int64_t>());
         HM_LAUNCH_CHECK();
-        for (int q = 0; q < 5; ++q)
-            tot[q] = exclusive_scan_i64(cnt.as<int64_t>() + q * (ng + 1), cx.as<int64_t>() + q * (ng + 1), ng + 1, s);
+        exclusive_scans_i64(cnt.as<int64_t>(), cx.as<int64_t>(), ng + 1, ng + 1, 5, tot, s);
     }
     const int64_t o = tot[0], c = tot[1], ntiles = tot[2], nred = tot[3], nslots = tot[4];
     const int64_t *d_off = cx.as<int64_t>(), *d_col0 = d_off + (ng + 1), *d_toff = d_off + 2 * (ng + 1),

@@ -353,11 +353,17 @@ QuadParams make_quad(int ss_order) {
 }
 
 // ----------------------------------------------------------------------------
-// exclusive scan of int64 (three passes: tile sums, scan of sums, tile scan)
+// exclusive scans of int64: tile sums, then a scan of every tile that starts at
+// the sum of the tiles before it.  Bound by launches and read-backs at the sizes
+// of the set-up (tens of thousands of values), so there are few of both: one
+// kernel for one tile, two up to SCAN_SELF tiles (every CTA adds up the sums of the
+// tiles before its own), and several scans of one length are one call and one
+// read-back.
 // ----------------------------------------------------------------------------
 constexpr int SCAN_THREADS = 512;
 constexpr int SCAN_ITEMS = 8;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
+constexpr int64_t SCAN_SELF = 4096;
 
 __device__ __forceinline__ int64_t block_exclusive_scan(int64_t v, int64_t *s_warp, int64_t *total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -382,8 +388,10 @@ __device__ __forceinline__ int64_t block_exclusive_scan(int64_t v, int64_t *s_wa
     return before + x - v;
 }
 
-__global__ void scan_tile_sums(const int64_t *in, int64_t n, int64_t *sums) {
+// blockIdx.y: which of the scans (in, out: `stride` values apart; sums: nb)
+__global__ void scan_tile_sums(const int64_t *in, int64_t stride, int64_t n, int64_t *sums) {
     __shared__ int64_t s_warp[32];
+    in += blockIdx.y * stride;
     int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
     int64_t acc = 0;
     for (int k = 0; k < SCAN_ITEMS; ++k) {
@@ -392,12 +400,14 @@ __global__ void scan_tile_sums(const int64_t *in, int64_t n, int64_t *sums) {
     }
     int64_t tot;
     block_exclusive_scan(acc, s_warp, &tot);
-    if (threadIdx.x == 0) sums[blockIdx.x] = tot;
+    if (threadIdx.x == 0) sums[blockIdx.y * (int64_t)gridDim.x + blockIdx.x] = tot;
 }
 
-__global__ void scan_sums_single(int64_t *sums, int64_t nb, int64_t *total) {
+// more than SCAN_SELF tiles: their sums, scanned in place
+__global__ void scan_sums_single(int64_t *sums, int64_t nb) {
     __shared__ int64_t s_warp[32];
     __shared__ int64_t s_carry;
+    sums += blockIdx.y * nb;
     if (threadIdx.x == 0) s_carry = 0;
     __syncthreads();
     for (int64_t b0 = 0; b0 < nb; b0 += blockDim.x) {
@@ -411,11 +421,15 @@ __global__ void scan_sums_single(int64_t *sums, int64_t nb, int64_t *total) {
         if (threadIdx.x == 0) s_carry = carry + tot;
         __syncthreads();
     }
-    if (threadIdx.x == 0 && total) *total = s_carry;
 }
 
-__global__ void scan_tiles(const int64_t *in, int64_t *out, int64_t n, const int64_t *sums) {
+// scanned: sums holds the exclusive scan of the tile sums
+__global__ void scan_tiles(const int64_t *in, int64_t *out, int64_t stride, int64_t n, const int64_t *sums,
+                           bool scanned, int64_t *totals) {
     __shared__ int64_t s_warp[32];
+    in += blockIdx.y * stride;
+    out += blockIdx.y * stride;
+    sums += blockIdx.y * (int64_t)gridDim.x;
     int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
     int64_t v[SCAN_ITEMS];
     int64_t acc = 0;
@@ -424,40 +438,85 @@ __global__ void scan_tiles(const int64_t *in, int64_t *out, int64_t n, const int
         v[k] = i < n ? in[i] : 0;
         acc += v[k];
     }
-    int64_t ex = block_exclusive_scan(acc, s_warp, nullptr) + sums[blockIdx.x];
+    int64_t first = 0;
+    if (scanned) {
+        first = sums[blockIdx.x];
+    } else if (blockIdx.x > 0) {
+        int64_t before = 0;
+        for (int64_t k = threadIdx.x; k < blockIdx.x; k += SCAN_THREADS) before += sums[k];
+        block_exclusive_scan(before, s_warp, &first);
+        __syncthreads();  // s_warp is used again
+    }
+    int64_t tot;
+    int64_t ex = block_exclusive_scan(acc, s_warp, &tot) + first;
     for (int k = 0; k < SCAN_ITEMS; ++k) {
         int64_t i = base + k;
         if (i < n) out[i] = ex;
         ex += v[k];
     }
+    if (totals && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) totals[blockIdx.y] = first + tot;
+}
+
+static int64_t scan_nb(int64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE; }
+
+// the scans, without a read-back; d_sums: batch * scan_nb(n) values, d_totals: batch values or null
+static void scan_launch(const int64_t *d_in, int64_t *d_out, int64_t stride, int64_t n, int batch, int64_t *d_sums,
+                        int64_t *d_totals, cudaStream_t s) {
+    const int64_t nb = scan_nb(n);
+    const dim3 grid((unsigned)nb, (unsigned)batch);
+    const bool scanned = nb > SCAN_SELF;
+    if (nb > 1) {
+        scan_tile_sums<<<grid, SCAN_THREADS, 0, s>>>(d_in, stride, n, d_sums);
+        HM_LAUNCH_CHECK();
+    }
+    if (scanned) {
+        scan_sums_single<<<dim3(1, (unsigned)batch), 1024, 0, s>>>(d_sums, nb);
+        HM_LAUNCH_CHECK();
+    }
+    scan_tiles<<<grid, SCAN_THREADS, 0, s>>>(d_in, d_out, stride, n, d_sums, scanned, d_totals);
+    HM_LAUNCH_CHECK();
+}
+
+void exclusive_scans_i64(const int64_t *d_in, int64_t *d_out, int64_t stride, int64_t n, int batch, int64_t *totals,
+                         cudaStream_t s) {
+    if (n <= 0) {
+        std::fill(totals, totals + batch, 0);
+        return;
+    }
+    DBuf sums;
+    const int64_t nb = scan_nb(n);
+    sums.alloc(sizeof(int64_t) * batch * (nb + 1));
+    int64_t *d_totals = sums.as<int64_t>() + batch * nb;
+    scan_launch(d_in, d_out, stride, n, batch, sums.as<int64_t>(), d_totals, s);
+    HM_CUDA_CHECK(cudaMemcpyAsync(totals, d_totals, sizeof(int64_t) * batch, cudaMemcpyDeviceToHost, s));
+    HM_CUDA_CHECK(cudaStreamSynchronize(s));
 }
 
 int64_t exclusive_scan_i64(const int64_t *d_in, int64_t *d_out, int64_t n, cudaStream_t s) {
-    if (n <= 0) return 0;
-    int64_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
-    DBuf sums;
-    sums.alloc(sizeof(int64_t) * (nb + 1));
-    int64_t *d_sums = sums.as<int64_t>();
-    scan_tile_sums<<<(unsigned)nb, SCAN_THREADS, 0, s>>>(d_in, n, d_sums);
-    HM_LAUNCH_CHECK();
-    scan_sums_single<<<1, 1024, 0, s>>>(d_sums, nb, d_sums + nb);
-    HM_LAUNCH_CHECK();
-    scan_tiles<<<(unsigned)nb, SCAN_THREADS, 0, s>>>(d_in, d_out, n, d_sums);
-    HM_LAUNCH_CHECK();
-    return read_scalar(d_sums + nb, s);
+    int64_t total = 0;
+    exclusive_scans_i64(d_in, d_out, n, n, 1, &total, s);
+    return total;
 }
 
 // ----------------------------------------------------------------------------
 // stable LSD radix sort, 8-bit digits.  Per pass: per-tile digit counts,
-// scan of the digit-major count matrix, then an in-order scatter in which
-// every tile ranks its keys stably (warp match + per-warp digit counts).
+// and an in-order scatter in which every tile ranks its keys stably (warp match
+// + per-warp digit counts).  Up to RS_SELF tiles every scatter CTA adds up the
+// counts in front of its own itself (two launches per pass); above that they
+// are scanned first, digit-major.  Digits that no key has bits in are passed
+// over, and no pass waits for the host.
+// Measured with the scans above, set-up of 5,120 panels (five sorts of up to 8
+// digits, thirteen levels of the block tree): 394 -> 141 launches, and the time
+// outside the assembly kernels 5.6 -> 3.3 ms (21,780 panels 7.5 -> 5.4 ms).
 // ----------------------------------------------------------------------------
 constexpr int RS_THREADS = 256;
 constexpr int RS_ITEMS = 8;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
 constexpr int RS_WARPS = RS_THREADS / 32;
+constexpr int64_t RS_SELF = 64;
 
-__global__ void radix_hist(const uint64_t *keys, int64_t n, int shift, int64_t *counts, int64_t ntiles) {
+// counts[tile][digit] (self) or counts[digit][tile]
+__global__ void radix_hist(const uint64_t *keys, int64_t n, int shift, int64_t *counts, int64_t ntiles, bool self) {
     __shared__ int s_cnt[256];
     s_cnt[threadIdx.x] = 0;
     __syncthreads();
@@ -467,16 +526,30 @@ __global__ void radix_hist(const uint64_t *keys, int64_t n, int shift, int64_t *
         if (i < n) atomicAdd(&s_cnt[(keys[i] >> shift) & 255u], 1);
     }
     __syncthreads();
-    counts[(int64_t)threadIdx.x * ntiles + blockIdx.x] = s_cnt[threadIdx.x];
+    counts[self ? (int64_t)blockIdx.x * 256 + threadIdx.x : (int64_t)threadIdx.x * ntiles + blockIdx.x] =
+        s_cnt[threadIdx.x];
 }
 
 __global__ void radix_scatter(const uint64_t *kin, const int32_t *vin, uint64_t *kout, int32_t *vout, int64_t n,
-                              int shift, const int64_t *offs, int64_t ntiles) {
+                              int shift, const int64_t *offs, int64_t ntiles, bool self) {
     __shared__ int64_t s_base[256];
     __shared__ int s_cnt[RS_WARPS][256];
     __shared__ int s_run[256];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    s_base[tid] = offs[(int64_t)tid * ntiles + blockIdx.x];
+    if (self) {
+        // keys of this digit in the tiles before this one, and in all tiles
+        __shared__ int64_t s_warp[32];
+        int64_t before = 0, all = 0;
+#pragma unroll 8
+        for (int64_t t = 0; t < ntiles; ++t) {
+            const int64_t c = offs[256 * t + tid];
+            before += t < blockIdx.x ? c : 0;
+            all += c;
+        }
+        s_base[tid] = block_exclusive_scan(all, s_warp, nullptr) + before;
+    } else {
+        s_base[tid] = offs[(int64_t)tid * ntiles + blockIdx.x];
+    }
     s_run[tid] = 0;
     const unsigned lt_mask = (1u << lane) - 1u;
     int64_t base = (int64_t)blockIdx.x * RS_TILE;
@@ -512,20 +585,21 @@ __global__ void radix_scatter(const uint64_t *kin, const int32_t *vin, uint64_t 
 }
 
 void radix_sort_u64(uint64_t *d_keys, int32_t *d_vals, uint64_t *d_tmp_keys, int32_t *d_tmp_vals, int64_t n,
-                    int key_bits, cudaStream_t s) {
+                    uint64_t key_bits, cudaStream_t s) {
     if (n <= 1) return;
-    int64_t ntiles = (n + RS_TILE - 1) / RS_TILE;
+    const int64_t ntiles = (n + RS_TILE - 1) / RS_TILE;
+    const bool self = ntiles <= RS_SELF;
     DBuf counts;
-    counts.alloc(sizeof(int64_t) * 256 * ntiles);
-    int passes = (key_bits + 7) / 8;
+    counts.alloc(sizeof(int64_t) * (256 * ntiles + scan_nb(256 * ntiles)));
+    int64_t *d_counts = counts.as<int64_t>(), *d_sums = d_counts + 256 * ntiles;
     uint64_t *ka = d_keys, *kb = d_tmp_keys;
     int32_t *va = d_vals, *vb = d_tmp_vals;
-    for (int p = 0; p < passes; ++p) {
-        int shift = 8 * p;
-        radix_hist<<<(unsigned)ntiles, RS_THREADS, 0, s>>>(ka, n, shift, counts.as<int64_t>(), ntiles);
+    for (int shift = 0; shift < 64; shift += 8) {
+        if (((key_bits >> shift) & 255u) == 0) continue;
+        radix_hist<<<(unsigned)ntiles, RS_THREADS, 0, s>>>(ka, n, shift, d_counts, ntiles, self);
         HM_LAUNCH_CHECK();
-        exclusive_scan_i64(counts.as<int64_t>(), counts.as<int64_t>(), 256 * ntiles, s);
-        radix_scatter<<<(unsigned)ntiles, RS_THREADS, 0, s>>>(ka, va, kb, vb, n, shift, counts.as<int64_t>(), ntiles);
+        if (!self) scan_launch(d_counts, d_counts, 0, 256 * ntiles, 1, d_sums, nullptr, s);
+        radix_scatter<<<(unsigned)ntiles, RS_THREADS, 0, s>>>(ka, va, kb, vb, n, shift, d_counts, ntiles, self);
         HM_LAUNCH_CHECK();
         std::swap(ka, kb);
         std::swap(va, vb);

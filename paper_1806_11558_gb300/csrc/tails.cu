@@ -252,9 +252,11 @@ void split_terms(hm_matrix *A, const DBuf &uw, const DBuf &uw_off, cudaStream_t 
                                                      c64.as<int64_t>());
     HM_LAUNCH_CHECK();
     int64_t *c = c64.as<int64_t>();
-    A->info.factor_tail_terms = exclusive_scan_i64(c, c, na + 1, s);
-    A->info.u_tail_entries = exclusive_scan_i64(c + (na + 1), c + (na + 1), na + 1, s);
-    A->info.lr_tail_entries = exclusive_scan_i64(c + 2 * (na + 1), c + 2 * (na + 1), na + 1, s);
+    int64_t tot[3];
+    exclusive_scans_i64(c, c, na + 1, na + 1, 3, tot, s);
+    A->info.factor_tail_terms = tot[0];
+    A->info.u_tail_entries = tot[1];
+    A->info.lr_tail_entries = tot[2];
 }
 
 // The row panels of the two parts (with the FP32 copy; A->rank32 set).
@@ -280,8 +282,7 @@ void build_tail_panels(hm_matrix *A, cudaStream_t s) {
     HM_CUDA_CHECK(cudaMemsetAsync(cnt.as<int64_t>() + 2 * nl1 + nl, 0, sizeof(int64_t), s));
     HM_CUDA_CHECK(cudaMemsetAsync(cnt.as<int64_t>() + 3 * nl1 + nl, 0, sizeof(int64_t), s));
     int64_t tot[4];
-    for (int q = 0; q < 4; ++q)
-        tot[q] = exclusive_scan_i64(cnt.as<int64_t>() + q * nl1, cx.as<int64_t>() + q * nl1, nl1, s);
+    exclusive_scans_i64(cnt.as<int64_t>(), cx.as<int64_t>(), nl1, nl1, 4, tot, s);
     P.entries = tot[0];
     R.entries = tot[2];
     P.off.alloc(sizeof(int64_t) * nl1);

@@ -510,15 +510,13 @@ hm_tree *build_tree_impl(const double *d_V, int64_t nv, const int32_t *d_T, int6
     HM_LAUNCH_CHECK();
     // a3: stable sort by (code, original index), then, for several
     // geometries, stable by geometry: the order is (geometry, code, index)
-    radix_sort_u64(code.as<uint64_t>(), tr->perm.as<int32_t>(), code_tmp.as<uint64_t>(), idx_tmp.as<int32_t>(), n, 63,
-                   s);
+    radix_sort_u64(code.as<uint64_t>(), tr->perm.as<int32_t>(), code_tmp.as<uint64_t>(), idx_tmp.as<int32_t>(), n,
+                   ~uint64_t(0) >> 1, s);
     if (G > 1) {
-        int bits = 1;
-        while ((1 << bits) < G) ++bits;
         gather_gid_kernel<<<grid_for(n), 256, 0, s>>>(gid.as<int32_t>(), tr->perm.as<int32_t>(), n, code.as<uint64_t>());
         HM_LAUNCH_CHECK();
         radix_sort_u64(code.as<uint64_t>(), tr->perm.as<int32_t>(), code_tmp.as<uint64_t>(), idx_tmp.as<int32_t>(), n,
-                       bits, s);
+                       bits_upto((uint64_t)G - 1), s);
     }
     tr->geom_off = goff;
 
@@ -606,26 +604,24 @@ hm_tree *build_tree_impl(const double *d_V, int64_t nv, const int32_t *d_T, int6
     int64_t ncand = G;
     const double eta2 = prm.eta * prm.eta;
     while (ncand > 0) {
-        DBuf flag, ca, cd, cs;
+        DBuf flag, cnt;  // counts of admissible and dense blocks and of children, each of ncand values
         flag.alloc(ncand);
-        ca.alloc(sizeof(int64_t) * ncand);
-        cd.alloc(sizeof(int64_t) * ncand);
-        cs.alloc(sizeof(int64_t) * ncand);
+        cnt.alloc(sizeof(int64_t) * 3 * ncand);
+        int64_t *ca = cnt.as<int64_t>(), *cd = ca + ncand, *cs = cd + ncand;
         bt_classify_kernel<<<grid_for(ncand), 256, 0, s>>>(
             cand.as<int32_t>(), ncand, tr->cl_range.as<int32_t>(), tr->cl_box.as<double>(), d_child.as<int32_t>(),
-            prm.leaf_size, eta2, flag.as<int8_t>(), ca.as<int64_t>(), cd.as<int64_t>(), cs.as<int64_t>());
+            prm.leaf_size, eta2, flag.as<int8_t>(), ca, cd, cs);
         HM_LAUNCH_CHECK();
-        const int64_t na = exclusive_scan_i64(ca.as<int64_t>(), ca.as<int64_t>(), ncand, s);
-        const int64_t nd = exclusive_scan_i64(cd.as<int64_t>(), cd.as<int64_t>(), ncand, s);
-        const int64_t ns = exclusive_scan_i64(cs.as<int64_t>(), cs.as<int64_t>(), ncand, s);
+        int64_t tot[3];
+        exclusive_scans_i64(ca, ca, ncand, ncand, 3, tot, s);
+        const int64_t na = tot[0], nd = tot[1], ns = tot[2];
         DBuf ao, dout, next;
         ao.alloc(sizeof(int32_t) * 4 * std::max<int64_t>(na, 1));
         dout.alloc(sizeof(int32_t) * 4 * std::max<int64_t>(nd, 1));
         next.alloc(sizeof(int32_t) * 2 * std::max<int64_t>(ns, 1));
         bt_emit_kernel<<<grid_for(ncand), 256, 0, s>>>(cand.as<int32_t>(), ncand, tr->cl_range.as<int32_t>(),
-                                                       d_child.as<int32_t>(), flag.as<int8_t>(), ca.as<int64_t>(),
-                                                       cd.as<int64_t>(), cs.as<int64_t>(), ao.as<int32_t>(),
-                                                       dout.as<int32_t>(), next.as<int32_t>());
+                                                       d_child.as<int32_t>(), flag.as<int8_t>(), ca, cd, cs,
+                                                       ao.as<int32_t>(), dout.as<int32_t>(), next.as<int32_t>());
         HM_LAUNCH_CHECK();
         if (na) { adm_parts.push_back(std::move(ao)); adm_cnt.push_back(na); }
         if (nd) { den_parts.push_back(std::move(dout)); den_cnt.push_back(nd); }
@@ -656,6 +652,8 @@ hm_tree *build_tree_impl(const double *d_V, int64_t nv, const int32_t *d_T, int6
     adm_parts.clear();
     den_parts.clear();
 
+    // bits of a key (row_begin, col_begin)
+    const uint64_t range_bits = bits_upto((uint64_t)n) << 32 | bits_upto((uint64_t)n);
     // dense leaves sorted by (row_begin, col_begin), grouped in leaf row panels
     {
         DBuf key, kt, idx, it, width;
@@ -667,7 +665,8 @@ hm_tree *build_tree_impl(const double *d_V, int64_t nv, const int32_t *d_T, int6
         dense_keys_kernel<<<grid_for(n_den), 256, 0, s>>>(den_all.as<int32_t>(), n_den, key.as<uint64_t>(),
                                                           idx.as<int32_t>());
         HM_LAUNCH_CHECK();
-        radix_sort_u64(key.as<uint64_t>(), idx.as<int32_t>(), kt.as<uint64_t>(), it.as<int32_t>(), n_den, 64, s);
+        radix_sort_u64(key.as<uint64_t>(), idx.as<int32_t>(), kt.as<uint64_t>(), it.as<int32_t>(), n_den, range_bits,
+                       s);
         tr->dense.alloc(sizeof(int32_t) * 4 * n_den);
         gather_rows4_kernel<<<grid_for(n_den), 256, 0, s>>>(den_all.as<int32_t>(), idx.as<int32_t>(), n_den,
                                                             tr->dense.as<int32_t>(), width.as<int64_t>());
@@ -759,8 +758,9 @@ hm_tree *build_tree_impl(const double *d_V, int64_t nv, const int32_t *d_T, int6
                                                                 cnt.as<int64_t>(), key.as<uint64_t>(),
                                                                 list.as<int32_t>());
                 HM_LAUNCH_CHECK();
-                radix_sort_u64(key.as<uint64_t>(), list.as<int32_t>(), kt.as<uint64_t>(), vt.as<int32_t>(), np, 64,
-                               s);
+                // by leaf cluster (the pairs are there in the order of the blocks)
+                radix_sort_u64(key.as<uint64_t>(), list.as<int32_t>(), kt.as<uint64_t>(), vt.as<int32_t>(), np,
+                               bits_upto((uint64_t)nl) << 32, s);
                 lr_rowcount_kernel<<<grid_for(np), 256, 0, s>>>(key.as<uint64_t>(), np, ptr.as<int64_t>());
                 HM_LAUNCH_CHECK();
                 exclusive_scan_i64(ptr.as<int64_t>(), ptr.as<int64_t>(), nl + 1, s);
@@ -780,7 +780,8 @@ hm_tree *build_tree_impl(const double *d_V, int64_t nv, const int32_t *d_T, int6
             leaf_keys_kernel<<<grid_for(n_adm), 256, 0, s>>>(tr->adm.as<int32_t>(), n_adm, k2.as<uint64_t>(),
                                                              i2.as<int32_t>());
             HM_LAUNCH_CHECK();
-            radix_sort_u64(k2.as<uint64_t>(), i2.as<int32_t>(), kt.as<uint64_t>(), it.as<int32_t>(), n_adm, 64, s);
+            radix_sort_u64(k2.as<uint64_t>(), i2.as<int32_t>(), kt.as<uint64_t>(), it.as<int32_t>(), n_adm, range_bits,
+                           s);
             partner_kernel<<<grid_for(n_adm), 256, 0, s>>>(tr->adm.as<int32_t>(), n_adm, k2.as<uint64_t>(),
                                                            i2.as<int32_t>(), tr->adm_tp.as<int32_t>());
             HM_LAUNCH_CHECK();
