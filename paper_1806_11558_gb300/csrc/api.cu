@@ -117,6 +117,7 @@ hm_status hm_build_tree(const double *d_vertices, int64_t n_vertices, const int3
         if (n_vertices < 3 || n_vertices > (1LL << 30)) fail(HM_EINVAL, "n_vertices must be in [3, 2^30]");
         if (!(params->eta >= 0.0) || !std::isfinite(params->eta)) fail(HM_EINVAL, "eta must be finite and >= 0");
         if (params->leaf_size < 1 || params->leaf_size > 254) fail(HM_EINVAL, "leaf_size must be in [1, 254]");
+        AllocScope scope;
         *out = build_tree_impl(d_vertices, n_vertices, d_tris, n_tris, *params, {}, (cudaStream_t)stream);
     });
 }
@@ -136,6 +137,7 @@ hm_status hm_build_forest(const double *d_vertices, int64_t n_vertices, const in
         if (goff[0] != 0 || goff[n_geom] != n_tris) fail(HM_EINVAL, "tri_offsets must start at 0 and end at n_tris");
         for (int g = 0; g < n_geom; ++g)
             if (goff[g + 1] <= goff[g]) fail(HM_EINVAL, "geometry %d has no triangle", g);
+        AllocScope scope;
         *out = build_tree_impl(d_vertices, n_vertices, d_tris, n_tris, *params, goff, (cudaStream_t)stream);
     });
 }
@@ -166,6 +168,7 @@ hm_status hm_assemble(const hm_tree *tree, const hm_assemble_params *params, hm_
             fail(HM_EINVAL, "factor_tail_bits must be 0 or in [8, 24]");
         cudaStream_t s = (cudaStream_t)stream;
         const auto t0 = std::chrono::steady_clock::now();
+        AllocScope scope;
         std::unique_ptr<hm_matrix> A(new hm_matrix());
         A->tree = tree;
         A->params = *params;
@@ -381,6 +384,7 @@ void hm_trim(void) {
 }
 
 void hm_free(void *handle) {
+    AllocScope scope(~size_t(0));  // one synchronisation for all buffers
     if (is_matrix(handle)) {
         hm_matrix *A = static_cast<hm_matrix *>(handle);
         A->magic = 0;

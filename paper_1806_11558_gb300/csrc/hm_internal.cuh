@@ -29,6 +29,7 @@
 
 #include <cstdint>
 #include <cstdio>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -100,7 +101,17 @@ std::vector<TraceTotal> trace_read();
 // cudaFree implies) and a later allocation takes the smallest cached block
 // that is large enough and at most 1/8 larger.  The cache holds at most a
 // quarter of the device memory; a failed cudaMalloc empties it and retries;
-// hm_trim() returns it to the driver.
+// hm_trim() returns it to the driver.  Smaller buffers are rounded up to a power
+// of two and cached the same way, up to SMALL_CAP bytes of them.
+//
+// Inside an AllocScope (a set-up call: some 150 buffers, most of them temporary
+// and small, and a cudaFree or a synchronisation for each would stop the stream
+// as often) a released buffer goes to a list of the scope instead, without a
+// wait, and the next allocation of the scope takes it from there.  That is safe
+// because a scope belongs to one thread and all its work is queued on one stream;
+// at the end of the scope, after one device synchronisation, the list goes to
+// the cache.  Set-up of 5,120 panels 6.1 -> 5.2 ms,
+// of 21,780 panels 15.0 -> 13.6 ms.
 // ----------------------------------------------------------------------------
 struct DBuf {
     void *p = nullptr;
@@ -132,6 +143,24 @@ struct DBuf {
     template <class T> T *as() const { return static_cast<T *>(p); }
 };
 void cache_trim();  // frees every cached block
+
+// See above.  Holds at most `cap` bytes; inside another scope of the thread it
+// does nothing.
+class AllocScope {
+  public:
+    explicit AllocScope(size_t cap = size_t(1) << 30);
+    ~AllocScope();
+    AllocScope(const AllocScope &) = delete;
+    AllocScope &operator=(const AllocScope &) = delete;
+
+  private:
+    friend struct DBuf;
+    void flush();  // one synchronisation, then everything to the cache
+    std::multimap<size_t, void *> blocks;
+    size_t held = 0, cap;
+    int dev = 0;
+    bool outer = false;
+};
 
 // Injected allocation failures (hm_set_fault_injection, HM_FAULT_INJECT): every
 // device allocation of the library (DBuf, SBuf) passes this checkpoint first;

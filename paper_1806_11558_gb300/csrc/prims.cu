@@ -157,10 +157,12 @@ void fail(hm_status s, const char *fmt, ...) {
 // device buffers
 // ----------------------------------------------------------------------------
 // block cache of DBuf (see hm_internal.cuh)
-constexpr size_t CACHE_MIN = size_t(1) << 20;
+constexpr size_t CACHE_MIN = size_t(1) << 20;   // smaller blocks are rounded up
+constexpr size_t SMALL_CAP = size_t(64) << 20;  // bytes of them in the cache
 static std::mutex g_cache_mu;
 static std::multimap<std::pair<int, size_t>, void *> g_cache;  // (device, size) -> block
-static size_t g_cache_bytes = 0;
+static size_t g_cache_bytes = 0, g_small_bytes = 0;
+static thread_local AllocScope *tl_scope = nullptr;
 
 static size_t cache_cap() {
     static size_t cap = 0;
@@ -181,7 +183,22 @@ void cache_trim() {
     }
     cudaSetDevice(cur);
     g_cache.clear();
-    g_cache_bytes = 0;
+    g_cache_bytes = g_small_bytes = 0;
+}
+
+// a block that no queued work uses: into the cache, or freed
+static void cache_put(int dev, size_t blk, void *p) {
+    {
+        std::lock_guard<std::mutex> lk(g_cache_mu);
+        const bool small = blk < CACHE_MIN;
+        if (g_cache_bytes + blk <= cache_cap() && (!small || g_small_bytes + blk <= SMALL_CAP)) {
+            g_cache.insert({{dev, blk}, p});
+            g_cache_bytes += blk;
+            if (small) g_small_bytes += blk;
+            return;
+        }
+    }
+    cudaFree(p);
 }
 
 // ----------------------------------------------------------------------------
@@ -225,23 +242,42 @@ void DBuf::alloc(size_t nbytes) {
     if (nbytes == 0) nbytes = 16;
     fault_checkpoint(nbytes);
     HM_CUDA_CHECK(cudaGetDevice(&dev));
-    if (nbytes >= CACHE_MIN) {
+    size_t want = nbytes, most = nbytes + nbytes / 8;
+    if (nbytes < CACHE_MIN) {
+        want = 512;
+        while (want < nbytes) want *= 2;
+        most = want;
+    }
+    if (tl_scope && tl_scope->dev == dev) {
+        auto it = tl_scope->blocks.lower_bound(want);
+        if (it != tl_scope->blocks.end() && it->first <= most) {
+            p = it->second;
+            blk = it->first;
+            bytes = nbytes;
+            tl_scope->held -= blk;
+            tl_scope->blocks.erase(it);
+            return;
+        }
+    }
+    {
         std::lock_guard<std::mutex> lk(g_cache_mu);
-        auto it = g_cache.lower_bound({dev, nbytes});
-        if (it != g_cache.end() && it->first.first == dev && it->first.second <= nbytes + nbytes / 8) {
+        auto it = g_cache.lower_bound({dev, want});
+        if (it != g_cache.end() && it->first.first == dev && it->first.second <= most) {
             p = it->second;
             blk = it->first.second;
             bytes = nbytes;
             g_cache_bytes -= blk;
+            if (blk < CACHE_MIN) g_small_bytes -= blk;
             g_cache.erase(it);
             return;
         }
     }
-    cudaError_t e = cudaMalloc(&p, nbytes);
+    cudaError_t e = cudaMalloc(&p, want);
     if (e == cudaErrorMemoryAllocation) {
         (void)cudaGetLastError();
+        if (tl_scope) tl_scope->flush();
         cache_trim();
-        e = cudaMalloc(&p, nbytes);
+        e = cudaMalloc(&p, want);
     }
     if (e != cudaSuccess) {
         p = nullptr;
@@ -250,7 +286,7 @@ void DBuf::alloc(size_t nbytes) {
              cudaGetErrorString(e));
     }
     bytes = nbytes;
-    blk = nbytes;
+    blk = want;
 }
 
 // Waits for the work queued on device `dev` (the device a block belongs to,
@@ -268,19 +304,39 @@ static bool sync_device(int dev) {
 
 void DBuf::release() {
     if (p) {
-        bool cached = false;
-        if (blk >= CACHE_MIN && sync_device(dev)) {
-            std::lock_guard<std::mutex> lk(g_cache_mu);
-            if (g_cache_bytes + blk <= cache_cap()) {
-                g_cache.insert({{dev, blk}, p});
-                g_cache_bytes += blk;
-                cached = true;
-            }
+        if (tl_scope && tl_scope->dev == dev && tl_scope->held + blk <= tl_scope->cap) {
+            tl_scope->blocks.insert({blk, p});
+            tl_scope->held += blk;
+        } else if (sync_device(dev)) {
+            cache_put(dev, blk, p);
+        } else {
+            cudaFree(p);
         }
-        if (!cached) cudaFree(p);
     }
     p = nullptr;
     bytes = blk = 0;
+}
+
+AllocScope::AllocScope(size_t cap_) : cap(cap_), outer(tl_scope == nullptr) {
+    if (!outer) return;
+    if (cudaGetDevice(&dev) != cudaSuccess) (void)cudaGetLastError();
+    tl_scope = this;
+}
+
+void AllocScope::flush() {
+    const bool idle = blocks.empty() || sync_device(dev);
+    for (auto &b : blocks) {
+        if (idle) cache_put(dev, b.first, b.second);
+        else cudaFree(b.second);
+    }
+    blocks.clear();
+    held = 0;
+}
+
+AllocScope::~AllocScope() {
+    if (!outer) return;
+    flush();
+    tl_scope = nullptr;
 }
 
 int num_sms() {
