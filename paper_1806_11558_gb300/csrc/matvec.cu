@@ -41,17 +41,36 @@ __global__ void scatter_perm_kernel(const double *ym, const int32_t *perm, int64
 // ---------------------------------------------------------------------------
 // packing of the ACA factors into low-rank row panels and the W arena
 // ---------------------------------------------------------------------------
+// The kernels of this part copy integers and factors; they are bound by chains of
+// dependent loads (a block of the list, its partner, its offset, its factors:
+// some hundred blocks per leaf cluster), so one warp takes one cluster or 32
+// columns of its panel and many are in flight.  Before (one thread per cluster, one
+// block after the other per CTA) -> now, the whole set-up, ms: 21,780 panels 13.6 ->
+// 12.4, 64,980 panels 40.4 -> 38.3, 327,680 panels 272 -> 264.
+
 // per leaf row cluster: padded width of its low-rank panel and the first
-// panel column of each of its (rho, block) pairs
+// panel column of each of its (rho, block) pairs; one warp per cluster
 __global__ void up_width_kernel(const int32_t *leaf_begin, int64_t nleaf, const int64_t *lr_rowptr,
                                 const int32_t *lr_list, const int32_t *rank, int32_t *koff, int32_t *up_K,
                                 int64_t *up_size, int64_t *up_kpad) {
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < nleaf; r += (int64_t)gridDim.x * blockDim.x) {
-        int64_t acc = 0;
-        for (int64_t q = lr_rowptr[r]; q < lr_rowptr[r + 1]; ++q) {
-            koff[q] = (int32_t)acc;
-            acc += rank[lr_list[q]];
+    const int lane = threadIdx.x & 31;
+    const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (r >= nleaf) return;
+    const int64_t q1 = lr_rowptr[r + 1];
+    int64_t acc = 0;
+    for (int64_t q0 = lr_rowptr[r]; q0 < q1; q0 += 32) {
+        const int64_t q = q0 + lane;
+        const int k = q < q1 ? rank[lr_list[q]] : 0;
+        int x = k;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
         }
+        if (q < q1) koff[q] = (int32_t)(acc + x - k);
+        acc += __shfl_sync(0xffffffffu, x, 31);
+    }
+    if (lane == 0) {
         const int64_t Kp = (acc + 7) / 8 * 8;
         up_K[r] = (int32_t)Kp;
         up_size[r] = (int64_t)(leaf_begin[r + 1] - leaf_begin[r]) * Kp;
@@ -65,104 +84,71 @@ __device__ __forceinline__ bool is_mirror(const int32_t *adm, const int32_t *tp,
     return tp[b] >= 0 && adm[4 * b] > adm[4 * b + 2];
 }
 
-__global__ void up_pack_kernel(const int32_t *leaf_begin, const int64_t *lr_rowptr, const int32_t *lr_list,
-                               const int32_t *adm, const int32_t *tp, const int32_t *rank, const int64_t *t_off,
-                               const int64_t *uw_off, const double *uw, const int32_t *koff, const int64_t *up_off,
-                               const int32_t *up_K, const int64_t *up_colptr, double *up, int32_t *tidx) {
+// Panels of one factor per leaf cluster: U_b(rows of the cluster, :) over the
+// admissible leaves whose rows cover it (ROWS, with the projections' indices
+// tidx), or W_b(columns of the cluster, :) over those whose columns cover it.
+// A warp takes 32 columns of a panel: each lane looks up its column's block once
+// and then walks down the rows of the factor, so every row is written as whole
+// 256-byte lines and there is no index arithmetic per element.
+template <bool ROWS>
+__global__ void __launch_bounds__(256) pack_kernel(const int32_t *leaf_begin, const int64_t *ptr, const int32_t *list,
+                                                   const int32_t *adm, const int32_t *tp, const int32_t *rank,
+                                                   const int64_t *t_off, const int64_t *uw_off, const double *uw,
+                                                   const int32_t *koff, const int64_t *off, const int32_t *K,
+                                                   const int64_t *colptr, double *panels, int32_t *tidx) {
     const int64_t r = blockIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x >> 5) * gridDim.y;
     const int32_t r0 = leaf_begin[r], mr = leaf_begin[r + 1] - r0;
-    const int Ku = up_K[r];
-    double *Q = up + up_off[r];
-    int32_t *ti = tidx + up_colptr[r];
-    for (int64_t q = lr_rowptr[r]; q < lr_rowptr[r + 1]; ++q) {
-        const int32_t b = lr_list[q];
-        const int k = rank[b], off = r0 - adm[4 * b], c = koff[q];
-        if (is_mirror(adm, tp, b)) {
-            const int32_t p = tp[b];
-            const int mp = adm[4 * p + 1] - adm[4 * p];
-            const double *Wp = uw + uw_off[p] + (int64_t)mp * k;
-            for (int e = threadIdx.x; e < mr * k; e += blockDim.x) {
-                const int i = e / k, l = e - (e / k) * k;
-                Q[(int64_t)i * Ku + c + l] = Wp[(int64_t)(off + i) * k + l];
-            }
-        } else {
-            const int m = adm[4 * b + 1] - adm[4 * b];
-            const double *U = uw + uw_off[b];
-            for (int e = threadIdx.x; e < mr * k; e += blockDim.x) {
-                const int i = e / k, l = e - (e / k) * k;
-                Q[(int64_t)i * Ku + c + l] = U[(int64_t)l * m + off + i];
-            }
+    const int ld = K[r];
+    const int64_t qa = ptr[r], qb = ptr[r + 1];
+    for (int c = 32 * (blockIdx.y * (blockDim.x >> 5) + warp) + lane; c < ld; c += 32 * nw) {
+        // the last block that starts at or before column c
+        int64_t lo = qa, hi = qb;
+        while (hi - lo > 1) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (koff[mid] <= c) lo = mid;
+            else hi = mid;
         }
-        for (int l = threadIdx.x; l < k; l += blockDim.x) ti[c + l] = (int32_t)(t_off[b] + l);
-    }
-    // the padding columns (the panel width rounded up to 8) are zeros
-    const int64_t qa = lr_rowptr[r], qb = lr_rowptr[r + 1];
-    const int kw = qb > qa ? koff[qb - 1] + rank[lr_list[qb - 1]] : 0, pw = Ku - kw;
-    for (int e = threadIdx.x; e < mr * pw; e += blockDim.x) {
-        const int i = e / pw;
-        Q[(int64_t)i * Ku + kw + (e - i * pw)] = 0.0;
-    }
-}
-
-// column panels of W: per leaf column cluster kappa, W_b(rows of kappa, :)
-// over the admissible leaves whose columns cover kappa
-__global__ void wp_pack_kernel(const int32_t *leaf_begin, const int64_t *lr_colptr, const int32_t *lr_collist,
-                               const int32_t *adm, const int32_t *tp, const int32_t *rank, const int64_t *uw_off,
-                               const double *uw, const int32_t *koff, const int64_t *wp_off, const int32_t *wp_K,
-                               double *wp) {
-    const int64_t kap = blockIdx.x;
-    const int32_t c0 = leaf_begin[kap], mc = leaf_begin[kap + 1] - c0;
-    const int Kw = wp_K[kap];
-    double *Wt = wp + wp_off[kap];
-    for (int64_t q = lr_colptr[kap]; q < lr_colptr[kap + 1]; ++q) {
-        const int32_t b = lr_collist[q];
-        const int k = rank[b], off = c0 - adm[4 * b + 2], c = koff[q];
-        if (is_mirror(adm, tp, b)) {
-            const int32_t p = tp[b];
-            const int mp = adm[4 * p + 1] - adm[4 * p];
-            const double *Up = uw + uw_off[p];  // column-major m_p x k
-            for (int e = threadIdx.x; e < mc * k; e += blockDim.x) {
-                const int j = e / k, l = e - (e / k) * k;
-                Wt[(int64_t)j * Kw + c + l] = Up[(int64_t)l * mp + off + j];
-            }
-        } else {
-            const int m = adm[4 * b + 1] - adm[4 * b];
-            const double *W = uw + uw_off[b] + (int64_t)m * k;  // row-major n x k
-            for (int e = threadIdx.x; e < mc * k; e += blockDim.x) {
-                const int j = e / k, l = e - (e / k) * k;
-                Wt[(int64_t)j * Kw + c + l] = W[(int64_t)(off + j) * k + l];
-            }
+        const int32_t b = list[lo];
+        const int k = rank[b], l = c - koff[lo];
+        double *dst = panels + off[r] + c;
+        if (l >= k) {  // the panel width is rounded up to 8; the padding columns are zeros
+            for (int i = 0; i < mr; ++i, dst += ld) *dst = 0.0;
+            continue;
         }
-    }
-    // the padding columns (the panel width rounded up to 8) are zeros
-    const int64_t qa = lr_colptr[kap], qb = lr_colptr[kap + 1];
-    const int kw = qb > qa ? koff[qb - 1] + rank[lr_collist[qb - 1]] : 0, pw = Kw - kw;
-    for (int e = threadIdx.x; e < mc * pw; e += blockDim.x) {
-        const int j = e / pw;
-        Wt[(int64_t)j * Kw + kw + (e - j * pw)] = 0.0;
+        if (ROWS) tidx[colptr[r] + c] = (int32_t)(t_off[b] + l);
+        const int64_t o = r0 - adm[4 * b + (ROWS ? 0 : 2)];  // first row of the cluster in the factor
+        const bool mirror = is_mirror(adm, tp, b);
+        const int32_t p = mirror ? tp[b] : b;
+        const int64_t mp = adm[4 * p + 1] - adm[4 * p];
+        // column l of the rows from o on of U_p (column-major) or of W_p behind it (row-major)
+        const bool wfac = ROWS == mirror;
+        const double *src = uw + uw_off[p] + (wfac ? (mp + o) * k + l : l * mp + o);
+        const int64_t step = wfac ? k : 1;
+#pragma unroll 8
+        for (int i = 0; i < mr; ++i, src += step, dst += ld) *dst = __ldg(src);
     }
 }
 
 // offset of the partial projection of each (block, leaf cluster) pair: the
 // column leaf clusters of the block (side = 2, projections through the W
 // panels, product with H) or its row leaf clusters (side = 0, through the U
-// panels, product with H^T)
+// panels, product with H^T); one warp per cluster
 __global__ void pofs_kernel(const int32_t *leaf_begin, int64_t nleaf, const int64_t *lr_colptr,
                             const int32_t *lr_collist, const int32_t *adm, int side, const int64_t *wp_colptr,
                             const int32_t *koff, const int64_t *bcolptr, int64_t *pofs) {
-    for (int64_t kap = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; kap < nleaf;
-         kap += (int64_t)gridDim.x * blockDim.x) {
-        for (int64_t q = lr_colptr[kap]; q < lr_colptr[kap + 1]; ++q) {
-            const int32_t b = lr_collist[q];
-            int64_t lo = 0, hi = nleaf;
-            const int32_t cb = adm[4 * b + side];
-            while (lo < hi) {
-                const int64_t mid = (lo + hi) >> 1;
-                if (leaf_begin[mid] < cb) lo = mid + 1;
-                else hi = mid;
-            }
-            pofs[bcolptr[b] + (kap - lo)] = wp_colptr[kap] + koff[q];
+    const int64_t kap = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (kap >= nleaf) return;
+    for (int64_t q = lr_colptr[kap] + (threadIdx.x & 31); q < lr_colptr[kap + 1]; q += 32) {
+        const int32_t b = lr_collist[q];
+        int64_t lo = 0, hi = nleaf;
+        const int32_t cb = adm[4 * b + side];
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (leaf_begin[mid] < cb) lo = mid + 1;
+            else hi = mid;
         }
+        pofs[bcolptr[b] + (kap - lo)] = wp_colptr[kap] + koff[q];
     }
 }
 
@@ -200,6 +186,8 @@ void build_lr_panels(hm_matrix *A, const DBuf &uw, const DBuf &uw_off, cudaStrea
     const hm_tree *tr = A->tree;
     const int64_t nl = tr->n_leaf, na = tr->n_adm;
     const int64_t np = read_scalar(tr->lr_rowptr.as<int64_t>() + nl, s);
+    // CTAs per cluster of the packing: eight CTAs of eight warps per SM, where there are that many columns
+    const dim3 pack_grid((unsigned)nl, (unsigned)std::max<int64_t>(1, std::min<int64_t>(16, 8LL * num_sms() / nl)));
     A->up_koff.alloc(sizeof(int32_t) * std::max<int64_t>(np, 1));
     A->up_K.alloc(sizeof(int32_t) * nl);
     A->up_off.alloc(sizeof(int64_t) * (nl + 1));
@@ -207,7 +195,7 @@ void build_lr_panels(hm_matrix *A, const DBuf &uw, const DBuf &uw_off, cudaStrea
     DBuf size, kpad;
     size.alloc(sizeof(int64_t) * (nl + 1));
     kpad.alloc(sizeof(int64_t) * (nl + 1));
-    up_width_kernel<<<grid1d(nl), 256, 0, s>>>(tr->leaf_begin.as<int32_t>(), nl, tr->lr_rowptr.as<int64_t>(),
+    up_width_kernel<<<(unsigned)((nl + 7) / 8), 256, 0, s>>>(tr->leaf_begin.as<int32_t>(), nl, tr->lr_rowptr.as<int64_t>(),
                                               tr->lr_list.as<int32_t>(), A->rank.as<int32_t>(),
                                               A->up_koff.as<int32_t>(), A->up_K.as<int32_t>(), size.as<int64_t>(),
                                               kpad.as<int64_t>());
@@ -221,7 +209,7 @@ void build_lr_panels(hm_matrix *A, const DBuf &uw, const DBuf &uw_off, cudaStrea
     A->tidx.alloc(sizeof(int32_t) * std::max<int64_t>(ncol, 8));
     HM_CUDA_CHECK(cudaMemsetAsync(A->tidx.p, 0, sizeof(int32_t) * std::max<int64_t>(ncol, 8), s));
     if (na > 0 && nl > 0) {
-        up_pack_kernel<<<(unsigned)nl, 256, 0, s>>>(
+        pack_kernel<true><<<pack_grid, 256, 0, s>>>(
             tr->leaf_begin.as<int32_t>(), tr->lr_rowptr.as<int64_t>(), tr->lr_list.as<int32_t>(),
             tr->adm.as<int32_t>(), tr->adm_tp.as<int32_t>(), A->rank.as<int32_t>(), A->t_off.as<int64_t>(),
             uw_off.as<int64_t>(),
@@ -234,7 +222,7 @@ void build_lr_panels(hm_matrix *A, const DBuf &uw, const DBuf &uw_off, cudaStrea
     A->wp_K.alloc(sizeof(int32_t) * nl);
     A->wp_off.alloc(sizeof(int64_t) * (nl + 1));
     A->wp_colptr.alloc(sizeof(int64_t) * (nl + 1));
-    up_width_kernel<<<grid1d(nl), 256, 0, s>>>(tr->leaf_begin.as<int32_t>(), nl, tr->lr_colptr.as<int64_t>(),
+    up_width_kernel<<<(unsigned)((nl + 7) / 8), 256, 0, s>>>(tr->leaf_begin.as<int32_t>(), nl, tr->lr_colptr.as<int64_t>(),
                                               tr->lr_collist.as<int32_t>(), A->rank.as<int32_t>(),
                                               A->wp_koff.as<int32_t>(), A->wp_K.as<int32_t>(), size.as<int64_t>(),
                                               kpad.as<int64_t>());
@@ -247,14 +235,13 @@ void build_lr_panels(hm_matrix *A, const DBuf &uw, const DBuf &uw_off, cudaStrea
     const int64_t npairs = read_scalar(tr->lr_bcolptr.as<int64_t>() + na, s);
     A->pofs.alloc(sizeof(int64_t) * std::max<int64_t>(npairs, 1));
     if (na > 0 && nl > 0) {
-        wp_pack_kernel<<<(unsigned)nl, 256, 0, s>>>(tr->leaf_begin.as<int32_t>(), tr->lr_colptr.as<int64_t>(),
-                                                   tr->lr_collist.as<int32_t>(), tr->adm.as<int32_t>(),
-                                                   tr->adm_tp.as<int32_t>(), A->rank.as<int32_t>(),
-                                                   uw_off.as<int64_t>(), uw.as<double>(),
-                                                   A->wp_koff.as<int32_t>(), A->wp_off.as<int64_t>(),
-                                                   A->wp_K.as<int32_t>(), A->wp.as<double>());
+        pack_kernel<false><<<pack_grid, 256, 0, s>>>(
+            tr->leaf_begin.as<int32_t>(), tr->lr_colptr.as<int64_t>(), tr->lr_collist.as<int32_t>(),
+            tr->adm.as<int32_t>(), tr->adm_tp.as<int32_t>(), A->rank.as<int32_t>(), A->t_off.as<int64_t>(),
+            uw_off.as<int64_t>(), uw.as<double>(), A->wp_koff.as<int32_t>(), A->wp_off.as<int64_t>(),
+            A->wp_K.as<int32_t>(), nullptr, A->wp.as<double>(), nullptr);
         HM_LAUNCH_CHECK();
-        pofs_kernel<<<grid1d(nl), 256, 0, s>>>(tr->leaf_begin.as<int32_t>(), nl, tr->lr_colptr.as<int64_t>(),
+        pofs_kernel<<<(unsigned)((nl + 7) / 8), 256, 0, s>>>(tr->leaf_begin.as<int32_t>(), nl, tr->lr_colptr.as<int64_t>(),
                                               tr->lr_collist.as<int32_t>(), tr->adm.as<int32_t>(), 2,
                                               A->wp_colptr.as<int64_t>(), A->wp_koff.as<int32_t>(),
                                               tr->lr_bcolptr.as<int64_t>(), A->pofs.as<int64_t>());
@@ -406,7 +393,7 @@ void build_transposed(const hm_matrix *Ac, cudaStream_t s) {
     A->tidx_t.alloc(sizeof(int32_t) * std::max<int64_t>(A->n_partials, 8));
     HM_CUDA_CHECK(cudaMemsetAsync(A->tidx_t.p, 0, sizeof(int32_t) * std::max<int64_t>(A->n_partials, 8), s));
     if (na > 0 && nl > 0) {
-        pofs_kernel<<<grid1d(nl), 256, 0, s>>>(tr->leaf_begin.as<int32_t>(), nl, tr->lr_rowptr.as<int64_t>(),
+        pofs_kernel<<<(unsigned)((nl + 7) / 8), 256, 0, s>>>(tr->leaf_begin.as<int32_t>(), nl, tr->lr_rowptr.as<int64_t>(),
                                               tr->lr_list.as<int32_t>(), tr->adm.as<int32_t>(), 0,
                                               A->up_colptr.as<int64_t>(), A->up_koff.as<int32_t>(),
                                               tr->lr_browptr.as<int64_t>(), A->pofs_t.as<int64_t>());
