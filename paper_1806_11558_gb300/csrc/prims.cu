@@ -325,9 +325,10 @@ AllocScope::AllocScope(size_t cap_) : cap(cap_), outer(tl_scope == nullptr) {
 
 void AllocScope::flush() {
     const bool idle = blocks.empty() || sync_device(dev);
-    for (auto &b : blocks) {
-        if (idle) cache_put(dev, b.first, b.second);
-        else cudaFree(b.second);
+    // the largest first: where not all fit, the ones that are freed are smaller and sooner mapped again
+    for (auto b = blocks.rbegin(); b != blocks.rend(); ++b) {
+        if (idle) cache_put(dev, b->first, b->second);
+        else cudaFree(b->second);
     }
     blocks.clear();
     held = 0;
