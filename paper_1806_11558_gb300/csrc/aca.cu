@@ -56,6 +56,7 @@ struct AcaArgs {
     const int32_t *adm;
     const int32_t *work;  // blocks to approximate, largest first: [0, n_big) CTA-wide, then warp-wide
     int64_t n_big, n_work;
+    int64_t n_share;  // work[n_big, n_big + n_share): small blocks that a CTA takes together
     double eps;
     int kmax;
     QuadParams qp;
@@ -74,7 +75,7 @@ struct AcaArgs {
     unsigned long long *arena_top;
     int32_t *rank;
     int64_t *uw_off;
-    unsigned long long *q_big, *q_small;
+    unsigned long long *q_big, *q_share, *q_small;
     int *kmax_hit;
     const int32_t *todo;  // optional subset of block ids (re-run after overflow)
     int64_t n_todo;
@@ -153,15 +154,18 @@ __device__ __forceinline__ float warp_sum8(const float (&a)[8]) {
 // decides when to stop): res[0] = |u_r|^2, res[1] = |w_r|^2,
 // res[2 + l] = u_r . u_l, res[2 + r + l] = w_l . w_r (l < r).  One pass over
 // the columns, per-warp shuffle reductions, one shared-memory round.
-template <bool CTA, int NT, class T>
+// SHARE (a CTA on a small block): the warps take eight terms each in turn and
+// form them as a warp alone would, so the sums have the same bits.
+template <bool CTA, int NT, bool SHARE, class T>
 __device__ __noinline__ void norm_terms(const T *Uf, const T *Wf, int m, int n, int r, const AcaShared &sh) {
-    const int gs = CTA ? NT : 32, t = CTA ? (int)threadIdx.x : (int)(threadIdx.x & 31);
+    constexpr bool ALL = CTA && !SHARE;  // all threads on every term
+    const int gs = ALL ? NT : 32, t = ALL ? (int)threadIdx.x : (int)(threadIdx.x & 31);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nvals = 2 + 2 * r;
     const T *ur = Uf + (int64_t)r * m, *wr = Wf + (int64_t)r * n;
-    float *st = CTA ? sh.stage + warp * NORM_STRIDE : sh.stage;
+    float *st = ALL ? sh.stage + warp * NORM_STRIDE : SHARE ? sh.res : sh.stage;
 #pragma unroll 1
-    for (int c0 = 0; c0 < nvals; c0 += 8) {
+    for (int c0 = SHARE ? 8 * warp : 0; c0 < nvals; c0 += SHARE ? NT / 4 : 8) {
         float acc[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) acc[c] = 0.0f;
@@ -190,8 +194,8 @@ __device__ __noinline__ void norm_terms(const T *Uf, const T *Wf, int m, int n, 
         const float a = warp_sum8(acc);
         if ((lane & 3) == 0 && c0 + (lane >> 2) < nvals) st[c0 + (lane >> 2)] = a;
     }
-    if (CTA) {
-        __syncthreads();
+    if (CTA) __syncthreads();
+    if (ALL) {
 #pragma unroll 1
         for (int v = t; v < nvals; v += gs) {
             float a = 0.0f;
@@ -200,7 +204,7 @@ __device__ __noinline__ void norm_terms(const T *Uf, const T *Wf, int m, int n, 
             sh.res[v] = a;
         }
         __syncthreads();
-    } else {
+    } else if (!CTA) {
         __syncwarp();
     }
 }
@@ -307,6 +311,7 @@ __device__ __forceinline__ FF aca_entry(const float *fix, bool fixed_is_row, int
 // themselves.
 struct FacPairs {
     using T = FF;
+    static constexpr bool SHARE = false;
     FF *U, *W;
     __device__ __forceinline__ FF residual(FF e, const FF *vec, const FF *p, int ld, int r) const {
         float hs = e.h, lo = e.l;
@@ -328,6 +333,7 @@ struct FacPairs {
 // terms, the rank-one updates in FP64; there the FP32 units are the busier pipe.
 struct FacDouble {
     using T = double;
+    static constexpr bool SHARE = true;  // in a CTA
     double *U, *W;
     float *Uf, *Wf;
     __device__ __forceinline__ double residual(FF e, const double *vec, const double *p, int ld, int r) const {
@@ -397,13 +403,17 @@ __device__ int aca_block(const AcaArgs &A, int rb, int m, int cb, int n, const F
             for (int l = t; l < r; l += gs) vec[l] = src[(int64_t)l * src_ld];
             G::sync();
             best = Best{-1, 0x7fffffff, 0.0};
+            // a CTA's warps take rounds of 32 in turn, where a CTA is on a block so that it ends sooner equal parts
+            constexpr bool PARTS = CTA && F::SHARE;
+            const int per = (nvar + NT / 32 - 1) / (NT / 32);
+            const int kb = PARTS ? (t - lane) / 32 * per : t - lane, ke = PARTS ? min(nvar, kb + per) : nvar;
 #pragma unroll 1
-            for (int k0 = t - lane; k0 < nvar; k0 += gs) {
-                const int cnt = min(32, nvar - k0);
+            for (int k0 = kb; k0 < ke; k0 += PARTS ? 32 : gs) {
+                const int cnt = min(32, ke - k0);
                 const int lg = cnt > 16 ? 0 : cnt > 8 ? 1 : cnt > 4 ? 2 : 3;
                 const int sub = lane & ((1 << lg) - 1), k = k0 + (lane >> lg);
-                const FF e = aca_entry(sh.fix, pass == 0, fp, v0 + min(k, nvar - 1), sub, lg, A);
-                if (sub == 0 && k < nvar) {
+                const FF e = aca_entry(sh.fix, pass == 0, fp, v0 + min(k, ke - 1), sub, lg, A);
+                if (sub == 0 && k < ke) {
                     const T v = fac.residual(e, vec, M + k, nvar, r);
                     dst[k] = v;
                     if (pass) fac.shadow(v, true, d0 + k);
@@ -449,7 +459,7 @@ __device__ int aca_block(const AcaArgs &A, int rb, int m, int cb, int n, const F
         if (t == 0) sh.ucol[jp >> 5] |= 1u << (jp & 31);
         G::sync();
         // ---- Frobenius norm of the approximant ----
-        norm_terms<CTA, NT>(fac.norm_u(), fac.norm_w(), m, n, r, sh);
+        norm_terms<CTA, NT, CTA && F::SHARE>(fac.norm_u(), fac.norm_w(), m, n, r, sh);
         const float *res = CTA ? sh.res : sh.stage;
         const double nu2 = res[0], nw2 = res[1];
         const double step2 = nu2 * nw2;  // exact
@@ -556,6 +566,39 @@ __global__ void __launch_bounds__(NT, MINB) aca_kernel(AcaArgs A) {
     }
     if (A.todo) return;
 
+    // ---- phase 1c: small blocks of a problem with fewer of them than warps ----
+    if (A.n_share > 0) {
+        AcaShared sh;
+        double *d = reinterpret_cast<double *>(smem_raw);
+        sh.fix = reinterpret_cast<float *>(d);
+        sh.vec = d + 32;
+        sh.bred = s_bred;
+        sh.ibc = &s_ibc;
+        sh.urow = reinterpret_cast<uint32_t *>(d + 32 + MAX_KMAX);
+        sh.ucol = sh.urow + (SMALL_MAX_DIM + 31) / 32;
+        sh.stage = reinterpret_cast<float *>(sh.ucol + (SMALL_MAX_DIM + 31) / 32);
+        sh.res = sh.stage;
+        double *U = A.scr_small + (int64_t)blockIdx.x * WARPS * A.small_stride;
+        for (;;) {
+            long long q = 0;
+            if (threadIdx.x == 0) q = (long long)atomicAdd(A.q_share, 1ull);
+            q = Grp<true, NT>::bcast(q, sh);
+            if (q >= A.n_share) break;
+            const int64_t b = A.work[A.n_big + q];
+            const int32_t rb = A.adm[4 * b], re = A.adm[4 * b + 1], cb = A.adm[4 * b + 2], ce = A.adm[4 * b + 3];
+            const int m = re - rb, n = ce - cb;
+            double *W = U + (int64_t)m * A.kmax;
+            float *Uf = reinterpret_cast<float *>(W + (int64_t)n * A.kmax);
+            const FacDouble fac{U, W, Uf, Uf + (int64_t)m * A.kmax};
+            bool hit = false;
+            const int k = aca_block<true, NT>(A, rb, m, cb, n, fac, sh, &hit);
+            if (hit && threadIdx.x == 0) atomicAdd(A.kmax_hit, 1);
+            __syncthreads();
+            aca_store<true, NT>(A, b, m, n, k, fac, sh);
+            __syncthreads();
+        }
+    }
+
     // ---------------- phase 2: small blocks, one warp each ----------------
     {
         AcaShared sh;
@@ -574,8 +617,8 @@ __global__ void __launch_bounds__(NT, MINB) aca_kernel(AcaArgs A) {
             int q = 0;
             if (lane == 0) q = (int)atomicAdd(A.q_small, 1ull);
             q = __shfl_sync(0xffffffffu, q, 0);
-            if (A.n_big + q >= A.n_work) break;
-            const int64_t b = A.work[A.n_big + q];
+            if (A.n_big + A.n_share + q >= A.n_work) break;
+            const int64_t b = A.work[A.n_big + A.n_share + q];
             const int32_t rb = A.adm[4 * b], re = A.adm[4 * b + 1], cb = A.adm[4 * b + 2], ce = A.adm[4 * b + 3];
             const int m = re - rb, n = ce - cb;
             double *W = U + (int64_t)m * A.kmax;
@@ -673,15 +716,20 @@ void assemble_aca(const hm_tree *tr, hm_matrix *A, const QuadParams &qp, cudaStr
     // work list for a split: blocks with both dims <= SMALL_MAX_DIM and
     // m + n <= small_sum go to single warps, the others to whole CTAs (first)
     // (huge blocks, m + n > HUGE_SUM, come first: only big_ctas CTAs hold scratch for them)
-    auto split = [&](const std::vector<int32_t> &blocks, int small_sum, std::vector<int32_t> &work, int64_t &n_big,
-                     int &max_sum_small, int64_t &n_huge) {
-        std::vector<int32_t> huge, big, small;
+    // Small blocks longer than a warp's share of all of them would end after all
+    // the others: a whole CTA takes each of those, with the same result (5,120
+    // panels, 2,851 blocks on 3,040 warps: 2.0 -> 1.1 ms).
+    auto split = [&](const std::vector<int32_t> &blocks, int small_sum, int64_t warps, std::vector<int32_t> &work,
+                     int64_t &n_big, int &max_sum_small, int64_t &n_huge, int64_t &n_share) {
+        std::vector<int32_t> huge, big, share, small;
         max_sum_small = 2;
+        int64_t sum_small = 0;
         for (int32_t b : blocks) {
             const int m = h_adm[4 * b + 1] - h_adm[4 * b], n = h_adm[4 * b + 3] - h_adm[4 * b + 2];
             if (m <= SMALL_MAX_DIM && n <= SMALL_MAX_DIM && m + n <= small_sum) {
                 small.push_back(b);
                 max_sum_small = std::max(max_sum_small, m + n);
+                sum_small += m + n;
             } else if (m + n > HUGE_SUM) {
                 huge.push_back(b);
             } else {
@@ -690,8 +738,14 @@ void assemble_aca(const hm_tree *tr, hm_matrix *A, const QuadParams &qp, cudaStr
         }
         n_huge = (int64_t)huge.size();
         n_big = n_huge + (int64_t)big.size();
+        const auto rest = std::stable_partition(small.begin(), small.end(),
+                                                [&](int32_t b) { return (int64_t)msum(b) * warps > sum_small; });
+        share.assign(small.begin(), rest);
+        small.erase(small.begin(), rest);
+        n_share = (int64_t)share.size();
         work = huge;
         work.insert(work.end(), big.begin(), big.end());
+        work.insert(work.end(), share.begin(), share.end());
         work.insert(work.end(), small.begin(), small.end());
     };
 
@@ -793,11 +847,12 @@ void assemble_aca(const hm_tree *tr, hm_matrix *A, const QuadParams &qp, cudaStr
         const Launch &L = launch_of(tc.nt);
         const int grid = sms * std::min(tc.ctas, L.occ);
         std::vector<int32_t> work;
-        int64_t n_big = 0, n_huge = 0;
+        int64_t n_big = 0, n_huge = 0, n_share = 0;
         int max_sum_small = 2;
-        split(blocks, tc.small_sum, work, n_big, max_sum_small, n_huge);
+        split(blocks, tc.small_sum, (int64_t)grid * (L.nt / 32), work, n_big, max_sum_small, n_huge, n_share);
         AcaArgs a = base;
         a.n_huge = n_huge;
+        a.n_share = n_share;
         a.big_ctas = huge_ctas(grid);
         scr_med.alloc(sizeof(double) * base.med_stride * grid);
         a.scr_med = scr_med.as<double>();
@@ -814,13 +869,14 @@ void assemble_aca(const hm_tree *tr, hm_matrix *A, const QuadParams &qp, cudaStr
         a.q_small = ctr4 + 2;
         a.kmax_hit = reinterpret_cast<int *>(ctr4 + 3);
         a.q_huge = ctr4 + 4;
+        a.q_share = ctr4 + 5;
         a.rank = rank;
         a.uw_off = uwo;
         a.arena = arena;
         a.arena_cap = cap;
         a.todo = nullptr;
         a.n_todo = 0;
-        HM_CUDA_CHECK(cudaMemsetAsync(ctr4, 0, sizeof(unsigned long long) * 5, s));
+        HM_CUDA_CHECK(cudaMemsetAsync(ctr4, 0, sizeof(unsigned long long) * 6, s));
         cudaEvent_t t0, t1;
         HM_CUDA_CHECK(cudaEventCreate(&t0));
         HM_CUDA_CHECK(cudaEventCreate(&t1));
@@ -860,7 +916,7 @@ void assemble_aca(const hm_tree *tr, hm_matrix *A, const QuadParams &qp, cudaStr
             t_rank.alloc(sizeof(int32_t) * na);
             t_uwo.alloc(sizeof(int64_t) * na);
             t_arena.alloc(sizeof(double) * sum_mn * kmax);
-            t_ctr.alloc(sizeof(unsigned long long) * 5);
+            t_ctr.alloc(sizeof(unsigned long long) * 6);
             auto time_of = [&](const Tune &tc) {
                 return run(sample, tc, t_rank.as<int32_t>(), t_uwo.as<int64_t>(), t_arena.as<double>(),
                            sum_mn * kmax, t_ctr.as<unsigned long long>(), t_scr, t_work, nullptr);
@@ -913,7 +969,7 @@ void assemble_aca(const hm_tree *tr, hm_matrix *A, const QuadParams &qp, cudaStr
     }
     DBuf arena, ctr, scr_small, d_work;
     arena.alloc(sizeof(double) * cap);
-    ctr.alloc(sizeof(unsigned long long) * 5);
+    ctr.alloc(sizeof(unsigned long long) * 6);
     // the arguments of that run are kept for an overflow re-run
     AcaArgs a{};
     const float ms = run(upper, cfg, A->rank.as<int32_t>(), uw_off.as<int64_t>(), arena.as<double>(), cap,

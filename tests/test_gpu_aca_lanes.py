@@ -48,3 +48,35 @@ def test_squares_below_the_normal_float_range():
         assert np.isfinite(ex["dense"]).all() and np.isfinite(ex["uw"]).all()
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("leaf,count", [(20, 40), (40, 100)])
+def test_blocks_shared_by_a_cta(orc, leaf, count):
+    # with fewer blocks than warps a CTA works on one block, with many copies of the geometry a warp does:
+    # the same ranks and factors, bit for bit
+    torch = need_gpu()
+    import paper_1806_11558_gb300 as hm
+    V, T = meshgen.bump_sphere(3, 1808)[:2]
+    g = GpuH(V, T, leaf=leaf, eta=1.5, eps=1e-6)
+    n, nv = T.shape[0], V.shape[0]
+    Vs = torch.from_numpy(np.tile(V, (count, 1))).cuda()
+    Ts = torch.from_numpy(np.ascontiguousarray((T[None] + nv * np.arange(count)[:, None, None]).reshape(-1, 3)
+                                               .astype(np.int32))).cuda()
+    tree = hm.hm_build_forest(Vs, Ts, [n * k for k in range(count + 1)], eta=1.5, leaf_size=leaf)
+    A = hm.hm_assemble(tree, aca_eps=1e-6)
+    try:
+        ti = hm.hm_tree_get_info(tree)
+        one, all_ = g.export(), hm.hm_matrix_export(A, ti["n_dense"], ti["n_adm"])
+        al = g.leaves(False).reshape(-1, 4)
+        ak = {tuple(b): k for k, b in enumerate(hm.hm_tree_get_leaves(tree, False).cpu().numpy().reshape(-1, 4).tolist())}
+        assert al.shape[0] > 0 and ti["n_adm"] == count * al.shape[0]
+        for b, blk in enumerate(al.tolist()):
+            c, k = ak[tuple(blk)], int(one["rank"][b])
+            assert int(all_["rank"][c]) == k
+            for off, size in (("u_off", blk[1] - blk[0]), ("w_off", blk[3] - blk[2])):
+                x = one["uw"][one[off][b]:one[off][b] + size * k]
+                assert np.array_equal(x, all_["uw"][all_[off][c]:all_[off][c] + size * k])
+    finally:
+        hm.hm_free(A)
+        hm.hm_free(tree)
+        g.close()
