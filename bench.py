@@ -42,7 +42,7 @@ LARGE = dict(workload="unit icosphere level 8, Galerkin single-layer Laplace, P0
              nrhs=16, sources="16 seeded exterior point sources, |p| uniform in [2, 4]", solve_rel_tol=1e-12,
              form="mixed: FP32 near field + FP32 factors; lockstep GMRES whose inner solves use the 16-RHS "
                   "tensor-core product; iterative refinement on the FP64 master, its residuals by the 16-RHS "
-                  "double-float product",
+                  "digit product (tensor cores)",
              inner_tol=1e-4, restart=128, precond=True, batched=True, resid_df=True, factor_tail_bits=0)
 PRECISION = dict(workload="bumped icosphere level 7, Galerkin single-layer Laplace, P0",
                  case="precision", panels=327680, leaf_size=64, eta=1.5, aca_eps=1e-7, aca_kmax=64, ss_order=8,
@@ -68,8 +68,8 @@ def _peaks():
 FP64_PEAK_TFLOPS = 152 * 2.07e9 * 2 * 2 / 1e12   # 1.26
 FP32_PEAK_TFLOPS = 152 * 2.07e9 * 128 * 2 / 1e12  # 80.5
 # FP32 flops of one pair evaluation in the double-float entry (ACA and the
-# regular near field; TwoSum 6, TwoProduct 2 with its FMA counted 2, ...): 93 per pair
-FF_FLOPS_PER_PAIR = 93
+# regular near field; TwoSum 6, or 3 of ordered positive terms, TwoProduct 3 with its FMA counted 2, ...): 78 per pair
+FF_FLOPS_PER_PAIR = 78
 
 # DRAM traffic per launch from an ncu capture, valid while the kernel's source
 # file is unchanged (sha256 of the file at capture time); null otherwise.
@@ -425,7 +425,7 @@ def run_large(args, world, hm, torch, W=LARGE, case="large"):
         byts = mi["dense_entries"] * 4 + mi["lr_entries"] * fb
         mv[name] = {"s": sec, "matrix_gb": byts / 1e9, "gbs_matrix": byts / sec / 1e9,
                     "s_per_rhs": sec / R}
-    # the FP64 master, 16 right-hand sides in double-float arithmetic (the residual product of the refinement)
+    # the FP64 master, 16 right-hand sides by exact digit products (the residual product of the refinement)
     hm.hm_matvec_block(A, Xr, Yr, prec=hm.HM_F64)
     a.record(stream)
     for _ in range(3):
@@ -1023,7 +1023,7 @@ def run_solve16(torch, hm, level=6):
 
 
 def run_dfmv(torch, hm, case):
-    """The FP64 master applied to 16 right-hand sides: the double-float
+    """The FP64 master applied to 16 right-hand sides: the exact-digit
     16-column product (hm_matvec_block, HM_F64) against 16 FP64 products
     (hm_matvec, one right-hand side each), and their difference."""
     import meshgen
