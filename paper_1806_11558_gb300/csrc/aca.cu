@@ -517,7 +517,9 @@ __device__ void aca_store(const AcaArgs &A, int64_t b, int m, int n, int k, cons
 // registers per thread).  Four CTAs of 128 threads with 128 registers evaluate
 // the entries 11% faster, but wait longer between them: 655,220 panels 357 ms
 // against 334.
-template <int NT, int MINB>
+// SHARED: with phase 1c, whose code costs the others registers (200,000 panels:
+// 94.2 ms with it in the kernel, 93.3 without).
+template <int NT, int MINB, bool SHARED>
 __global__ void __launch_bounds__(NT, MINB) aca_kernel(AcaArgs A) {
     constexpr int WARPS = NT / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -567,7 +569,7 @@ __global__ void __launch_bounds__(NT, MINB) aca_kernel(AcaArgs A) {
     if (A.todo) return;
 
     // ---- phase 1c: small blocks of a problem with fewer of them than warps ----
-    if (A.n_share > 0) {
+    if constexpr (SHARED) {
         AcaShared sh;
         double *d = reinterpret_cast<double *>(smem_raw);
         sh.fix = reinterpret_cast<float *>(d);
@@ -753,23 +755,28 @@ void assemble_aca(const hm_tree *tr, hm_matrix *A, const QuadParams &qp, cudaStr
     // launch configurations: CTA sizes of 64, 128 and 256 threads, each with
     // the register budget of about 100 per thread
     struct Launch {
-        void (*kern)(AcaArgs);
+        void (*kern)(AcaArgs), (*kern_shared)(AcaArgs);
         int nt, occ;
         size_t smem;
     };
-    auto make_launch = [&](void (*kern)(AcaArgs), int nt) {
+    auto make_launch = [&](void (*kern)(AcaArgs), void (*kern_shared)(AcaArgs), int nt) {
         const int warps = nt / 32;
         const size_t smem_big = sizeof(double) * (32 + MAX_KMAX) + sizeof(uint32_t) * (words_r + words_c + 1) +
                                 sizeof(float) * (warps + 1) * NORM_STRIDE;
         const size_t smem_small = (size_t)warps * sizeof(double) * WARP_SMEM_DOUBLES;
-        Launch L{kern, nt, 0, std::max(smem_big, smem_small)};
-        HM_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem));
-        HM_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&L.occ, kern, nt, L.smem));
+        Launch L{kern, kern_shared, nt, 1 << 30, std::max(smem_big, smem_small)};
+        for (auto k : {kern, kern_shared}) {
+            int occ = 0;
+            HM_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem));
+            HM_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, nt, L.smem));
+            L.occ = std::min(L.occ, occ);
+        }
         if (L.occ < 1) fail(HM_EINTERNAL, "ACA kernel (%d threads) does not fit on an SM", nt);
         return L;
     };
-    const Launch launches[3] = {make_launch(aca_kernel<64, 10>, 64), make_launch(aca_kernel<128, 5>, 128),
-                                make_launch(aca_kernel<256, 2>, 256)};
+    const Launch launches[3] = {make_launch(aca_kernel<64, 10, false>, aca_kernel<64, 10, true>, 64),
+                                make_launch(aca_kernel<128, 5, false>, aca_kernel<128, 5, true>, 128),
+                                make_launch(aca_kernel<256, 2, false>, aca_kernel<256, 2, true>, 256)};
     auto launch_of = [&](int nt) -> const Launch & { return launches[nt == 64 ? 0 : nt == 256 ? 2 : 1]; };
     const int sms = num_sms();
 
@@ -883,7 +890,7 @@ void assemble_aca(const hm_tree *tr, hm_matrix *A, const QuadParams &qp, cudaStr
         HM_CUDA_CHECK(cudaEventRecord(t0, s));
         {
             Trace trace("aca_kernel", s);
-            L.kern<<<grid, L.nt, L.smem, s>>>(a);
+            (n_share > 0 ? L.kern_shared : L.kern)<<<grid, L.nt, L.smem, s>>>(a);
             HM_LAUNCH_CHECK();
         }
         HM_CUDA_CHECK(cudaEventRecord(t1, s));
