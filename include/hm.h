@@ -435,11 +435,11 @@ HM_API hm_status hm_matvec_scaled(const hm_matrix *A, int32_t trans, int32_t nrh
                                   const double *d_right, const double *d_x, double *d_y, double alpha, double beta,
                                   hm_stream_t stream);
 
-/* Frees an hm_tree or hm_matrix handle (NULL is a no-op).  Device buffers of
- * 1 MiB or more are not unmapped but kept by the library for its later
- * allocations (unmapping costs ~0.4 ms per GB), up to a quarter of the
- * device memory; the library empties that cache by itself when one of its
- * own allocations fails. */
+/* Frees an hm_tree or hm_matrix handle (NULL is a no-op).  Its device buffers
+ * are not unmapped but kept by the library for its later allocations
+ * (unmapping costs ~0.4 ms per GB), up to a quarter of the device memory, and
+ * 64 MiB of buffers below 1 MiB; the library empties that cache by itself when
+ * one of its own allocations fails. */
 HM_API void hm_free(void *handle);
 
 /* Adds a low-precision copy to an assembled matrix, made from its FP64
