@@ -413,7 +413,16 @@ __global__ void __launch_bounds__(32 * CW, 4) col_fx_kernel(int parts, const int
 // b0[c] (the block holding entry 32 c) by a search over the next 32 blocks'
 // offsets, or over t_off beyond them.
 // ---------------------------------------------------------------------------
-constexpr int T_EMIN = -70;  // smallest exponent of a non-zero row of t (2^(54 - e) stays a float)
+// x 2^k to the nearest integer, by integer operations, for finite x with |x| 2^k < 2^62
+__device__ __forceinline__ long long scaled_int(float x, int k) {
+    const uint32_t b = __float_as_uint(x);
+    const int eb = max((int)(b >> 23) & 0xff, 1);
+    const long long m = (long long)((b & 0x7fffffu) | (b & 0x7f800000u ? 0x800000u : 0u));  // |x| = m 2^(eb - 150)
+    const int sh = eb - 150 + k;
+    const int dn = min(-sh, 32);
+    const long long v = sh >= 0 ? m << sh : (m + (1ll << (dn - 1))) >> dn;
+    return (int)b < 0 ? -v : v;
+}
 
 template <int NT>
 __global__ void __launch_bounds__(256) tsum_fx_kernel(int64_t na, int64_t nt, const int32_t *__restrict__ b0tab,
@@ -472,25 +481,16 @@ __global__ void __launch_bounds__(256) tsum_fx_kernel(int64_t na, int64_t nt, co
             norm2(s[r], c[r], h, lo);
             s[r] = h;
             c[r] = lo;
-            const int eb = (int)(__float_as_uint(h) >> 23) & 0xff;
-            if (eb == 0xff) bad |= 1u << r;
-            else if (eb) ex = max(ex, max(eb - 126, T_EMIN));
+            const uint32_t hb = __float_as_uint(h) & 0x7fffffffu;
+            if (hb >= 0x7f800000u) bad |= 1u << r;
+            else if (hb) ex = max(ex, max((int)(hb >> 23), 1) - 126);  // |h| < 2^ex, subnormal h too
         }
         Te[e] = make_uint2((uint32_t)(ex + E_BIAS) << 20, bad);
-        const float sc = __uint_as_float((uint32_t)(127 + QB - max(ex, T_EMIN)) << 23);  // 2^(54 - ex)
         unsigned long long u[NR];
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
-            const uint32_t hb = __float_as_uint(s[r]);
-            const int eb = (int)(hb >> 23) & 0xff;
             long long q = 0;
-            if (eb != 0 && eb != 0xff) {
-                const int sh = QB - 24 - (ex - (eb - 126));  // h = mantissa 2^(eb - 126 - 24)
-                const long long mant = (long long)((hb & 0x7fffffu) | 0x800000u);
-                q = sh >= 0 ? mant << sh : sh > -25 ? mant >> -sh : 0;
-                if ((int)hb < 0) q = -q;
-                q += __float2int_rn(__fmul_rn(c[r], sc));
-            }
+            if (ex > E_ZERO && !(bad >> r & 1)) q = scaled_int(s[r], QB - ex) + scaled_int(c[r], QB - ex);
             u[r] = (unsigned long long)(q + DIGIT_BIAS);
         }
         uint4 *o = reinterpret_cast<uint4 *>(Td + e * DIG);
