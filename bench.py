@@ -139,9 +139,9 @@ def algorithmic_work(mi, ti, dense_leaves, n):
         "col_bcp_kernel.bf16": ("hbm", (2.0 * w16 + xr * (n + K16)) if K16 else (2.0 * w + xr * (n + K)), "byte"),
         "nearfield_kernel": ("alu32", float(nf_entries) * PAIRS_PER_ENTRY * FF_FLOPS_PER_PAIR, "flop"),
         # product of the FP64 master with 16 right-hand sides: every entry once, the digits and exponents of the
-        # rows of x and t (7 x 16 x 2 + 8 B), the rows of y (16 x 8 B), the partials (float pairs)
-        "row_fx_kernel": ("hbm", 8.0 * (d + u) + 232.0 * (n + K) + 128.0 * n, "byte"),
-        "col_fx_kernel": ("hbm", 8.0 * w + 232.0 * n + 128.0 * w * nl / n, "byte"),
+        # rows of x and t (8 x 16 x 2 + 8 B), the rows of y (16 x 8 B), the partials (float pairs)
+        "row_fx_kernel": ("hbm", 8.0 * (d + u) + 264.0 * (n + K) + 128.0 * n, "byte"),
+        "col_fx_kernel": ("hbm", 8.0 * w + 264.0 * n + 128.0 * w * nl / n, "byte"),
         "nearfield_kernel.f64": ("alu", float(nf_entries) * PAIRS_PER_ENTRY * FLOPS_PER_PAIR, "flop"),
         "aca_kernel": ("alu32", float(mi["aca_entries"]) * PAIRS_PER_ENTRY * FF_FLOPS_PER_PAIR, "flop"),
     }

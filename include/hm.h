@@ -180,9 +180,10 @@ typedef struct {
                            b - H x of all systems by the 16-right-hand-side
                            product of the FP64 master on the tensor cores
                            (hm_matvec_block with HM_F64: each stored entry
-                           read once per 16 systems; a few 1e-15 of |H||x|
-                           instead of ~1e-16), and the stopping test on them; 0 = one FP64 product
-                           per system.  Other values: HM_EINVAL. */
+                           read once per 16 systems; a few 1e-15 of each
+                           system's |H||x| instead of ~1e-16), and the
+                           stopping test on them; 0 = one FP64 product per
+                           system.  Other values: HM_EINVAL. */
 } hm_solve_params;
 
 typedef struct {
@@ -353,14 +354,18 @@ HM_API hm_status hm_matvec(const hm_matrix *A, int32_t trans, int32_t nrhs, hm_d
  *  about 16 significant bits (relative error ~1e-5 on top of the copy's own
  *  rounding) — accurate enough for the inner solves of the refinement.
  *  prec = HM_F64: the FP64 master on the tensor cores, every entry and x cut
- *  into seven digits base 256 whose products are summed without rounding
+ *  into eight digits base 256 whose products are summed without rounding
  *  (Ozaki, Ogita, Oishi and Rump): a few 1e-15 of the row sums of |H||x| — the
- *  FP64 residuals of the batched refinement (hm_solve_params.resid_df).  Each
- *  x_r is scaled by itself; a right-hand side whose entries are small beside
- *  the others' in the same panels keeps fewer of the 54 bits there.
+ *  FP64 residuals of the batched refinement (hm_solve_params.resid_df).  Leaf
+ *  clusters where a right-hand side is far smaller than others of its 16 (by 2^7
+ *  in x or by 2^9 in the terms of a row) are formed in pairs of floats with
+ *  compensated sums, ~1e-14 of its own |H||x|, at up to four times the time.  Sums
+ *  are carried in the range of FP32, each x_r scaled by its largest entry: terms
+ *  below 2^-149 of that count as zero, a sum beyond 2^128 is NaN.
  * Stream-ordered (working vectors from the stream-ordered pool; HM_F64 uses
- * 360 bytes per panel, 128 per partial projection and 232 per unit of total
- * rank).
+ * 392 bytes per panel, 128 per partial projection, 264 per unit of total rank and,
+ * for leaf clusters whose panels are split over several work items, 136 per row and
+ * item).
  * Errors: HM_EINVAL for NULL pointers, nrhs < 1, an unknown precision, or a
  * low precision whose copy was not assembled. */
 HM_API hm_status hm_matvec_block(const hm_matrix *A, int32_t nrhs, hm_dtype prec, const double *d_x, double *d_y,

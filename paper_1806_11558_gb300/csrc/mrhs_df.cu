@@ -12,33 +12,45 @@
 // multiplication and its applications", Numer. Algorithms 2012):
 //   * column k of a panel has the exponent e_k of its largest x_r (each x_r
 //     scaled by its own largest entry first) and x_r 2^-e_k becomes an integer
-//     of 54 bits and sign, seven balanced digits d in [-128, 127], as FP16;
-//   * a term w 2^e_k of a row becomes an integer of 54 bits or less and sign on
+//     of 62 bits and sign, eight balanced digits d in [-128, 127], as FP16;
+//   * a term w 2^e_k of a row becomes an integer of 62 bits or less and sign on
 //     the scale of the row's largest term so far, in integer operations on the
-//     bits of w: seven digits, the top one signed, the others in [0, 255], as
+//     bits of w: eight digits, the top one signed, the others in [0, 255], as
 //     FP16 subnormals (u 2^-24, which are the digit's own bits);
-//   * of the 49 products of digits the 34 of order i + j <= 7 are formed by
+//   * of the 64 products of digits the 36 of order i + j <= 7 are formed by
 //     mma.m16n8k16 and summed by order: integers below 2^24 times 2^-24, exact
 //     in FP32 over 128 columns (orders 4 to 7, worth 2^-32 and less, may round);
 //   * the sums are put together as a float pair, without loss for the orders 0
-//     to 3, and added to a running pair (TwoSum): every 128 columns, or where a
+//     to 4, and added to a running pair (TwoSum): every 128 columns, or where a
 //     larger term raises the row's scale.
-// Against the exact product (16 right-hand sides, 1,280 to 2,880 panels) the
-// error is 4e-16 of |H||x| in norm for random and 2.5e-15 for positive x; the
-// compensated sums of float pairs that this replaces had 3e-15 and 1e-14 to
-// 1.4e-13.  Time per pass, before -> now (HBM alone): 64,980 panels, leaves of 64 rows:
-// row 3.93 -> 1.00 ms (0.33), column 0.97 -> 0.50 ms (0.15); 327,680 panels,
-// leaves of 80: row 16.1 -> 7.2 ms (2.3), column 6.4 -> 3.6 ms (1.1).
+// The scales of columns and rows are those of the largest of 16 right-hand sides.
+// Eight digits leave 15 bits for a right-hand side that is smaller there than
+// others and has still what a pair of floats keeps (48 bits of an entry and of an x);
+// each sum keeps a record of the right-hand sides that had a term of their own
+// of that size (X_OWN, ROW_OWN), and the clusters where one had none are formed
+// again in pairs of floats, where no right-hand side sees another.  Seven digits
+// and no record were 11% to 22% faster (64,980 panels 1.73 ms a pass) and lost a unit
+// vector's entries 10^7 below another's to 2e-9.
+// Against the exact product (16 right-hand sides, 1,280 and 2,880 panels) the
+// error is 2e-16 of |H||x| in norm for random, 2.3e-15 for positive x and 1.7e-15
+// for unit vectors; float pairs throughout have 2e-15, 1.1e-14 and 2.2e-15.
+// Time of a pass with 16 right-hand sides, float pairs -> this (HBM alone), ms:
+// 5,120 panels 0.415 -> 0.186, 64,980 panels, leaves of 64 rows, 4.59 -> 1.92 (0.48; row
+// pass 1.12, column pass 0.56), 327,680 panels, leaves of 80, 26.8 -> 15.4 (3.4; row 9.3,
+// column 5.1).  Vectors whose sizes differ by 1e10 between the halves of the sphere,
+// so that most clusters are formed again: 0.50, 7.0 and 35 ms.
 // Non-finite x or entries give NaN in the rows they reach.
 //
 //   scale_x / digits_x    : the scale of each x_r, the digits of x
 //   col_fx_kernel         : per leaf column cluster kappa the partials
 //                           x_kappa^T W of its column panel
+//   col_pairs_kernel      : the partials of the listed clusters, in float pairs
 //   tsum_fx_kernel        : t_b = sum of b's partials in increasing cluster
 //                           order, and its digits
 //   row_fx_kernel         : per leaf row cluster, the near-field panel times
 //                           the gathered x and the U panel times the gathered t
 //   row_reduce_kernel     : the sums of the rows whose panels were split
+//   pairs / row_pairs     : the rows of the listed clusters, in float pairs
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -50,15 +62,23 @@ namespace hm {
 namespace fx {
 
 constexpr int MR = 16;              // right-hand sides of a pass
-constexpr int NA = 7;               // digits of an entry, and of an x
+constexpr int NA = 8;               // digits of an entry, and of an x
 constexpr int NO = 6;               // sums kept: the orders 0 to 5, and with the last 6 / 2^8 and 7 / 2^16
 constexpr int DIG = NA * MR;        // halves per row of digits ([digit, top first][rhs])
 constexpr int XSTRIDE = 2 * DIG + 16;  // bytes per staged row: 8 rows hit different banks (ldmatrix)
-constexpr int QB = 54;              // bits of an integer x
+constexpr int QB = 62;              // bits of an integer x
 constexpr int E_ZERO = -900;        // exponent of a column of zeros, and the smallest one
 constexpr int E_BIAS = 1000;        // added to the exponents of columns, which makes them positive
 constexpr int F_EXP = 884;          // a row's factor 2^(E - 1011) as a float: exponent field E - 884
 constexpr int E_NAN = F_EXP + 255;  // biased term exponents from here on: not finite, or beyond FP32
+// A sum is taken as it is where one of its terms has an x_r within 2^X_OWN of the
+// column's largest and an entry within 2^ROW_OWN (COL_OWN) of the row's scale, or in a
+// row within RAISE_OWN more by later terms that raised the scale: the 2^-61.5 of the
+// scale that a term may be off is then 2^-46.5 of that term or less, which is what
+// pairs of floats make of a product.  Within a row the scale is mostly raised by
+// the diagonal, or late in U by 2; without RAISE_OWN one row in some 10,000 of random
+// vectors was unsure.
+constexpr int X_OWN = 6, ROW_OWN = 5, RAISE_OWN = 3, COL_OWN = 8;
 
 // (s, c) += (s2, c2)
 __device__ __forceinline__ void dadd(float &s, float &c, float s2, float c2) {
@@ -112,17 +132,19 @@ __global__ void __launch_bounds__(256) scale_x_kernel(const double *__restrict__
 // |x_r| < 2^scale
 __device__ __forceinline__ int scale_of(unsigned int sc) { return sc >= 0x100000u ? (int)(sc >> 20) - 1022 : 0; }
 
-// the seven digits of q, |q| <= 2^54, as halves at o[0], o[MR], ... (top first)
-constexpr long long DIGIT_BIAS = 0x80808080808080ll;
+// the eight digits of q, |q| <= 2^62, as halves at o[0], o[MR], ... (top first)
+constexpr unsigned long long DIGIT_BIAS = 0x8080808080808080ull;
 __device__ __forceinline__ void store_digits(long long q, __half *o) {
-    const unsigned long long u = (unsigned long long)(q + DIGIT_BIAS);
+    const unsigned long long u = (unsigned long long)q + DIGIT_BIAS;
 #pragma unroll
     for (int j = 0; j < NA; ++j) o[(NA - 1 - j) * MR] = __int2half_rn((int)((u >> (8 * j)) & 0xffu) - 128);
 }
 
-// Xd[m] = the digits of x_r 2^-(scale_r + e), Xe[m] = ((e + E_BIAS) 2^20, bits of the r
-// whose x_r is not finite), for position m (x is [nr][n], original order
-// when perm is given); zeros for r >= nr.  16 lanes per position.
+// Xd[m] = the digits of x_r 2^-(scale_r + e), Xe[m] = ((e + E_BIAS) 2^20, state of
+// the x_r), for position m (x is [nr][n], original order when perm is given);
+// zeros for r >= nr.  16 lanes per position.  State: bit r and bit r + 16 of x_r are
+// 00 zero, 01 (the upper) small beside the column's largest, 11 within 2^X_OWN of
+// it, 10 not finite.
 __global__ void __launch_bounds__(256) digits_x_kernel(const double *__restrict__ x, int64_t n, int nr,
                                                        const int32_t *__restrict__ perm,
                                                        const unsigned int *__restrict__ sc, __half *__restrict__ Xd,
@@ -140,10 +162,11 @@ __global__ void __launch_bounds__(256) digits_x_kernel(const double *__restrict_
         int e = ex;
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-        const unsigned int bm = __ballot_sync(0xffffffffu, bad) >> (threadIdx.x & 16) & 0xffffu;
         // the mantissa (53 bits) on the column's scale, rounded to nearest
         long long q = 0;
         const int sh = e - ex;
+        const unsigned int lo = __ballot_sync(0xffffffffu, bad || (eb != 0 && sh <= X_OWN));
+        const unsigned int up = __ballot_sync(0xffffffffu, !bad && eb != 0);
         if (eb != 0 && !bad && sh < 63) {
             const unsigned long long mant = (b & 0xfffffffffffffull) | 0x10000000000000ull;
             q = (long long)(((mant << (QB - 53)) + ((1ull << sh) >> 1)) >> sh);
@@ -151,7 +174,9 @@ __global__ void __launch_bounds__(256) digits_x_kernel(const double *__restrict_
         }
         if (m < n) {
             store_digits(q, Xd + m * DIG + r);
-            if (r == 0) Xe[m] = make_uint2((uint32_t)(e + E_BIAS) << 20, bm);
+            if (r == 0)
+                Xe[m] = make_uint2((uint32_t)(e + E_BIAS) << 20,
+                                   (lo >> (threadIdx.x & 16) & 0xffffu) | (up >> (threadIdx.x & 16)) << 16);
         }
     }
 }
@@ -177,37 +202,43 @@ __device__ __forceinline__ uint32_t raise_exp(uint32_t tm, uint32_t E20) {
     return tm < E20 + 0x100000u ? E20 : (tm & 0xfff00000u) + HEADROOM;
 }
 
-// w 2^(e - E) as 55-bit fixed point plus 2^55: bytes 6..0 are the digits (the
-// top one plus 128)
-__device__ __forceinline__ void fixed_point(double w, uint32_t E20, uint32_t e20, uint32_t &lo, uint32_t &hi) {
+// w 2^(e - E) as 63-bit fixed point plus 2^63: bytes 7..0 are the digits (the
+// top one plus 128); returns E minus the term's exponent
+__device__ __forceinline__ uint32_t fixed_point(double w, uint32_t E20, uint32_t e20, uint32_t &lo, uint32_t &hi) {
     const int h = __double2hiint(w);
     const uint32_t s = min((E20 - e20 - ((uint32_t)h & 0x7ff00000u)) >> 20, 63u);
     const unsigned long long v =
-        ((((unsigned long long)(uint32_t)((h & 0xfffff) | 0x100000) << 32) | (uint32_t)__double2loint(w)) << 2) >> s;
+        ((((unsigned long long)(uint32_t)((h & 0xfffff) | 0x100000) << 32) | (uint32_t)__double2loint(w)) << 10) >> s;
     const uint32_t sg = (uint32_t)(h >> 31);
     lo = (uint32_t)v ^ sg;
-    hi = (uint32_t)(v >> 32) ^ sg ^ 0x00800000u;
+    hi = (uint32_t)(v >> 32) ^ sg ^ 0x80000000u;
+    return s;
 }
 
-// the seven digits of two entries of consecutive k (columns with e20 = ea,
-// eb), packed for an A fragment (lower k in the low half): o[i][reg], top
-// digit first, as FP16 subnormals
-__device__ __forceinline__ void digit_pair(double a, double b, uint32_t E20, uint32_t ea, uint32_t eb, uint32_t (&o)[NA][4], int reg) {
+// the eight digits of two entries of consecutive k (a's column with e20 = e.x and
+// state e.y, b's with e.z and e.w), packed for an A fragment (lower k in the
+// low half): o[i][reg], top digit first, as FP16 subnormals.  own: the states
+// of the columns whose term is within 2^OWN of the row's scale.
+template <int OWN>
+__device__ __forceinline__ void digit_pair(double a, double b, uint32_t E20, const uint4 &e, uint32_t (&o)[NA][4], int reg,
+                                           uint32_t &own) {
     uint32_t al, ah, bl, bh;
-    fixed_point(a, E20, ea, al, ah);
-    fixed_point(b, E20, eb, bl, bh);
-    const uint32_t t = __byte_perm(ah, bh, 0x6521);  // a5 a6 b5 b6
-    const uint32_t p = __byte_perm(al, bl, 0x6521);  // a1 a2 b1 b2
-    const uint32_t q = __byte_perm(al, bl, 0x7430);  // a0 a3 b0 b3
+    if (fixed_point(a, E20, e.x, al, ah) <= OWN) own |= e.y;
+    if (fixed_point(b, E20, e.z, bl, bh) <= OWN) own |= e.w;
+    const uint32_t t = __byte_perm(ah, bh, 0x7632);  // a6 a7 b6 b7
+    const uint32_t u = __byte_perm(ah, bh, 0x5410);  // a4 a5 b4 b5
+    const uint32_t p = __byte_perm(al, bl, 0x7632);  // a2 a3 b2 b3
+    const uint32_t q = __byte_perm(al, bl, 0x5410);  // a0 a1 b0 b1
     const uint32_t top = __byte_perm(t, 0, 0x4341);
     const __half2 c = __hsub2(*reinterpret_cast<const __half2 *>(&top), __half2half2(__ushort_as_half(0x80)));
     o[0][reg] = *reinterpret_cast<const uint32_t *>(&c);
-    o[1][reg] = __byte_perm(t, 0, 0x4240);
-    o[2][reg] = __byte_perm(ah, bh, 0x0400) & 0x00ff00ffu;  // a4 . b4 .
-    o[3][reg] = __byte_perm(q, 0, 0x4341);
+    o[1][reg] = t & 0x00ff00ffu;
+    o[2][reg] = __byte_perm(u, 0, 0x4341);
+    o[3][reg] = u & 0x00ff00ffu;
     o[4][reg] = __byte_perm(p, 0, 0x4341);
-    o[5][reg] = __byte_perm(p, 0, 0x4240);
-    o[6][reg] = __byte_perm(q, 0, 0x4240);
+    o[5][reg] = p & 0x00ff00ffu;
+    o[6][reg] = __byte_perm(q, 0, 0x4341);
+    o[7][reg] = q & 0x00ff00ffu;
 }
 
 // acc[i + j] += A_i X_j over 16 rows of staged digits (row k at xs + k
@@ -232,25 +263,26 @@ __device__ __forceinline__ void mma_orders(float (&acc)[NO][NT][4], const uint32
         for (int i = 0; i + j < NO; ++i)
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) mma_f16(acc[i + j][nt], a[i], b[2 * nt], b[2 * nt + 1]);
-        // orders NO (from j = 0) and NO + 1 (from j = 1) on the scale of the last sum
+        // orders NO (up to j = NO) and NO + 1 on the scale of the last sum
 #pragma unroll
         for (int m = 0; m < 2; ++m) {
-            if (m == 1 && j == 0) continue;
 #pragma unroll
             for (int k = 0; k < 2 * NT; ++k) {
                 const __half2 v = __hmul2(*reinterpret_cast<const __half2 *>(&b[k]), __float2half2_rn(0x1p-8f));
                 b[k] = *reinterpret_cast<const uint32_t *>(&v);
             }
+            if (j <= NO + m)
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) mma_f16(acc[NO - 1][nt], a[NO + m - j], b[2 * nt], b[2 * nt + 1]);
+                for (int nt = 0; nt < NT; ++nt) mma_f16(acc[NO - 1][nt], a[max(NO + m - j, 0)], b[2 * nt], b[2 * nt + 1]);
         }
     }
 }
 
 __device__ __forceinline__ int exp_of(uint32_t E20) { return (int)(E20 >> 20) - E_BIAS; }
+// 2^(E - 1011), subnormal too
 __device__ __forceinline__ float row_factor(uint32_t E20) {
-    const int E = exp_of(E20);
-    return E > F_EXP && E < E_NAN ? __uint_as_float((uint32_t)(E - F_EXP) << 23) : 0.0f;
+    const int e = exp_of(E20) - F_EXP;
+    return e > 0 ? __uint_as_float((uint32_t)min(e, 255) << 23) : e > -23 ? __uint_as_float(1u << (e + 22)) : 0.0f;
 }
 
 // (h, l) += x with the rounding of h kept in l
@@ -261,11 +293,13 @@ __device__ __forceinline__ void add_exact(float &h, float &l, float x) {
     h = t;
 }
 
-// (s, c) += 2^(E - 1011) sum_d acc_d 2^-8d for the rows g (E20 = e0) and g + 8
-// (e1) of a fragment; acc_d to zero.  The orders 0 to 3 are added without
-// loss (24 bits each, their rounding kept), the rest is below 2^-26 of order 0.
-template <int NT>
-__device__ __forceinline__ void flush(float (&acc)[NO][NT][4], uint32_t e0, uint32_t e1, float (&s)[NT][4], float (&c)[NT][4]) {
+// the running sums += 2^(E - 1011) sum_d acc_d 2^-8d for the rows g (E20 = e0) and g + 8
+// (e1) of a fragment; acc_d to zero.  The orders 0 to 4 are added without
+// loss (24 bits each, their rounding kept) and the pair is normalised, so that
+// a right-hand side whose sums begin in a lower order keeps its 48 bits.
+// add(nt, e, h, l): the running pair of sum (nt, e) += (h, l).
+template <int NT, class Add>
+__device__ __forceinline__ void flush(float (&acc)[NO][NT][4], uint32_t e0, uint32_t e1, const Add &add) {
     const float f0 = row_factor(e0), f1 = row_factor(e1);
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
@@ -273,20 +307,48 @@ __device__ __forceinline__ void flush(float (&acc)[NO][NT][4], uint32_t e0, uint
         for (int e = 0; e < 4; ++e) {
             const float f = e < 2 ? f0 : f1;
             float h = acc[0][nt][e];
-            float l = __fmul_rn(__fmaf_rn(acc[5][nt][e], 0x1p-8f, acc[4][nt][e]), 0x1p-32f);
+            float l = __fmul_rn(acc[5][nt][e], 0x1p-40f);
             add_exact(h, l, __fmul_rn(acc[1][nt][e], 0x1p-8f));
             add_exact(h, l, __fmul_rn(acc[2][nt][e], 0x1p-16f));
             add_exact(h, l, __fmul_rn(acc[3][nt][e], 0x1p-24f));
-            dadd(s[nt][e], c[nt][e], __fmul_rn(h, f), __fmul_rn(l, f));
+            add_exact(h, l, __fmul_rn(acc[4][nt][e], 0x1p-32f));
+            norm2(h, l, h, l);
+            add(nt, e, __fmul_rn(h, f), __fmul_rn(l, f));
 #pragma unroll
             for (int d = 0; d < NO; ++d) acc[d][nt][e] = 0.0f;
         }
+}
+
+// bits of the right-hand sides whose sum in a row or column of exponent E20 is not
+// sure to be good to 2^-46.5 of its own terms: all of them are small beside others'.
+// all: the states of the columns together.  A row that is zero or not finite has none.
+__device__ __forceinline__ uint32_t unsure(uint32_t E20, uint32_t all, uint32_t own) {
+    return E20 == E20_START || exp_of(E20) >= E_NAN ? 0u : all >> 16 & ~own;
+}
+
+// E = the new scale; own is kept while the raises (of this row in the bits from sh
+// on of raised) come to RAISE_OWN at most
+__device__ __forceinline__ void raise_own(uint32_t &E, uint32_t to, uint32_t &own, uint32_t &raised, int sh) {
+    uint32_t sum = (raised >> sh & 0xffffu) + ((to - E) >> 20);
+    if (sum > RAISE_OWN) own = sum = 0;
+    raised = (raised & ~(0xffffu << sh)) | sum << sh;
+    E = to;
+}
+
+// the cluster goes to the list of those to be formed again, once
+__device__ __forceinline__ void note_cluster(int32_t *todo, int64_t nl, int64_t cluster) {
+    if (atomicExch(todo + 1 + nl + cluster, 1) == 0) todo[1 + atomicAdd(todo, 1)] = (int32_t)cluster;
 }
 
 // largest of the four lanes of a quad (one fragment row)
 __device__ __forceinline__ uint32_t quad_max(uint32_t v) {
     v = max(v, __shfl_xor_sync(0xffffffffu, v, 1));
     return max(v, __shfl_xor_sync(0xffffffffu, v, 2));
+}
+
+__device__ __forceinline__ uint32_t quad_or(uint32_t v) {
+    v |= __shfl_xor_sync(0xffffffffu, v, 1);
+    return v | __shfl_xor_sync(0xffffffffu, v, 2);
 }
 
 // ---------------------------------------------------------------------------
@@ -308,7 +370,8 @@ __global__ void __launch_bounds__(32 * CW, 4) col_fx_kernel(int parts, const int
                                                          const int64_t *__restrict__ wp_colptr,
                                                          const double *__restrict__ wp, const __half *__restrict__ Xd,
                                                          const uint2 *__restrict__ Xe, float2 *__restrict__ P,
-                                                         const int32_t *__restrict__ order) {
+                                                         const int32_t *__restrict__ order, int64_t nl,
+                                                         int32_t *__restrict__ todo) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int q = blockIdx.x / parts, part = blockIdx.x - q * parts;
     const int64_t kap = order ? order[q] : q;
@@ -318,6 +381,8 @@ __global__ void __launch_bounds__(32 * CW, 4) col_fx_kernel(int parts, const int
     const int mp = (mc + KC - 1) / KC * KC;
     uint2 *se = reinterpret_cast<uint2 *>(smem);      // [mp]
     unsigned char *xs = smem + 8 * mp;              // [mp][XSTRIDE]
+    // the running sums, touched once in 128 rows, which would not fit the registers: [4 NT][threads]
+    float2 *ss = reinterpret_cast<float2 *>(xs + mp * XSTRIDE) + threadIdx.x;
     for (int e = threadIdx.x; e < mp * 2; e += 32 * CW) {
         const int j = e >> 1, p = NA * (e & 1);
 #pragma unroll
@@ -330,24 +395,33 @@ __global__ void __launch_bounds__(32 * CW, 4) col_fx_kernel(int parts, const int
     for (int j = threadIdx.x; j < mp; j += 32 * CW) se[j] = j < mc ? __ldg(Xe + c0 + j) : make_uint2(0, 0);
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-    unsigned int bad = 0;
-    for (int j = lane; j < mp; j += 32) bad |= se[j].y;
-    bad = __reduce_or_sync(0xffffffffu, bad);
+    unsigned int bad = 0, all = 0;
+    for (int j = lane; j < mp; j += 32) {
+        const unsigned int y = se[j].y;
+        all |= y;
+        bad |= y & ~(y >> 16);
+    }
+    bad = __reduce_or_sync(0xffffffffu, bad);  // in the lower half
+    all = __reduce_or_sync(0xffffffffu, all);
     const double *W = wp + wp_off[kap];
     for (int v0 = 16 * (part * CW + warp); v0 < Kw; v0 += 16 * CW * parts) {
         const int v = v0 + 2 * g;
         const bool ok = v < Kw;  // Kw is even
         const double *col = W + (ok ? v : 0) + (int64_t)(2 * t) * Kw;
-        float acc[NO][NT][4], s[NT][4], c[NT][4];
+        float acc[NO][NT][4];
+        auto add = [&](int nt, int e, float h, float l) {
+            float2 &v = ss[(4 * nt + e) * 32 * CW];
+            dadd(v.x, v.y, h, l);
+        };
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                s[nt][e] = c[nt][e] = 0.0f;
+                ss[(4 * nt + e) * 32 * CW] = make_float2(0.0f, 0.0f);
 #pragma unroll
                 for (int d = 0; d < NO; ++d) acc[d][nt][e] = 0.0f;
             }
-        uint32_t E0 = E20_START, E1 = E20_START;
+        uint32_t E0 = E20_START, E1 = E20_START, own0 = 0, own1 = 0;
         int held = 0;
 #pragma unroll 1
         for (int k0 = 0; k0 < mc; k0 += KC, col += (int64_t)KC * Kw) {
@@ -367,8 +441,10 @@ __global__ void __launch_bounds__(32 * CW, 4) col_fx_kernel(int parts, const int
             }
             const uint32_t n0 = raise_exp(quad_max(m0), E0), n1 = raise_exp(quad_max(m1), E1);
             if (__any_sync(0xffffffffu, n0 != E0 || n1 != E1) || held == FLUSH) {
-                if (held) flush<NT>(acc, E0, E1, s, c);
+                if (held) flush<NT>(acc, E0, E1, add);
                 held = 0;
+                if (n0 != E0) own0 = 0;
+                if (n1 != E1) own1 = 0;
                 E0 = n0;
                 E1 = n1;
             }
@@ -381,14 +457,16 @@ __global__ void __launch_bounds__(32 * CW, 4) col_fx_kernel(int parts, const int
                 for (int hf = 0; hf < 2; ++hf) {
                     const uint4 e = *reinterpret_cast<const uint4 *>(se + k0 + kk + 8 * hf + 2 * t);
                     const double2 x = w[kk / 4 + 2 * hf], y = w[kk / 4 + 2 * hf + 1];
-                    digit_pair(x.x, y.x, E0, e.x, e.z, a, 2 * hf);
-                    digit_pair(x.y, y.y, E1, e.x, e.z, a, 2 * hf + 1);
+                    digit_pair<COL_OWN>(x.x, y.x, E0, e, a, 2 * hf, own0);
+                    digit_pair<COL_OWN>(x.y, y.y, E1, e, a, 2 * hf + 1, own1);
                 }
                 mma_orders<NT>(acc, a, xs + (k0 + kk) * XSTRIDE);
             }
         }
-        flush<NT>(acc, E0, E1, s, c);
+        flush<NT>(acc, E0, E1, add);
         const int worst = (exp_of(E0) >= E_NAN ? 1 : 0) | (exp_of(E1) >= E_NAN ? 2 : 0);
+        if (__any_sync(0xffffffffu, (unsure(E0, all, quad_or(own0)) | unsure(E1, all, quad_or(own1))) != 0) && lane == 0)
+            note_cluster(todo, nl, kap);
         if (!ok) continue;
         const float nan = __uint_as_float(0x7fffffffu);
 #pragma unroll
@@ -397,7 +475,8 @@ __global__ void __launch_bounds__(32 * CW, 4) col_fx_kernel(int parts, const int
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) {
                 const int r = 8 * nt + 2 * t;
-                float4 w = make_float4(s[nt][2 * h], c[nt][2 * h], s[nt][2 * h + 1], c[nt][2 * h + 1]);
+                const float2 s0 = ss[(4 * nt + 2 * h) * 32 * CW], s1 = ss[(4 * nt + 2 * h + 1) * 32 * CW];
+                float4 w = make_float4(s0.x, s0.y, s1.x, s1.y);
                 if ((worst >> h & 1) || (bad >> r & 1)) w.x = nan;
                 if ((worst >> h & 1) || (bad >> (r + 1) & 1)) w.z = nan;
                 o[r / 2] = w;
@@ -424,6 +503,49 @@ __device__ __forceinline__ long long scaled_int(float x, int k) {
     return (int)b < 0 ? -v : v;
 }
 
+// the block of entry e = 32 ch + lane of t (whole warps; any block where e is past the end)
+__device__ __forceinline__ int64_t block_of(int64_t ch, int64_t e, int64_t na, const int32_t *__restrict__ b0tab,
+                                            const int64_t *__restrict__ t_off) {
+    const unsigned full = 0xffffffffu;
+    const int64_t b0 = b0tab[ch];
+    const int64_t to = t_off[min(b0 + (threadIdx.x & 31), na)];  // t_off has na + 1 entries
+    int j = 0;
+#pragma unroll
+    for (int st = 16; st > 0; st >>= 1) {
+        const int64_t tj = __shfl_sync(full, to, j + st);
+        if (tj <= e) j += st;
+    }
+    const int64_t to31 = __shfl_sync(full, to, 31);
+    if (to31 > e || b0 + 31 >= na) return b0 + j;
+    int64_t lo = b0 + 31, hi = na;
+    while (hi - lo > 1) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (t_off[mid] <= e) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// entry l of t_b for 8 NT right-hand sides, as normalised pairs
+template <int NT>
+__device__ __forceinline__ void sum_partials(int64_t b, int64_t l, const int64_t *__restrict__ bcolptr,
+                                             const int64_t *__restrict__ pofs, const float2 *__restrict__ P,
+                                             float (&s)[8 * NT], float (&c)[8 * NT]) {
+#pragma unroll
+    for (int r = 0; r < 8 * NT; ++r) s[r] = c[r] = 0.0f;
+    for (int64_t q = bcolptr[b]; q < bcolptr[b + 1]; ++q) {
+        const float4 *pp = reinterpret_cast<const float4 *>(P + (pofs[q] + l) * MR);
+#pragma unroll
+        for (int k = 0; k < 4 * NT; ++k) {
+            const float4 v = __ldg(pp + k);
+            dadd(s[2 * k], c[2 * k], v.x, v.y);
+            dadd(s[2 * k + 1], c[2 * k + 1], v.z, v.w);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < 8 * NT; ++r) norm2(s[r], c[r], s[r], c[r]);
+}
+
 template <int NT>
 __global__ void __launch_bounds__(256) tsum_fx_kernel(int64_t na, int64_t nt, const int32_t *__restrict__ b0tab,
                                                       const int64_t *__restrict__ t_off,
@@ -431,67 +553,39 @@ __global__ void __launch_bounds__(256) tsum_fx_kernel(int64_t na, int64_t nt, co
                                                       const int64_t *__restrict__ pofs, const float2 *__restrict__ P,
                                                       __half *__restrict__ Td, uint2 *__restrict__ Te) {
     constexpr int NR = 8 * NT;
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int64_t nchunk = (nt + 31) / 32;
     for (int64_t ch = w0; ch < nchunk; ch += nw) {
-        const int64_t b0 = b0tab[ch];
-        const int64_t bl = min(b0 + lane, na);
-        const int64_t to = t_off[bl];  // t_off has na + 1 entries
-        const int64_t e = ch * 32 + lane;
-        int j = 0;
-#pragma unroll
-        for (int st = 16; st > 0; st >>= 1) {
-            const int64_t tj = __shfl_sync(full, to, j + st);
-            if (tj <= e) j += st;
-        }
-        const int64_t to31 = __shfl_sync(full, to, 31);
+        const int64_t e = ch * 32 + (threadIdx.x & 31);
+        const int64_t b = block_of(ch, e, na, b0tab, t_off);
         if (e >= nt) continue;
-        int64_t b = b0 + j;
-        if (to31 <= e && b0 + 31 < na) {
-            int64_t lo = b0 + 31, hi = na;
-            while (hi - lo > 1) {
-                const int64_t mid = (lo + hi) >> 1;
-                if (t_off[mid] <= e) lo = mid;
-                else hi = mid;
-            }
-            b = lo;
-        }
         const int64_t l = e - t_off[b];
         float s[NR], c[NR];
-#pragma unroll
-        for (int r = 0; r < NR; ++r) s[r] = c[r] = 0.0f;
-        for (int64_t q = bcolptr[b]; q < bcolptr[b + 1]; ++q) {
-            const float4 *pp = reinterpret_cast<const float4 *>(P + (pofs[q] + l) * MR);
-#pragma unroll
-            for (int k = 0; k < NR / 2; ++k) {
-                const float4 v = __ldg(pp + k);
-                dadd(s[2 * k], c[2 * k], v.x, v.y);
-                dadd(s[2 * k + 1], c[2 * k + 1], v.z, v.w);
-            }
-        }
-        // (s, c) normalised; the exponent of the largest
+        sum_partials<NT>(b, l, bcolptr, pofs, P, s, c);
+        // the exponent of the largest, and the states (as of x: digits_x_kernel)
         int ex = E_ZERO;
         unsigned int bad = 0;
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
-            float h, lo;
-            norm2(s[r], c[r], h, lo);
-            s[r] = h;
-            c[r] = lo;
-            const uint32_t hb = __float_as_uint(h) & 0x7fffffffu;
+            const uint32_t hb = __float_as_uint(s[r]) & 0x7fffffffu;
             if (hb >= 0x7f800000u) bad |= 1u << r;
-            else if (hb) ex = max(ex, max((int)(hb >> 23), 1) - 126);  // |h| < 2^ex, subnormal h too
+            else if (hb) ex = max(ex, max((int)(hb >> 23), 1) - 126);  // |s| < 2^ex, subnormal s too
         }
-        Te[e] = make_uint2((uint32_t)(ex + E_BIAS) << 20, bad);
+        unsigned int state = bad;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const uint32_t hb = __float_as_uint(s[r]) & 0x7fffffffu;
+            if (hb == 0u || hb >= 0x7f800000u) continue;
+            state |= (max((int)(hb >> 23), 1) - 126 + X_OWN >= ex ? 0x10001u : 0x10000u) << r;
+        }
+        Te[e] = make_uint2((uint32_t)(ex + E_BIAS) << 20, state);
         unsigned long long u[NR];
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
             long long q = 0;
             if (ex > E_ZERO && !(bad >> r & 1)) q = scaled_int(s[r], QB - ex) + scaled_int(c[r], QB - ex);
-            u[r] = (unsigned long long)(q + DIGIT_BIAS);
+            u[r] = (unsigned long long)q + DIGIT_BIAS;
         }
         uint4 *o = reinterpret_cast<uint4 *>(Td + e * DIG);
 #pragma unroll
@@ -520,11 +614,11 @@ __global__ void __launch_bounds__(256) tsum_fx_kernel(int64_t na, int64_t nt, co
 // filled by cp.async: the FP64 rows of the chunk, and the digits and exponents
 // of the gathered rows of x or t.  A warp takes the largest term of each of its
 // rows in the chunk, forms the digits of its entries (each entry by one lane)
-// and multiplies.  Per 16 x 16 entries: 68 products of 16 x 8 x 16 (~150 cycles of an
-// SM), ~22 integer operations per entry (~80 cycles of the ALU pipe), 2 KB from
+// and multiplies.  Per 16 x 16 entries: 72 products of 16 x 8 x 16 (~160 cycles of an
+// SM), ~26 integer operations per entry (~95 cycles of the ALU pipe), 2 KB from
 // HBM (~95 cycles).
 // ---------------------------------------------------------------------------
-constexpr int AST = KC * 8 + 64;          // bytes per staged panel row: row pairs fill the banks
+constexpr int AST = KC * 8;               // bytes per staged panel row; odd rows have their 64-byte halves swapped (banks)
 template <int MT> struct RowCfg {
     static constexpr int THREADS = 32 * MT;
     static constexpr int A_BYTES = 16 * MT * AST;
@@ -541,7 +635,8 @@ __global__ void __launch_bounds__(32 * MT, RowCfg<MT>::CTAS) row_fx_kernel(
     const int64_t *__restrict__ up_colptr, const int32_t *__restrict__ tidx, const double *__restrict__ up,
     const __half *__restrict__ Xd, const uint2 *__restrict__ Xe, const __half *__restrict__ Td,
     const uint2 *__restrict__ Te, const unsigned int *__restrict__ sc, double *__restrict__ Y,
-    const int4 *__restrict__ items, float2 *__restrict__ Ypart, int prow) {
+    const int4 *__restrict__ items, float2 *__restrict__ Ypart, uint2 *__restrict__ part_state, int prow,
+    int64_t nl, int32_t *__restrict__ todo) {
     using C = RowCfg<MT>;
     extern __shared__ __align__(16) unsigned char smem[];
     int32_t *s_idx = reinterpret_cast<int32_t *>(smem + 2 * C::STAGE);  // [2][KC]
@@ -575,7 +670,7 @@ __global__ void __launch_bounds__(32 * MT, RowCfg<MT>::CTAS) row_fx_kernel(
         const double *P = u ? Pu : Pd;
         const bool in = k0 + acol < K;
         const double *src = P + (int64_t)arow * K + k0 + acol;
-        unsigned char *dst = st + arow * AST + acol * 8;
+        unsigned char *dst = st + arow * AST + ((acol * 8) ^ ((arow & 1) << 6));  // the rows below have the same parity
 #pragma unroll
         for (int v = 0; v < 8; ++v, src += (C::THREADS / 16) * (int64_t)K) {
             const bool ok = in && arow + (C::THREADS / 16) * v < rows;
@@ -610,8 +705,9 @@ __global__ void __launch_bounds__(32 * MT, RowCfg<MT>::CTAS) row_fx_kernel(
 #pragma unroll
             for (int d = 0; d < NO; ++d) acc[d][nt][e] = 0.0f;
         }
-    unsigned int bad = 0;
-    uint32_t E0 = E20_START, E1 = E20_START;
+    auto add = [&](int nt, int e, float h, float l) { dadd(s[nt][e], c[nt][e], h, l); };
+    unsigned int bad = 0, all = 0;
+    uint32_t E0 = E20_START, E1 = E20_START, own0 = 0, own1 = 0, raised = 0;
     int held = 0;
     load_idx(it.y);
     load_idx(it.y + 1);
@@ -623,25 +719,29 @@ __global__ void __launch_bounds__(32 * MT, RowCfg<MT>::CTAS) row_fx_kernel(
         __syncthreads();  // chunk ch has landed for every thread; every thread is done with chunk ch - 1
         if (ch + 1 < cend) issue(ch + 1);
         const unsigned char *st = smem + (ch & 1) * C::STAGE;
+        // columns 8 i + 2 t, + 1 of a row: the i-th 64 bytes, i's lowest bit flipped in odd rows
         const double *a0 = reinterpret_cast<const double *>(st + (16 * warp + g) * AST) + 2 * t;
-        const double *a1 = reinterpret_cast<const double *>(st + (16 * warp + g + 8) * AST) + 2 * t;
+        const double *a1 = a0 + 8 * KC;
+        const int flip = 8 * (g & 1);
         const unsigned char *sb = st + C::A_BYTES;
         const uint2 *se = reinterpret_cast<const uint2 *>(sb + KC * XSTRIDE) + 2 * t;
         uint32_t m0 = 0, m1 = 0;
 #pragma unroll
         for (int k = 0; k < KC; k += 8) {
-            const double2 w0 = *reinterpret_cast<const double2 *>(a0 + k), w1 = *reinterpret_cast<const double2 *>(a1 + k);
+            const double2 w0 = *reinterpret_cast<const double2 *>(a0 + (k ^ flip));
+            const double2 w1 = *reinterpret_cast<const double2 *>(a1 + (k ^ flip));
             const uint4 e = *reinterpret_cast<const uint4 *>(se + k);
-            bad |= e.y | e.w;
+            all |= e.y | e.w;
+            bad |= (e.y & ~(e.y >> 16)) | (e.w & ~(e.w >> 16));
             m0 = max(m0, max(term_exp(w0.x, e.x), term_exp(w0.y, e.z)));
             m1 = max(m1, max(term_exp(w1.x, e.x), term_exp(w1.y, e.z)));
         }
         const uint32_t n0 = raise_exp(quad_max(m0), E0), n1 = raise_exp(quad_max(m1), E1);
         if (__any_sync(0xffffffffu, n0 != E0 || n1 != E1) || held == FLUSH) {
-            if (held) flush<NT>(acc, E0, E1, s, c);
+            if (held) flush<NT>(acc, E0, E1, add);
             held = 0;
-            E0 = n0;
-            E1 = n1;
+            raise_own(E0, n0, own0, raised, 0);
+            raise_own(E1, n1, own1, raised, 16);
         }
         ++held;
 #pragma unroll
@@ -649,20 +749,32 @@ __global__ void __launch_bounds__(32 * MT, RowCfg<MT>::CTAS) row_fx_kernel(
             uint32_t a[NA][4];
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {
-                const double2 w0 = *reinterpret_cast<const double2 *>(a0 + k + 8 * hf);
-                const double2 w1 = *reinterpret_cast<const double2 *>(a1 + k + 8 * hf);
+                const double2 w0 = *reinterpret_cast<const double2 *>(a0 + ((k + 8 * hf) ^ flip));
+                const double2 w1 = *reinterpret_cast<const double2 *>(a1 + ((k + 8 * hf) ^ flip));
                 const uint4 e = *reinterpret_cast<const uint4 *>(se + k + 8 * hf);
-                digit_pair(w0.x, w0.y, E0, e.x, e.z, a, 2 * hf);
-                digit_pair(w1.x, w1.y, E1, e.x, e.z, a, 2 * hf + 1);
+                digit_pair<ROW_OWN>(w0.x, w0.y, E0, e, a, 2 * hf, own0);
+                digit_pair<ROW_OWN>(w1.x, w1.y, E1, e, a, 2 * hf + 1, own1);
             }
             mma_orders<NT>(acc, a, sb + k * XSTRIDE);
         }
         // the indices of chunk ch + 2 (chunk ch's were read by issue(ch), an iteration ago)
         load_idx(ch + 2);
     }
-    flush<NT>(acc, E0, E1, s, c);
+    flush<NT>(acc, E0, E1, add);
     const int worst = (exp_of(E0) >= E_NAN ? 1 : 0) | (exp_of(E1) >= E_NAN ? 2 : 0);
-    bad = __reduce_or_sync(0xffffffffu, bad);
+    bad = __reduce_or_sync(0xffffffffu, bad);  // in the lower half
+    all = __reduce_or_sync(0xffffffffu, all);
+    own0 = quad_or(own0);
+    own1 = quad_or(own1);
+    if (it.w >= 0) {  // a part of the row: row_reduce_kernel looks at all of them
+        if (t == 0) {
+            uint2 *o = part_state + (int64_t)it.w * prow + part * 16 * MT + 16 * warp + g;
+            if (16 * warp + g < rows) o[0] = make_uint2(E0 | (raised & 0xffffu), (all & 0xffff0000u) | (own0 & 0xffffu));
+            if (16 * warp + g + 8 < rows) o[8] = make_uint2(E1 | raised >> 16, (all & 0xffff0000u) | (own1 & 0xffffu));
+        }
+    } else if (__any_sync(0xffffffffu, (unsure(E0, all, own0) | unsure(E1, all, own1)) != 0) && lane == 0) {
+        note_cluster(todo, nl, rho);
+    }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int row = 16 * warp + g + 8 * h;
@@ -684,11 +796,14 @@ __global__ void __launch_bounds__(32 * MT, RowCfg<MT>::CTAS) row_fx_kernel(
 }
 
 // rows of the clusters whose panels were split: Y = the sum of the partials
-// in slot order (red: cluster, first slot, slots)
+// in slot order (red: cluster, first slot, slots).  A part's own terms speak for the
+// row where its scale is within RAISE_OWN of the row's, raises included.
 template <int NT>
 __global__ void __launch_bounds__(256) row_reduce_kernel(const int4 *__restrict__ red, const int32_t *__restrict__ leaf_begin,
                                                          const float2 *__restrict__ Ypart, int prow,
-                                                         const unsigned int *__restrict__ sc, double *__restrict__ Y) {
+                                                         const uint2 *__restrict__ part_state,
+                                                         const unsigned int *__restrict__ sc, double *__restrict__ Y,
+                                                         int64_t nl, int32_t *__restrict__ todo) {
     const int4 rd = red[blockIdx.x];
     const int32_t r0 = leaf_begin[rd.x], mr = leaf_begin[rd.x + 1] - r0;
     for (int e = threadIdx.x; e < mr * 8 * NT; e += 256) {
@@ -700,6 +815,196 @@ __global__ void __launch_bounds__(256) row_reduce_kernel(const int4 *__restrict_
             dadd(s, c, v.x, v.y);
         }
         Y[(int64_t)(r0 + row) * MR + r] = scalbn((double)s + (double)c, scale_of(sc[r]));
+    }
+    for (int row = threadIdx.x; row < mr; row += 256) {
+        const uint2 *p = part_state + (int64_t)rd.y * prow + row;
+        uint32_t E = E20_START, all = 0, own = 0;
+        for (int k = 0; k < rd.z; ++k) E = max(E, p[(int64_t)k * prow].x & 0xfff00000u);
+        for (int k = 0; k < rd.z; ++k) {
+            const uint2 v = p[(int64_t)k * prow];
+            all |= v.y;
+            if ((E >> 20) - (v.x >> 20) + (v.x & 0xffffu) <= RAISE_OWN) own |= v.y;
+        }
+        if (unsure(E, all, own)) note_cluster(todo, nl, rd.x);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The clusters where right-hand sides of unlike sizes meet (unsure), formed again
+// with pairs of floats: every entry and x_r is split by itself, w = h + l to
+// 2^-47 |w|, and each term is added with an error-free product and sum (the
+// compensated dot product of Ogita, Rump and Oishi, "Accurate sum and dot product",
+// SIAM J. Sci. Comput. 2005, Algorithm 5.3), so no right-hand side sees another.
+// Few or no clusters as a rule (of random vectors a few column clusters of 1,000 and a
+// row cluster of some 10,000): the lists (todo: length, clusters, marks) are walked by a
+// fixed number of CTAs, which end at once where they are empty (3 us a kernel).  Bound
+// by the FP32 pipe where all clusters are listed, by latency where few are.
+// ---------------------------------------------------------------------------
+constexpr int PAIR_CTAS = 8;  // per SM
+
+// h: w truncated to 24 bits, l: the rest, from the bits of w where both are normal
+// floats; (0, 0) below the floats, NaN above them
+__device__ __forceinline__ void split(double w, float &h, float &l) {
+    const uint32_t hi32 = (uint32_t)__double2hiint(w), lo32 = (uint32_t)__double2loint(w);
+    const uint32_t mag = hi32 & 0x7fffffffu, sgn = hi32 & 0x80000000u;
+    if (mag >= 0x3b500000u && mag < 0x47f00000u) {  // biased exponent in [949, 1151)
+        h = __uint_as_float(sgn | ((mag - 0x38000000u) << 3) | (lo32 >> 29));
+        const float sc = __uint_as_float((uint32_t)((int)(mag >> 20) - 948) << 23);  // 2^(exponent - 52)
+        l = __uint_as_float(__float_as_uint(__fmul_rn(__uint2float_rn(lo32 & 0x1fffffffu), sc)) | sgn);
+    } else if (mag >= 0x47f00000u) {
+        h = l = __uint_as_float(0x7fffffffu);
+    } else {
+        h = __double2float_rz(w);
+        l = __double2float_rn(w - (double)h);
+    }
+}
+
+// (s, c) += (ah + al)(xh + xl)
+__device__ __forceinline__ void dfma(float &s, float &c, float ah, float al, float xh, float xl) {
+    const float p = __fmul_rn(ah, xh);
+    const float e = __fmaf_rn(ah, xh, -p);
+    const float t = __fadd_rn(s, p);
+    const float bp = __fsub_rn(t, s);
+    const float sg = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(p, bp));
+    s = t;
+    c = __fadd_rn(c, __fmaf_rn(al, xh, __fmaf_rn(ah, xl, __fadd_rn(e, sg))));
+}
+
+// (s, c)_r += w z_r for the pairs of z at z[r], z[MR + r]
+template <int NT>
+__device__ __forceinline__ void pair_step(double w, const float4 *z, float (&s)[8 * NT], float (&c)[8 * NT]) {
+    float ah, al;
+    split(w, ah, al);
+#pragma unroll
+    for (int q = 0; q < 2 * NT; ++q) {
+        const float4 xh = z[q], xl = z[MR / 4 + q];
+        dfma(s[4 * q], c[4 * q], ah, al, xh.x, xl.x);
+        dfma(s[4 * q + 1], c[4 * q + 1], ah, al, xh.y, xl.y);
+        dfma(s[4 * q + 2], c[4 * q + 2], ah, al, xh.z, xl.z);
+        dfma(s[4 * q + 3], c[4 * q + 3], ah, al, xh.w, xl.w);
+    }
+}
+
+// x_r at position m on its own scale, as a pair
+__device__ __forceinline__ void x_pair(const double *__restrict__ x, int64_t n, int nr, const int32_t *__restrict__ perm,
+                                       const unsigned int *__restrict__ sc, int64_t m, int r, float &h, float &l) {
+    const double v = r < nr ? scalbn(x[(int64_t)r * n + (perm ? perm[m] : m)], -scale_of(sc[r])) : 0.0;
+    h = __double2float_rn(v);
+    l = __double2float_rn(v - (double)h);
+}
+
+// the partials of the listed column clusters; one thread per panel column
+constexpr int CP_THREADS = 128;
+template <int NT>
+__global__ void __launch_bounds__(CP_THREADS) col_pairs_kernel(
+    int parts, const int32_t *__restrict__ todo, const int32_t *__restrict__ leaf_begin,
+    const int64_t *__restrict__ wp_off, const int32_t *__restrict__ wp_K, const int64_t *__restrict__ wp_colptr,
+    const double *__restrict__ wp, const double *__restrict__ x, int64_t n, int nr, const int32_t *__restrict__ perm,
+    const unsigned int *__restrict__ sc, float2 *__restrict__ P) {
+    __shared__ float4 sx[MAX_LEAF * MR / 2];
+    float *sf = reinterpret_cast<float *>(sx);
+    const int64_t count = (int64_t)todo[0] * parts;
+    for (int64_t q = blockIdx.x; q < count; q += gridDim.x) {
+        const int64_t kap = todo[1 + q / parts];
+        const int Kw = wp_K[kap], v0 = (int)(q % parts) * CP_THREADS;
+        if (v0 >= Kw) continue;
+        const int32_t c0 = leaf_begin[kap], mc = leaf_begin[kap + 1] - c0;
+        __syncthreads();  // the last cluster's x has been read
+        for (int e = threadIdx.x; e < mc * MR; e += CP_THREADS) {
+            const int j = e / MR, r = e % MR;
+            x_pair(x, n, nr, perm, sc, c0 + j, r, sf[2 * MR * j + r], sf[2 * MR * j + MR + r]);
+        }
+        __syncthreads();
+        const int v = v0 + threadIdx.x;
+        if (v >= Kw) continue;
+        float s[8 * NT], c[8 * NT];
+#pragma unroll
+        for (int r = 0; r < 8 * NT; ++r) s[r] = c[r] = 0.0f;
+        const double *col = wp + wp_off[kap] + v;
+#pragma unroll 4
+        for (int j = 0; j < mc; ++j) pair_step<NT>(__ldg(col + (int64_t)j * Kw), sx + j * MR / 2, s, c);
+        float4 *o = reinterpret_cast<float4 *>(P + (wp_colptr[kap] + v) * MR);
+#pragma unroll
+        for (int r = 0; r < 8 * NT; r += 2) o[r / 2] = make_float4(s[r], c[r], s[r + 1], c[r + 1]);
+    }
+}
+
+// where a row cluster is listed: x and t as pairs ([row][hi 16, lo 16]), in the place of their digits
+template <int NT>
+__global__ void __launch_bounds__(256) pairs_kernel(const int32_t *__restrict__ todo, int64_t na, int64_t nt,
+                                                    const int32_t *__restrict__ b0tab, const int64_t *__restrict__ t_off,
+                                                    const int64_t *__restrict__ bcolptr, const int64_t *__restrict__ pofs,
+                                                    const float2 *__restrict__ P, const double *__restrict__ x, int64_t n,
+                                                    int nr, const int32_t *__restrict__ perm,
+                                                    const unsigned int *__restrict__ sc, float *__restrict__ Xp,
+                                                    float *__restrict__ Tp) {
+    if (todo[0] == 0) return;
+    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t e = t0; e < n * MR; e += nth)
+        x_pair(x, n, nr, perm, sc, e / MR, (int)(e % MR), Xp[e / MR * 2 * MR + e % MR], Xp[e / MR * 2 * MR + MR + e % MR]);
+    for (int64_t ch = t0 >> 5; ch < (nt + 31) / 32; ch += nth >> 5) {
+        const int64_t e = ch * 32 + (threadIdx.x & 31);
+        const int64_t b = block_of(ch, e, na, b0tab, t_off);
+        if (e >= nt) continue;
+        float s[8 * NT], c[8 * NT];
+        sum_partials<NT>(b, e - t_off[b], bcolptr, pofs, P, s, c);
+        float4 *o = reinterpret_cast<float4 *>(Tp + e * 2 * MR);
+#pragma unroll
+        for (int k = 0; k < 2 * NT; ++k) {
+            o[k] = make_float4(s[4 * k], s[4 * k + 1], s[4 * k + 2], s[4 * k + 3]);
+            o[MR / 4 + k] = make_float4(c[4 * k], c[4 * k + 1], c[4 * k + 2], c[4 * k + 3]);
+        }
+    }
+}
+
+// the rows of the listed row clusters, eight per CTA and one per warp; the gathered
+// pairs of 64 columns at a time in shared memory
+constexpr int RP_ROWS = 8, RP_COLS = 64, RP_STRIDE = MR / 2 + 1;  // float4 per column: eight lanes hit different banks
+template <int NT>
+__global__ void __launch_bounds__(32 * RP_ROWS) row_pairs_kernel(
+    int parts, const int32_t *__restrict__ todo, const int32_t *__restrict__ leaf_begin,
+    const int64_t *__restrict__ rho_off, const int32_t *__restrict__ rho_K, const int64_t *__restrict__ rho_colptr,
+    const int32_t *__restrict__ colidx, const double *__restrict__ dense, const int64_t *__restrict__ up_off,
+    const int32_t *__restrict__ up_K, const int64_t *__restrict__ up_colptr, const int32_t *__restrict__ tidx,
+    const double *__restrict__ up, const float4 *__restrict__ Xp, const float4 *__restrict__ Tp,
+    const unsigned int *__restrict__ sc, double *__restrict__ Y) {
+    __shared__ float4 sz[RP_COLS * RP_STRIDE];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t count = (int64_t)todo[0] * parts;
+    for (int64_t q = blockIdx.x; q < count; q += gridDim.x) {
+        const int64_t rho = todo[1 + q / parts];
+        const int32_t r0 = leaf_begin[rho], mr = leaf_begin[rho + 1] - r0;
+        const int row = (int)(q % parts) * RP_ROWS + warp;
+        if (row - warp >= mr) continue;
+        float s[8 * NT], c[8 * NT];
+#pragma unroll
+        for (int r = 0; r < 8 * NT; ++r) s[r] = c[r] = 0.0f;
+#pragma unroll 1
+        for (int u = 0; u < 2; ++u) {  // the near field, then the U panel
+            const int K = u ? up_K[rho] : rho_K[rho];
+            const int32_t *idx = u ? tidx + up_colptr[rho] : colidx + rho_colptr[rho];
+            const double *p = (u ? up + up_off[rho] : dense + rho_off[rho]) + (int64_t)min(row, mr - 1) * K;
+            const float4 *z = u ? Tp : Xp;
+            for (int k0 = 0; k0 < K; k0 += RP_COLS) {
+                const int kc = min(RP_COLS, K - k0);
+                __syncthreads();
+                for (int e = threadIdx.x; e < kc * MR / 2; e += 32 * RP_ROWS)
+                    sz[e / (MR / 2) * RP_STRIDE + e % (MR / 2)] =
+                        __ldg(z + (int64_t)idx[k0 + e / (MR / 2)] * (MR / 2) + e % (MR / 2));
+                __syncthreads();
+                for (int k = lane; k < kc; k += 32) pair_step<NT>(__ldg(p + k0 + k), sz + k * RP_STRIDE, s, c);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 8 * NT; ++r) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float s2 = __shfl_xor_sync(0xffffffffu, s[r], o), c2 = __shfl_xor_sync(0xffffffffu, c[r], o);
+                dadd(s[r], c[r], s2, c2);
+            }
+            if (lane == r && row < mr)
+                Y[(int64_t)(r0 + row) * MR + r] = scalbn((double)s[r] + (double)c[r], scale_of(sc[r]));
+        }
     }
 }
 
@@ -725,16 +1030,20 @@ static unsigned grid_for(int64_t n) {
 struct Work {
     __half *Xd, *Td;
     float2 *P, *Ypart;
-    uint2 *Xe, *Te;
+    uint2 *Xe, *Te, *part_state;
     unsigned int *sc;
+    int32_t *todo_c, *todo_r;  // column and row clusters to be formed again: length, clusters [nl], marks [nl]
 };
+static int64_t todo_ints(int64_t nl) { return (1 + 2 * nl + 3) / 4 * 4; }
 
 template <int NT>
 static void block_product(const hm_matrix *A, const double *x, int nr, const int32_t *perm, double *Y, const Work &w,
                           cudaStream_t s) {
     const hm_tree *tr = A->tree;
     const int64_t n = tr->n, nl = tr->n_leaf;
-    HM_CUDA_CHECK(cudaMemsetAsync(w.sc, 0, sizeof(unsigned int) * MR, s));
+    // (the lists follow the scales)
+    HM_CUDA_CHECK(cudaMemsetAsync(w.sc, 0, sizeof(unsigned int) * MR + sizeof(int32_t) * 2 * todo_ints(nl), s));
+    const unsigned pair_grid = (unsigned)(PAIR_CTAS * num_sms());
     const dim3 gs((unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, 256)), (unsigned)nr);
     scale_x_kernel<<<gs, 256, 0, s>>>(x, n, w.sc);
     HM_LAUNCH_CHECK();
@@ -743,13 +1052,19 @@ static void block_product(const hm_matrix *A, const double *x, int nr, const int
     const int32_t *ord = A->mv_order.as<int32_t>();
     if (tr->n_adm > 0) {
         {
-            const int smem = (tr->max_leaf + KC - 1) / KC * KC * (XSTRIDE + 8);
+            const int smem = (tr->max_leaf + KC - 1) / KC * KC * (XSTRIDE + 8) + 4 * NT * 32 * CW * (int)sizeof(float2);
             HM_CUDA_CHECK(cudaFuncSetAttribute(col_fx_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
             const int parts = ((A->wp_kmax + 16 * CW * 4 - 1) / (16 * CW * 4)) | 1;  // odd: see col_kernel
             Trace trace("col_fx_kernel", s);
             col_fx_kernel<NT><<<(unsigned)(nl * parts), 32 * CW, smem, s>>>(
                 parts, tr->leaf_begin.as<int32_t>(), A->wp_off.as<int64_t>(), A->wp_K.as<int32_t>(),
-                A->wp_colptr.as<int64_t>(), A->wp.as<double>(), w.Xd, w.Xe, w.P, ord ? ord + nl : nullptr);
+                A->wp_colptr.as<int64_t>(), A->wp.as<double>(), w.Xd, w.Xe, w.P, ord ? ord + nl : nullptr, nl,
+                w.todo_c);
+            HM_LAUNCH_CHECK();
+            col_pairs_kernel<NT><<<pair_grid, CP_THREADS, 0, s>>>(
+                (A->wp_kmax + CP_THREADS - 1) / CP_THREADS, w.todo_c, tr->leaf_begin.as<int32_t>(),
+                A->wp_off.as<int64_t>(), A->wp_K.as<int32_t>(), A->wp_colptr.as<int64_t>(), A->wp.as<double>(), x, n, nr,
+                perm, w.sc, w.P);
             HM_LAUNCH_CHECK();
         }
         Trace trace("tsum_fx_kernel", s);
@@ -767,7 +1082,8 @@ static void block_product(const hm_matrix *A, const double *x, int nr, const int
             parts, tr->leaf_begin.as<int32_t>(), tr->rho_off.as<int64_t>(), tr->rho_K.as<int32_t>(),
             tr->rho_colptr.as<int64_t>(), tr->colidx.as<int32_t>(), A->dense.as<double>(), A->up_off.as<int64_t>(),
             A->up_K.as<int32_t>(), A->up_colptr.as<int64_t>(), A->tidx.as<int32_t>(), A->up.as<double>(), w.Xd, w.Xe,
-            w.Td, w.Te, w.sc, Y, A->fx_items.as<int4>(), w.Ypart, prow);
+            w.Td, w.Te, w.sc, Y, A->fx_items.as<int4>(), w.Ypart,
+            w.part_state, prow, nl, w.todo_r);
         HM_LAUNCH_CHECK();
     };
     switch (mt) {
@@ -779,9 +1095,22 @@ static void block_product(const hm_matrix *A, const double *x, int nr, const int
     }
     if (A->fx_nred > 0) {
         row_reduce_kernel<NT><<<(unsigned)A->fx_nred, 256, 0, s>>>(A->fx_red.as<int4>(), tr->leaf_begin.as<int32_t>(),
-                                                                   w.Ypart, prow, w.sc, Y);
+                                                                   w.Ypart, prow, w.part_state, w.sc, Y, nl, w.todo_r);
         HM_LAUNCH_CHECK();
     }
+    float *Xp = reinterpret_cast<float *>(w.Xd), *Tp = reinterpret_cast<float *>(w.Td);
+    static_assert(DIG * sizeof(__half) >= 2 * MR * sizeof(float), "pairs in the place of digits");
+    pairs_kernel<NT><<<pair_grid, 256, 0, s>>>(w.todo_r, tr->n_adm, tr->n_adm > 0 ? A->total_rank : 0,
+                                               A->tsum_b0.as<int32_t>(), A->t_off.as<int64_t>(),
+                                               tr->lr_bcolptr.as<int64_t>(), A->pofs.as<int64_t>(), w.P, x, n, nr, perm,
+                                               w.sc, Xp, Tp);
+    HM_LAUNCH_CHECK();
+    row_pairs_kernel<NT><<<pair_grid, 32 * RP_ROWS, 0, s>>>(
+        (tr->max_leaf + RP_ROWS - 1) / RP_ROWS, w.todo_r, tr->leaf_begin.as<int32_t>(), tr->rho_off.as<int64_t>(),
+        tr->rho_K.as<int32_t>(), tr->rho_colptr.as<int64_t>(), tr->colidx.as<int32_t>(), A->dense.as<double>(),
+        A->up_off.as<int64_t>(), A->up_K.as<int32_t>(), A->up_colptr.as<int64_t>(), A->tidx.as<int32_t>(),
+        A->up.as<double>(), reinterpret_cast<float4 *>(Xp), reinterpret_cast<float4 *>(Tp), w.sc, Y);
+    HM_LAUNCH_CHECK();
 }
 
 }  // namespace fx
@@ -822,13 +1151,15 @@ void build_fx_items(hm_matrix *A, const std::vector<int32_t> &begin, const std::
 }
 
 // floats of the working arrays of one 16-right-hand-side pass: digits of x
-// and t (56 each per row), partials of t (32 each), exponents of x and t (2
-// each, a multiple of 4 in all), scales (16), partials of split rows (32 per
-// row of a slot), Y (16 doubles per row)
+// and t (64 each per row), partials of t (32 each), exponents of x and t (2
+// each, a multiple of 4 in all), scales (16) and the two lists of clusters,
+// partials and states of split rows (32 and 2 per row of a slot, a multiple of 16
+// rows), Y (16 doubles per row)
 int64_t df_work_floats(const hm_matrix *A) {
     const int64_t n = A->tree->n, K = std::max<int64_t>(A->total_rank, 1), P = std::max<int64_t>(A->n_partials, 1);
-    return 56 * n + 32 * P + 56 * K + (2 * n + 3) / 4 * 4 + (2 * K + 3) / 4 * 4 + fx::MR +
-           32 * A->fx_nslots * ((A->tree->max_leaf + 15) / 16 * 16) + 32 * n;
+    return 64 * n + 32 * P + 64 * K + (2 * n + 3) / 4 * 4 + (2 * K + 3) / 4 * 4 + fx::MR +
+           2 * fx::todo_ints(A->tree->n_leaf) +
+           34 * A->fx_nslots * ((A->tree->max_leaf + 15) / 16 * 16) + 32 * n;
 }
 
 // Y (Morton [n][16] FP64) = H_64 x for the nr <= 16 vectors x_r = x[r * n +
@@ -841,18 +1172,24 @@ void matvec_df_block(const hm_matrix *A, const double *x, int nr, const int32_t 
     Work w;
     float *p = work;
     w.Xd = reinterpret_cast<__half *>(p);
-    p += 56 * n;
+    p += fx::DIG / 2 * n;
     w.P = reinterpret_cast<float2 *>(p);
     p += 32 * P;
     w.Td = reinterpret_cast<__half *>(p);
-    p += 56 * K;
+    p += fx::DIG / 2 * K;
     w.Xe = reinterpret_cast<uint2 *>(p);
     p += (2 * n + 3) / 4 * 4;
     w.Te = reinterpret_cast<uint2 *>(p);
     p += (2 * K + 3) / 4 * 4;
     w.sc = reinterpret_cast<unsigned int *>(p);
     p += MR;
+    w.todo_c = reinterpret_cast<int32_t *>(p);
+    p += todo_ints(A->tree->n_leaf);
+    w.todo_r = reinterpret_cast<int32_t *>(p);
+    p += todo_ints(A->tree->n_leaf);
     w.Ypart = reinterpret_cast<float2 *>(p);
+    p += 2 * MR * A->fx_nslots * ((A->tree->max_leaf + 15) / 16 * 16);
+    w.part_state = reinterpret_cast<uint2 *>(p);
     // at most 8 right-hand sides need one fragment column of the products, not two
     if (nr <= 8) block_product<1>(A, x, nr, perm, Y, w, s);
     else block_product<2>(A, x, nr, perm, Y, w, s);
