@@ -1,5 +1,6 @@
 // prims.cu -- errors, device buffers, quadrature constants, scan, radix sort,
 // TMA descriptors.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
@@ -162,7 +163,9 @@ constexpr size_t SMALL_CAP = size_t(64) << 20;  // bytes of them in the cache
 static std::mutex g_cache_mu;
 static std::multimap<std::pair<int, size_t>, void *> g_cache;  // (device, size) -> block
 static size_t g_cache_bytes = 0, g_small_bytes = 0;
+static std::vector<AllocScope *> g_scopes;  // open scopes of all threads; their lists are behind g_cache_mu too
 static thread_local AllocScope *tl_scope = nullptr;
+static bool sync_device(int dev);
 
 static size_t cache_cap() {
     static size_t cap = 0;
@@ -174,16 +177,28 @@ static size_t cache_cap() {
 }
 
 void cache_trim() {
-    std::lock_guard<std::mutex> lk(g_cache_mu);
+    std::multimap<std::pair<int, size_t>, void *> out;
+    std::vector<int> wait;  // devices whose work may still use a scope's blocks
+    {
+        std::lock_guard<std::mutex> lk(g_cache_mu);
+        out.swap(g_cache);
+        g_cache_bytes = g_small_bytes = 0;
+        for (AllocScope *sc : g_scopes) {
+            if (sc->blocks.empty()) continue;
+            for (auto &b : sc->blocks) out.insert({{sc->dev, b.first}, b.second});
+            wait.push_back(sc->dev);
+            sc->blocks.clear();
+            sc->held = 0;
+        }
+    }
+    for (int dev : wait) sync_device(dev);
     int cur = 0;
     cudaGetDevice(&cur);
-    for (auto &kv : g_cache) {
+    for (auto &kv : out) {
         cudaSetDevice(kv.first.first);
         cudaFree(kv.second);
     }
     cudaSetDevice(cur);
-    g_cache.clear();
-    g_cache_bytes = g_small_bytes = 0;
 }
 
 // a block that no queued work uses: into the cache, or freed
@@ -248,19 +263,19 @@ void DBuf::alloc(size_t nbytes) {
         while (want < nbytes) want *= 2;
         most = want;
     }
-    if (tl_scope && tl_scope->dev == dev) {
-        auto it = tl_scope->blocks.lower_bound(want);
-        if (it != tl_scope->blocks.end() && it->first <= most) {
-            p = it->second;
-            blk = it->first;
-            bytes = nbytes;
-            tl_scope->held -= blk;
-            tl_scope->blocks.erase(it);
-            return;
-        }
-    }
     {
         std::lock_guard<std::mutex> lk(g_cache_mu);
+        if (tl_scope && tl_scope->dev == dev) {
+            auto it = tl_scope->blocks.lower_bound(want);
+            if (it != tl_scope->blocks.end() && it->first <= most) {
+                p = it->second;
+                blk = it->first;
+                bytes = nbytes;
+                tl_scope->held -= blk;
+                tl_scope->blocks.erase(it);
+                return;
+            }
+        }
         auto it = g_cache.lower_bound({dev, want});
         if (it != g_cache.end() && it->first.first == dev && it->first.second <= most) {
             p = it->second;
@@ -275,7 +290,6 @@ void DBuf::alloc(size_t nbytes) {
     cudaError_t e = cudaMalloc(&p, want);
     if (e == cudaErrorMemoryAllocation) {
         (void)cudaGetLastError();
-        if (tl_scope) tl_scope->flush();
         cache_trim();
         e = cudaMalloc(&p, want);
     }
@@ -304,13 +318,18 @@ static bool sync_device(int dev) {
 
 void DBuf::release() {
     if (p) {
-        if (tl_scope && tl_scope->dev == dev && tl_scope->held + blk <= tl_scope->cap) {
-            tl_scope->blocks.insert({blk, p});
-            tl_scope->held += blk;
-        } else if (sync_device(dev)) {
-            cache_put(dev, blk, p);
-        } else {
-            cudaFree(p);
+        bool kept = false;
+        if (tl_scope && tl_scope->dev == dev) {
+            std::lock_guard<std::mutex> lk(g_cache_mu);
+            kept = tl_scope->held + blk <= tl_scope->cap;
+            if (kept) {
+                tl_scope->blocks.insert({blk, p});
+                tl_scope->held += blk;
+            }
+        }
+        if (!kept) {
+            if (sync_device(dev)) cache_put(dev, blk, p);
+            else cudaFree(p);
         }
     }
     p = nullptr;
@@ -320,24 +339,26 @@ void DBuf::release() {
 AllocScope::AllocScope(size_t cap_) : cap(cap_), outer(tl_scope == nullptr) {
     if (!outer) return;
     if (cudaGetDevice(&dev) != cudaSuccess) (void)cudaGetLastError();
+    std::lock_guard<std::mutex> lk(g_cache_mu);
+    g_scopes.push_back(this);
     tl_scope = this;
-}
-
-void AllocScope::flush() {
-    const bool idle = blocks.empty() || sync_device(dev);
-    // the largest first: where not all fit, the ones that are freed are smaller and sooner mapped again
-    for (auto b = blocks.rbegin(); b != blocks.rend(); ++b) {
-        if (idle) cache_put(dev, b->first, b->second);
-        else cudaFree(b->second);
-    }
-    blocks.clear();
-    held = 0;
 }
 
 AllocScope::~AllocScope() {
     if (!outer) return;
-    flush();
     tl_scope = nullptr;
+    std::multimap<size_t, void *> out;
+    {
+        std::lock_guard<std::mutex> lk(g_cache_mu);
+        g_scopes.erase(std::find(g_scopes.begin(), g_scopes.end(), this));
+        out.swap(blocks);
+    }
+    const bool idle = out.empty() || sync_device(dev);
+    // the largest first: where not all fit, the ones that are freed are smaller and sooner mapped again
+    for (auto b = out.rbegin(); b != out.rend(); ++b) {
+        if (idle) cache_put(dev, b->first, b->second);
+        else cudaFree(b->second);
+    }
 }
 
 int num_sms() {
