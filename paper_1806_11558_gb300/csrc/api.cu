@@ -76,6 +76,22 @@ template <class F> static hm_status guard(F &&f) {
 static bool is_tree(const void *p) { return p && static_cast<const hm_tree *>(p)->magic == HM_TREE_MAGIC; }
 static bool is_matrix(const void *p) { return p && static_cast<const hm_matrix *>(p)->magic == HM_MATRIX_MAGIC; }
 
+using Clock = std::chrono::steady_clock;
+static double seconds_since(Clock::time_point t0) { return std::chrono::duration<double>(Clock::now() - t0).count(); }
+
+// build_tree_impl with the time of the whole call, the return of its temporary buffers included
+static hm_tree *build_timed(const double *d_V, int64_t nv, const int32_t *d_T, int64_t n, const hm_tree_params &prm,
+                            const std::vector<int64_t> &goff, cudaStream_t s) {
+    const auto t0 = Clock::now();
+    hm_tree *t;
+    {
+        AllocScope scope;
+        t = build_tree_impl(d_V, nv, d_T, n, prm, goff, s);
+    }
+    t->seconds = seconds_since(t0);
+    return t;
+}
+
 static void check_matvec_args(const hm_matrix *A, int32_t trans, int32_t nrhs, hm_dtype prec, const double *d_x,
                               const double *d_y) {
     if (!is_matrix(A)) fail(HM_EINVAL, "not a matrix handle");
@@ -117,8 +133,7 @@ hm_status hm_build_tree(const double *d_vertices, int64_t n_vertices, const int3
         if (n_vertices < 3 || n_vertices > (1LL << 30)) fail(HM_EINVAL, "n_vertices must be in [3, 2^30]");
         if (!(params->eta >= 0.0) || !std::isfinite(params->eta)) fail(HM_EINVAL, "eta must be finite and >= 0");
         if (params->leaf_size < 1 || params->leaf_size > 254) fail(HM_EINVAL, "leaf_size must be in [1, 254]");
-        AllocScope scope;
-        *out = build_tree_impl(d_vertices, n_vertices, d_tris, n_tris, *params, {}, (cudaStream_t)stream);
+        *out = build_timed(d_vertices, n_vertices, d_tris, n_tris, *params, {}, (cudaStream_t)stream);
     });
 }
 
@@ -137,8 +152,7 @@ hm_status hm_build_forest(const double *d_vertices, int64_t n_vertices, const in
         if (goff[0] != 0 || goff[n_geom] != n_tris) fail(HM_EINVAL, "tri_offsets must start at 0 and end at n_tris");
         for (int g = 0; g < n_geom; ++g)
             if (goff[g + 1] <= goff[g]) fail(HM_EINVAL, "geometry %d has no triangle", g);
-        AllocScope scope;
-        *out = build_tree_impl(d_vertices, n_vertices, d_tris, n_tris, *params, goff, (cudaStream_t)stream);
+        *out = build_timed(d_vertices, n_vertices, d_tris, n_tris, *params, goff, (cudaStream_t)stream);
     });
 }
 
@@ -167,29 +181,31 @@ hm_status hm_assemble(const hm_tree *tree, const hm_assemble_params *params, hm_
         if (params->factor_tail_bits != 0 && (params->factor_tail_bits < 8 || params->factor_tail_bits > 24))
             fail(HM_EINVAL, "factor_tail_bits must be 0 or in [8, 24]");
         cudaStream_t s = (cudaStream_t)stream;
-        const auto t0 = std::chrono::steady_clock::now();
-        AllocScope scope;
+        const auto t0 = Clock::now();
         std::unique_ptr<hm_matrix> A(new hm_matrix());
         A->tree = tree;
         A->params = *params;
-        const QuadParams qp = make_quad(params->ss_order);
-        DBuf err;
-        err.alloc(sizeof(int));
-        HM_CUDA_CHECK(cudaMemsetAsync(err.p, 0, sizeof(int), s));
         double sr = 0, ss = 0, sa = 0;
-        assemble_nearfield(tree, A.get(), qp, s, err.as<int>(), &sr, &ss, params->nearfield_fp64 != 0);
         {
-            DBuf uw, uw_off;
-            assemble_aca(tree, A.get(), qp, s, &sa, uw, uw_off);
-            build_lr_panels(A.get(), uw, uw_off, s);
-            if (params->factor_tail_bits > 0) split_terms(A.get(), uw, uw_off, s);
+            AllocScope scope;
+            const QuadParams qp = make_quad(params->ss_order);
+            DBuf err;
+            err.alloc(sizeof(int));
+            HM_CUDA_CHECK(cudaMemsetAsync(err.p, 0, sizeof(int), s));
+            assemble_nearfield(tree, A.get(), qp, s, err.as<int>(), &sr, &ss, params->nearfield_fp64 != 0);
+            {
+                DBuf uw, uw_off;
+                assemble_aca(tree, A.get(), qp, s, &sa, uw, uw_off);
+                build_lr_panels(A.get(), uw, uw_off, s);
+                if (params->factor_tail_bits > 0) split_terms(A.get(), uw, uw_off, s);
+                HM_CUDA_CHECK(cudaStreamSynchronize(s));
+            }
+            make_low_copies(A.get(), s);
             HM_CUDA_CHECK(cudaStreamSynchronize(s));
+            const int e = read_scalar(err.as<int>(), s);
+            if (e == 2) fail(HM_ETIMEOUT, "a panel staging wait timed out");
+            if (e) fail(HM_EINTERNAL, "device error code %d during assembly", e);
         }
-        make_low_copies(A.get(), s);
-        HM_CUDA_CHECK(cudaStreamSynchronize(s));
-        const int e = read_scalar(err.as<int>(), s);
-        if (e == 2) fail(HM_ETIMEOUT, "a panel staging wait timed out");
-        if (e) fail(HM_EINTERNAL, "device error code %d during assembly", e);
         hm_matrix_info &I = A->info;  // mean / max rank, kmax hits and ACA entries are set by the ACA
         I.dense_entries = tree->dense_true;
         I.lr_entries = A->lr_entries;
@@ -199,7 +215,7 @@ hm_status hm_assemble(const hm_tree *tree, const hm_assemble_params *params, hm_
         I.bytes_f64 = (int64_t)(A->dense.bytes + A->up.bytes + A->wp.bytes);
         I.bytes_low = (int64_t)(A->dense32.bytes + A->up32.bytes + A->upbf.bytes + A->wp32.bytes + A->wpbf.bytes +
                                 A->ut32.data.bytes + A->ut16.data.bytes);
-        I.s_total = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
+        I.s_total = seconds_since(t0);
         *out = A.release();
     });
 }

@@ -7,7 +7,6 @@
 // with explicitly rounded operations (__dadd_rn etc.), so no FMA contraction
 // can change a decision.
 #include <algorithm>
-#include <chrono>
 #include <cmath>
 #include <memory>
 #include <numeric>
@@ -447,7 +446,6 @@ hm_tree *build_tree_impl(const double *d_V, int64_t nv, const int32_t *d_T, int6
     // geometries: triangle ranges [goff[g], goff[g + 1]) of the input (one geometry by default)
     std::vector<int64_t> goff = goff_in.empty() ? std::vector<int64_t>{0, n} : goff_in;
     const int G = (int)goff.size() - 1;
-    auto t0 = std::chrono::steady_clock::now();
     std::unique_ptr<hm_tree> tr(new hm_tree());
     tr->n = n;
     tr->nv = nv;
@@ -817,7 +815,6 @@ hm_tree *build_tree_impl(const double *d_V, int64_t nv, const int32_t *d_T, int6
     else
         tr->box_cols_f = 0;
     HM_CUDA_CHECK(cudaStreamSynchronize(s));
-    tr->seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     return tr.release();
 }
 
