@@ -209,27 +209,16 @@ __device__ __noinline__ void norm_terms(const T *Uf, const T *Wf, int m, int n, 
     }
 }
 
-// sum_l ur_l wr_l over the r cross terms, lanes over l, in double-float
-// arithmetic (2^-44 of the largest term); the same value on every lane
+// sum_l ur_l wr_l over the r cross terms in FP64 (the products are exact), lanes
+// over l; the same value on every lane.  In pairs of floats the ACA of 200,000 panels
+// took 94.4 ms instead of 94.5.
 __device__ __forceinline__ double cross_terms(const float *res, int r) {
-    float h = 0.0f, lo = 0.0f;
+    double a = 0.0;
 #pragma unroll 1
-    for (int l = threadIdx.x & 31; l < r; l += 32) {
-        float p, e, s, f;
-        two_prod(res[2 + l], res[2 + r + l], p, e);
-        two_sum(h, p, s, f);
-        h = s;
-        lo = __fadd_rn(lo, __fadd_rn(e, f));
-    }
+    for (int l = threadIdx.x & 31; l < r; l += 32) a += (double)res[2 + l] * (double)res[2 + r + l];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float p = __shfl_xor_sync(0xffffffffu, h, o), e = __shfl_xor_sync(0xffffffffu, lo, o);
-        float s, f;
-        two_sum(h, p, s, f);
-        h = s;
-        lo = __fadd_rn(__fadd_rn(lo, e), f);
-    }
-    return (double)h + (double)lo;
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a;
 }
 
 template <bool CTA, int NT>
