@@ -357,11 +357,13 @@ HM_API hm_status hm_matvec(const hm_matrix *A, int32_t trans, int32_t nrhs, hm_d
  *  into eight digits base 256 whose products are summed without rounding
  *  (Ozaki, Ogita, Oishi and Rump): a few 1e-15 of the row sums of |H||x| — the
  *  FP64 residuals of the batched refinement (hm_solve_params.resid_df).  Leaf
- *  clusters where a right-hand side is far smaller than others of its 16 (by 2^7
- *  in x or by 2^9 in the terms of a row) are formed in pairs of floats with
- *  compensated sums, ~1e-14 of its own |H||x|, at up to four times the time.  Sums
- *  are carried in the range of FP32, each x_r scaled by its largest entry: terms
- *  below 2^-149 of that count as zero, a sum beyond 2^128 is NaN.
+ *  clusters where a right-hand side is far smaller than others of its 16 (some
+ *  2^7 in x, 2^12 in the terms of a row) are formed in pairs of floats with
+ *  compensated sums, ~1e-14 of its own |H||x|, at up to four times the time; the
+ *  last bits of a result can depend on the right-hand sides beside it.  Sums are
+ *  carried in the range of FP32, each x_r scaled by its mean exponent (or so that
+ *  its largest entry is 2^30): what is below 2^-149 of that counts as zero, a sum
+ *  beyond 2^128 is NaN.
  * Stream-ordered (working vectors from the stream-ordered pool; HM_F64 uses
  * 392 bytes per panel, 128 per partial projection, 264 per unit of total rank and,
  * for leaf clusters whose panels are split over several work items, 136 per row and

@@ -11,7 +11,7 @@
 // transformations of matrix multiplication by using fast routines of matrix
 // multiplication and its applications", Numer. Algorithms 2012):
 //   * column k of a panel has the exponent e_k of its largest x_r (each x_r
-//     scaled by its own largest entry first) and x_r 2^-e_k becomes an integer
+//     scaled by its own mean exponent first) and x_r 2^-e_k becomes an integer
 //     of 62 bits and sign, eight balanced digits d in [-128, 127], as FP16;
 //   * a term w 2^e_k of a row becomes an integer of 62 bits or less and sign on
 //     the scale of the row's largest term so far, in integer operations on the
@@ -27,18 +27,18 @@
 // Eight digits leave 15 bits for a right-hand side that is smaller there than
 // others and has still what a pair of floats keeps (48 bits of an entry and of an x);
 // each sum keeps a record of the right-hand sides that had a term of their own
-// of that size (X_OWN, ROW_OWN), and the clusters where one had none are formed
+// of that size (NEAR_X and after), and the clusters where one had none are formed
 // again in pairs of floats, where no right-hand side sees another.  Seven digits
-// and no record were 11% to 22% faster (64,980 panels 1.73 ms a pass) and lost a unit
+// and no record were 12% to 19% faster (64,980 panels 1.73 ms a pass) and lost a unit
 // vector's entries 10^7 below another's to 2e-9.
 // Against the exact product (16 right-hand sides, 1,280 and 2,880 panels) the
 // error is 2e-16 of |H||x| in norm for random, 2.3e-15 for positive x and 1.7e-15
 // for unit vectors; float pairs throughout have 2e-15, 1.1e-14 and 2.2e-15.
 // Time of a pass with 16 right-hand sides, float pairs -> this (HBM alone), ms:
-// 5,120 panels 0.415 -> 0.186, 64,980 panels, leaves of 64 rows, 4.59 -> 1.92 (0.48; row
-// pass 1.12, column pass 0.56), 327,680 panels, leaves of 80, 26.8 -> 15.4 (3.4; row 9.3,
-// column 5.1).  Vectors whose sizes differ by 1e10 between the halves of the sphere,
-// so that most clusters are formed again: 0.50, 7.0 and 35 ms.
+// 5,120 panels 0.415 -> 0.189, 64,980 panels, leaves of 64 rows, 4.59 -> 1.94 (0.48; row
+// pass 1.14, column pass 0.57), 327,680 panels, leaves of 80, 26.8 -> 15.6 (3.4; row 9.4,
+// column 5.2).  Vectors whose sizes differ by 1e10 between the halves of the sphere,
+// so that most clusters are formed again: 0.43, 6.1 and 34 ms.
 // Non-finite x or entries give NaN in the rows they reach.
 //
 //   scale_x / digits_x    : the scale of each x_r, the digits of x
@@ -71,14 +71,16 @@ constexpr int E_ZERO = -900;        // exponent of a column of zeros, and the sm
 constexpr int E_BIAS = 1000;        // added to the exponents of columns, which makes them positive
 constexpr int F_EXP = 884;          // a row's factor 2^(E - 1011) as a float: exponent field E - 884
 constexpr int E_NAN = F_EXP + 255;  // biased term exponents from here on: not finite, or beyond FP32
-// A sum is taken as it is where one of its terms has an x_r within 2^X_OWN of the
-// column's largest and an entry within 2^ROW_OWN (COL_OWN) of the row's scale, or in a
-// row within RAISE_OWN more by later terms that raised the scale: the 2^-61.5 of the
-// scale that a term may be off is then 2^-46.5 of that term or less, which is what
-// pairs of floats make of a product.  Within a row the scale is mostly raised by
-// the diagonal, or late in U by 2; without RAISE_OWN one row in some 10,000 of random
-// vectors was unsure.
-constexpr int X_OWN = 6, ROW_OWN = 5, RAISE_OWN = 3, COL_OWN = 8;
+// A sum is taken as it is where one of its terms has an x_r within 2^NEAR_X of the
+// column's largest and an entry within 2^NEAR_W of the row's scale, or within 2^FAR_X
+// and 2^FAR_W (a column of a panel: RAISED more), or in a row within RAISED more by later
+// terms that raised the scale: the 2^-61.5 of the scale that a term may be off is then
+// 2^-46.5 of that term or less, which is what pairs of floats make of a product.  The
+// first kind finds right-hand sides beside another's peak, whose own terms are
+// elsewhere and of full size; the second finds those that are smooth and small in a
+// whole cluster.  Within a row the scale is mostly raised by the diagonal, or late in U
+// by 2; without RAISED one row cluster in some 1,000 of random vectors was unsure.
+constexpr int NEAR_X = 2, NEAR_W = 9, FAR_X = 6, FAR_W = 5, RAISED = 3;
 
 // (s, c) += (s2, c2)
 __device__ __forceinline__ void dadd(float &s, float &c, float s2, float c2) {
@@ -116,21 +118,45 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], u
 // ---------------------------------------------------------------------------
 // digits of the vectors
 // ---------------------------------------------------------------------------
-// sc[r] = the largest high word of |x_r| (finite entries)
-__global__ void __launch_bounds__(256) scale_x_kernel(const double *__restrict__ x, int64_t n,
-                                                      unsigned int *__restrict__ sc) {
+// What the scale of an x_r is taken from: its largest exponent, the sum and the
+// number of the exponents of its entries (finite and not zero; the exponent of x is e
+// where 2^(e-1) <= |x| < 2^e).  All zero at the start.
+struct Scale {
+    long long sum;
+    unsigned int count;
+    unsigned int top;  // largest e + 1100
+};
+
+__global__ void __launch_bounds__(256) scale_x_kernel(const double *__restrict__ x, int64_t n, Scale *__restrict__ sc) {
     const double *xr = x + (int64_t)blockIdx.y * n;
-    unsigned int m = 0;
+    int sum = 0, count = 0;  // 256 CTAs: less than 2^20 entries a thread
+    unsigned int top = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const unsigned int h = (unsigned int)__double2hiint(xr[i]) & 0x7fffffffu;
-        if (h < 0x7ff00000u) m = max(m, h);
+        const int eb = (__double2hiint(xr[i]) >> 20) & 0x7ff;
+        if (eb != 0 && eb != 0x7ff) {
+            sum += eb - 1022;
+            ++count;
+            top = max(top, (unsigned int)(eb - 1022 + 1100));
+        }
     }
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(sc + blockIdx.y, m);
+    top = __reduce_max_sync(0xffffffffu, top);
+    count = __reduce_add_sync(0xffffffffu, count);
+    const int lo = __reduce_add_sync(0xffffffffu, sum & 0xffff), hi = __reduce_add_sync(0xffffffffu, sum >> 16);
+    if ((threadIdx.x & 31) == 0 && count) {
+        Scale *o = sc + blockIdx.y;
+        atomicMax(&o->top, top);
+        atomicAdd(&o->count, (unsigned int)count);
+        atomicAdd(reinterpret_cast<unsigned long long *>(&o->sum), (unsigned long long)((long long)hi * 65536 + lo));
+    }
 }
 
-// |x_r| < 2^scale
-__device__ __forceinline__ int scale_of(unsigned int sc) { return sc >= 0x100000u ? (int)(sc >> 20) - 1022 : 0; }
+// x_r is scaled by 2^-scale: its mean exponent, so that right-hand sides of like size have
+// like digits where one of them has a peak (by the largest entry instead, a
+// peak of 4,096 in 40 of 655,220 panels made all clusters unsure), but no peak above 2^30
+__device__ __forceinline__ int scale_of(const Scale &sc) {
+    if (sc.count == 0) return 0;
+    return max((int)(sc.sum / (long long)sc.count), (int)sc.top - 1100 - 30);
+}
 
 // the eight digits of q, |q| <= 2^62, as halves at o[0], o[MR], ... (top first)
 constexpr unsigned long long DIGIT_BIAS = 0x8080808080808080ull;
@@ -143,11 +169,11 @@ __device__ __forceinline__ void store_digits(long long q, __half *o) {
 // Xd[m] = the digits of x_r 2^-(scale_r + e), Xe[m] = ((e + E_BIAS) 2^20, state of
 // the x_r), for position m (x is [nr][n], original order when perm is given);
 // zeros for r >= nr.  16 lanes per position.  State: bit r and bit r + 16 of x_r are
-// 00 zero, 01 (the upper) small beside the column's largest, 11 within 2^X_OWN of
-// it, 10 not finite.
+// 00 zero, 01 (the upper) small beside the column's largest, 11 within 2^NEAR_X of
+// it, 10 not finite; and bit r of the exponent's word: within 2^FAR_X or not finite.
 __global__ void __launch_bounds__(256) digits_x_kernel(const double *__restrict__ x, int64_t n, int nr,
                                                        const int32_t *__restrict__ perm,
-                                                       const unsigned int *__restrict__ sc, __half *__restrict__ Xd,
+                                                       const Scale *__restrict__ sc, __half *__restrict__ Xd,
                                                        uint2 *__restrict__ Xe) {
     const int r = threadIdx.x & 15;
     const int S = r < nr ? scale_of(sc[r]) : 0;
@@ -165,7 +191,8 @@ __global__ void __launch_bounds__(256) digits_x_kernel(const double *__restrict_
         // the mantissa (53 bits) on the column's scale, rounded to nearest
         long long q = 0;
         const int sh = e - ex;
-        const unsigned int lo = __ballot_sync(0xffffffffu, bad || (eb != 0 && sh <= X_OWN));
+        const unsigned int lo = __ballot_sync(0xffffffffu, bad || (eb != 0 && sh <= NEAR_X));
+        const unsigned int lf = __ballot_sync(0xffffffffu, bad || (eb != 0 && sh <= FAR_X));
         const unsigned int up = __ballot_sync(0xffffffffu, !bad && eb != 0);
         if (eb != 0 && !bad && sh < 63) {
             const unsigned long long mant = (b & 0xfffffffffffffull) | 0x10000000000000ull;
@@ -175,7 +202,7 @@ __global__ void __launch_bounds__(256) digits_x_kernel(const double *__restrict_
         if (m < n) {
             store_digits(q, Xd + m * DIG + r);
             if (r == 0)
-                Xe[m] = make_uint2((uint32_t)(e + E_BIAS) << 20,
+                Xe[m] = make_uint2((uint32_t)(e + E_BIAS) << 20 | (lf >> (threadIdx.x & 16) & 0xffffu),
                                    (lo >> (threadIdx.x & 16) & 0xffffu) | (up >> (threadIdx.x & 16)) << 16);
         }
     }
@@ -192,7 +219,8 @@ __global__ void __launch_bounds__(256) digits_x_kernel(const double *__restrict_
 constexpr uint32_t HEADROOM = 1u << 20;
 constexpr uint32_t E20_START = (uint32_t)(E_BIAS + 320) << 20;
 
-// exponent (biased by 1023 + E_BIAS, times 2^20, plus some fraction bits) of the term w 2^e
+// exponent (biased by 1023 + E_BIAS, times 2^20, plus some fraction bits) of the term w 2^e;
+// the states in the lower bits of e20 may make it one more, no less
 __device__ __forceinline__ uint32_t term_exp(double w, uint32_t e20) {
     return ((uint32_t)__double2hiint(w) & 0x7fffffffu) + e20;
 }
@@ -203,7 +231,8 @@ __device__ __forceinline__ uint32_t raise_exp(uint32_t tm, uint32_t E20) {
 }
 
 // w 2^(e - E) as 63-bit fixed point plus 2^63: bytes 7..0 are the digits (the
-// top one plus 128); returns E minus the term's exponent
+// top one plus 128); returns E minus the term's exponent.  E20: with its lower 20
+// bits set, over what is in those of e20.
 __device__ __forceinline__ uint32_t fixed_point(double w, uint32_t E20, uint32_t e20, uint32_t &lo, uint32_t &hi) {
     const int h = __double2hiint(w);
     const uint32_t s = min((E20 - e20 - ((uint32_t)h & 0x7ff00000u)) >> 20, 63u);
@@ -218,13 +247,17 @@ __device__ __forceinline__ uint32_t fixed_point(double w, uint32_t E20, uint32_t
 // the eight digits of two entries of consecutive k (a's column with e20 = e.x and
 // state e.y, b's with e.z and e.w), packed for an A fragment (lower k in the
 // low half): o[i][reg], top digit first, as FP16 subnormals.  own: the states
-// of the columns whose term is within 2^OWN of the row's scale.
-template <int OWN>
+// of the columns whose term is near enough to the row's scale for them (MORE: bits
+// beyond NEAR_W and FAR_W).  E20 as in fixed_point.
+template <int MORE>
 __device__ __forceinline__ void digit_pair(double a, double b, uint32_t E20, const uint4 &e, uint32_t (&o)[NA][4], int reg,
                                            uint32_t &own) {
     uint32_t al, ah, bl, bh;
-    if (fixed_point(a, E20, e.x, al, ah) <= OWN) own |= e.y;
-    if (fixed_point(b, E20, e.z, bl, bh) <= OWN) own |= e.w;
+    const uint32_t sa = fixed_point(a, E20, e.x, al, ah), sb = fixed_point(b, E20, e.z, bl, bh);
+    if (sa <= NEAR_W + MORE) own |= e.y;
+    if (sa <= FAR_W + MORE) own |= e.x;
+    if (sb <= NEAR_W + MORE) own |= e.w;
+    if (sb <= FAR_W + MORE) own |= e.z;
     const uint32_t t = __byte_perm(ah, bh, 0x7632);  // a6 a7 b6 b7
     const uint32_t u = __byte_perm(ah, bh, 0x5410);  // a4 a5 b4 b5
     const uint32_t p = __byte_perm(al, bl, 0x7632);  // a2 a3 b2 b3
@@ -327,10 +360,10 @@ __device__ __forceinline__ uint32_t unsure(uint32_t E20, uint32_t all, uint32_t 
 }
 
 // E = the new scale; own is kept while the raises (of this row in the bits from sh
-// on of raised) come to RAISE_OWN at most
+// on of raised) come to RAISED at most
 __device__ __forceinline__ void raise_own(uint32_t &E, uint32_t to, uint32_t &own, uint32_t &raised, int sh) {
     uint32_t sum = (raised >> sh & 0xffffu) + ((to - E) >> 20);
-    if (sum > RAISE_OWN) own = sum = 0;
+    if (sum > RAISED) own = sum = 0;
     raised = (raised & ~(0xffffu << sh)) | sum << sh;
     E = to;
 }
@@ -457,8 +490,8 @@ __global__ void __launch_bounds__(32 * CW, 4) col_fx_kernel(int parts, const int
                 for (int hf = 0; hf < 2; ++hf) {
                     const uint4 e = *reinterpret_cast<const uint4 *>(se + k0 + kk + 8 * hf + 2 * t);
                     const double2 x = w[kk / 4 + 2 * hf], y = w[kk / 4 + 2 * hf + 1];
-                    digit_pair<COL_OWN>(x.x, y.x, E0, e, a, 2 * hf, own0);
-                    digit_pair<COL_OWN>(x.y, y.y, E1, e, a, 2 * hf + 1, own1);
+                    digit_pair<RAISED>(x.x, y.x, E0 | 0xfffffu, e, a, 2 * hf, own0);
+                    digit_pair<RAISED>(x.y, y.y, E1 | 0xfffffu, e, a, 2 * hf + 1, own1);
                 }
                 mma_orders<NT>(acc, a, xs + (k0 + kk) * XSTRIDE);
             }
@@ -572,14 +605,16 @@ __global__ void __launch_bounds__(256) tsum_fx_kernel(int64_t na, int64_t nt, co
             if (hb >= 0x7f800000u) bad |= 1u << r;
             else if (hb) ex = max(ex, max((int)(hb >> 23), 1) - 126);  // |s| < 2^ex, subnormal s too
         }
-        unsigned int state = bad;
+        unsigned int state = bad, far = bad;
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
             const uint32_t hb = __float_as_uint(s[r]) & 0x7fffffffu;
             if (hb == 0u || hb >= 0x7f800000u) continue;
-            state |= (max((int)(hb >> 23), 1) - 126 + X_OWN >= ex ? 0x10001u : 0x10000u) << r;
+            const int below = ex - (max((int)(hb >> 23), 1) - 126);
+            state |= (below <= NEAR_X ? 0x10001u : 0x10000u) << r;
+            far |= (below <= FAR_X ? 1u : 0u) << r;
         }
-        Te[e] = make_uint2((uint32_t)(ex + E_BIAS) << 20, state);
+        Te[e] = make_uint2((uint32_t)(ex + E_BIAS) << 20 | far, state);
         unsigned long long u[NR];
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
@@ -615,7 +650,7 @@ __global__ void __launch_bounds__(256) tsum_fx_kernel(int64_t na, int64_t nt, co
 // of the gathered rows of x or t.  A warp takes the largest term of each of its
 // rows in the chunk, forms the digits of its entries (each entry by one lane)
 // and multiplies.  Per 16 x 16 entries: 72 products of 16 x 8 x 16 (~160 cycles of an
-// SM), ~26 integer operations per entry (~95 cycles of the ALU pipe), 2 KB from
+// SM), ~28 integer operations per entry (~100 cycles of the ALU pipe), 2 KB from
 // HBM (~95 cycles).
 // ---------------------------------------------------------------------------
 constexpr int AST = KC * 8;               // bytes per staged panel row; odd rows have their 64-byte halves swapped (banks)
@@ -634,7 +669,7 @@ __global__ void __launch_bounds__(32 * MT, RowCfg<MT>::CTAS) row_fx_kernel(
     const double *__restrict__ dense, const int64_t *__restrict__ up_off, const int32_t *__restrict__ up_K,
     const int64_t *__restrict__ up_colptr, const int32_t *__restrict__ tidx, const double *__restrict__ up,
     const __half *__restrict__ Xd, const uint2 *__restrict__ Xe, const __half *__restrict__ Td,
-    const uint2 *__restrict__ Te, const unsigned int *__restrict__ sc, double *__restrict__ Y,
+    const uint2 *__restrict__ Te, const Scale *__restrict__ sc, double *__restrict__ Y,
     const int4 *__restrict__ items, float2 *__restrict__ Ypart, uint2 *__restrict__ part_state, int prow,
     int64_t nl, int32_t *__restrict__ todo) {
     using C = RowCfg<MT>;
@@ -752,8 +787,8 @@ __global__ void __launch_bounds__(32 * MT, RowCfg<MT>::CTAS) row_fx_kernel(
                 const double2 w0 = *reinterpret_cast<const double2 *>(a0 + ((k + 8 * hf) ^ flip));
                 const double2 w1 = *reinterpret_cast<const double2 *>(a1 + ((k + 8 * hf) ^ flip));
                 const uint4 e = *reinterpret_cast<const uint4 *>(se + k + 8 * hf);
-                digit_pair<ROW_OWN>(w0.x, w0.y, E0, e, a, 2 * hf, own0);
-                digit_pair<ROW_OWN>(w1.x, w1.y, E1, e, a, 2 * hf + 1, own1);
+                digit_pair<0>(w0.x, w0.y, E0 | 0xfffffu, e, a, 2 * hf, own0);
+                digit_pair<0>(w1.x, w1.y, E1 | 0xfffffu, e, a, 2 * hf + 1, own1);
             }
             mma_orders<NT>(acc, a, sb + k * XSTRIDE);
         }
@@ -797,12 +832,12 @@ __global__ void __launch_bounds__(32 * MT, RowCfg<MT>::CTAS) row_fx_kernel(
 
 // rows of the clusters whose panels were split: Y = the sum of the partials
 // in slot order (red: cluster, first slot, slots).  A part's own terms speak for the
-// row where its scale is within RAISE_OWN of the row's, raises included.
+// row where its scale is within RAISED of the row's, raises included.
 template <int NT>
 __global__ void __launch_bounds__(256) row_reduce_kernel(const int4 *__restrict__ red, const int32_t *__restrict__ leaf_begin,
                                                          const float2 *__restrict__ Ypart, int prow,
                                                          const uint2 *__restrict__ part_state,
-                                                         const unsigned int *__restrict__ sc, double *__restrict__ Y,
+                                                         const Scale *__restrict__ sc, double *__restrict__ Y,
                                                          int64_t nl, int32_t *__restrict__ todo) {
     const int4 rd = red[blockIdx.x];
     const int32_t r0 = leaf_begin[rd.x], mr = leaf_begin[rd.x + 1] - r0;
@@ -823,7 +858,7 @@ __global__ void __launch_bounds__(256) row_reduce_kernel(const int4 *__restrict_
         for (int k = 0; k < rd.z; ++k) {
             const uint2 v = p[(int64_t)k * prow];
             all |= v.y;
-            if ((E >> 20) - (v.x >> 20) + (v.x & 0xffffu) <= RAISE_OWN) own |= v.y;
+            if ((E >> 20) - (v.x >> 20) + (v.x & 0xffffu) <= RAISED) own |= v.y;
         }
         if (unsure(E, all, own)) note_cluster(todo, nl, rd.x);
     }
@@ -835,9 +870,9 @@ __global__ void __launch_bounds__(256) row_reduce_kernel(const int4 *__restrict_
 // 2^-47 |w|, and each term is added with an error-free product and sum (the
 // compensated dot product of Ogita, Rump and Oishi, "Accurate sum and dot product",
 // SIAM J. Sci. Comput. 2005, Algorithm 5.3), so no right-hand side sees another.
-// Few or no clusters as a rule (of random vectors a few column clusters of 1,000 and a
-// row cluster of some 10,000): the lists (todo: length, clusters, marks) are walked by a
-// fixed number of CTAs, which end at once where they are empty (3 us a kernel).  Bound
+// Few or no clusters as a rule (none of random or smooth vectors of like size): the
+// lists (todo: length, clusters, marks) are walked by a fixed number of CTAs, which
+// end at once where they are empty (3 us a kernel).  Bound
 // by the FP32 pipe where all clusters are listed, by latency where few are.
 // ---------------------------------------------------------------------------
 constexpr int PAIR_CTAS = 8;  // per SM
@@ -887,7 +922,7 @@ __device__ __forceinline__ void pair_step(double w, const float4 *z, float (&s)[
 
 // x_r at position m on its own scale, as a pair
 __device__ __forceinline__ void x_pair(const double *__restrict__ x, int64_t n, int nr, const int32_t *__restrict__ perm,
-                                       const unsigned int *__restrict__ sc, int64_t m, int r, float &h, float &l) {
+                                       const Scale *__restrict__ sc, int64_t m, int r, float &h, float &l) {
     const double v = r < nr ? scalbn(x[(int64_t)r * n + (perm ? perm[m] : m)], -scale_of(sc[r])) : 0.0;
     h = __double2float_rn(v);
     l = __double2float_rn(v - (double)h);
@@ -900,7 +935,7 @@ __global__ void __launch_bounds__(CP_THREADS) col_pairs_kernel(
     int parts, const int32_t *__restrict__ todo, const int32_t *__restrict__ leaf_begin,
     const int64_t *__restrict__ wp_off, const int32_t *__restrict__ wp_K, const int64_t *__restrict__ wp_colptr,
     const double *__restrict__ wp, const double *__restrict__ x, int64_t n, int nr, const int32_t *__restrict__ perm,
-    const unsigned int *__restrict__ sc, float2 *__restrict__ P) {
+    const Scale *__restrict__ sc, float2 *__restrict__ P) {
     __shared__ float4 sx[MAX_LEAF * MR / 2];
     float *sf = reinterpret_cast<float *>(sx);
     const int64_t count = (int64_t)todo[0] * parts;
@@ -929,82 +964,166 @@ __global__ void __launch_bounds__(CP_THREADS) col_pairs_kernel(
     }
 }
 
-// where a row cluster is listed: x and t as pairs ([row][hi 16, lo 16]), in the place of their digits
+// where a row cluster is listed: x and t as pairs ([row][hi 16, lo 16]), in the place of their digits.
+// Few listed clusters: only the rows that they read, a warp per entry of t with its lanes over the
+// partials (a block of the top levels has thousands, and one lane's chain of them is what the whole
+// sum takes: 1,310,720 panels 2.7 ms).  Else all rows, as tsum_fx_kernel forms them.
+constexpr int FEW = 64;  // listed clusters of one in so many
 template <int NT>
-__global__ void __launch_bounds__(256) pairs_kernel(const int32_t *__restrict__ todo, int64_t na, int64_t nt,
-                                                    const int32_t *__restrict__ b0tab, const int64_t *__restrict__ t_off,
-                                                    const int64_t *__restrict__ bcolptr, const int64_t *__restrict__ pofs,
-                                                    const float2 *__restrict__ P, const double *__restrict__ x, int64_t n,
-                                                    int nr, const int32_t *__restrict__ perm,
-                                                    const unsigned int *__restrict__ sc, float *__restrict__ Xp,
-                                                    float *__restrict__ Tp) {
-    if (todo[0] == 0) return;
+__global__ void __launch_bounds__(256) pairs_kernel(
+    const int32_t *__restrict__ todo, int64_t nl, int64_t na, int64_t nt, const int32_t *__restrict__ b0tab,
+    const int64_t *__restrict__ t_off, const int64_t *__restrict__ bcolptr, const int64_t *__restrict__ pofs,
+    const float2 *__restrict__ P, const int32_t *__restrict__ rho_K, const int64_t *__restrict__ rho_colptr,
+    const int32_t *__restrict__ colidx, const int32_t *__restrict__ up_K, const int64_t *__restrict__ up_colptr,
+    const int32_t *__restrict__ tidx, const double *__restrict__ x, int64_t n, int nr, const int32_t *__restrict__ perm,
+    const Scale *__restrict__ sc, float *__restrict__ Xp, float *__restrict__ Tp) {
+    const int count = todo[0];
+    if (count == 0) return;
     const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nth = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t e = t0; e < n * MR; e += nth)
-        x_pair(x, n, nr, perm, sc, e / MR, (int)(e % MR), Xp[e / MR * 2 * MR + e % MR], Xp[e / MR * 2 * MR + MR + e % MR]);
-    for (int64_t ch = t0 >> 5; ch < (nt + 31) / 32; ch += nth >> 5) {
-        const int64_t e = ch * 32 + (threadIdx.x & 31);
-        const int64_t b = block_of(ch, e, na, b0tab, t_off);
-        if (e >= nt) continue;
-        float s[8 * NT], c[8 * NT];
-        sum_partials<NT>(b, e - t_off[b], bcolptr, pofs, P, s, c);
-        float4 *o = reinterpret_cast<float4 *>(Tp + e * 2 * MR);
+    const int lane = threadIdx.x & 31;
+    auto x_row = [&](int64_t m, int r) { x_pair(x, n, nr, perm, sc, m, r, Xp[m * 2 * MR + r], Xp[m * 2 * MR + MR + r]); };
+    if ((int64_t)count * FEW > nl) {
+        for (int64_t e = t0; e < n * MR; e += nth) x_row(e / MR, (int)(e % MR));
+        for (int64_t ch = t0 >> 5; ch < (nt + 31) / 32; ch += nth >> 5) {
+            const int64_t e = ch * 32 + lane;
+            const int64_t b = block_of(ch, e, na, b0tab, t_off);
+            if (e >= nt) continue;
+            float s[8 * NT], c[8 * NT];
+            sum_partials<NT>(b, e - t_off[b], bcolptr, pofs, P, s, c);
+            float4 *o = reinterpret_cast<float4 *>(Tp + e * 2 * MR);
 #pragma unroll
-        for (int k = 0; k < 2 * NT; ++k) {
-            o[k] = make_float4(s[4 * k], s[4 * k + 1], s[4 * k + 2], s[4 * k + 3]);
-            o[MR / 4 + k] = make_float4(c[4 * k], c[4 * k + 1], c[4 * k + 2], c[4 * k + 3]);
+            for (int k = 0; k < 2 * NT; ++k) {
+                o[k] = make_float4(s[4 * k], s[4 * k + 1], s[4 * k + 2], s[4 * k + 3]);
+                o[MR / 4 + k] = make_float4(c[4 * k], c[4 * k + 1], c[4 * k + 2], c[4 * k + 3]);
+            }
+        }
+        return;
+    }
+    for (int i = 0; i < count; ++i) {
+        const int64_t rho = todo[1 + i];
+        const int32_t *ci = colidx + rho_colptr[rho], *ti = tidx + up_colptr[rho];
+        for (int64_t e = t0; e < (int64_t)rho_K[rho] * MR; e += nth) x_row(ci[e / MR], (int)(e % MR));
+        for (int64_t v = t0 >> 5; v < up_K[rho]; v += nth >> 5) {
+            const int64_t e = ti[v];
+            // the block of e: from the one that holds entry 32 (e / 32) to the one that holds the next such entry
+            int64_t b = b0tab[e / 32], hi = (e / 32 + 1) * 32 < nt ? b0tab[e / 32 + 1] + 1 : na;
+            while (hi - b > 1) {
+                const int64_t mid = (b + hi) >> 1;
+                if (t_off[mid] <= e) b = mid;
+                else hi = mid;
+            }
+            const int64_t l = e - t_off[b];
+            float s[8 * NT], c[8 * NT];
+#pragma unroll
+            for (int r = 0; r < 8 * NT; ++r) s[r] = c[r] = 0.0f;
+            for (int64_t q = bcolptr[b] + lane; q < bcolptr[b + 1]; q += 32) {
+                const float4 *pp = reinterpret_cast<const float4 *>(P + (pofs[q] + l) * MR);
+#pragma unroll
+                for (int k = 0; k < 4 * NT; ++k) {
+                    const float4 w = __ldg(pp + k);
+                    dadd(s[2 * k], c[2 * k], w.x, w.y);
+                    dadd(s[2 * k + 1], c[2 * k + 1], w.z, w.w);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < 8 * NT; ++r) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const float s2 = __shfl_xor_sync(0xffffffffu, s[r], o), c2 = __shfl_xor_sync(0xffffffffu, c[r], o);
+                    dadd(s[r], c[r], s2, c2);
+                }
+                if (lane == r) norm2(s[r], c[r], Tp[e * 2 * MR + r], Tp[e * 2 * MR + MR + r]);
+            }
         }
     }
 }
 
-// the rows of the listed row clusters, eight per CTA and one per warp; the gathered
-// pairs of 64 columns at a time in shared memory
-constexpr int RP_ROWS = 8, RP_COLS = 64, RP_STRIDE = MR / 2 + 1;  // float4 per column: eight lanes hit different banks
+// the rows of the listed row clusters, sixteen per CTA and two per warp (a column's pairs, read from
+// shared memory once, serve both); the gathered pairs of 64 columns at a time in shared memory, the next
+// 64 and their entries on the way meanwhile
+constexpr int RP_WARPS = 8, RP_ROWS = 2 * RP_WARPS, RP_COLS = 64;
+constexpr int RP_STRIDE = MR / 2 + 1;  // float4 per column: eight lanes hit different banks
 template <int NT>
-__global__ void __launch_bounds__(32 * RP_ROWS) row_pairs_kernel(
+__global__ void __launch_bounds__(32 * RP_WARPS, 2) row_pairs_kernel(
     int parts, const int32_t *__restrict__ todo, const int32_t *__restrict__ leaf_begin,
     const int64_t *__restrict__ rho_off, const int32_t *__restrict__ rho_K, const int64_t *__restrict__ rho_colptr,
     const int32_t *__restrict__ colidx, const double *__restrict__ dense, const int64_t *__restrict__ up_off,
     const int32_t *__restrict__ up_K, const int64_t *__restrict__ up_colptr, const int32_t *__restrict__ tidx,
     const double *__restrict__ up, const float4 *__restrict__ Xp, const float4 *__restrict__ Tp,
-    const unsigned int *__restrict__ sc, double *__restrict__ Y) {
+    const Scale *__restrict__ sc, double *__restrict__ Y) {
+    constexpr int PIECES = RP_COLS * MR / 2 / (32 * RP_WARPS);  // float4 of a chunk per thread
     __shared__ float4 sz[RP_COLS * RP_STRIDE];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t count = (int64_t)todo[0] * parts;
     for (int64_t q = blockIdx.x; q < count; q += gridDim.x) {
         const int64_t rho = todo[1 + q / parts];
         const int32_t r0 = leaf_begin[rho], mr = leaf_begin[rho + 1] - r0;
-        const int row = (int)(q % parts) * RP_ROWS + warp;
-        if (row - warp >= mr) continue;
-        float s[8 * NT], c[8 * NT];
+        const int row = (int)(q % parts) * RP_ROWS + 2 * warp;
+        if (row - 2 * warp >= mr) continue;
+        float s[2][8 * NT], c[2][8 * NT];
 #pragma unroll
-        for (int r = 0; r < 8 * NT; ++r) s[r] = c[r] = 0.0f;
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int r = 0; r < 8 * NT; ++r) s[i][r] = c[i][r] = 0.0f;
 #pragma unroll 1
         for (int u = 0; u < 2; ++u) {  // the near field, then the U panel
             const int K = u ? up_K[rho] : rho_K[rho];
             const int32_t *idx = u ? tidx + up_colptr[rho] : colidx + rho_colptr[rho];
-            const double *p = (u ? up + up_off[rho] : dense + rho_off[rho]) + (int64_t)min(row, mr - 1) * K;
+            const double *p0 = (u ? up + up_off[rho] : dense + rho_off[rho]);
+            const double *p[2] = {p0 + (int64_t)min(row, mr - 1) * K, p0 + (int64_t)min(row + 1, mr - 1) * K};
             const float4 *z = u ? Tp : Xp;
+            float4 zn[PIECES];
+            double wn[2][RP_COLS / 32];
+            auto fetch = [&](int k0) {
+#pragma unroll
+                for (int i = 0; i < PIECES; ++i) {
+                    const int e = threadIdx.x + 32 * RP_WARPS * i, k = k0 + e / (MR / 2);
+                    if (k < K) zn[i] = __ldg(z + (int64_t)idx[k] * (MR / 2) + e % (MR / 2));
+                }
+#pragma unroll
+                for (int h = 0; h < RP_COLS / 32; ++h)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const int k = k0 + 32 * h + lane;
+                        wn[i][h] = k < K ? __ldg(p[i] + k) : 0.0;
+                    }
+            };
+            fetch(0);
+#pragma unroll 1
             for (int k0 = 0; k0 < K; k0 += RP_COLS) {
-                const int kc = min(RP_COLS, K - k0);
+                __syncthreads();  // the last chunk has been read
+                double w[2][RP_COLS / 32];
+#pragma unroll
+                for (int i = 0; i < PIECES; ++i) {
+                    const int e = threadIdx.x + 32 * RP_WARPS * i;
+                    sz[e / (MR / 2) * RP_STRIDE + e % (MR / 2)] = zn[i];
+                }
+#pragma unroll
+                for (int h = 0; h < RP_COLS / 32; ++h)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) w[i][h] = wn[i][h];
                 __syncthreads();
-                for (int e = threadIdx.x; e < kc * MR / 2; e += 32 * RP_ROWS)
-                    sz[e / (MR / 2) * RP_STRIDE + e % (MR / 2)] =
-                        __ldg(z + (int64_t)idx[k0 + e / (MR / 2)] * (MR / 2) + e % (MR / 2));
-                __syncthreads();
-                for (int k = lane; k < kc; k += 32) pair_step<NT>(__ldg(p + k0 + k), sz + k * RP_STRIDE, s, c);
+                if (k0 + RP_COLS < K) fetch(k0 + RP_COLS);
+#pragma unroll
+                for (int h = 0; h < RP_COLS / 32; ++h) {
+                    if (k0 + 32 * h + lane >= K) continue;
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) pair_step<NT>(w[i][h], sz + (32 * h + lane) * RP_STRIDE, s[i], c[i]);
+                }
             }
         }
 #pragma unroll
-        for (int r = 0; r < 8 * NT; ++r) {
+        for (int i = 0; i < 2; ++i)
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float s2 = __shfl_xor_sync(0xffffffffu, s[r], o), c2 = __shfl_xor_sync(0xffffffffu, c[r], o);
-                dadd(s[r], c[r], s2, c2);
+            for (int r = 0; r < 8 * NT; ++r) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const float s2 = __shfl_xor_sync(0xffffffffu, s[i][r], o), c2 = __shfl_xor_sync(0xffffffffu, c[i][r], o);
+                    dadd(s[i][r], c[i][r], s2, c2);
+                }
+                if (lane == r && row + i < mr)
+                    Y[(int64_t)(r0 + row + i) * MR + r] = scalbn((double)s[i][r] + (double)c[i][r], scale_of(sc[r]));
             }
-            if (lane == r && row < mr)
-                Y[(int64_t)(r0 + row) * MR + r] = scalbn((double)s[r] + (double)c[r], scale_of(sc[r]));
-        }
     }
 }
 
@@ -1031,9 +1150,10 @@ struct Work {
     __half *Xd, *Td;
     float2 *P, *Ypart;
     uint2 *Xe, *Te, *part_state;
-    unsigned int *sc;
+    Scale *sc;
     int32_t *todo_c, *todo_r;  // column and row clusters to be formed again: length, clusters [nl], marks [nl]
 };
+constexpr int SCALE_FLOATS = MR * (int)(sizeof(Scale) / sizeof(float));
 static int64_t todo_ints(int64_t nl) { return (1 + 2 * nl + 3) / 4 * 4; }
 
 template <int NT>
@@ -1042,7 +1162,7 @@ static void block_product(const hm_matrix *A, const double *x, int nr, const int
     const hm_tree *tr = A->tree;
     const int64_t n = tr->n, nl = tr->n_leaf;
     // (the lists follow the scales)
-    HM_CUDA_CHECK(cudaMemsetAsync(w.sc, 0, sizeof(unsigned int) * MR + sizeof(int32_t) * 2 * todo_ints(nl), s));
+    HM_CUDA_CHECK(cudaMemsetAsync(w.sc, 0, sizeof(Scale) * MR + sizeof(int32_t) * 2 * todo_ints(nl), s));
     const unsigned pair_grid = (unsigned)(PAIR_CTAS * num_sms());
     const dim3 gs((unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, 256)), (unsigned)nr);
     scale_x_kernel<<<gs, 256, 0, s>>>(x, n, w.sc);
@@ -1100,12 +1220,13 @@ static void block_product(const hm_matrix *A, const double *x, int nr, const int
     }
     float *Xp = reinterpret_cast<float *>(w.Xd), *Tp = reinterpret_cast<float *>(w.Td);
     static_assert(DIG * sizeof(__half) >= 2 * MR * sizeof(float), "pairs in the place of digits");
-    pairs_kernel<NT><<<pair_grid, 256, 0, s>>>(w.todo_r, tr->n_adm, tr->n_adm > 0 ? A->total_rank : 0,
-                                               A->tsum_b0.as<int32_t>(), A->t_off.as<int64_t>(),
-                                               tr->lr_bcolptr.as<int64_t>(), A->pofs.as<int64_t>(), w.P, x, n, nr, perm,
-                                               w.sc, Xp, Tp);
+    pairs_kernel<NT><<<pair_grid, 256, 0, s>>>(
+        w.todo_r, nl, tr->n_adm, tr->n_adm > 0 ? A->total_rank : 0, A->tsum_b0.as<int32_t>(), A->t_off.as<int64_t>(),
+        tr->lr_bcolptr.as<int64_t>(), A->pofs.as<int64_t>(), w.P, tr->rho_K.as<int32_t>(), tr->rho_colptr.as<int64_t>(),
+        tr->colidx.as<int32_t>(), A->up_K.as<int32_t>(), A->up_colptr.as<int64_t>(), A->tidx.as<int32_t>(), x, n, nr,
+        perm, w.sc, Xp, Tp);
     HM_LAUNCH_CHECK();
-    row_pairs_kernel<NT><<<pair_grid, 32 * RP_ROWS, 0, s>>>(
+    row_pairs_kernel<NT><<<pair_grid, 32 * RP_WARPS, 0, s>>>(
         (tr->max_leaf + RP_ROWS - 1) / RP_ROWS, w.todo_r, tr->leaf_begin.as<int32_t>(), tr->rho_off.as<int64_t>(),
         tr->rho_K.as<int32_t>(), tr->rho_colptr.as<int64_t>(), tr->colidx.as<int32_t>(), A->dense.as<double>(),
         A->up_off.as<int64_t>(), A->up_K.as<int32_t>(), A->up_colptr.as<int64_t>(), A->tidx.as<int32_t>(),
@@ -1120,8 +1241,10 @@ static void block_product(const hm_matrix *A, const double *x, int nr, const int
 // the Morton order tears apart has a near field ten times the mean width, and
 // one CTA walking it would be the pass (21,780 panels: mean 93 chunks, widest
 // 336): an item gets at most half of what an SM's share of CTAs would do one
-// after the other, 24 to 256 chunks.  Items by decreasing work; K: host copies
-// of the panel widths.
+// after the other, 24 to 256 chunks.  A pass with 16 right-hand sides, ms: 21,780
+// panels 0.687 (the whole share 0.769, a quarter 0.698); 5,120 panels 0.183 (at least 12
+// chunks 0.179, 48 0.222); 259,920 panels, leaves of 128, 10.52 (at most 128 10.51, 512
+// 10.57).  Items by decreasing work; K: host copies of the panel widths.
 void build_fx_items(hm_matrix *A, const std::vector<int32_t> &begin, const std::vector<int32_t> &kd,
                     const std::vector<int32_t> &ku, cudaStream_t s) {
     const int64_t nl = (int64_t)kd.size();
@@ -1152,12 +1275,12 @@ void build_fx_items(hm_matrix *A, const std::vector<int32_t> &begin, const std::
 
 // floats of the working arrays of one 16-right-hand-side pass: digits of x
 // and t (64 each per row), partials of t (32 each), exponents of x and t (2
-// each, a multiple of 4 in all), scales (16) and the two lists of clusters,
+// each, a multiple of 4 in all), scales (64) and the two lists of clusters,
 // partials and states of split rows (32 and 2 per row of a slot, a multiple of 16
 // rows), Y (16 doubles per row)
 int64_t df_work_floats(const hm_matrix *A) {
     const int64_t n = A->tree->n, K = std::max<int64_t>(A->total_rank, 1), P = std::max<int64_t>(A->n_partials, 1);
-    return 64 * n + 32 * P + 64 * K + (2 * n + 3) / 4 * 4 + (2 * K + 3) / 4 * 4 + fx::MR +
+    return 64 * n + 32 * P + 64 * K + (2 * n + 3) / 4 * 4 + (2 * K + 3) / 4 * 4 + fx::SCALE_FLOATS +
            2 * fx::todo_ints(A->tree->n_leaf) +
            34 * A->fx_nslots * ((A->tree->max_leaf + 15) / 16 * 16) + 32 * n;
 }
@@ -1181,8 +1304,8 @@ void matvec_df_block(const hm_matrix *A, const double *x, int nr, const int32_t 
     p += (2 * n + 3) / 4 * 4;
     w.Te = reinterpret_cast<uint2 *>(p);
     p += (2 * K + 3) / 4 * 4;
-    w.sc = reinterpret_cast<unsigned int *>(p);
-    p += MR;
+    w.sc = reinterpret_cast<Scale *>(p);
+    p += SCALE_FLOATS;
     w.todo_c = reinterpret_cast<int32_t *>(p);
     p += todo_ints(A->tree->n_leaf);
     w.todo_r = reinterpret_cast<int32_t *>(p);

@@ -62,6 +62,22 @@ def test_unit_vectors_on_a_graded_mesh(orc, nrhs, leaf):
         g.close()
 
 
+# peaks on 20 of 5,120 panels in all right-hand sides but one: 256 leaves a few of the 256 clusters' rows unsure (only what they
+# read is formed again), 16,384 all of them
+@pytest.mark.parametrize("nrhs,peak", [(16, 2 ** 8), (7, 2 ** 8), (16, 2 ** 14)])
+def test_peaks_beside_a_vector_without(orc, nrhs, peak):
+    need_gpu()
+    V, T = meshgen.icosphere(4)
+    g = GpuH(V, T, leaf=20, eta=1.5, eps=1e-6)
+    try:
+        at = np.argsort(-(V[T].mean(1) @ np.array([0.3, 0.5, 0.8])))[:20]
+        X = np.random.default_rng(9).standard_normal((nrhs, g.n))
+        X[1:, at] *= peak
+        _check(orc, g, X)
+    finally:
+        g.close()
+
+
 def test_sizes_that_cross_within_one_cluster(orc):
     need_gpu()  # 80 panels, no far field
     V, T = meshgen.icosphere(1)
