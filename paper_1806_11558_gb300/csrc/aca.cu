@@ -351,8 +351,8 @@ struct FacDouble {
 // instruction cache.  A warp's last round of an odd length (cnt of 32 entries)
 // is spread over the idle lanes, 2, 4 or 8 lanes per entry: rows of 40 entries
 // take 9 outer points' time instead of 14.  Before -> now, ms (eps 1e-6): 5,120
-// panels 2.49 -> 2.10, 21,780 panels 7.76 -> 6.06, 200,000 panels 114.6 -> 93.3,
-// 655,220 panels (leaves of 80) 381 -> 334; the schedulers issue 77% of the time,
+// panels 1.92 -> 1.20, 21,780 panels 7.83 -> 6.18, 200,000 panels 115.8 -> 94.5,
+// 655,220 panels (leaves of 80) 385 -> 337; the schedulers issue 76% of the time,
 // and at 96 registers wait for results of the unrolled chains the rest.
 template <bool CTA, int NT, class F>
 __device__ int aca_block(const AcaArgs &A, int rb, int m, int cb, int n, const F &fac, const AcaShared &sh,

@@ -277,7 +277,7 @@ hm_status hm_matvec_block(const hm_matrix *A, int32_t nrhs, hm_dtype prec, const
         if (!d_x || !d_y) fail(HM_EINVAL, "NULL argument");
         if (nrhs < 1) fail(HM_EINVAL, "nrhs must be >= 1");
         if (prec != HM_F64 && prec != HM_F32 && prec != HM_BF16) fail(HM_EINVAL, "unknown precision %d", (int)prec);
-        if (prec == HM_F64) {  // the FP64 master in double-float arithmetic (mrhs_df.cu)
+        if (prec == HM_F64) {  // the FP64 master by exact digit products (mrhs_df.cu)
             matvec_df(A, nrhs, d_x, d_y, alpha, beta, (cudaStream_t)stream);
             return;
         }
