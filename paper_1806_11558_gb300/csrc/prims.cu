@@ -161,6 +161,9 @@ void fail(hm_status s, const char *fmt, ...) {
 constexpr size_t CACHE_MIN = size_t(1) << 20;   // smaller blocks are rounded up
 constexpr size_t SMALL_CAP = size_t(64) << 20;  // bytes of them in the cache
 static std::mutex g_cache_mu;
+// held while blocks taken from the lists are given back to the driver, so that another
+// thread whose allocation failed meanwhile waits for them (taken before g_cache_mu)
+static std::mutex g_trim_mu;
 static std::multimap<std::pair<int, size_t>, void *> g_cache;  // (device, size) -> block
 static size_t g_cache_bytes = 0, g_small_bytes = 0;
 static std::vector<AllocScope *> g_scopes;  // open scopes of all threads; their lists are behind g_cache_mu too
@@ -179,6 +182,7 @@ static size_t cache_cap() {
 void cache_trim() {
     std::multimap<std::pair<int, size_t>, void *> out;
     std::vector<int> wait;  // devices whose work may still use a scope's blocks
+    std::lock_guard<std::mutex> trim(g_trim_mu);
     {
         std::lock_guard<std::mutex> lk(g_cache_mu);
         out.swap(g_cache);
@@ -201,17 +205,21 @@ void cache_trim() {
     cudaSetDevice(cur);
 }
 
-// a block that no queued work uses: into the cache, or freed
+// a block that no queued work uses into the cache, where it fits (g_cache_mu is held)
+static bool cache_keep(int dev, size_t blk, void *p) {
+    const bool small = blk < CACHE_MIN;
+    if (g_cache_bytes + blk > cache_cap() || (small && g_small_bytes + blk > SMALL_CAP)) return false;
+    g_cache.insert({{dev, blk}, p});
+    g_cache_bytes += blk;
+    if (small) g_small_bytes += blk;
+    return true;
+}
+
+// the same, or freed
 static void cache_put(int dev, size_t blk, void *p) {
     {
         std::lock_guard<std::mutex> lk(g_cache_mu);
-        const bool small = blk < CACHE_MIN;
-        if (g_cache_bytes + blk <= cache_cap() && (!small || g_small_bytes + blk <= SMALL_CAP)) {
-            g_cache.insert({{dev, blk}, p});
-            g_cache_bytes += blk;
-            if (small) g_small_bytes += blk;
-            return;
-        }
+        if (cache_keep(dev, blk, p)) return;
     }
     cudaFree(p);
 }
@@ -347,18 +355,24 @@ AllocScope::AllocScope(size_t cap_) : cap(cap_), outer(tl_scope == nullptr) {
 AllocScope::~AllocScope() {
     if (!outer) return;
     tl_scope = nullptr;
-    std::multimap<size_t, void *> out;
+    // the list is there for other threads' failed allocations until it has gone to the cache
+    bool idle = true;
+    {
+        std::lock_guard<std::mutex> lk(g_cache_mu);
+        idle = blocks.empty();
+    }
+    idle = idle || sync_device(dev);
+    std::vector<void *> rest;
+    std::lock_guard<std::mutex> trim(g_trim_mu);
     {
         std::lock_guard<std::mutex> lk(g_cache_mu);
         g_scopes.erase(std::find(g_scopes.begin(), g_scopes.end(), this));
-        out.swap(blocks);
+        // the largest first: where not all fit, the ones that are freed are smaller and sooner mapped again
+        for (auto b = blocks.rbegin(); b != blocks.rend(); ++b)
+            if (!idle || !cache_keep(dev, b->first, b->second)) rest.push_back(b->second);
+        blocks.clear();
     }
-    const bool idle = out.empty() || sync_device(dev);
-    // the largest first: where not all fit, the ones that are freed are smaller and sooner mapped again
-    for (auto b = out.rbegin(); b != out.rend(); ++b) {
-        if (idle) cache_put(dev, b->first, b->second);
-        else cudaFree(b->second);
-    }
+    for (void *p : rest) cudaFree(p);
 }
 
 int num_sms() {

@@ -1,7 +1,8 @@
 """The library's allocator against a device of 3 GiB that exists only on the
 host (its runtime calls replaced at link time): memory that a set-up call of one
 thread has released but still holds must be there for another thread's
-allocation, and no block may be freed that queued work could still use."""
+allocation, memory that one thread is giving back for another that fails at the same
+time, and no block may be freed that queued work could still use."""
 import os
 import shutil
 import subprocess
@@ -16,6 +17,7 @@ RUNTIME = r"""
 #include <cstdlib>
 #include <map>
 #include <mutex>
+#include <unistd.h>
 typedef unsigned long size_type;
 std::mutex mu;
 std::map<void *, size_type> live;
@@ -31,6 +33,7 @@ int cudaMalloc(void **p, size_type n) {
     return 0;
 }
 int cudaFree(void *p) {
+    usleep(2000);
     std::lock_guard<std::mutex> lk(mu);
     if (!live.count(p)) { printf("freed twice\n"); exit(3); }
     in_use -= live[p];
@@ -93,6 +96,33 @@ int main() {
     CHECK(ok);
     CHECK(again);
     cache_trim();
+    CHECK(in_use == 0);
+    // two threads that need the cached memory at once
+    for (int k = 0; k < 20; ++k) {
+        DBuf fixed;
+        fixed.alloc(1660 * MiB);
+        {
+            AllocScope scope;
+            DBuf b[7];
+            for (auto &x : b) x.alloc(109 * MiB);
+        }
+        CHECK(in_use == (1660 + 763) * MiB);
+        bool had[2] = {false, false};
+        std::promise<void> done[2];
+        auto ask = [&](int i) {
+            DBuf a;
+            try { a.alloc(700 * MiB); had[i] = true; }
+            catch (...) {}
+            done[i].set_value();
+            done[1 - i].get_future().wait();
+        };
+        std::thread one(ask, 0), two(ask, 1);
+        one.join();
+        two.join();
+        CHECK(had[0] && had[1]);
+        fixed.release();
+        cache_trim();
+    }
     CHECK(in_use == 0);
     // an allocation that cannot be had fails and leaves the scope usable
     {
